@@ -120,36 +120,49 @@ def _draw_activation(g, M, K, heavy):
     return x
 
 
-def prepare(case, seed):
+def _draw_inputs(case, seed):
+    """The numbers of a case: per linear (W, A, B) with A, B None at rank 0, and per linear its fp32 activation (one tensor where
+    a group shares it)."""
     g = torch.Generator(device=DEV)
     g.manual_seed(int(seed))
-    cfg = L.default_config()
-    cfg.w_bits = case["w_bits"]
-    M, rank, heavy, io = case["rows"], case["rank"], case["heavy"], _IO[case["io"]]
+    M, rank, heavy = case["rows"], case["rank"], case["heavy"]
     shapes, groups = _shapes(case)
-    if case["kind"] == "calibrate":
-        K, N = shapes[0]
-        W, X = _draw_weight(g, K, N, heavy), _draw_activation(g, M, K, heavy)
-        omega = torch.randn((N, L.factor_sketch_columns(K, N, rank)), generator=g, device=DEV)
-        return {"kind": "calibrate", "W": W, "samples": [X], "rank": rank, "omega": omega, "cfg": cfg}
-
-    packed, Xs, Ys = [], [None] * len(shapes), []
+    weights, Xs = [], [None] * len(shapes)
     for K, N in shapes:
         W = _draw_weight(g, K, N, heavy)
         A = B = None
-        if rank:                                  # factors of the magnitude that real ones have
+        if rank and case["kind"] != "calibrate":  # factors of the magnitude that real ones have
             A = torch.randn((K, rank), generator=g, device=DEV) / K ** 0.5
             B = torch.randn((rank, N), generator=g, device=DEV) * (0.004 * (K ** 0.5 + N ** 0.5) / N ** 0.5)
-        packed.append(L.prepare_weights(W, A, B, cfg))
-        Ys.append(torch.zeros(L.mxint8_bytes(M, N), dtype=torch.uint8, device=DEV) if io == L.MXINT8
-                  else torch.zeros((M, N), dtype=io, device=DEV))
+        weights.append((W, A, B))
     for group in groups:
         shared = None
         for j in group:
             if shared is None or case["kind"] == "stack":
-                x = _draw_activation(g, M, shapes[j][0], heavy)
-                shared = L.to_mxint8(*L.quantize_activations(x, cfg)) if io == L.MXINT8 else x.to(io)
+                shared = _draw_activation(g, M, shapes[j][0], heavy)
             Xs[j] = shared
+    return g, weights, Xs
+
+
+def prepare(case, seed):
+    cfg = L.default_config()
+    cfg.w_bits = case["w_bits"]
+    M, rank, io = case["rows"], case["rank"], _IO[case["io"]]
+    shapes, groups = _shapes(case)
+    g, weights, drawn = _draw_inputs(case, seed)
+    if case["kind"] == "calibrate":
+        K, N = shapes[0]
+        omega = torch.randn((N, L.factor_sketch_columns(K, N, rank)), generator=g, device=DEV)
+        return {"kind": "calibrate", "W": weights[0][0], "samples": [drawn[0]], "rank": rank, "omega": omega, "cfg": cfg}
+
+    packed, Xs, Ys, made = [], [], [], {}
+    for (K, N), x in zip(shapes, drawn):
+        packed.append(L.prepare_weights(*weights.pop(0), cfg))
+        Ys.append(torch.zeros(L.mxint8_bytes(M, N), dtype=torch.uint8, device=DEV) if io == L.MXINT8
+                  else torch.zeros((M, N), dtype=io, device=DEV))
+        if id(x) not in made:
+            made[id(x)] = L.to_mxint8(*L.quantize_activations(x, cfg)) if io == L.MXINT8 else x.to(io)
+        Xs.append(made[id(x)])
 
     plan, need = [], max(L.workspace_bytes(M, K, N, rank, cfg) for K, N in shapes)
     for group in groups:
@@ -206,3 +219,34 @@ def tolerance(case):
     if case["kind"] == "calibrate":               # fp64 sums throughout; the factors are rounded to fp32 at the end
         return {"rel": 1e-5, "max": 1e-3, "differ": 1e-3}
     return {"f32": {"rel": 1e-6, "max": 2e-5}, "bf16": {"rel": 1e-4, "max": 8e-3}, "mxint8": {"differ": 2e-4}}[case["io"]]
+
+
+def _blocks(v, bits, dim):
+    """MXINT: blocks of 16 along dim share e = floor(log2(max |v|)) in [-56, 55]; the mantissas are round-to-even of
+    v / 2^(e - bits + 2), at most 2^(bits-1) - 1 in magnitude.  -> (mantissas and values as v lies, exponents), in fp64."""
+    b = v.double().movedim(dim, -1).unflatten(-1, (-1, 16))
+    amax = b.abs().amax(-1, keepdim=True)
+    e = torch.where(amax > 0, torch.frexp(amax)[1].double() - 1, -56.0).clamp_(-56, 55)
+    step = torch.exp2(e - (bits - 2))
+    m = torch.round(b / step).clamp_(1 - 2 ** (bits - 1), 2 ** (bits - 1) - 1)
+    return m.flatten(-2).movedim(-1, dim), (m * step).flatten(-2).movedim(-1, dim), e.squeeze(-1)
+
+
+def exact(case, seed):
+    if case["kind"] == "calibrate":               # singular vectors of a nearly flat spectrum: no such values
+        return None
+    _, weights, drawn = _draw_inputs(case, seed)
+    rank, out = case["rank"], []
+    for x in drawn:
+        W, A, B = weights.pop(0)
+        x = _blocks(x.bfloat16() if case["io"] == "bf16" else x, 8, 1)[1]
+        y = x @ _blocks(W, case["w_bits"], 0)[1]
+        if rank:
+            pad = -rank % 16
+            t = torch.nn.functional.pad(x @ _blocks(A, 8, 0)[1], (0, pad))
+            y += _blocks(t, 8, 1)[1] @ _blocks(torch.nn.functional.pad(B, (0, 0, 0, pad)), 8, 0)[1]
+        if case["io"] == "mxint8":
+            m, _, e = _blocks(y, 8, 1)
+            y = torch.cat([m.to(torch.int8).view(torch.uint8).flatten(), (e + 127).to(torch.uint8).flatten()])
+        out.append(y)
+    return out
