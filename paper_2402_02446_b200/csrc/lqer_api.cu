@@ -173,11 +173,21 @@ static size_t small_bytes(const PackedMeta& m, int M) {
   const size_t a = small_slice_bytes(m, M), b = decode_cols_slot_bytes(m);
   return a > b ? a : b;
 }
-// Bytes a call with M rows needs: the persistent head plus the scratch of the path it takes.
+// Scratch of a larger batch's prologue behind its Xcat: partial sums of T (ranks up to 64), or digit planes and sums.
+static size_t prologue_scratch(const PackedMeta& m, int M) {
+  return align_up(prologue_digits_applies(m) ? prologue_digits_scratch_bytes(m, M) : prologue_tc_scratch_bytes(m, M), 256);
+}
+// The least a call with M rows is taken with: the persistent head plus the scratch of the path it takes (ranks above 64 run
+// launch_prologue, which needs none, where the room is too small for the digit planes).
 static size_t call_bytes(const PackedMeta& m, int M, bool small) {
   return align_up(persist_bytes(m), 256) +
          (small ? small_bytes(m, M)
                 : xcat_bytes(m, M) + align_up(prologue_tc_scratch_bytes(m, M), 256) + gemm_splitk_bytes(m, M));
+}
+// What it asks for.
+static size_t call_bytes_wanted(const PackedMeta& m, int M, bool small) {
+  if (small) return call_bytes(m, M, small);
+  return align_up(persist_bytes(m), 256) + xcat_bytes(m, M) + prologue_scratch(m, M) + gemm_splitk_bytes(m, M);
 }
 // Whether a call with M rows takes the small-batch kernels under the current path setting.
 static bool takes_small_path(int path, int M) {
@@ -194,7 +204,8 @@ lqer_status_t call_workspace_bytes(const void* packed, int M, size_t* bytes) {
 }
 // Bytes that fit every call of up to M_max rows, whichever path it takes.
 static size_t workspace_total(const PackedMeta& m, int M_max) {
-  const size_t a = xcat_bytes(m, M_max) + align_up(prologue_tc_scratch_bound(m, M_max), 256) + gemm_splitk_bound(m, M_max);
+  const size_t a = xcat_bytes(m, M_max) + gemm_splitk_bound(m, M_max) +
+                   (prologue_digits_applies(m) ? prologue_scratch(m, M_max) : align_up(prologue_tc_scratch_bound(m, M_max), 256));
   const size_t b = small_bytes(m, M_max < kSmallMaxM ? M_max : kSmallMaxM);
   return align_up(persist_bytes(m), 256) + (a > b ? a : b);
 }
@@ -253,7 +264,10 @@ static lqer_status_t run_linear(const void* X, int M, const void* packed, void* 
   int path = g_path.load();
   if ((path == 2 || path == 5 || path == 7) && M > kSmallMaxM) return LQER_ERR_SHAPE;
   const bool small = takes_small_path(path, M);
-  if (project_only && !small) path = 3;
+  // Paths 1 and 3 keep the mma.sync prologue, as does a workspace without room for the digit planes.
+  const bool digits = !small && path != 1 && path != 3 && prologue_digits_applies(m) &&
+                      (path == 6 || prologue_work(m, M) >= kDigitMinWork) && workspace_bytes >= call_bytes_wanted(m, M, small);
+  if (project_only && !small && !digits) path = 3;
   // Paths 1 and 3 keep the SIMT-style prologue at every batch size; the others take the tensor-core one where it fits.
   const bool tc_prologue = path != 1 && path != 3 && prologue_tc_fits(m, M, X, path == 6);
   if (path == 6) path = 4;
@@ -275,24 +289,25 @@ static lqer_status_t run_linear(const void* X, int M, const void* packed, void* 
     }
   } else {
     if (path == 1 && (M > 65535 || io.y_type != kYF32)) return LQER_ERR_SHAPE;   // the checking kernel writes fp32 only
-    err = tc_prologue ? launch_prologue_tc(X, io.x_type, M, m, packed, xcat, Tm, Te, dst,
-                                           reinterpret_cast<double*>(static_cast<uint8_t*>(xcat) + xcat_bytes(m, M)),
-                                           reinterpret_cast<int*>(wsb + pcount_offset(m)), kChainAlone, s)
-                      : launch_prologue(X, io.x_type, M, m, packed, xcat, Tm, Te, dst, s);
+    GemmActs acts = plain_acts(xcat, m);
+    const DigitCall dc{X, packed, &m};
+    err = digits ? launch_prologue_digits(&dc, 1, M, io.x_type, xcat, &acts, Tm, Te, dst, s)
+          : tc_prologue ? launch_prologue_tc(X, io.x_type, M, m, packed, xcat, Tm, Te, dst,
+                                             reinterpret_cast<double*>(static_cast<uint8_t*>(xcat) + xcat_bytes(m, M)),
+                                             reinterpret_cast<int*>(wsb + pcount_offset(m)), kChainAlone, s)
+                        : launch_prologue(X, io.x_type, M, m, packed, xcat, Tm, Te, dst, s);
+    const size_t behind = xcat_bytes(m, M) + (digits ? prologue_scratch(m, M) : align_up(prologue_tc_scratch_bytes(m, M), 256));
     if (err == cudaSuccess && !project_only)
       err = (path == 1) ? launch_gemm_simt(xcat, M, m, packed, static_cast<float*>(Y), s)
-                        : launch_gemm_tc2_splitk(xcat, M, m, packed, Y, io.y_type,
-                                                 reinterpret_cast<float*>(static_cast<uint8_t*>(xcat) + xcat_bytes(m, M) +
-                                                                          align_up(prologue_tc_scratch_bytes(m, M), 256)),
-                                                 dst, s);
+                        : launch_gemm_tc2_splitk(acts, M, m, packed, Y, io.y_type,
+                                                 reinterpret_cast<float*>(static_cast<uint8_t*>(xcat) + behind), dst, s);
   }
   return err == cudaSuccess ? LQER_OK : LQER_ERR_CUDA;
 }
 
-// Scratch one layer of a grouped prefill launch needs: its own Xcat and its own prologue partial sums.
-static size_t group_slice_bytes(const PackedMeta& m, int M) {
-  return xcat_bytes(m, M) + align_up(prologue_tc_scratch_bytes(m, M), 256);
-}
+// Scratch one layer of a grouped prefill launch needs: its own Xcat and its own prologue scratch (layers of rank above 64
+// that share an X take less together).
+static size_t group_slice_bytes(const PackedMeta& m, int M) { return xcat_bytes(m, M) + prologue_scratch(m, M); }
 // Consecutive prefill calls from `first` on that may share a GEMM launch with it (auto path only): the same M > 256,
 // the same formats, any shapes; at most `limit`, and only as many as the workspace has slices for.
 static bool same_formats(const PackedMeta& a, const PackedMeta& b) {
@@ -427,9 +442,24 @@ static lqer_status_t run_prefill_group(const lqer_call_t* calls, int n, const Pa
   DeviceStatus* dst = static_cast<DeviceStatus*>(workspace);
   size_t head = 0;
   for (int g = 0; g < n; ++g) head = std::max(head, align_up(persist_bytes(metas[g]), 256));
-  const void* xcats[8];
+  GemmActs acts[8];
   const void* packed[8];
   void* Ys[8];
+  bool digits = n > 1;
+  long long work = 0;
+  for (int g = 0; g < n; ++g) {
+    digits = digits && prologue_digits_applies(metas[g]);
+    work += prologue_work(metas[g], M);
+  }
+  if (digits && work >= kDigitMinWork) {
+    DigitCall dc[8];
+    for (int g = 0; g < n; ++g) {
+      dc[g] = DigitCall{calls[g].X, calls[g].packed, &metas[g]};
+      packed[g] = calls[g].packed; Ys[g] = calls[g].Y;
+    }
+    if (launch_prologue_digits(dc, n, M, io.x_type, wsb + head, acts, nullptr, nullptr, dst, s) != cudaSuccess) return LQER_ERR_CUDA;
+    return launch_gemm_tc2_group(acts, packed, Ys, io.y_type, metas, n, M, dst, s) == cudaSuccess ? LQER_OK : LQER_ERR_CUDA;
+  }
   // The prologues of the group share nothing but the status word: each has its slice of the workspace, and, while the
   // counter pairs last, its own range of them, so that each may overlap the tail of the one before.
   size_t count_base = 0;
@@ -438,7 +468,7 @@ static lqer_status_t run_prefill_group(const lqer_call_t* calls, int n, const Pa
   const bool own_counters = (long long)row_tiles * n <= kPrologueRowTiles;
   size_t off = head;
   for (int g = 0; g < n; ++g) {
-    xcats[g] = wsb + off;
+    acts[g] = plain_acts(wsb + off, metas[g]);
     off += group_slice_bytes(metas[g], M);
     packed[g] = calls[g].packed; Ys[g] = calls[g].Y;
   }
@@ -493,7 +523,7 @@ static lqer_status_t run_prefill_group(const lqer_call_t* calls, int n, const Pa
         if (!take) continue;
         Xs[cnt] = calls[g].X;
         pk[cnt] = packed[g];
-        xc[cnt] = const_cast<void*>(xcats[g]);
+        xc[cnt] = acts[g].xcat;
         parts[cnt] = reinterpret_cast<double*>(static_cast<uint8_t*>(xc[cnt]) + xcat_bytes(metas[g], M));
         counts[cnt] = reinterpret_cast<int*>(wsb + count_base) + (size_t)g * row_tiles * 2;
         ms[cnt] = metas[g];
@@ -509,7 +539,7 @@ static lqer_status_t run_prefill_group(const lqer_call_t* calls, int n, const Pa
   } else {
     for (int g = 0; g < n; ++g) {
       const PackedMeta& m = metas[g];
-      uint8_t* xcat = static_cast<uint8_t*>(const_cast<void*>(xcats[g]));
+      uint8_t* xcat = static_cast<uint8_t*>(acts[g].xcat);
       const float* X = calls[g].X;
       int* counters = reinterpret_cast<int*>(wsb + count_base) + (own_counters ? (size_t)g * row_tiles * 2 : 0);
       const int order = !own_counters ? kChainAlone : g == 0 ? kChainFirst : kChainLater;
@@ -520,7 +550,7 @@ static lqer_status_t run_prefill_group(const lqer_call_t* calls, int n, const Pa
       if (err != cudaSuccess) return LQER_ERR_CUDA;
     }
   }
-  return launch_gemm_tc2_group(xcats, packed, Ys, io.y_type, metas, n, M, dst, s) == cudaSuccess ? LQER_OK : LQER_ERR_CUDA;
+  return launch_gemm_tc2_group(acts, packed, Ys, io.y_type, metas, n, M, dst, s) == cudaSuccess ? LQER_OK : LQER_ERR_CUDA;
 }
 
 }  // namespace lqer
@@ -584,7 +614,7 @@ lqer_status_t lqer_call_workspace_bytes(int M, int K, int N, int k, const lqer_c
   if (M <= 0 || M > (1 << 24)) return LQER_ERR_SHAPE;
   PackedMeta m;
   fill_meta(m, K, N, k, *cfg);
-  *bytes = call_bytes(m, M, M <= kSmallMaxM);
+  *bytes = call_bytes_wanted(m, M, M <= kSmallMaxM);
   return LQER_OK;
 }
 

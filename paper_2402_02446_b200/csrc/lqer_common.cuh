@@ -468,20 +468,47 @@ cudaError_t launch_prologue_tc_group(const void* const* Xs, int x_type, int M, c
                                      void* const* xcats, double* const* partials, int* const* counters,
                                      const int* splits, int n, int8_t* Tm, uint8_t* Te, DeviceStatus* st, int order,
                                      cudaStream_t s);
+// What the main GEMM reads of a layer: [X_q | T_q] as bf16 rows of ld values, X_q from column 0, T_q from t_col.
+struct GemmActs {
+  void* xcat;
+  int ld, t_col;
+};
+inline GemmActs plain_acts(void* xcat, const PackedMeta& m) { return GemmActs{xcat, (int)xcat_cols(m), m.K64}; }
+// The prologue with the projection as one integer contraction over all of K on the int8 tensor cores, for ranks above 64:
+// three launches for up to kDigitMaxLayers layers with one M and one set of formats, any shapes; layers with the same X
+// share its quantisation.  `scratch`: at most the sum over the layers of their Xcat bytes and
+// prologue_digits_scratch_bytes (each rounded up to 256); places[g] says where layer g's activations are.
+constexpr int kDigitMaxLayers = 8, kDigitMaxUnits = 8;
+struct DigitCall {
+  const void* X;
+  const void* packed;
+  const PackedMeta* meta;
+};
+// It serves ranks above 64 (below, launch_prologue_tc), from this much work M K k_pad on, summed over the layers of a call:
+// three launches take some 20 us whatever the shape.  Measured, launch_prologue against this, K = 4096: rank 80 at 512 rows
+// 18.9 / 19.5 us, at 768 rows 33.2 / 21.4; rank 256 at 129 rows 25.2 / 25.0, at 512 rows 31.3 / 26.2, at 4096 rows 187 / 68;
+// K = 1024: rank 80 at 1024 rows 17.0 / 19.8, at 2048 rows 23.0 / 20.3; rank 256 at 512 rows 16.5 / 20.7, at 768 rows
+// 26.7 / 22.4; K = 11008: rank 80 at 129 rows 31.3 / 23.3, rank 256 at 4096 rows 464 / 141.
+inline bool prologue_digits_applies(const PackedMeta& m) { return m.k_pad > 64; }
+constexpr long long kDigitMinWork = 150LL * 1000 * 1000;
+inline long long prologue_work(const PackedMeta& m, int M) { return (long long)M * m.K * m.k_pad; }
+size_t prologue_digits_scratch_bytes(const PackedMeta& m, int M);
+cudaError_t launch_prologue_digits(const DigitCall* calls, int n, int M, int x_type, void* scratch, GemmActs* places, int8_t* Tm,
+                                   uint8_t* Te, DeviceStatus* st, cudaStream_t s);
 cudaError_t launch_gemm_simt(const void* xcat, int M, const PackedMeta& m, const void* packed, float* Y,
                              cudaStream_t s);
 // y_type: element type of Y (kYF32, kYBF16, kYMXINT8: mantissas [M,N] then exponent bytes [M,N/16], N % 16 == 0).
 constexpr int kYF32 = 0, kYBF16 = 1, kYMXINT8 = 2;
 inline size_t y_bytes(int y_type, size_t M, size_t N) { return y_type == kYMXINT8 ? M * N + M * N / 16 : M * N * (y_type == kYBF16 ? 2 : 4); }
-cudaError_t launch_gemm_tc2(const void* xcat, int M, const PackedMeta& m, const void* packed, void* Y, int y_type,
+cudaError_t launch_gemm_tc2(const GemmActs& acts, int M, const PackedMeta& m, const void* packed, void* Y, int y_type,
                             DeviceStatus* st, cudaStream_t s);
 // Small batches: the layer's K range cut into gemm_splitk_ranges(m, M) ranges that run as layers of one launch;
 // `partials` holds (ranges - 1) * M * N floats (gemm_splitk_bytes).
-cudaError_t launch_gemm_tc2_splitk(const void* xcat, int M, const PackedMeta& m, const void* packed, void* Y, int y_type,
+cudaError_t launch_gemm_tc2_splitk(const GemmActs& acts, int M, const PackedMeta& m, const void* packed, void* Y, int y_type,
                                    float* partials, DeviceStatus* st, cudaStream_t s);
-// Up to gemm_tc2_max_group() layers with one M in one launch (xcats, packed, Ys, metas: host arrays of n entries).
+// Up to gemm_tc2_max_group() layers with one M in one launch (acts, packed, Ys, metas: host arrays of n entries).
 int gemm_tc2_max_group();
-cudaError_t launch_gemm_tc2_group(const void* const* xcats, const void* const* packed, void* const* Ys, int y_type,
+cudaError_t launch_gemm_tc2_group(const GemmActs* acts, const void* const* packed, void* const* Ys, int y_type,
                                   const PackedMeta* metas, int n, int M, DeviceStatus* st, cudaStream_t s);
 // Factor preparation (Section 3.1 / 3.2, Appendix A): A_k, B_k from W and calibration samples, by randomised subspace
 // iteration with factor_sketch_rank columns; Omega [N, that many] fp32 is the caller's random test matrix.

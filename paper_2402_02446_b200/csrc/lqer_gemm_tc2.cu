@@ -66,7 +66,7 @@ struct Layer {
   void* Y;                     // [M, N] fp32; bf16 or the MXINT8 sections by Params::y_type (never for the K ranges of a split layer)
   size_t y_extent;             // bytes of the buffer behind Y, for the checked build
   size_t w_extent, b_extent;   // bytes of the packed W and B sections
-  int N, K64;
+  int N, t_col;                // columns of Y; first column of T_q in the activation matrix
   int n_tiles, k_slabs, r_blocks;
   int slab0, slab_stride;      // a layer may be a K range of a real layer (split K): its first weight slab, and the
                                // real layer's slab count (the stride between column tiles of the packed weights)
@@ -161,7 +161,7 @@ gemm_tc2_kernel(const __grid_constant__ TensorMaps tmaps, const Params p) {
         const CUtensorMap* tmap_x = &tmaps.m[layer];
         const uint8_t* wsec = p.L[layer].wsec;
         const uint8_t* bsec = p.L[layer].bsec;
-        const int k_slabs = p.L[layer].k_slabs, r_blocks = p.L[layer].r_blocks, K64 = p.L[layer].K64;
+        const int k_slabs = p.L[layer].k_slabs, r_blocks = p.L[layer].r_blocks, t_col = p.L[layer].t_col;
         const int stages_per_tile = p.L[layer].spt, n_tiles = p.L[layer].n_tiles;
         const int slab0 = p.L[layer].slab0, slab_stride = p.L[layer].slab_stride;
         const int b_tile_stride = r_blocks * kTileN * 17;
@@ -184,7 +184,7 @@ gemm_tc2_kernel(const __grid_constant__ TensorMaps tmaps, const Params p) {
             if (has_w && !LQER_IN_BOUNDS(p.status, (size_t)my_ntile * b_tile_stride + (size_t)r_blocks * kTileN * 16 + rb0 * kTileN,
                                          nb * kTileN, p.L[layer].b_extent, 606)) { ok = false; break; }
             mbar_expect_tx(loaded(st), A_TILE_BYTES + (has_w ? nb * (kTileN * 17) : 0));
-            tma_load_2d(a_dst, tmap_x, K64 + rs * RANK_PER_STAGE, row0, loaded(st));
+            tma_load_2d(a_dst, tmap_x, t_col + rs * RANK_PER_STAGE, row0, loaded(st));
             if (has_w) {
               const uint8_t* tile = bsec + (size_t)my_ntile * b_tile_stride;
               bulk_load(a_dst + PK_OFFSET, tile + (size_t)rb0 * kTileN * 16, nb * kTileN * 16, loaded(st));
@@ -443,22 +443,22 @@ __global__ void __launch_bounds__(256) splitk_sum_kernel(float4* __restrict__ Y,
 
 // Small batches have few tiles; their K range is cut into ranges that run as layers of one launch, the first into Y,
 // the others into scratch that a second kernel adds to Y in a fixed order.
-cudaError_t launch_gemm_tc2_splitk(const void* xcat, int M, const PackedMeta& m, const void* packed, void* Yv, int y_type,
+cudaError_t launch_gemm_tc2_splitk(const GemmActs& acts, int M, const PackedMeta& m, const void* packed, void* Yv, int y_type,
                                    float* partials, DeviceStatus* st, cudaStream_t s) {
   using namespace tc2;
   const int C = gemm_splitk_ranges(m, M);
   // only an fp32 Y can collect the ranges' sums: a layer with another output type runs whole
-  if (C < 2 || y_type != kYF32) return launch_gemm_tc2(xcat, M, m, packed, Yv, y_type, st, s);
+  if (C < 2 || y_type != kYF32) return launch_gemm_tc2(acts, M, m, packed, Yv, y_type, st, s);
   float* Y = static_cast<float*>(Yv);
   if ((m.N & 3) != 0) return cudaErrorInvalidValue;
   EncodeTiledFn enc = encode_fn();
   if (enc == nullptr) return cudaErrorNotSupported;
   TensorMaps tmaps;
-  const cuuint64_t dims[2] = {(cuuint64_t)xcat_cols(m), (cuuint64_t)M};
-  const cuuint64_t strides[1] = {(cuuint64_t)xcat_cols(m) * 2};
+  const cuuint64_t dims[2] = {(cuuint64_t)acts.ld, (cuuint64_t)M};
+  const cuuint64_t strides[1] = {(cuuint64_t)acts.ld * 2};
   const cuuint32_t box[2] = {BK, BM};
   const cuuint32_t estr[2] = {1, 1};
-  if (enc(&tmaps.m[0], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(xcat), dims, strides, box, estr,
+  if (enc(&tmaps.m[0], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, acts.xcat, dims, strides, box, estr,
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
@@ -477,7 +477,7 @@ cudaError_t launch_gemm_tc2_splitk(const void* xcat, int M, const PackedMeta& m,
     ly.Y = c == 0 ? Y : partials + (size_t)(c - 1) * M * m.N;
     ly.y_extent = (size_t)M * m.N * 4;
     ly.w_extent = m.off_b - m.off_w; ly.b_extent = m.off_a - m.off_b;
-    ly.N = m.N; ly.K64 = m.K64;
+    ly.N = m.N; ly.t_col = acts.t_col;
     ly.n_tiles = m.n_tiles; ly.k_slabs = hi - lo;
     ly.r_blocks = c == C - 1 ? m.r_blocks : 0;
     ly.slab0 = lo; ly.slab_stride = m.k_slabs;
@@ -502,9 +502,9 @@ cudaError_t launch_gemm_tc2_splitk(const void* xcat, int M, const PackedMeta& m,
   return cudaGetLastError();
 }
 
-cudaError_t launch_gemm_tc2(const void* xcat, int M, const PackedMeta& m, const void* packed, void* Y, int y_type,
+cudaError_t launch_gemm_tc2(const GemmActs& acts, int M, const PackedMeta& m, const void* packed, void* Y, int y_type,
                             DeviceStatus* st, cudaStream_t s) {
-  return launch_gemm_tc2_group(&xcat, &packed, &Y, y_type, &m, 1, M, st, s);
+  return launch_gemm_tc2_group(&acts, &packed, &Y, y_type, &m, 1, M, st, s);
 }
 
 int gemm_tc2_max_group() { return tc2::MAX_GROUP; }
@@ -512,7 +512,7 @@ int gemm_tc2_max_group() { return tc2::MAX_GROUP; }
 // n layers with one M (shapes may differ, formats must not) as ONE launch: the tiles of all layers form one list that
 // the CTA pairs walk, so the pairs idle only at the end of the whole list, and set-up and the last epilogue are paid
 // once.  Layers with more K stages per tile come first in the list.
-cudaError_t launch_gemm_tc2_group(const void* const* xcats, const void* const* packed, void* const* Ys, int y_type,
+cudaError_t launch_gemm_tc2_group(const GemmActs* acts, const void* const* packed, void* const* Ys, int y_type,
                                   const PackedMeta* metas, int n, int M, DeviceStatus* st, cudaStream_t s) {
   using namespace tc2;
   if (n < 1 || n > MAX_GROUP) return cudaErrorInvalidValue;
@@ -533,11 +533,11 @@ cudaError_t launch_gemm_tc2_group(const void* const* xcats, const void* const* p
     const int g = order[slot < n ? slot : 0];
     const PackedMeta& m = metas[g];
     if (m.lr_bits != metas[0].lr_bits || m.w_bits != metas[0].w_bits) return cudaErrorInvalidValue;
-    const cuuint64_t dims[2] = {(cuuint64_t)xcat_cols(m), (cuuint64_t)M};
-    const cuuint64_t strides[1] = {(cuuint64_t)xcat_cols(m) * 2};
+    const cuuint64_t dims[2] = {(cuuint64_t)acts[g].ld, (cuuint64_t)M};
+    const cuuint64_t strides[1] = {(cuuint64_t)acts[g].ld * 2};
     const cuuint32_t box[2] = {BK, BM};
     const cuuint32_t estr[2] = {1, 1};
-    if (enc(&tmaps.m[slot], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(xcats[g]), dims, strides, box, estr,
+    if (enc(&tmaps.m[slot], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, acts[g].xcat, dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
@@ -549,7 +549,7 @@ cudaError_t launch_gemm_tc2_group(const void* const* xcats, const void* const* p
     ly.y_extent = y_bytes(y_type, (size_t)M, (size_t)m.N);
     if (kDebugBounds) ly.y_extent -= std::min(ly.y_extent, debug_y_shrink());
     ly.w_extent = m.off_b - m.off_w; ly.b_extent = m.off_a - m.off_b;
-    ly.N = m.N; ly.K64 = m.K64;
+    ly.N = m.N; ly.t_col = acts[g].t_col;
     ly.n_tiles = m.n_tiles; ly.k_slabs = m.k_slabs; ly.r_blocks = m.r_blocks;
     ly.slab0 = 0; ly.slab_stride = m.k_slabs;
     ly.spt = m.k_slabs + (m.r_blocks + 1) / 2;

@@ -1,0 +1,770 @@
+// Activation prologue of larger batches with ranks above 64 (paper Section 4.1: X_q in MXINT8, blocks [1,16]; Section 3.1:
+// the small high-precision product T = X_q A_k), in three launches:
+//   quantise_kernel  X -> Xcat[:, 0:K64] (the exact bf16 values of X_q), one exponent byte per 16-block, and per row the
+//                    range of its exponents; A_q -> digit planes (below);
+//   project_kernel   T = X_q A_q as ONE integer contraction on the tcgen05 int8 tensor cores, into 64-bit sums;
+//   finish_kernel    T re-quantised along the rank, appended to Xcat.
+//
+// The projection has to be exact (T is re-quantised, and its rounding decisions must be those of a 64-bit sum), but the
+// blocks of a row have exponents of their own, so the int32 products of different blocks cannot simply be added up.  Here
+// a row is written in ONE fixed-point format instead: with E the top of the row's window of exponents [E - 8, E], a value
+// m * 2^(e-6) of a block with E - 8 <= e <= E is the integer m * 2^(8-(E-e)), at most 127 * 2^8 in magnitude, times
+// 2^(E-14): sixteen bits, i.e. two signed base-256 digits.  A column of A_q takes the same form over its blocks.  T is then
+// three integer contractions (high x high, the two mixed ones into one accumulator, low x low) over the WHOLE of K, exact
+// in int32 for up to 32768 K per CTA, and one 64-bit combination per element of T.  Partial sums of different K ranges
+// are integers with a common scale, so they are added with 64-bit integer atomics, in any order: exact and reproducible.
+// Blocks outside their row's (or column's) window - it is the one that holds most of them - are zero in the digit planes
+// and are added in fp64 at the end, for rows and columns that have such a block at all.
+// Scaling every block's products in fp64 instead, as the other prologues do, is bound by 14.7 block products per clock and
+// SM: 115 us for 2048 rows of 4096 columns at rank 256.
+#include <algorithm>
+
+#include "lqer_tc_ptx.cuh"
+
+namespace lqer {
+namespace pdg {
+using namespace tc;
+
+constexpr int kWindow = 8;                        // a window holds the exponents [E - 8, E]
+constexpr int kColsPerWarp = 2;                   // columns of A_q one warp turns into digits,
+constexpr int kColShares = 4;                     // in one of so many shares of K
+constexpr int ROWS = 128;
+constexpr int PANEL = 128;                        // K per stage: one 128-byte swizzled row of int8
+constexpr int MAX_NT = 128;                       // T columns per CTA: three int32 accumulators of 128 columns in tensor memory
+constexpr int STAGES = 3;
+constexpr int X_PLANE = ROWS * PANEL;             // 16384
+constexpr int A_PLANE = MAX_NT * PANEL;           // 16384
+constexpr int STAGE_BYTES = 2 * X_PLANE + 2 * A_PLANE;
+constexpr int CONV_WARPS = 16;
+constexpr int WORKERS = CONV_WARPS * 32;          // threads of the converter warps; they do phase 1 too
+constexpr int NUM_THREADS = (2 + CONV_WARPS) * 32;
+constexpr int kParts = CONV_WARPS;                // shares of a row in phase 1, at most
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + CONV_WARPS * 1024 + 256 + 1024;
+constexpr int kQuantThreads = 256;
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
+constexpr int kFinishRows = 16;
+constexpr int TMEM_COLS = 512;
+
+struct LayerA {                                   // one layer's A section and its place among the unit's T columns
+  const uint8_t* asec;
+  int8_t* Tm;                                     // optional exports
+  uint8_t* Te;
+  int k_pad, col0;
+};
+struct Unit {                                     // one X and the layers that multiply it
+  const void* X;
+  uint16_t* xcat;                                 // [M, ld]: X_q values, then T columns
+  uint8_t* ebytes;                                // [M, ep] exponent bytes of X_q's blocks; 0: a block of zeros
+  uint16_t* rowparts;                             // [M][kParts]: largest | smallest << 8 exponent byte in each share of a row
+  int* rowinfo;                                   // [M]: E + 1024, bit 16: the row has blocks outside its window (phase 2 writes it)
+  int* colinfo;                                   // [ktot]: E + 1024 of A_q's columns, bit 16: it has blocks outside its window
+  uint8_t* planes;                                // digit planes of A_q: [column tile][panel][hi, lo][columns][128], swizzled
+  unsigned long long* tacc;                       // [row tile][ktot][128] sums (splits > 1)
+  LayerA layer[kDigitMaxLayers];
+  int n_layers, ktot;
+  int K, K64, ld, ep, panels;
+  int row_tiles, col_tiles, splits;
+  int first_a, first_rows;                        // quantise_kernel: this unit's first warp of each kind
+  int first_item, first_finish;                   // project_kernel, finish_kernel: its first CTA
+  size_t xcat_extent;                             // bytes, for the checked build
+};
+struct Params {
+  Unit U[kDigitMaxUnits];
+  int n, M, x_type;
+  int warps_per_row;                              // a power of two up to kParts
+  int rows_begin, n_warps;                        // warps of quantise_kernel: A_q of all units, then (from rows_begin) their rows
+  int a_bits, lr_bits, exp_min, exp_max, w_exp_min;
+  DeviceStatus* status;
+  long long wait_limit;
+  int stall;                                      // test hook: the last panel's A digits are withheld
+};
+
+__device__ __forceinline__ const Unit& unit_of(const Params& p, int index, int Unit::* first) {
+  int u = 0;
+  for (int i = 1; i < p.n; ++i)
+    if (index >= p.U[i].*first) u = i;
+  return p.U[u];
+}
+__device__ __forceinline__ void tile_columns(int ktot, int col_tiles, int ct, int& c0, int& nt) {
+  const unsigned nb = (unsigned)ktot >> 4;                             // at most 128
+  c0 = (int)((unsigned)ct * nb / (unsigned)col_tiles) << 4;
+  nt = ((int)((unsigned)(ct + 1) * nb / (unsigned)col_tiles) << 4) - c0;
+}
+__device__ __forceinline__ bool outside(int eb, int E) { return eb != 0 && (eb - 127 > E || eb - 127 < E - kWindow); }
+
+// The window [E - 8, E] that holds most of the blocks counted in hist[exponent byte], for one warp.
+__device__ __forceinline__ int best_window(const int* hist, int lane) {
+  int best = -1, at = 0;
+  for (int eb = 1 + lane; eb < 256; eb += 32) {   // the lowest top that holds the most
+    int n = 0;
+    for (int d = 0; d <= kWindow; ++d) n += eb - d >= 1 ? hist[eb - d] : 0;
+    if (n > best) { best = n; at = eb; }
+  }
+  for (int s = 16; s > 0; s >>= 1) {
+    const int ob = __shfl_xor_sync(0xFFFFFFFFu, best, s), oa = __shfl_xor_sync(0xFFFFFFFFu, at, s);
+    if (ob > best || (ob == best && oa < at)) { best = ob; at = oa; }
+  }
+  return at - 127;
+}
+
+// Two base-256 digits of four integers xi = v * scale (|xi| <= 32512): xi = hi * 256 + lo, both signed bytes.
+// The sum v * scale + (1.5 * 2^23 + 128) is exact and carries xi + 128 in its low 16 bits.
+__device__ __forceinline__ void digits_of(float v0, float v1, float v2, float v3, float scale, uint32_t& hi, uint32_t& lo) {
+  const float kMagic = 12583040.0f;
+  const uint32_t u0 = __float_as_uint(fmaf(v0, scale, kMagic)), u1 = __float_as_uint(fmaf(v1, scale, kMagic));
+  const uint32_t u2 = __float_as_uint(fmaf(v2, scale, kMagic)), u3 = __float_as_uint(fmaf(v3, scale, kMagic));
+  const uint32_t a = __byte_perm(u0, u1, 0x5410), b = __byte_perm(u2, u3, 0x5410);
+  hi = __byte_perm(a, b, 0x7531);
+  lo = __byte_perm(a, b, 0x6420) ^ 0x80808080u;
+}
+
+// One signed byte of a word as a float without a conversion instruction (they run at an eighth of the rate): offset by 128
+// it is the low byte of the float 1.5 * 2^23 + 128 + value.
+__device__ __forceinline__ float byte_value(uint32_t w, uint32_t select) {
+  return __uint_as_float(__byte_perm(w ^ 0x80808080u, 0x4B400000u, select)) - 12583040.0f;
+}
+
+// The window of one row or column whose non-zero blocks' exponent bytes reach from mn to mx: E, and bit 16 if some lie
+// outside.  byte_of(b): block b's exponent byte, 0 for a block of zeros.  One warp; hist: 256 ints of its own.
+template <class F>
+__device__ __forceinline__ int window_of(int mx, int mn, int blocks, int* hist, int lane, F&& byte_of) {
+  if (mx - mn <= kWindow || mx == 0) return mx - 127 + 1024;
+  for (int i = lane; i < 256; i += 32) hist[i] = 0;
+  __syncwarp();
+  for (int b = lane; b < blocks; b += 32) {
+    const int eb = byte_of(b);
+    if (eb != 0) atomicAdd(&hist[eb], 1);
+  }
+  __syncwarp();
+  const int E = best_window(hist, lane);
+  __syncwarp();
+  return (E + 1024) | 1 << 16;
+}
+
+// One warp: a share of K of two columns of a layer's A_q -> windows (every share works them out) and digit planes.
+__device__ __forceinline__ void a_digits(const Params& p, const Unit& u, int part, int lane, int* hist) {
+  const int share = part % kColShares;
+  part /= kColShares;
+  int l = 0;
+  for (; l + 1 < u.n_layers && part >= u.layer[l].k_pad / kColsPerWarp; ++l) part -= u.layer[l].k_pad / kColsPerWarp;
+  const LayerA& la = u.layer[l];
+  if (part >= la.k_pad / kColsPerWarp) return;
+  const int c = part * kColsPerWarp, kb = u.K / 16, kp = la.k_pad;
+  const uint4* mant = reinterpret_cast<const uint4*>(la.asec);
+  const uint8_t* aexp = la.asec + (size_t)kb * kp * 16;
+  auto zero = [&](int b, int j) {
+    const uint4 v = mant[(size_t)b * kp + c + j];
+    return (v.x | v.y | v.z | v.w) == 0u;
+  };
+  int mx[2] = {0, 0}, mn[2] = {255, 255};
+  for (int b0 = lane; b0 < kb; b0 += 8 * 32) {
+    uint32_t e2[8];                                                    // eight loads in flight before the first is looked at
+#pragma unroll
+    for (int i = 0; i < 8; ++i) e2[i] = b0 + 32 * i < kb ? *reinterpret_cast<const uint16_t*>(aexp + (size_t)(b0 + 32 * i) * kp + c) : 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int eb = (int)((e2[i] >> (8 * j)) & 0xFFu);
+        // (only the lowest exponent may be a block of zeros)
+        if (eb != 0 && (eb - 127 > p.w_exp_min || !zero(b0 + 32 * i, j))) { mx[j] = max(mx[j], eb); mn[j] = min(mn[j], eb); }
+      }
+  }
+  int info[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    mx[j] = __reduce_max_sync(0xFFFFFFFFu, mx[j]);
+    mn[j] = __reduce_min_sync(0xFFFFFFFFu, mn[j]);
+    info[j] = window_of(mx[j], mn[j], kb, hist, lane, [&](int b) { return zero(b, j) ? 0 : (int)aexp[(size_t)b * kp + c + j]; });
+  }
+  const int col = la.col0 + c;
+  if (lane == 0 && share == 0) { u.colinfo[col] = info[0]; u.colinfo[col + 1] = info[1]; }
+  int c0 = 0, nt = 0;
+  for (int ct = 0; ct < u.col_tiles; ++ct) {                           // (tiles are whole 16-blocks: both columns lie in one)
+    tile_columns(u.ktot, u.col_tiles, ct, c0, nt);
+    if (col < c0 + nt) break;
+  }
+  uint8_t* img = u.planes + (size_t)u.panels * 2 * PANEL * c0;
+  const int n = col - c0;
+  for (int b0 = share * 32 + lane; b0 < u.ep; b0 += 2 * 32 * kColShares) {
+    uint4 v[2][2];
+    int d[2][2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int b = b0 + 32 * kColShares * i;
+        v[i][j] = make_uint4(0u, 0u, 0u, 0u);
+        d[i][j] = -1;
+        if (b < kb) {
+          v[i][j] = mant[(size_t)b * kp + c + j];
+          d[i][j] = (info[j] & 0xFFFF) - 1024 - ((int)aexp[(size_t)b * kp + c + j] - 127);
+        }
+      }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int b = b0 + 32 * kColShares * i;
+      if (b >= u.ep) break;
+      uint8_t* tile = img + (size_t)(b >> 3) * (2 * PANEL * nt);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        uint4 hi = make_uint4(0u, 0u, 0u, 0u), lo = hi;
+        if (d[i][j] >= 0 && d[i][j] <= kWindow) {
+          const float scale = pow2f(kWindow - d[i][j]);
+          const uint32_t w[4] = {v[i][j].x, v[i][j].y, v[i][j].z, v[i][j].w};
+          uint32_t h[4], o[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            digits_of(byte_value(w[q], 0x7640), byte_value(w[q], 0x7641), byte_value(w[q], 0x7642), byte_value(w[q], 0x7643), scale, h[q], o[q]);
+          hi = make_uint4(h[0], h[1], h[2], h[3]);
+          lo = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+        uint8_t* at = tile + (n + j) * PANEL + (((b & 7) ^ ((n + j) & 7)) << 4);
+        *reinterpret_cast<uint4*>(at) = hi;
+        *reinterpret_cast<uint4*>(at + nt * PANEL) = lo;
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void load16(const void* X, int x_type, int M, int K, int row, int col, const QuantConsts& qc, int a_bits,
+                                       float (&v)[16]) {
+  const size_t idx = (size_t)row * K + col;
+  if (x_type == kXBF16) {
+    const uint4* src = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(X) + idx);
+    const uint4 a = __ldg(src), b = __ldg(src + 1);
+    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { v[2 * i] = __uint_as_float(w[i] << 16); v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u); }
+  } else if (x_type == kXMXINT8) {
+    const uint8_t* xb = static_cast<const uint8_t*>(X);
+    const uint4 a = __ldg(reinterpret_cast<const uint4*>(xb + idx));
+    const uint32_t eb = __ldg(xb + (size_t)M * K + (size_t)row * (K / 16) + (col >> 4));
+    const uint32_t w[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 q = mxint_quad_values(w[i], eb, a_bits, qc.emin, qc.emax);
+      v[4 * i] = q.x; v[4 * i + 1] = q.y; v[4 * i + 2] = q.z; v[4 * i + 3] = q.w;
+    }
+  } else {
+    const float4* src = reinterpret_cast<const float4*>(static_cast<const float*>(X) + idx);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 q = __ldg(src + i);
+      v[4 * i] = q.x; v[4 * i + 1] = q.y; v[4 * i + 2] = q.z; v[4 * i + 3] = q.w;
+    }
+  }
+}
+
+// One warp: share `part` of a row.  A lane owns a whole 16-block; kBatch blocks of a lane are loaded together.
+constexpr int kBatch = 2;
+__device__ __forceinline__ void quantise_row(const Params& p, const Unit& u, int row, int part, int lane) {
+  if (u.splits > 1) {
+    // the sums start at zero: any share of them will do (the last row takes those of the last row tile's missing rows too)
+    const int rows_here = row == p.M - 1 ? u.row_tiles * ROWS - row : 1;
+    unsigned long long* acc = u.tacc + (size_t)row * u.ktot;
+    for (int i = part * 32 + lane; i < rows_here * u.ktot; i += p.warps_per_row * 32) acc[i] = 0ull;
+  }
+  const QuantConsts qc = quant_consts(p.a_bits, p.exp_min, p.exp_max);
+  const int kb = u.K / 16, xb = u.K64 / 16, stride = p.warps_per_row * 32;
+  int mx = 0, mn = 255;
+  uint8_t* erow = u.ebytes + (size_t)row * u.ep;
+  uint16_t* xrow = u.xcat + (size_t)row * u.ld;
+  float v[kBatch][16];
+#pragma unroll
+  for (int h = 0; h < kBatch; ++h) {
+    const int b = part * 32 + lane + h * stride;
+    if (b < kb) load16(u.X, p.x_type, p.M, u.K, row, b * 16, qc, p.a_bits, v[h]);
+  }
+  for (int b0 = part * 32 + lane; b0 < u.ep; b0 += kBatch * stride) {
+#pragma unroll
+    for (int h = 0; h < kBatch; ++h) {
+      const int b = b0 + h * stride;
+      if (b >= u.ep) break;
+      uint4 m8 = make_uint4(0u, 0u, 0u, 0u), x0 = m8, x1 = m8;
+      int e = 0, eb = 0;
+      if (b < kb) {
+        quantize_block16(v[h], qc, e, m8, x0, x1);
+        // (a block of narrower mantissas is a block of 8-bit ones with trailing zeros: the windows count in those)
+        if ((m8.x | m8.y | m8.z | m8.w) != 0u) { eb = e + 127; mx = max(mx, eb); mn = min(mn, eb); }
+      }
+      const int bn = b + kBatch * stride;                              // the next block is on its way while this one is stored
+      if (bn < kb) load16(u.X, p.x_type, p.M, u.K, row, bn * 16, qc, p.a_bits, v[h]);
+      if (b < xb && LQER_IN_BOUNDS(p.status, ((size_t)row * u.ld + b * 16) * 2, 32, u.xcat_extent, 331)) {
+        *reinterpret_cast<uint4*>(xrow + b * 16) = x0;
+        *reinterpret_cast<uint4*>(xrow + b * 16 + 8) = x1;
+      }
+      erow[b] = (uint8_t)eb;
+    }
+  }
+  mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+  mn = __reduce_min_sync(0xFFFFFFFFu, mn);
+  if (lane == 0) u.rowparts[(size_t)row * kParts + part] = (uint16_t)(mx | mn << 8);
+}
+
+// Bound by reading X and writing Xcat; no warp waits for another.
+__global__ void __launch_bounds__(kQuantThreads, 3) quantise_kernel(const __grid_constant__ Params p) {
+  __shared__ int s_hist[kQuantThreads / 32][256];
+  pdl_wait();
+  pdl_launch_dependents();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int w = (int)blockIdx.x * (kQuantThreads / 32) + warp;
+  if (w >= p.n_warps) return;
+  if (w < p.rows_begin) {
+    const Unit& u = unit_of(p, w, &Unit::first_a);
+    a_digits(p, u, w - u.first_a, lane, s_hist[warp]);
+  } else {
+    const Unit& u = unit_of(p, w, &Unit::first_rows);
+    const int share = w - u.first_rows;
+    quantise_row(p, u, share / p.warps_per_row, share % p.warps_per_row, lane);
+  }
+}
+
+__device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}\n"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
+}
+// int8 x int8 -> int32, both operands K-major, M = m, N = n.
+__host__ __device__ constexpr uint32_t make_idesc_i8(int m, int n) {
+  return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr) : "memory");
+}
+
+// The terms of T[row, col] that the digit planes leave out, in fp64: blocks outside the row's or the column's window.
+__device__ __noinline__ double outside_terms(const Params& p, const Unit& u, int row, int col, int rinfo, int cinfo) {
+  if (row >= p.M) return 0.0;
+  int l = 0;
+  while (l + 1 < u.n_layers && col >= u.layer[l + 1].col0) ++l;
+  const LayerA& la = u.layer[l];
+  const int kb = u.K / 16, c = col - la.col0;
+  const uint8_t* aexp = la.asec + (size_t)kb * la.k_pad * 16;
+  const int E = (rinfo & 0xFFFF) - 1024, CE = (cinfo & 0xFFFF) - 1024;
+  const bool wide = (cinfo >> 16) != 0;
+  double t = 0.0;
+  for (int b = 0; b < kb; ++b) {
+    const int eb = u.ebytes[(size_t)row * u.ep + b];
+    if (eb == 0 || (!outside(eb, E) && !wide)) continue;
+    const int ae = aexp[(size_t)b * la.k_pad + c];
+    if (!outside(eb, E) && !outside(ae, CE)) continue;
+    // the block's 8-bit mantissas from its bf16 values
+    const uint16_t* xv = u.xcat + (size_t)row * u.ld + b * 16;
+    const uint4 a = *reinterpret_cast<const uint4*>(la.asec + ((size_t)b * la.k_pad + c) * 16);
+    const uint32_t aw[4] = {a.x, a.y, a.z, a.w};
+    const float inv = pow2f(6 - (eb - 127));
+    int s = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      uint32_t w = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)                                      // the low byte of 1.5 * 2^23 + mantissa
+        w |= (__float_as_uint(fmaf(__uint_as_float((uint32_t)xv[4 * i + k] << 16), inv, 12582912.0f)) & 0xFFu) << (8 * k);
+      s = __dp4a((int)w, (int)aw[i], s);
+    }
+    t += (double)s * pow2d(eb - 127 + ae - 127 - 6 - (p.lr_bits - 2));
+  }
+  return t;
+}
+
+// kFinishRows rows of a tile's columns: the 64-bit sums -> T -> T_q.  Sixteen lanes hold a 16-block of T.
+__global__ void __launch_bounds__(WORKERS) finish_kernel(const __grid_constant__ Params p) {
+  pdl_launch_dependents();
+  const Unit& u = unit_of(p, blockIdx.x, &Unit::first_finish);
+  int item = (int)blockIdx.x - u.first_finish;
+  const int rg = item % (ROWS / kFinishRows); item /= ROWS / kFinishRows;
+  const int ct = item % u.col_tiles, rt = item / u.col_tiles;
+  int c0, nt;
+  tile_columns(u.ktot, u.col_tiles, ct, c0, nt);
+  const int tid = threadIdx.x, j16 = tid & 15;
+  pdl_wait();
+  if (rt * ROWS + rg * kFinishRows >= p.M) return;
+  const LayerA& la = u.layer[0];                                       // exports: a unit of one layer only
+#pragma unroll 1
+  for (int o = tid >> 4; o < kFinishRows * (nt >> 4); o += 4 * (WORKERS / 16)) {
+    long long s[4];
+    int ri[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = o + i * (WORKERS / 16), r = rg * kFinishRows + (k % kFinishRows), col = c0 + (k / kFinishRows) * 16 + j16;
+      const bool in = k < kFinishRows * (nt >> 4) && rt * ROWS + r < p.M;
+      s[i] = in ? (long long)__ldcg(u.tacc + ((size_t)rt * u.ktot + col) * ROWS + r) : 0;
+      ri[i] = in ? __ldcg(u.rowinfo + rt * ROWS + r) : 1024;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = o + i * (WORKERS / 16);
+      if (k >= kFinishRows * (nt >> 4)) break;                         // the same for all lanes of a warp but its half
+      const int row = rt * ROWS + rg * kFinishRows + (k % kFinishRows), col = c0 + (k / kFinishRows) * 16 + j16;
+      const int ci = u.colinfo[col];
+      const unsigned half = 0xFFFFu << (tid & 16);
+      const int p2 = (ri[i] & 0xFFFF) + (ci & 0xFFFF) - 2048 - 14 - kWindow - (p.lr_bits - 2);     // T = s * 2^p2
+      int e, m;
+      if (__any_sync(half, ((ri[i] | ci) >> 16) != 0)) {
+        double t = (double)s[i] * pow2d(p2);
+        if (((ri[i] | ci) >> 16) != 0) t += outside_terms(p, u, row, col, ri[i], ci);
+        double amax = fabs(t);
+#pragma unroll 1
+        for (int d = 1; d < 16; d <<= 1) amax = fmax(amax, __shfl_xor_sync(half, amax, d));
+        e = block_exponent(amax, p.exp_min, p.exp_max);
+        m = quant_mantissa(t, e, p.a_bits);
+      } else {
+        // the same decisions in integers (64-bit integers become doubles and doubles integers at a few per clock only)
+        const unsigned long long mag = (unsigned long long)(s[i] < 0 ? -s[i] : s[i]);
+        const int top = mag == 0 ? -(1 << 20) : 63 - __clzll((long long)mag) + p2;                // floor(log2 |T|)
+        const int bt = __reduce_max_sync(half, top);
+        e = min(max(bt, p.exp_min), p.exp_max);
+        const int qmax = (1 << (p.a_bits - 1)) - 1, sh = e - (p.a_bits - 2) - p2;                 // |T| in steps = mag * 2^-sh
+        if (top > e) {
+          m = qmax;
+        } else if (sh <= 0) {
+          m = mag == 0 ? 0 : (int)(mag << min(-sh, 63));
+        } else if (sh > 62) {
+          m = 0;
+        } else {                                                                                  // half to even
+          const unsigned long long q = mag >> sh, rest = mag & ((1ull << sh) - 1ull), tie = 1ull << (sh - 1);
+          m = (int)q + (rest > tie || (rest == tie && (q & 1ull)) ? 1 : 0);
+        }
+        m = min(m, qmax);
+        if (s[i] < 0) m = -m;
+      }
+      const size_t at = (size_t)row * u.ld + u.K64 + col;
+      if (row < p.M && LQER_IN_BOUNDS(p.status, at * 2, 2, u.xcat_extent, 332)) {
+        u.xcat[at] = (uint16_t)bf16_bits_of(m, e - (p.a_bits - 2));
+        if (la.Tm != nullptr) la.Tm[(size_t)row * la.k_pad + col] = (int8_t)m;
+        if (la.Te != nullptr && j16 == 0) la.Te[(size_t)row * (la.k_pad / 16) + col / 16] = (uint8_t)(e + 127);
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(NUM_THREADS, 1) project_kernel(const __grid_constant__ Params p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 1);
+  volatile WaitState* ws = reinterpret_cast<volatile WaitState*>(tmem_slot + 2);
+  int* s_hist = reinterpret_cast<int*>(smem + STAGES * STAGE_BYTES + 256);    // [CONV_WARPS][256]
+  const uint32_t bar0 = smem_u32(bars);
+  auto full = [&](int s) { return bar0 + 8u * s; };
+  auto empty = [&](int s) { return bar0 + 8u * (STAGES + s); };
+  const uint32_t done = bar0 + 8u * (2 * STAGES);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+  if (tid == 0) {
+    for (int s = 0; s < STAGES; ++s) { mbar_init(full(s), CONV_WARPS + 1); mbar_init(empty(s), 1); }
+    mbar_init(done, 1);
+    ws->abort = 0;
+    ws->limit = p.wait_limit;
+    fence_barrier_init();
+    fence_proxy_async_smem();
+  }
+  if (warp == 1) tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
+  const Unit& u = unit_of(p, blockIdx.x, &Unit::first_item);
+  int item = (int)blockIdx.x - u.first_item;
+  const int sp = item % u.splits; item /= u.splits;
+  const int ct = item % u.col_tiles, rt = item / u.col_tiles;
+  int c0, nt;
+  tile_columns(u.ktot, u.col_tiles, ct, c0, nt);
+  const int pn0 = (int)((long long)sp * u.panels / u.splits), pn1 = (int)((long long)(sp + 1) * u.panels / u.splits);
+  const int np = pn1 - pn0;
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  pdl_launch_dependents();
+  pdl_wait();
+
+  if (warp == 0) {
+    // -------------------------------------------------------------- A digits: one bulk copy per plane pair
+    if (lane == 0) {
+      const uint8_t* img = u.planes + (size_t)u.panels * 2 * PANEL * c0;
+      const uint32_t bytes = (uint32_t)(2 * PANEL * nt);
+      for (int i = 0; i < np; ++i) {
+        const int st = i % STAGES;
+        if (p.stall != 0 && pn0 + i == u.panels - 1) break;
+        if (!mbar_wait<true>(empty(st), (uint32_t)((i / STAGES) & 1) ^ 1u, ws)) break;
+        mbar_expect_tx(full(st), bytes);
+        bulk_load(smem_u32(smem + st * STAGE_BYTES + 2 * X_PLANE), img + (size_t)(pn0 + i) * bytes, bytes, full(st));
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // -------------------------------------------------------------- MMA issuer: the whole warp loops, one lane issues
+    const uint32_t idesc = make_idesc_i8(ROWS, nt);
+    const uint64_t xd0 = make_desc(smem_u32(smem)), ad0 = make_desc(smem_u32(smem + 2 * X_PLANE));
+    bool ok = true;
+    for (int i = 0; i < np; ++i) {
+      const int st = i % STAGES;
+      const uint64_t xh = xd0 + (uint64_t)(st * (STAGE_BYTES >> 4)), xl = xh + (X_PLANE >> 4);
+      const uint64_t ah = ad0 + (uint64_t)(st * (STAGE_BYTES >> 4)), al = ah + (uint64_t)((nt * PANEL) >> 4);
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(full(st), (uint32_t)((i / STAGES) & 1), ws)) != 0;
+      if (!ok) break;
+      tc_fence_after();
+      if (elect_one()) {
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {                           // 32 K = 32 bytes per instruction
+          const uint32_t acc = i > 0 || ks > 0 ? 1u : 0u;
+          umma_i8(tmem, xh + 2 * ks, ah + 2 * ks, idesc, acc);
+          umma_i8(tmem + MAX_NT, xh + 2 * ks, al + 2 * ks, idesc, acc);
+          umma_i8(tmem + MAX_NT, xl + 2 * ks, ah + 2 * ks, idesc, 1u);
+          umma_i8(tmem + 2 * MAX_NT, xl + 2 * ks, al + 2 * ks, idesc, acc);
+        }
+        umma_commit(empty(st));
+      }
+      __syncwarp();
+    }
+    if (ok && elect_one()) umma_commit(done);
+    __syncwarp();
+  } else {
+    // -------------------------------------------------------------- X_q values -> digit planes of the stage
+    const int cw = warp - 2;
+    const int r = cw * 8 + (lane >> 2), q = lane & 3;              // row of the tile; blocks 2q, 2q + 1 of a panel
+    const int row = rt * ROWS + r;
+    const bool live = row < p.M;
+    const uint16_t* xrow = u.xcat + (size_t)(live ? row : 0) * u.ld + q * 32;
+    const uint8_t* erow = u.ebytes + (size_t)(live ? row : 0) * u.ep + q * 2;
+    const uint32_t dst0 = (uint32_t)(r * PANEL + (((2 * q) ^ (r & 7)) << 4)), dst1 = (uint32_t)(r * PANEL + (((2 * q + 1) ^ (r & 7)) << 4));
+    uint4 x[2][4];
+    uint32_t eb[2];
+    auto fetch = [&](int pn, int w) {
+      eb[w] = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[w][i] = make_uint4(0u, 0u, 0u, 0u);
+      if (live && pn < pn1) {
+        eb[w] = *reinterpret_cast<const uint16_t*>(erow + pn * 8);
+        const uint4* src = reinterpret_cast<const uint4*>(xrow + pn * PANEL);
+        if (pn * PANEL + q * 32 < u.K64) { x[w][0] = src[0]; x[w][1] = src[1]; x[w][2] = src[2]; x[w][3] = src[3]; }
+      }
+    };
+    fetch(pn0, 0);
+    fetch(pn0 + 1, 1);
+    // the row's window from its shares (the row's four lanes look at four of them each)
+    int info;
+    {
+      int mx = 0, mn = 255;
+      for (int i = q; live && i < p.warps_per_row; i += 4) {
+        const int v = u.rowparts[(size_t)row * kParts + i];
+        mx = max(mx, v & 0xFF); mn = min(mn, v >> 8);
+      }
+      mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1)); mn = min(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, 1));
+      mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 2)); mn = min(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, 2));
+      info = mx - 127 + 1024;
+      unsigned wide = __ballot_sync(0xFFFFFFFFu, mx != 0 && mx - mn > kWindow);
+      while (wide != 0) {                                          // a row at a time, all lanes
+        const int src = __ffs(wide) - 1;
+        wide &= ~(0xFu << (src & ~3));
+        const uint8_t* er = u.ebytes + (size_t)__shfl_sync(0xFFFFFFFFu, row, src) * u.ep;
+        const int w = window_of(__shfl_sync(0xFFFFFFFFu, mx, src), __shfl_sync(0xFFFFFFFFu, mn, src), u.K / 16, s_hist + 256 * cw, lane,
+                                [&](int b) { return (int)er[b]; });
+        if ((lane & ~3) == (src & ~3)) info = w;
+      }
+      if (q == 0 && live && sp == 0) u.rowinfo[row] = info;
+    }
+    const int E = (info & 0xFFFF) - 1024;
+    const float base = pow2f(14 - max(E, -56));
+    bool ok = true;
+    auto put = [&](int i, int w) {
+      const int st = i % STAGES;
+      if (!mbar_wait(empty(st), (uint32_t)((i / STAGES) & 1) ^ 1u, ws)) { ok = false; return; }
+      uint8_t* hi_p = smem + st * STAGE_BYTES;
+      uint8_t* lo_p = hi_p + X_PLANE;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int e = (int)((eb[w] >> (8 * h)) & 0xFFu);
+        const float scale = e == 0 || outside(e, E) ? 0.0f : base;
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint4& v = x[w][2 * h + (k >> 1)];
+          const uint32_t a = (k & 1) ? v.z : v.x, b = (k & 1) ? v.w : v.y;
+          digits_of(__uint_as_float(a << 16), __uint_as_float(a & 0xFFFF0000u), __uint_as_float(b << 16), __uint_as_float(b & 0xFFFF0000u),
+                    scale, hi[k], lo[k]);
+        }
+        *reinterpret_cast<uint4*>(hi_p + (h ? dst1 : dst0)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *reinterpret_cast<uint4*>(lo_p + (h ? dst1 : dst0)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full(st));
+    };
+    for (int i = 0; i < np && ok; i += 2) {
+      put(i, 0);
+      fetch(pn0 + i + 2, 0);
+      if (ok && i + 1 < np) {
+        put(i + 1, 1);
+        fetch(pn0 + i + 3, 1);
+      }
+    }
+    // -------------------------------------------------------------- the sums: 64-bit combination, exchange, T_q
+    if (ok) ok = mbar_wait(done, 0u, ws);
+    tc_fence_after();
+    ok = __all_sync(0xFFFFFFFFu, ok) != 0;
+    // 16 columns of a tensor memory lane's row at a time, to the sums in memory
+    if (ok) {
+      const int tr = (warp & 3) * 32 + lane;                       // a warp reads the lanes of its number mod 4
+      unsigned long long* acc = u.tacc + ((size_t)rt * u.ktot + c0) * ROWS + tr;
+      for (int cb = (cw >> 2) * 16; cb < nt; cb += 64) {
+        uint32_t hh[16], mid[16], ll[16];
+        const uint32_t base_t = tmem + ((uint32_t)((warp & 3) * 32) << 16) + cb;
+        tmem_ld16(base_t, hh);
+        tmem_ld16(base_t + MAX_NT, mid);
+        tmem_ld16(base_t + 2 * MAX_NT, ll);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const long long v = (long long)(int)hh[j] * 65536 + (long long)(int)mid[j] * 256 + (long long)(int)ll[j];
+          if (u.splits > 1) atomicAdd(acc + (size_t)(cb + j) * ROWS, (unsigned long long)v);
+          else acc[(size_t)(cb + j) * ROWS] = (unsigned long long)v;
+        }
+      }
+      __threadfence();
+    }
+    tc_fence_before();
+  }
+
+  __syncthreads();                                          // every role is done or has given up
+  if (ws->abort != 0) {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 400000) { }                     // copies in flight land before the CTA's shared memory goes
+    if (tid == 0) report_error(p.status, LQER_ERR_TIMEOUT, 330, blockIdx.x);
+  }
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, TMEM_COLS);
+  }
+}
+
+static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
+
+}  // namespace pdg
+
+// Scratch of a unit whose layers' rank paddings sum to ktot (behind its Xcat): exponent bytes, windows, digit planes of A_q,
+// counters and 64-bit sums.
+static size_t digit_unit_scratch(int K64, int ktot, int M) {
+  using namespace pdg;
+  const size_t panels = (size_t)(K64 + PANEL - 1) / PANEL, rt = (size_t)(M + ROWS - 1) / ROWS;
+  return align256((size_t)M * panels * 8) + align256((size_t)M * kParts * 2) + align256((size_t)M * 4) + align256((size_t)ktot * 4) + align256(panels * 2 * PANEL * ktot) +
+         align256(rt * ktot * ROWS * 8);
+}
+// A group of layers needs at most the sum of this over its layers, whichever of them share an X.
+size_t prologue_digits_scratch_bytes(const PackedMeta& m, int M) { return digit_unit_scratch(m.K64, m.k_pad, M); }
+
+cudaError_t launch_prologue_digits(const DigitCall* calls, int n, int M, int x_type, void* scratch, GemmActs* places, int8_t* Tm,
+                                   uint8_t* Te, DeviceStatus* st, cudaStream_t s) {
+  using namespace pdg;
+  if (n < 1 || n > kDigitMaxLayers) return cudaErrorInvalidValue;
+  static OncePerDevice once;
+  cudaError_t err = once.run([] { return cudaFuncSetAttribute(project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES); });
+  if (err != cudaSuccess) return err;
+  const PackedMeta& m0 = *calls[0].meta;
+  Params p;
+  p.n = 0; p.M = M; p.x_type = x_type;
+  p.a_bits = m0.a_bits; p.lr_bits = m0.lr_bits; p.exp_min = m0.exp_min; p.exp_max = m0.exp_max; p.w_exp_min = m0.w_exp_min;
+  p.status = st;
+  p.wait_limit = wait_limit_cycles();
+  // layers that multiply the same X share its quantised values
+  int unit_at[kDigitMaxLayers];
+  for (int g = 0; g < n; ++g) {
+    const PackedMeta& m = *calls[g].meta;
+    if (m.k_pad == 0) return cudaErrorInvalidValue;
+    int q = 0;
+    while (q < p.n && !(p.U[q].X == calls[g].X && p.U[q].K == m.K)) ++q;
+    unit_at[g] = q;
+    Unit& u = p.U[q];
+    if (q == p.n) {
+      ++p.n;
+      u.X = calls[g].X; u.K = m.K; u.K64 = m.K64;
+      u.panels = (m.K64 + PANEL - 1) / PANEL;
+      u.ep = u.panels * 8;
+      u.row_tiles = (M + ROWS - 1) / ROWS;
+      u.n_layers = 0; u.ktot = 0;
+    }
+    LayerA& la = u.layer[u.n_layers++];
+    la.asec = static_cast<const uint8_t*>(calls[g].packed) + m.off_a;
+    la.Tm = n == 1 ? Tm : nullptr; la.Te = n == 1 ? Te : nullptr;
+    la.k_pad = m.k_pad; la.col0 = u.ktot;
+    places[g].t_col = m.K64 + u.ktot;
+    u.ktot += m.k_pad;
+  }
+  uint8_t* at = static_cast<uint8_t*>(scratch);
+  int items = 0, longest = 0;
+  for (int q = 0; q < p.n; ++q) {
+    Unit& u = p.U[q];
+    u.ld = u.K64 + u.ktot;
+    u.col_tiles = (u.ktot + MAX_NT - 1) / MAX_NT;
+    u.splits = (u.K64 + 32767) / 32768;                     // int32 sums: at most 32768 K per CTA
+    items += u.row_tiles * u.col_tiles * u.splits;
+    longest = std::max(longest, u.ep);
+    u.xcat = reinterpret_cast<uint16_t*>(at);
+    u.xcat_extent = (size_t)M * u.ld * 2;
+    at += align256(u.xcat_extent);
+    u.ebytes = at; at += align256((size_t)M * u.ep);
+    u.rowparts = reinterpret_cast<uint16_t*>(at); at += align256((size_t)M * kParts * 2);
+    u.rowinfo = reinterpret_cast<int*>(at); at += align256((size_t)M * 4);
+    u.colinfo = reinterpret_cast<int*>(at); at += align256((size_t)u.ktot * 4);
+    u.planes = at; at += align256((size_t)u.panels * 2 * PANEL * u.ktot);
+    u.tacc = reinterpret_cast<unsigned long long*>(at); at += align256((size_t)u.row_tiles * u.ktot * ROWS * 8);
+  }
+  for (int g = 0; g < n; ++g) {
+    places[g].xcat = p.U[unit_at[g]].xcat;
+    places[g].ld = p.U[unit_at[g]].ld;
+  }
+  // K ranges: CTAs for one round over the SMs, and at least two panels a range
+  const int sms = std::max(sm_count(), 1);
+  for (;;) {
+    int pick = -1;
+    double len = 2.0;
+    for (int q = 0; q < p.n; ++q) {
+      const Unit& u = p.U[q];
+      const double l = (double)u.panels / u.splits;
+      if (l > len && items + u.row_tiles * u.col_tiles <= sms) { len = l; pick = q; }
+    }
+    if (pick < 0) break;
+    ++p.U[pick].splits;
+    items += p.U[pick].row_tiles * p.U[pick].col_tiles;
+  }
+  // A row to a warp where the rows fill the SMs (32 warps each), to several warps otherwise, down to one block per lane.
+  p.warps_per_row = 1;
+  while (p.warps_per_row < kParts && (long long)p.n * M * p.warps_per_row < (long long)32 * sms && longest > 32 * kBatch * p.warps_per_row)
+    p.warps_per_row *= 2;
+  int warps = 0, finish = 0;
+  items = 0;
+  for (int q = 0; q < p.n; ++q) { p.U[q].first_a = warps; warps += p.U[q].ktot / kColsPerWarp * kColShares; }
+  p.rows_begin = warps;
+  for (int q = 0; q < p.n; ++q) {
+    Unit& u = p.U[q];
+    u.first_rows = warps; warps += M * p.warps_per_row;
+    u.first_item = items; items += u.row_tiles * u.col_tiles * u.splits;
+    u.first_finish = finish; finish += u.row_tiles * u.col_tiles * (ROWS / kFinishRows);
+  }
+  p.n_warps = warps;
+  for (int q = p.n; q < kDigitMaxUnits; ++q) p.U[q] = p.U[0];
+  p.stall = take_stall(kFamPrologue) ? 1 : 0;
+  LaunchScope scope(kFamPrologue, s, 3);
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3((warps + kQuantThreads / 32 - 1) / (kQuantThreads / 32));
+  cfg.blockDim = dim3(kQuantThreads);
+  if ((err = cudaLaunchKernelEx(&cfg, quantise_kernel, p)) != cudaSuccess) return err;
+  cfg.gridDim = dim3(items);
+  cfg.blockDim = dim3(NUM_THREADS);
+  cfg.dynamicSmemBytes = SMEM_BYTES;
+  if ((err = cudaLaunchKernelEx(&cfg, project_kernel, p)) != cudaSuccess) return err;
+  cfg.gridDim = dim3(finish);
+  cfg.blockDim = dim3(WORKERS);
+  cfg.dynamicSmemBytes = 0;
+  return cudaLaunchKernelEx(&cfg, finish_kernel, p);
+}
+
+}  // namespace lqer

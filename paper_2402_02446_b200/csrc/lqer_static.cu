@@ -51,5 +51,5 @@ extern "C" lqer_status_t lqer_linear_static(const float* X, int M, const void* p
   // The array keeps whatever the previous call left: the head of the workspace (status area,
   // arrival counters, accumulator) must start at zero.
   if ((st = lqer_workspace_init(scratch, need, stream)) != LQER_OK) return st;
-  return lqer_linear_stream(X, M, packed, Y, scratch, need, stream);
+  return lqer_linear_stream(X, M, packed, Y, scratch, (size_t)LQER_STATIC_SCRATCH_BYTES, stream);
 }

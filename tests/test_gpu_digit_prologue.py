@@ -1,0 +1,107 @@
+"""The prologue of larger batches with ranks above 64 (Section 3.1: T = X_q A_k as one integer contraction over digit planes)
+against the oracle: T_q has to be bit-exact, whatever the blocks' exponents."""
+import numpy as np
+import pytest
+import torch
+
+import lqer_inputs as gen
+import paper_2402_02446_b200 as L
+from paper_2402_02446_b200 import binding
+from helpers import exp_bytes, worst_ratio
+from oracle import lqer as olqer
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _t(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+
+
+def _spread(v, axis, bits, seed):
+    """v with every 16-block along `axis` scaled by a power of two from [-bits, bits]."""
+    g = np.random.default_rng(seed)
+    n = list(v.shape)
+    n[axis] //= 16
+    return (v * np.exp2(g.integers(-bits, bits + 1, size=n)).repeat(16, axis=axis)).astype(np.float32)
+
+
+# row tiles that end inside a tile, K with a part of a panel of 128 (and a single 16-block), ranks that end inside a block or
+# are cut into two column tiles, K ranges of one and of several panels
+@pytest.mark.parametrize("M,K,k", [(129, 80, 72), (129, 272, 65), (130, 1040, 100), (257, 2048, 128), (300, 1200, 200), (1030, 512, 256)])
+@pytest.mark.parametrize("wide", ["plain", "rows", "columns", "both"])
+def test_t_is_exact_inside_and_outside_the_windows(M, K, k, wide):
+    N = 264
+    spec = gen.LayerSpec("digits", M=M, K=K, N=N, k=k, calib_rows=32, outlier_frac=0.01, outlier_scale=50.0, seed=900 + K)
+    W = gen.make_weight(spec)
+    A, B = gen.make_random_factors(spec)
+    X = gen.make_activations(spec)
+    if wide in ("rows", "both"):                       # every third row: block exponents over 25 binades
+        X[::3] = _spread(X[::3], 1, 12, 1)
+        X[1, :16] = 0.0
+        X[2] = 0.0
+        X[4, 3] = np.inf
+    if wide in ("columns", "both"):
+        A[:, ::5] = _spread(A[:, ::5], 0, 10, 2)
+        A[:, 1] = 0.0
+    P, Pg = olqer.prepare_weights(W, A, B), L.prepare_weights(_t(W), _t(A), _t(B))
+    ref = olqer.forward(X, P)
+    ws = L.new_workspace(M, Pg)
+    L.set_path(binding.PATH_TENSOR_PROLOGUE)           # whatever the amount of work
+    try:
+        Tm, Te = L.project_lowrank(_t(X), Pg, ws)
+        Y = L.linear(_t(X), Pg, ws).cpu().numpy()
+    finally:
+        L.set_path(binding.PATH_AUTO)
+    assert L.poll_status(ws) == 0
+    assert np.array_equal(Tm.cpu().numpy(), ref.Tm)
+    assert np.array_equal(Te.cpu().numpy(), exp_bytes(ref.Te))
+    assert np.all(Y[ref.tol == 0.0] == 0.0)            # a row of zeros
+    ref.tol[ref.tol == 0.0] = 1.0
+    assert worst_ratio(Y, ref) <= 1.0
+    # the other prologue of these ranks gives the same result
+    L.set_path(binding.PATH_TENSOR)
+    try:
+        assert np.array_equal(L.linear(_t(X), Pg, ws).cpu().numpy(), Y)
+    finally:
+        L.set_path(binding.PATH_AUTO)
+    Pg.release()
+
+
+@pytest.mark.parametrize("x_type", ["f32", "bf16", "mxint8"])
+def test_layers_that_share_an_activation_equal_single_calls(x_type):
+    # three calls on one X, one on another, ranks of two widths: one group; each result is the single call's, bit for bit
+    M = 300
+    specs = [gen.LayerSpec(f"share{i}", M=M, K=2064, N=n, k=k, calib_rows=32, outlier_frac=0.01, outlier_scale=20.0, seed=950 + i)
+             for i, (n, k) in enumerate([(256, 80), (520, 256), (264, 112), (256, 80)])]
+    packs = []
+    for s in specs:
+        A, B = gen.make_random_factors(s)
+        packs.append(L.prepare_weights(_t(gen.make_weight(s)), _t(A), _t(B)))
+    Xs = [_t(gen.make_activations(specs[0])), _t(gen.make_activations(specs[3]))]
+    dt = {"f32": torch.float32, "bf16": torch.bfloat16, "mxint8": L.MXINT8}[x_type]
+    Xs = [L.to_mxint8(*L.quantize_activations(x)) if dt == L.MXINT8 else x.to(dt) for x in Xs]
+    Xc = [Xs[0], Xs[0], Xs[1], Xs[0]]
+    Ys = [torch.full((M, s.N), float("nan"), device=DEV) for s in specs]
+    calls = L.make_calls(list(zip(Xc, packs, Ys)), dt, torch.float32)
+    ws = torch.zeros(L.batched_workspace_bytes(calls), dtype=torch.uint8, device=DEV)
+    for _ in range(2):
+        L.linear_batched_ex(calls, ws, dt, torch.float32)
+    assert L.poll_status(ws) == 0
+    for x, Pg, y in zip(Xc, packs, Ys):
+        assert torch.equal(L.linear_ex(x, Pg, ws, M=M), y)
+        Pg.release()
+
+
+def test_a_workspace_without_room_for_the_planes_is_taken_as_before():
+    spec = gen.LayerSpec("tight", M=300, K=4112, N=264, k=128, calib_rows=32, outlier_frac=0.01, outlier_scale=20.0, seed=970)
+    A, B = gen.make_random_factors(spec)
+    Pg = L.prepare_weights(_t(gen.make_weight(spec)), _t(A), _t(B))
+    X = _t(gen.make_activations(spec))
+    Y = L.linear(X, Pg, L.new_workspace(spec.M, Pg))
+    least = 168192 + (spec.M * (4160 + 128) * 2 + 255) // 256 * 256       # the head and [X_q | T_q]
+    ws = torch.zeros(least, dtype=torch.uint8, device=DEV)
+    assert torch.equal(L.linear(X, Pg, ws), Y) and L.poll_status(ws) == 0
+    with pytest.raises(binding.LqerError):
+        L.linear(X, Pg, ws[: least - 256])
+    Pg.release()
