@@ -9,10 +9,9 @@
 //            Z = orth(G^T Q), Q = orth(G Z); then Bt = G^T Q = Q_b R (Cholesky factor of Bt^T Bt), the right
 //            singular vectors V of the small matrix R (one-sided Jacobi in one CTA), and
 //            A = diag(1/s) Q V_k,   B = (Bt V_k)^T = Sigma_k V_k^T.
-// The large products read G as fp32 and accumulate in fp64; everything of rank size is fp64.  orth() is
-// Cholesky QR applied twice.  Omega (the random test matrix) is an input, so the caller owns the random numbers.
-// None of this is on the inference path; the kernels are plain CUDA-core code built for clarity and a fixed
-// summation order.
+// The large products read G as fp32 and accumulate in fp64 (on the fp64 tensor pipe); everything of rank size is fp64.
+// orth() is Cholesky QR applied twice.  Omega (the random test matrix) is an input, so the caller owns the random numbers.
+// None of this is on the inference path; every sum has a fixed order.
 #include "lqer_common.cuh"
 
 namespace lqer {
@@ -21,6 +20,7 @@ namespace fac {
 constexpr int kOversample = 16;
 constexpr int kIters = 4;
 constexpr int kMaxR = 272;                 // 256 + oversample
+constexpr int kGramChunks = 32;            // partial Gram matrices (the workspace has room for 64)
 
 // ---------------------------------------------------------------------------- calibration (Appendix A)
 // Partial sums of |X| over a chunk of rows: grid (column blocks of 256, row chunks), one thread per column.
@@ -92,58 +92,142 @@ __global__ void __launch_bounds__(256) scaled_error_kernel(const float* __restri
 }
 
 // ---------------------------------------------------------------------------- products with G
+__global__ void __launch_bounds__(256) widen_kernel(const float* __restrict__ x, size_t n, double* __restrict__ y) {
+  const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (i < n) y[i] = (double)x[i];
+}
 // C[m, r] = op(G) X, fp64 accumulation.  TRANS = false: op(G) = G [m = K, inner = N], X [N, r].
-// TRANS = true: op(G) = G^T [m = N, inner = K], X [K, r].  X may be fp32 (the test matrix) or fp64.
-// CTA tile 64 (m) x 64 (r), inner step 16, 256 threads with 4 x 4 outputs each.
-template <bool TRANS, typename XT>
-__global__ void __launch_bounds__(256) g_times_kernel(const float* __restrict__ G, int K, int N, const XT* __restrict__ X, int r,
-                                                      double* __restrict__ C) {
-  __shared__ double s_g[16][65];     // [inner][m]
-  __shared__ double s_x[16][65];     // [inner][r]
+// TRANS = true: op(G) = G^T [m = N, inner = K], X [K, r].
+// Bound by the fp64 multiply-adds (2 K N r flop; 43 us for a 4096 x 4096 G at r = 48 and 37 TFLOP/s): they run as
+// mma.sync.m16n8k8 in fp64, whose fragments come straight from global memory.  A CTA owns 16 MT rows of C and up to 48
+// columns for the whole inner dimension; its eight warps take inner chunks of 16 (8 for G^T) in turn, each holds a full
+// tile of sums, and the eight are added in warp order at the end.  The inner positions of an MMA and the rows of its A
+// operand may be any, as long as both operands agree and the store knows: a lane takes neighbouring elements of G, one
+// vector load each, instead of the fragment's strided ones.
+// Measured (4096 x 4096, r = 48): 101 us (G^T) and 87 us (G) per product, against 1250 - 1320 us for a 64 x 64 tile per CTA
+// with 4 x 4 outputs per thread, which left 84 SMs without a tile.
+constexpr int kGCols = 48, kGTiles = kGCols / 8, kGWarps = 8;
+__device__ __forceinline__ void dmma(double (&c)[4], const double (&a)[4], double b0, double b1) {
+  asm volatile("mma.sync.aligned.m16n8k8.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3]) : "d"(a[0]), "d"(a[1]), "d"(a[2]), "d"(a[3]), "d"(b0), "d"(b1));
+}
+template <bool TRANS, int MT>
+__global__ void __launch_bounds__(kGWarps * 32) g_times_kernel(const float* __restrict__ G, int K, int N, const double* __restrict__ X, int r,
+                                                               double* __restrict__ C) {
+  extern __shared__ double s_part[];                         // [warp][16 MT][kGCols]
+  constexpr int STEP = TRANS ? 8 : 16;                       // inner positions of a chunk
   const int m_total = TRANS ? N : K, inner = TRANS ? K : N;
-  const int m0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4];
+  const int m0 = blockIdx.x * 16 * MT, c0 = blockIdx.y * kGCols;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int n_tiles = min(kGTiles, (r - c0 + 7) / 8);
+  double acc[MT][kGTiles][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < MT; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  for (int i0 = 0; i0 < inner; i0 += 16) {
-    for (int q = threadIdx.x; q < 64 * 16; q += 256) {
-      int mi, ii;
-      if (TRANS) { mi = q & 63; ii = q >> 6; } else { ii = q & 15; mi = q >> 4; }   // coalesced along G's rows
-      const int m = m0 + mi, i = i0 + ii;
-      float g = 0.0f;
-      if (m < m_total && i < inner) g = TRANS ? G[(size_t)i * N + m] : G[(size_t)m * N + i];
-      s_g[ii][mi] = (double)g;
+    for (int n = 0; n < kGTiles; ++n)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][n][j] = 0.0;
+
+  // one chunk of both operands: gv[i][...] G's elements of m tile i, xv[h][n] X's rows of the chunk's k positions
+  constexpr int KS = STEP / 8;                               // MMAs along the inner dimension
+  float gv[MT][KS][4];
+  double xv[KS][2][kGTiles];
+  auto load = [&](int i0) {
+    if (TRANS) {
+      // lane g: columns 2 MT g + .. of the CTA's 16 MT; its rows are inner positions i0 + t and i0 + t + 4
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = i0 + t + 4 * h, m = m0 + 2 * MT * g;
+        float v[2 * MT];
+#pragma unroll
+        for (int q = 0; q < 2 * MT; ++q) v[q] = 0.0f;
+        if (i < inner && m < m_total) {                      // (N is a multiple of 8)
+          const float* src = G + (size_t)i * N + m;
+          if (MT == 2) {
+            const float4 w = *reinterpret_cast<const float4*>(src);
+            v[0] = w.x; v[1] = w.y; v[2 * MT - 2] = w.z; v[2 * MT - 1] = w.w;
+          } else {
+            const float2 w = *reinterpret_cast<const float2*>(src);
+            v[0] = w.x; v[1] = w.y;
+          }
+        }
+#pragma unroll
+        for (int i2 = 0; i2 < MT; ++i2) { gv[i2][0][2 * h] = v[2 * i2]; gv[i2][0][2 * h + 1] = v[2 * i2 + 1]; }
+      }
+    } else {
+      // lane t: inner positions i0 + 4 t + {0, 1, 2, 3}: k slots t and t + 4 of two MMAs
+#pragma unroll
+      for (int i2 = 0; i2 < MT; ++i2)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int m = m0 + 16 * i2 + 8 * h + g, i = i0 + 4 * t;
+          float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (m < m_total && i < inner) w = *reinterpret_cast<const float4*>(G + (size_t)m * N + i);
+          gv[i2][0][h] = w.x; gv[i2][0][2 + h] = w.y; gv[i2][KS - 1][h] = w.z; gv[i2][KS - 1][2 + h] = w.w;
+        }
     }
-    for (int q = threadIdx.x; q < 16 * 64; q += 256) {
-      const int rr = q & 63, ii = q >> 6;
-      const int i = i0 + ii, c = r0 + rr;
-      s_x[ii][rr] = (i < inner && c < r) ? (double)X[(size_t)i * r + c] : 0.0;
-    }
-    __syncthreads();
 #pragma unroll
-    for (int ii = 0; ii < 16; ++ii) {
-      double a[4], b[4];
+    for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = s_g[ii][ty * 4 + i];
+      for (int h = 0; h < 2; ++h) {
+        const int i = TRANS ? i0 + t + 4 * h : i0 + 4 * t + 2 * ks + h;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = s_x[ii][tx * 4 + j];
+        for (int n = 0; n < kGTiles; ++n) {
+          const int c = c0 + 8 * n + g;
+          xv[ks][h][n] = i < inner && c < r ? X[(size_t)i * r + c] : 0.0;
+        }
+      }
+  };
+  for (int i0 = warp * STEP; i0 < inner; i0 += kGWarps * STEP) {
+    load(i0);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+    for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
+      for (int i2 = 0; i2 < MT; ++i2) {
+        // a fragment: (row g, k t), (g + 8, t), (g, t + 4), (g + 8, t + 4)
+        const double a[4] = {(double)gv[i2][ks][0], (double)gv[i2][ks][1], (double)gv[i2][ks][2], (double)gv[i2][ks][3]};
+#pragma unroll
+        for (int n = 0; n < kGTiles; ++n)
+          if (n < n_tiles) dmma(acc[i2][n], a, xv[ks][0][n], xv[ks][1][n]);
+      }
   }
+  double* mine = s_part + (size_t)warp * 16 * MT * kGCols;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i2 = 0; i2 < MT; ++i2)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int m = m0 + ty * 4 + i, c = r0 + tx * 4 + j;
-      if (m < m_total && c < r) C[(size_t)m * r + c] = acc[i][j];
-    }
+    for (int n = 0; n < kGTiles; ++n)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        // accumulator row g + 8 (j / 2) of m tile i2, column 2 t + j % 2
+        const int row = TRANS ? 2 * MT * g + 2 * i2 + (j >> 1) : 16 * i2 + 8 * (j >> 1) + g;
+        mine[row * kGCols + 8 * n + 2 * t + (j & 1)] = acc[i2][n][j];
+      }
+  __syncthreads();
+  for (int o = threadIdx.x; o < 16 * MT * kGCols; o += kGWarps * 32) {
+    const int m = m0 + o / kGCols, c = c0 + o % kGCols;
+    if (m >= m_total || c >= r) continue;
+    double v = 0.0;
+#pragma unroll
+    for (int w = 0; w < kGWarps; ++w) v += s_part[(size_t)w * 16 * MT * kGCols + o];
+    C[(size_t)m * r + c] = v;
+  }
+}
+// 32 rows per CTA where that gives a CTA to most SMs, 16 otherwise.
+template <bool TRANS>
+static cudaError_t g_times(const float* G, int K, int N, const double* X, int r, double* C, cudaStream_t s) {
+  const int m = TRANS ? N : K, cols = (r + kGCols - 1) / kGCols;
+  static OncePerDevice once;
+  const cudaError_t e = once.run([] {
+    const cudaError_t e1 = cudaFuncSetAttribute(g_times_kernel<TRANS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGWarps * 16 * kGCols * 8);
+    return e1 != cudaSuccess ? e1
+                             : cudaFuncSetAttribute(g_times_kernel<TRANS, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGWarps * 32 * kGCols * 8);
+  });
+  if (e != cudaSuccess) return e;
+  if ((m + 31) / 32 * cols >= 96)
+    g_times_kernel<TRANS, 2><<<dim3((m + 31) / 32, cols), kGWarps * 32, kGWarps * 32 * kGCols * 8, s>>>(G, K, N, X, r, C);
+  else
+    g_times_kernel<TRANS, 1><<<dim3((m + 15) / 16, cols), kGWarps * 32, kGWarps * 16 * kGCols * 8, s>>>(G, K, N, X, r, C);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------- tall-skinny helpers (fp64)
@@ -170,44 +254,77 @@ __global__ void __launch_bounds__(256) gram_partial_kernel(const double* __restr
   }
   if (i0 + ti < r && j0 + tj < r) part[((size_t)blockIdx.z * r + i0 + ti) * r + j0 + tj] = acc;
 }
-__global__ void __launch_bounds__(256) gram_sum_kernel(const double* __restrict__ part, int chunks, int r, double* __restrict__ C) {
-  const int idx = blockIdx.x * 256 + threadIdx.x;
-  if (idx >= r * r) return;
-  double acc = 0.0;
-  for (int q = 0; q < chunks; ++q) acc += part[(size_t)q * r * r + idx];
-  C[idx] = acc;
-}
-// C = R^T R (upper-triangular R by Cholesky), then Rinv = R^-1; one CTA, column by column.  A pivot that is not
-// positive (rank-deficient Y) is replaced by a tiny one so that the run stays finite; status records it.
-__global__ void __launch_bounds__(1024) cholesky_inverse_kernel(double* __restrict__ C, int r, double* __restrict__ Rinv,
-                                                                int* __restrict__ status) {
-  // in place: the upper triangle of C becomes R
-  for (int j = 0; j < r; ++j) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double d = C[(size_t)j * r + j];
-      for (int p = 0; p < j; ++p) d -= C[(size_t)p * r + j] * C[(size_t)p * r + j];
-      if (!(d > 0.0)) { d = 1e-300; atomicMax(status, 2); }
-      C[(size_t)j * r + j] = sqrt(d);
-    }
-    __syncthreads();
-    const double djj = C[(size_t)j * r + j];
-    for (int c = j + 1 + threadIdx.x; c < r; c += 1024) {
-      double v = C[(size_t)j * r + c];
-      for (int p = 0; p < j; ++p) v -= C[(size_t)p * r + j] * C[(size_t)p * r + c];
-      C[(size_t)j * r + c] = v / djj;
-    }
+// C = the sum of the partial Gram matrices (in chunk order) = R^T R (upper-triangular R by Cholesky), then Rinv = R^-1; one
+// CTA.  A pivot that is not positive (rank-deficient Y) is replaced by a tiny one so that the run stays finite; status
+// records it.
+// A chain of 2 r short steps, bound by their latency: a step is one update of a whole triangle by all threads (the trailing
+// part of C minus the outer product of a finished row; the rows of R^-1 above a finished one) and ONE barrier - the
+// division of a row by its pivot is left to whoever reads the row, and done for good at the end -, with both matrices in
+// shared memory where they fit (r <= kSharedR).  67 us at r = 48, the sum of the partial matrices included; dot products
+// along rows and columns in global memory took 150 us and the sum 15 us in a kernel of its own.
+constexpr int kSharedR = 112;              // two r x r fp64 matrices within 200 KB
+__global__ void __launch_bounds__(1024) cholesky_inverse_kernel(const double* __restrict__ part, int chunks, double* __restrict__ Cg, int r,
+                                                                double* __restrict__ Rinvg, int* __restrict__ status) {
+  extern __shared__ double s_mat[];
+  __shared__ double s_inv[kMaxR];                            // 1 / pivot of each row
+  const bool shared = r <= kSharedR;
+  double* C = shared ? s_mat : Cg;
+  double* Rinv = shared ? s_mat + r * r : Rinvg;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int q = threadIdx.x; q < r * r; q += 1024) {
+    double acc = 0.0;
+#pragma unroll 8
+    for (int i = 0; i < chunks; ++i) acc += part[(size_t)i * r * r + q];
+    C[q] = acc;
+    Rinv[q] = q / r == q % r ? 1.0 : 0.0;
   }
   __syncthreads();
-  // Rinv: column c solves R x = e_c by back substitution (a thread per column)
-  for (int c = threadIdx.x; c < r; c += 1024) {
-    for (int i = r - 1; i >= 0; --i) {
-      double v = i == c ? 1.0 : 0.0;
-      if (i > c) { Rinv[(size_t)i * r + c] = 0.0; continue; }
-      for (int p = i + 1; p <= c; ++p) v -= C[(size_t)i * r + p] * Rinv[(size_t)p * r + c];
-      Rinv[(size_t)i * r + c] = v / C[(size_t)i * r + i];
+  // row j of the upper triangle of C becomes pivot_j times row j of R; the warp that has row j + 1 works out its pivot
+  // (all warps doing it would keep the fp64 pipe busy for longer than the update)
+  const auto pivot = [&](double d) {
+    if (!(d > 0.0)) { d = 1e-300; atomicMax(status, 2); }
+    return 1.0 / sqrt(d);
+  };
+  if (threadIdx.x == 0) s_inv[0] = pivot(C[0]);
+  __syncthreads();
+  for (int j = 0; j + 1 < r; ++j) {
+    const double inv2 = s_inv[j] * s_inv[j];
+    for (int i = j + 1 + ty; i < r; i += 32) {
+      const double f = C[j * r + i] * inv2;
+      for (int c = (i & ~31) + tx; c < r; c += 32)
+        if (c >= i) {
+          const double v = fma(-f, C[j * r + c], C[i * r + c]);
+          C[i * r + c] = v;
+          if (c == j + 1) s_inv[j + 1] = pivot(v);
+        }
     }
+    __syncthreads();
   }
+  // R Rinv = I from the last row up: Z (here in Rinv) with Rinv row i = Z row i / pivot_i
+  for (int i = r - 1; i > 0; --i) {
+    const double inv = s_inv[i];
+    for (int q = ty; q < i; q += 32) {
+      const double f = C[q * r + i] * (s_inv[q] * inv);      // R[q, i] / pivot_i
+      for (int c = (i & ~31) + tx; c < r; c += 32)
+        if (c >= i) Rinv[q * r + c] = fma(-f, Rinv[i * r + c], Rinv[q * r + c]);
+    }
+    __syncthreads();
+  }
+  for (int q = threadIdx.x; q < r * r; q += 1024) {
+    const int row = q / r, col = q % r;
+    const double inv = s_inv[row];
+    if (shared || col >= row) Cg[q] = col == row ? 1.0 / inv : C[q] * inv;
+    Rinvg[q] = Rinv[q] * inv;
+  }
+}
+static cudaError_t cholesky_inverse(const double* part, int chunks, double* C, int r, double* Rinv, int* status, cudaStream_t s) {
+  static OncePerDevice once;
+  const cudaError_t e = once.run([] {
+    return cudaFuncSetAttribute(cholesky_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kSharedR * kSharedR * 8);
+  });
+  if (e != cudaSuccess) return e;
+  cholesky_inverse_kernel<<<1, 1024, r <= kSharedR ? 2 * r * r * 8 : 0, s>>>(part, chunks, C, r, Rinv, status);
+  return cudaGetLastError();
 }
 // Out[m, c] = rowscale[m] * sum_j Y[m, j] T[j, c] for c < cols (T is [r, ldt]); fp64 in, OutT out, optionally
 // written transposed (Out[c, m]).  One CTA = 64 rows; T's used columns are walked in tiles of 64.
@@ -267,9 +384,13 @@ __global__ void __launch_bounds__(256) tall_times_small_kernel(const double* __r
 // triangle of C, row-major) by one-sided Jacobi: pairs of columns are rotated until all are mutually orthogonal,
 // V collects the rotations.  A warp per pair, the pairs of a step disjoint (round-robin tournament).  Mt, Vt: r x r
 // scratch, column-major.  Out: Vs row-major [r][r] with the columns in falling order of singular value, sigma[r].
-__global__ void __launch_bounds__(1024) jacobi_right_kernel(const double* __restrict__ C, int r, double* __restrict__ Mt,
-                                                            double* __restrict__ Vt, double* __restrict__ Vs, double* __restrict__ sigma,
+// Bound by the latency of its steps (r - 1 per sweep, one barrier each): both matrices sit in shared memory where they fit.
+__global__ void __launch_bounds__(1024) jacobi_right_kernel(const double* __restrict__ C, int r, double* __restrict__ Mtg,
+                                                            double* __restrict__ Vtg, double* __restrict__ Vs, double* __restrict__ sigma,
                                                             int* __restrict__ status) {
+  extern __shared__ double s_mat[];
+  double* Mt = r <= kSharedR ? s_mat : Mtg;
+  double* Vt = r <= kSharedR ? s_mat + r * r : Vtg;
   __shared__ int s_rotated;
   __shared__ double s_norm[kMaxR];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -376,11 +497,11 @@ static cudaError_t orthonormalise(const double* Yin, double* Yout, int m, int r,
   const double* src = Yin;
   double* bufs[2] = {Yout, const_cast<double*>(Yin)};
   for (int pass = 0; pass < 2; ++pass) {
-    const int chunks = 64, rows_per_chunk = (m + chunks - 1) / chunks;
+    const int chunks = kGramChunks, rows_per_chunk = (m + chunks - 1) / chunks;
     const int rt = (r + 15) / 16;
     gram_partial_kernel<<<dim3(rt, rt, chunks), 256, 0, s>>>(src, m, r, rows_per_chunk, gram_part);
-    gram_sum_kernel<<<(r * r + 255) / 256, 256, 0, s>>>(gram_part, chunks, r, C);
-    cholesky_inverse_kernel<<<1, 1024, 0, s>>>(C, r, Rinv, status);
+    const cudaError_t e = cholesky_inverse(gram_part, chunks, C, r, Rinv, status, s);
+    if (e != cudaSuccess) return e;
     double* dst = bufs[pass];
     tall_times_small_kernel<double, false><<<dim3((m + 63) / 64, (r + 63) / 64), 256, 0, s>>>(src, m, r, Rinv, r, r, nullptr, 0, dst);
     src = dst;
@@ -438,24 +559,29 @@ cudaError_t launch_factorize(const float* W, const float* const* Xs, const int* 
   // ---- G = S (W - W_q)
   scaled_error_kernel<<<dim3((N + 255) / 256, K / 16), 256, 0, s>>>(W, K, N, w_bits, emin, emax, sc, G);
   // ---- subspace iteration
-  const dim3 gK((K + 63) / 64, (r + 63) / 64), gN((N + 63) / 64, (r + 63) / 64);
-  g_times_kernel<false, float><<<gK, 256, 0, s>>>(G, K, N, Omega, r, T0);             // Y = G Omega      [K, r]
-  cudaError_t e = orthonormalise(T0, T1, K, r, gram_part, C, Rinv, status, s);           // Q in T1
+  widen_kernel<<<(int)(((size_t)N * r + 255) / 256), 256, 0, s>>>(Omega, (size_t)N * r, T1);
+  cudaError_t e = g_times<false>(G, K, N, T1, r, T0, s);                                 // Y = G Omega      [K, r]
+  if (e != cudaSuccess) return e;
+  e = orthonormalise(T0, T1, K, r, gram_part, C, Rinv, status, s);           // Q in T1
   if (e != cudaSuccess) return e;
   for (int it = 0; it < kIters; ++it) {
-    g_times_kernel<true, double><<<gN, 256, 0, s>>>(G, K, N, T1, r, T0);                // Z = G^T Q        [N, r]
+    if ((e = g_times<true>(G, K, N, T1, r, T0, s)) != cudaSuccess) return e;     // Z = G^T Q        [N, r]
     if ((e = orthonormalise(T0, Bt, N, r, gram_part, C, Rinv, status, s)) != cudaSuccess) return e;   // Z in Bt
-    g_times_kernel<false, double><<<gK, 256, 0, s>>>(G, K, N, Bt, r, T0);               // Y = G Z          [K, r]
+    if ((e = g_times<false>(G, K, N, Bt, r, T0, s)) != cudaSuccess) return e;    // Y = G Z          [K, r]
     if ((e = orthonormalise(T0, T1, K, r, gram_part, C, Rinv, status, s)) != cudaSuccess) return e;   // Q in T1
   }
-  g_times_kernel<true, double><<<gN, 256, 0, s>>>(G, K, N, T1, r, Bt);                  // Bt = G^T Q       [N, r]
+  if ((e = g_times<true>(G, K, N, T1, r, Bt, s)) != cudaSuccess) return e;       // Bt = G^T Q       [N, r]
   // ---- small SVD: Bt^T Bt = R^T R, R = U Sigma V^T  ->  G ~ (Q V) Sigma (...)^T
   {
-    const int chunks = 64, rpc = (N + chunks - 1) / chunks, rt = (r + 15) / 16;
+    const int chunks = kGramChunks, rpc = (N + chunks - 1) / chunks, rt = (r + 15) / 16;
     gram_partial_kernel<<<dim3(rt, rt, chunks), 256, 0, s>>>(Bt, N, r, rpc, gram_part);
-    gram_sum_kernel<<<(r * r + 255) / 256, 256, 0, s>>>(gram_part, chunks, r, C);
-    cholesky_inverse_kernel<<<1, 1024, 0, s>>>(C, r, Rinv, status);
-    jacobi_right_kernel<<<1, 1024, 0, s>>>(C, r, Mt, Vt, Vs, sigma, status);
+    if ((e = cholesky_inverse(gram_part, chunks, C, r, Rinv, status, s)) != cudaSuccess) return e;
+    static OncePerDevice once;
+    e = once.run([] {
+      return cudaFuncSetAttribute(jacobi_right_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kSharedR * kSharedR * 8);
+    });
+    if (e != cudaSuccess) return e;
+    jacobi_right_kernel<<<1, 1024, r <= kSharedR ? 2 * r * r * 8 : 0, s>>>(C, r, Mt, Vt, Vs, sigma, status);
   }
   // ---- A = S^-1 Q V_k  [K, k];  B = (Bt V_k)^T  [k, N]
   tall_times_small_kernel<float, false><<<dim3((K + 63) / 64, (k + 63) / 64), 256, 0, s>>>(T1, K, r, Vs, r, k, sc, 1, A);
