@@ -1,15 +1,16 @@
 // Small-batch form of the layer's contraction (paper Section 3.1 / 3.2: Y = [X_q | T_q] . [W_q ; B_q];
 // Section 2.1: few tokens per step make the layer memory bound on its weights).
 //
-// The 5th-generation tensor core takes one row of the M-side operand per cycle against up to 256 columns of
-// the N-side operand (measured: a tcgen05.mma of M = 128, K = 16 takes 134 cycles whether N is 16 or 256).  So
-// with few tokens the tokens go on the M side, padded to the smallest tile (64 rows, or 128), and the weights
-// take the full 256-wide N side:
-//     D[MT tokens, 256 weight columns] += Xtile[MT, 16 K] . Wtile[256, 16 K]^T      (tcgen05.mma, bf16 -> fp32)
-// A CTA streams packed weight tiles exactly once (two 128-column tiles = 256 columns x 64 K per stage, one bulk
-// copy each), converts the 4-bit mantissas to their exact bf16 values in shared memory (as the large-batch
-// GEMM does) and multiplies them with an [MT, 64] tile of the quantised activations that TMA brings from
-// Xcat (rows beyond the batch arrive as zeros).
+// The weights are the MMA's 128-row operand and the tokens its narrow one:
+//     D[128 weight columns, N tokens] += Wtile[128, 16 K] . Xtile[N, 16 K]^T        (tcgen05.mma, bf16 -> fp32)
+// and the weight operand comes from TENSOR MEMORY: a converter thread owns a weight column, turns its packed mantissas
+// into their exact bf16 values in registers and stores them to its lane (tcgen05.st), so the converted weights never
+// touch shared memory.  An MMA of K = 16 then takes 17 cycles at N = 16, 19 at 32, 32 at 64, 64 at 128 (measured; with
+// the operand in shared memory 39 at N = 16, and 128 with the tokens on the 64- or 128-row side against 256 weight
+// columns).  A CTA streams packed weight tiles exactly once into a ring of some 200 KB, in batches of four slabs of 64 K:
+// one bulk copy for each 128-column half of the tile and one TMA load for the four [N, 64] activation tiles (every copy
+// costs its issuing thread and the copy engine a hundred cycles and more, so a slab at a time held the ring back).
+// What bounds it is the stream of weights and, close behind, the instructions that expand them (1.8 per weight).
 //
 // Work items are (layer, 256-column tile, K chunk).  The chunks of a tile are fixed by the shape alone (so a
 // result never depends on the number of SMs or on which layers share a launch); each chunk is summed from
@@ -20,11 +21,13 @@
 //               depend on no earlier kernel) and TMA loads of activation tiles (after it)
 //   warp 1      tensor memory allocation, MMA issue (the whole warp runs the loop, one elected lane issues)
 //   warps 2-5   epilogue (tcgen05.ld, Y or partial sums, the last-arriver reduction)
-//   warps 6-29  converters in three groups of 256 threads (a weight column each); group g converts the stages
-//               with index = g (mod 3), so it meets one CV slot only and its PK slots in phase order
-// Two rings: PK slots hold {activation tile, two packed weight tiles}, with a barrier for the weights and one for
-// the activations (the converters need only the former, so they work while the prologue still runs); CV slots
-// hold converted weight tiles.
+//   warps 6-29  converters in three groups of 256 threads (a weight column each); group g converts the steps
+//               with index = g (mod 3)
+// Two rings: PK slots hold a batch {four activation tiles, two halves of four packed weight tiles}, with a barrier for the
+// weights and one for the activations (the converters need only the former, so they work while the prologue still runs);
+// CV slots (tensor memory) hold a step's converted weights: two slabs, one where 128 tokens leave no room.  A step costs the
+// MMA warp some 450 cycles beside the MMAs themselves (waits, the commit, the loop): with a slab to a step that was more
+// than the eight MMAs of 32 cycles.
 #include <algorithm>
 
 #include "lqer_gemm_small.cuh"
@@ -35,42 +38,76 @@ namespace sg {
 using namespace tc;
 
 constexpr int BK = 64;
-constexpr int CV_TILE_BYTES = BN * BK * 2; // 32768
-constexpr int CV_SLOTS = 3;
+constexpr int BATCH = 4;                   // slabs of 64 K (or of 64 ranks) per PK slot
+constexpr int CV_COLS = 64;                // tensor memory columns of a converted slab: 32 for each 128-column half
+constexpr int W_HALF_BYTES = BATCH * kWTileBytes;
 constexpr int CONVERTER_GROUPS = 3;
 constexpr int WARPS_PER_GROUP = 8;
 constexpr int NUM_THREADS = (6 + CONVERTER_GROUPS * WARPS_PER_GROUP) * 32;
-constexpr int RANK_PER_STAGE = 32;
 
 __device__ __forceinline__ void epilogue_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
-template <int MT, int PK_SLOTS>
+// NT: the most tokens of the class (32, 64, 128); a launch multiplies N = M rounded up to 16 of them.
+template <int NT>
 struct Cfg {
-  static constexpr int X_TILE_BYTES = MT * 128;
-  static constexpr int PK_SLOT_BYTES = (X_TILE_BYTES + 2 * kWTileBytes + 1023) / 1024 * 1024;
-  static constexpr int OFF_PK = CV_SLOTS * CV_TILE_BYTES;
-  static constexpr int OFF_BARS = OFF_PK + PK_SLOTS * PK_SLOT_BYTES;
+  static constexpr int X_BYTES = BATCH * NT * 128;
+  static constexpr int PK_SLOT_BYTES = X_BYTES + 2 * W_HALF_BYTES;
+  static constexpr int PK_SLOTS = NT == 32 ? 4 : NT == 64 ? 3 : 2;
+  static constexpr int ACCS = NT == 32 ? 2 : 1;      // accumulators of two halves x NT columns
+  static constexpr int CV_COL0 = ACCS * 2 * NT;      // the converted weights behind them
+  static constexpr int STEP = NT == 128 ? 1 : 2;     // slabs of a CV slot: what the MMA warp waits for, issues and commits at once
+  static constexpr int CV_SLOTS = CONVERTER_GROUPS;  // one for each group
+  static constexpr int OFF_BARS = PK_SLOTS * PK_SLOT_BYTES;
   static constexpr int NUM_BARS = 3 * PK_SLOTS + 2 * CV_SLOTS + 4;
   static constexpr int SMEM_BYTES = OFF_BARS + NUM_BARS * 8 + 64 + 1024;
-  static constexpr int TMEM_COLS = 512;    // two accumulators of 256 columns
-  static_assert(MT == 64 || MT == 128, "MMA tile rows");
-  static_assert(PK_SLOTS % CONVERTER_GROUPS == 0, "a converter group must meet a PK slot in phase order");
+  static constexpr int TMEM_COLS = 512;
+  static_assert(CV_COL0 + CV_SLOTS * STEP * CV_COLS <= TMEM_COLS, "tensor memory budget");
+  static_assert(BATCH % STEP == 0, "a step lies in one batch");
+  static_assert(PK_SLOT_BYTES % 1024 == 0, "swizzled activation tiles");
   static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
 };
 
+// The X descriptor comes in halves: only its low word (the address) changes from MMA to MMA.
+__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b64 b;\n setp.ne.b32 p, %5, 0;\n mov.b64 b, {%2, %3};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n}\n"
+      ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint4& a, const uint4& b, const uint4& c, const uint4& d) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+      ::"r"(taddr), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w), "r"(c.x), "r"(c.y), "r"(c.z),
+        "r"(c.w), "r"(d.x), "r"(d.y), "r"(d.z), "r"(d.w) : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z) : "memory");
+}
+
 struct TensorMaps {
-  CUtensorMap m[MAX_LAYERS];   // Xcat of each layer: bf16 [M, K64 + k_pad], box 64 x x_rows
+  CUtensorMap m[MAX_LAYERS];   // Xcat of each layer, bf16 [M, K64 + k_pad], as [slab][row][64]: box 4 x x_rows x 64
 };
 
 
-template <int MT, int PK_SLOTS>
+// The batch that starts with slab s: up to BATCH slabs of weights, or two slabs of B_q (8-bit mantissas: eight blocks of 16
+// ranks, 16 KB, then their exponent bytes).
+__device__ __forceinline__ int batch_end(int s, int s_hi, int k_slabs) {
+  return s < k_slabs ? min(s + BATCH, min(s_hi, k_slabs)) : min(s + 2, s_hi);
+}
+constexpr int RANK_EXP_OFFSET = 8 * kTileN * 16;
+static_assert(RANK_EXP_OFFSET + 8 * kTileN <= W_HALF_BYTES, "two rank slabs");
+template <int NT>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constant__ Params p) {
-  using C = Cfg<MT, PK_SLOTS>;
+  using C = Cfg<NT>;
+  constexpr int PK_SLOTS = C::PK_SLOTS, CV_SLOTS = C::CV_SLOTS, STEP = C::STEP;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint8_t* cv_base = smem;
-  uint8_t* pk_base = smem + C::OFF_PK;
+  uint8_t* pk_base = smem;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BARS);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::NUM_BARS);
   int* last_flag = reinterpret_cast<int*>(tmem_slot + 1);
@@ -101,12 +138,6 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     fence_proxy_async_smem();
   }
   if (warp == 1) tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
-  // rows of the activation tiles beyond the batch are zero for the whole launch: TMA only ever writes the first x_rows
-  for (int i = threadIdx.x; i < PK_SLOTS * (C::X_TILE_BYTES / 16); i += NUM_THREADS) {
-    const int slot = i / (C::X_TILE_BYTES / 16), o = i % (C::X_TILE_BYTES / 16);
-    if (o * 16 >= p.x_rows * 128) *reinterpret_cast<uint4*>(pk_base + slot * C::PK_SLOT_BYTES + o * 16) = make_uint4(0u, 0u, 0u, 0u);
-  }
-  fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -116,23 +147,24 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
   if (warp == 0) {
     // ------------------------------------------------------------------ producer
     if (lane == 0) {
-      // Packed weights depend on no earlier kernel: the first PK_SLOTS stages are requested at once, and only
+      // Packed weights depend on no earlier kernel: the first PK_SLOTS batches are requested at once, and only
       // then does the producer wait for the kernel before (the prologue that writes Xcat) and request the
-      // activation tiles of those stages.
-      int pend_slot[PK_SLOTS], pend_x[PK_SLOTS], pend_layer[PK_SLOTS];
-      int npend = 0;
+      // activation tiles of those batches.  They land on a barrier of their own (x_full, used once per slot); later
+      // ones share the weights' barrier, so that the MMA warp has one barrier to watch.
+      const uint32_t x_bytes = (uint32_t)BATCH * p.x_rows * 128u;   // (slabs and rows beyond the matrix arrive as zeros)
+      int npend = 0;                                           // batches requested without their activations: the first ones
       bool waited = false;
-      // the activation tiles of the stages requested before the wait land on a barrier of their own (x_full, used
-      // once per slot); later ones share the weights' barrier, so that the MMA warp has one barrier to watch
-      auto load_x = [&](int slot, int layer, int xcol) {
-        mbar_expect_tx(x_full(slot), p.x_rows * 128);        // rows of the box beyond the batch arrive as zeros
-        tma_load_2d(smem_u32(pk_base + slot * C::PK_SLOT_BYTES), &tmaps.m[layer], xcol, 0, x_full(slot));
-      };
       auto flush = [&]() {
         pdl_wait();
-        for (int q = 0; q < npend; ++q) load_x(pend_slot[q], pend_layer[q], pend_x[q]);
-        npend = 0;
         waited = true;
+        for (int i = cta, q = 0; q < npend; i += num_ctas) {
+          const Item it = item_of(p, i);
+          const int k_slabs = p.L[it.layer].k_slabs;
+          for (int s = it.s_lo; s < it.s_hi && q < npend; s = batch_end(s, it.s_hi, k_slabs), ++q) {
+            mbar_expect_tx(x_full(q), x_bytes);
+            tma_load_3d(smem_u32(pk_base + q * C::PK_SLOT_BYTES), &tmaps.m[it.layer], 0, 0, s, x_full(q));
+          }
+        }
       };
       int pk = 0;
       uint32_t ph = 0;
@@ -141,42 +173,38 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
       for (int i = cta; i < num_items && ok; i += num_ctas) {
         const Item it = item_of(p, i);
         const Layer& ly = p.L[it.layer];
-        const int b_tile_stride = ly.r_blocks * kTileN * 17;
+        const int k_slabs = ly.k_slabs, r_blocks = ly.r_blocks, b_tile_stride = r_blocks * kTileN * 17;
         const int nt0 = 2 * it.tile;
         const int n_half = nt0 + 1 < ly.n_tiles ? 2 : 1;       // 128-column tiles of this 256-column tile that exist
-        for (int s = it.s_lo; s < it.s_hi; ++s) {
-          if (p.stall != 0 && s == it.s_hi - 1 && i + num_ctas >= num_items) { ok = false; break; }
+        for (int s = it.s_lo; s < it.s_hi;) {
+          const int e = batch_end(s, it.s_hi, k_slabs);
+          if (p.stall != 0 && e == it.s_hi && i + num_ctas >= num_items) { ok = false; break; }
           if (!waited && npend == PK_SLOTS) flush();
           if (!mbar_wait<true>(pk_free(pk), ph ^ 1, abort_flag)) { ok = false; break; }
-          const uint32_t dst = smem_u32(pk_base + pk * C::PK_SLOT_BYTES) + C::X_TILE_BYTES;
-          int xcol;
-          const uint32_t x_bytes = waited ? (uint32_t)p.x_rows * 128u : 0u;
-          if (s < ly.k_slabs) {
-            if (!LQER_IN_BOUNDS(p.status, ((size_t)(nt0 + n_half - 1) * ly.k_slabs + s) * w_tile, w_tile, ly.w_extent, 705)) { ok = false; break; }
-            mbar_expect_tx(w_full(pk), n_half * w_tile + x_bytes);
-            for (int h = 0; h < n_half; ++h)
-              bulk_load(dst + h * kWTileBytes, ly.wsec + ((size_t)(nt0 + h) * ly.k_slabs + s) * w_tile, w_tile, w_full(pk));
-            xcol = s * BK;
+          const uint32_t slot = smem_u32(pk_base + pk * C::PK_SLOT_BYTES), dst = slot + C::X_BYTES;
+          const uint32_t bar = w_full(pk);
+          if (s < k_slabs) {
+            const size_t off = ((size_t)nt0 * k_slabs + s) * w_tile, half = (size_t)k_slabs * w_tile;
+            const uint32_t bytes = (uint32_t)(e - s) * w_tile;
+            if (!LQER_IN_BOUNDS(p.status, off + (n_half - 1) * half, bytes, ly.w_extent, 705)) { ok = false; break; }
+            mbar_expect_tx(bar, n_half * bytes + (waited ? x_bytes : 0u));
+            bulk_load(dst, ly.wsec + off, bytes, bar);
+            if (n_half > 1) bulk_load(dst + W_HALF_BYTES, ly.wsec + off + half, bytes, bar);
           } else {
-            const int rs = s - ly.k_slabs;
-            const int rb0 = rs * 2, nb = min(2, ly.r_blocks - rb0);
-            if (!LQER_IN_BOUNDS(p.status, (size_t)(nt0 + n_half - 1) * b_tile_stride + (size_t)ly.r_blocks * kTileN * 16 + rb0 * kTileN,
+            const int rb0 = (s - k_slabs) * 4, nb = min((e - s) * 4, r_blocks - rb0);
+            if (!LQER_IN_BOUNDS(p.status, (size_t)(nt0 + n_half - 1) * b_tile_stride + (size_t)r_blocks * kTileN * 16 + rb0 * kTileN,
                                 nb * kTileN, ly.b_extent, 706)) { ok = false; break; }
-            mbar_expect_tx(w_full(pk), n_half * nb * (kTileN * 17) + x_bytes);
+            mbar_expect_tx(bar, n_half * nb * (kTileN * 17) + (waited ? x_bytes : 0u));
             for (int h = 0; h < n_half; ++h) {
               const uint8_t* tile = ly.bsec + (size_t)(nt0 + h) * b_tile_stride;
-              bulk_load(dst + h * kWTileBytes, tile + (size_t)rb0 * kTileN * 16, nb * kTileN * 16, w_full(pk));
-              bulk_load(dst + h * kWTileBytes + 4096, tile + (size_t)ly.r_blocks * kTileN * 16 + rb0 * kTileN, nb * kTileN, w_full(pk));
+              bulk_load(dst + h * W_HALF_BYTES, tile + (size_t)rb0 * kTileN * 16, nb * kTileN * 16, bar);
+              bulk_load(dst + h * W_HALF_BYTES + RANK_EXP_OFFSET, tile + (size_t)r_blocks * kTileN * 16 + rb0 * kTileN, nb * kTileN, bar);
             }
-            xcol = ly.K64 + rs * RANK_PER_STAGE;
           }
-          if (waited) {
-            tma_load_2d(smem_u32(pk_base + pk * C::PK_SLOT_BYTES), &tmaps.m[it.layer], xcol, 0, w_full(pk));
-          } else {
-            pend_slot[npend] = pk; pend_x[npend] = xcol; pend_layer[npend] = it.layer;
-            ++npend;
-          }
+          if (waited) tma_load_3d(slot, &tmaps.m[it.layer], 0, 0, s, bar);
+          else ++npend;
           if (++pk == PK_SLOTS) { pk = 0; ph ^= 1; }
+          s = e;
         }
       }
       if (!waited) flush();
@@ -186,47 +214,82 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     // The tensor pipe queues very few MMAs, so what the issuing warp spends between two of them beyond the pipe's
     // own time is idle time of the pipe: the whole warp runs the loop (barrier addresses and descriptors are
     // warp-uniform values) and one elected lane issues.
-    constexpr uint32_t idesc = make_idesc(MT, BN);
-    const uint32_t cv0 = smem_u32(cv_base), pk0 = smem_u32(pk_base);
-    uint32_t it_no = 0, tile_it = 0;
-    bool ok = true;
-    for (int i = cta; i < num_items && ok; i += num_ctas, ++tile_it) {
+    const uint32_t idesc = make_idesc(128, (p.M + 15) / 16 * 16);
+    // This warp shares its scheduler with six converter warps and gets every sixth or seventh issue slot, so its loop is
+    // kept short: counters instead of divisions, 32-bit descriptor arithmetic, and tensor memory addresses from the
+    // constant 0 (an allocation of all 512 columns begins there) that the compiler can keep in uniform registers.
+    const uint32_t x_tile = (uint32_t)p.x_rows * (128u >> 4);           // in descriptor units of 16 bytes
+    const uint64_t desc0 = make_desc(smem_u32(pk_base));
+    const uint32_t b_hi = (uint32_t)(desc0 >> 32), b_lo0 = (uint32_t)desc0;
+    uint32_t cv = 0, cv_ph = 0, pk = 0, acc = 0, acc_ph = 1;
+    bool first_pass = true, ok = true;
+    for (int i = cta; i < num_items && ok; i += num_ctas) {
       const Item it = item_of(p, i);
-      const Layer& ly = p.L[it.layer];
-      const int acc = tile_it & 1;
-      ok = __all_sync(0xFFFFFFFFu, mbar_wait(acc_empty(acc), ((tile_it >> 1) & 1) ^ 1, abort_flag)) != 0;
+      const int k_slabs = p.L[it.layer].k_slabs, r_blocks = p.L[it.layer].r_blocks;
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(acc_empty(acc), acc_ph, abort_flag)) != 0;
       if (!ok) break;
       tc_fence_after();
-      const uint32_t d_tmem = tmem_base + acc * BN;
-      for (int s = it.s_lo; s < it.s_hi; ++s, ++it_no) {
-        const int cv = it_no % CV_SLOTS, pk = it_no % PK_SLOTS;
-        const uint64_t a_desc = make_desc(pk0 + pk * C::PK_SLOT_BYTES);
-        const uint64_t b_desc = make_desc(cv0 + cv * CV_TILE_BYTES);
-        const int nk = s < ly.k_slabs ? 4 : min(2, ly.r_blocks - (s - ly.k_slabs) * 2);
-        // a converted tile implies its packed tile had landed, and with it (from the second pass over the ring on) the
-        // activation tile; on the first pass the activation tiles have their own barrier
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(cv_ready(cv), (it_no / CV_SLOTS) & 1, abort_flag) &&
-                                         (it_no >= (uint32_t)PK_SLOTS || mbar_wait(x_full(pk), 0, abort_flag))) != 0;
-        if (!ok) break;
-        tc_fence_after();
-        if (elect_one()) {
-          for (int j = 0; j < nk; ++j)              // +2 in the address field = 32 bytes = 16 K
-            umma_bf16(d_tmem, a_desc + 2 * j, b_desc + 2 * j, idesc, (s > it.s_lo || j > 0) ? 1u : 0u);
-          umma_commit(cv_free(cv));
-          umma_commit(pk_free(pk));
+      const uint32_t d_tmem = acc * 2 * NT;
+      uint32_t add = 0u;
+      for (int s = it.s_lo; s < it.s_hi && ok;) {
+        const int e = batch_end(s, it.s_hi, k_slabs);
+        // a converted slab implies its batch had landed, and with it (from the second pass over the ring on) the
+        // activation tiles; on the first pass the activation tiles have their own barrier
+        if (first_pass) {
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(x_full(pk), 0, abort_flag)) != 0;
+          if (!ok) break;
         }
-        __syncwarp();
+        uint32_t b_lo = b_lo0 + pk * (C::PK_SLOT_BYTES >> 4);
+        const int whole_end = s < k_slabs ? e : s;                       // steps up to here are whole slabs of weights
+        for (; s < e; s += STEP) {
+          const uint32_t w = C::CV_COL0 + cv * (STEP * CV_COLS);
+          const uint32_t free_bar = cv_free(cv);
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(cv_ready(cv), cv_ph, abort_flag)) != 0;
+          if (!ok) break;
+          tc_fence_after();
+          if (elect_one()) {
+            // 16 K = 8 tensor memory columns; +2 in the address field = 32 bytes.  (Unrolled with constant offsets: a loop over
+            // the K steps and the halves issued one MMA per 130 cycles.)
+            if (s + STEP <= whole_end) {
+              umma_bf16_ts(d_tmem, w, b_lo, b_hi, idesc, add);
+              umma_bf16_ts(d_tmem + NT, w + 32, b_lo, b_hi, idesc, add);
+#pragma unroll
+              for (int j = 1; j < 4 * STEP; ++j) {
+                const uint32_t x = b_lo + (j >= 4 ? x_tile : 0u) + 2 * (j & 3);
+                umma_bf16_ts(d_tmem, w + (j >> 2) * CV_COLS + (j & 3) * 8, x, b_hi, idesc, 1u);
+                umma_bf16_ts(d_tmem + NT, w + (j >> 2) * CV_COLS + (j & 3) * 8 + 32, x, b_hi, idesc, 1u);
+              }
+            } else {
+              for (int t = 0; t < STEP && s + t < e; ++t) {
+                const int nk = s + t < k_slabs ? 4 : min(4, r_blocks - (s + t - k_slabs) * 4);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                  if (j < nk) {
+                    const uint32_t on = t + j > 0 ? 1u : add, x = b_lo + t * x_tile + 2 * j;
+                    umma_bf16_ts(d_tmem, w + t * CV_COLS + j * 8, x, b_hi, idesc, on);
+                    umma_bf16_ts(d_tmem + NT, w + t * CV_COLS + j * 8 + 32, x, b_hi, idesc, on);
+                  }
+              }
+            }
+            umma_commit(free_bar);
+            if (s + STEP >= e) umma_commit(pk_free(pk));
+          }
+          __syncwarp();
+          add = 1u;
+          b_lo += STEP * x_tile;
+          if (++cv == CV_SLOTS) { cv = 0; cv_ph ^= 1; }
+        }
+        s = e;
+        if (++pk == PK_SLOTS) { pk = 0; first_pass = false; }
       }
       if (ok && elect_one()) umma_commit(acc_full(acc));
       __syncwarp();
+      if (++acc == C::ACCS) { acc = 0; acc_ph ^= 1; }
     }
   } else if (warp < 6) {
     // ------------------------------------------------------------------ epilogue
-    // A lane of tensor memory holds a token: the 128-row MMA puts row r in lane r, the 64-row MMA puts rows
-    // 16 q .. 16 q + 15 in the first 16 lanes of lane quarter q.
+    // A lane of tensor memory holds a weight column, its columns the tokens: a token's 32 values of a warp are neighbours.
     const int q = warp & 3;
-    const int token = MT == 128 ? q * 32 + lane : (lane < 16 ? q * 16 + lane : p.M);
-    const bool warp_has_rows = (MT == 128 ? q * 32 : q * 16) < p.M;
     const int et = threadIdx.x - 64;               // 0..127: index among the epilogue threads
     uint32_t tile_it = 0;
     bool ok = true;
@@ -234,52 +297,54 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     for (int i = cta; i < num_items && ok; i += num_ctas, ++tile_it) {
       const Item it = item_of(p, i);
       const Layer& ly = p.L[it.layer];
-      const int acc = tile_it & 1;
-      if (!mbar_wait<true>(acc_full(acc), (tile_it >> 1) & 1, abort_flag)) { ok = false; break; }
+      const int acc = tile_it % C::ACCS;
+      if (!mbar_wait<true>(acc_full(acc), (tile_it / C::ACCS) & 1, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      const int col0 = it.tile * BN;
       const bool direct = ly.chunks == 1;
-      if (warp_has_rows) {
-        float* prow = direct ? nullptr : ly.partials + ((size_t)(it.tile * ly.chunks + it.chunk) * p.M + token) * BN;
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 32) {
-          if (col0 + c0 >= ly.N) break;
-          uint32_t r[32];
-          tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + c0, r);
+      for (int h = 0; h < 2; ++h) {
+        const int ccol = h * 128 + q * 32 + lane, col = it.tile * BN + ccol;
+        if (it.tile * BN + h * 128 >= ly.N) break;
+        const size_t pbase = (size_t)(it.tile * ly.chunks + it.chunk) * p.M * BN + ccol;
+#pragma unroll 1
+        for (int t0 = 0; t0 < p.M; t0 += 16) {
+          uint32_t r[16];
+          tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + acc * 2 * NT + h * NT + t0, r);
           tmem_ld_wait();
-          if (token < p.M) {
-            if (direct && p.y_type == kYMXINT8) {
-              // a token's 32 columns are two whole 16-blocks of its row
-              const QuantConsts qc = quant_consts(p.a_bits, p.exp_min, p.exp_max);
-              uint8_t* yq = static_cast<uint8_t*>(ly.Y);
+          if (!direct) {
 #pragma unroll
-              for (int j = 0; j < 2; ++j)
-                if (col0 + c0 + 16 * j < ly.N) {          // N is a multiple of 16 here
-                  float v[16];
+            for (int t = 0; t < 16; ++t) {
+              const size_t idx = pbase + (size_t)(t0 + t) * BN;
+              if (t0 + t < p.M && LQER_IN_BOUNDS(p.status, idx * 4, 4, ly.partial_extent, 704)) ly.partials[idx] = __uint_as_float(r[t]);
+            }
+          } else if (p.y_type == kYMXINT8) {
+            // sixteen lanes hold a 16-block of a token's row (N is a multiple of 16 here)
+            uint8_t* yq = static_cast<uint8_t*>(ly.Y);
 #pragma unroll
-                  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[16 * j + i]);
-                  uint4 m8, b0, b1;
-                  int e;
-                  quantize_block16(v, qc, e, m8, b0, b1);
-                  const size_t idx = (size_t)token * ly.N + col0 + c0 + 16 * j;
-                  if (LQER_IN_BOUNDS(p.status, (size_t)p.M * ly.N + idx / 16, 1, ly.y_extent, 703)) {
-                    *reinterpret_cast<uint4*>(yq + idx) = m8;
-                    yq[(size_t)p.M * ly.N + idx / 16] = (uint8_t)(e + 127);
-                  }
-                }
-            } else {
+            for (int t = 0; t < 16; ++t) {
+              const float v = __uint_as_float(r[t]);
+              float amax = fmaxf(fabsf(v), 0.0f);            // (a NaN counts as zero)
 #pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const float4 v = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]), __uint_as_float(r[4 * j + 2]),
-                                             __uint_as_float(r[4 * j + 3]));
-                if (!direct) {
-                  if (LQER_IN_BOUNDS(p.status, (size_t)(prow + c0 + 4 * j - ly.partials) * 4, 16, ly.partial_extent, 704))
-                    *reinterpret_cast<float4*>(prow + c0 + 4 * j) = v;
-                }
-                else if (col0 + c0 + 4 * j < ly.N) store_y4(ly.Y, (size_t)token * ly.N + col0 + c0 + 4 * j, v, p.y_type, p.status, ly.y_extent);   // N is a multiple of 8
+              for (int d = 1; d < 16; d <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, d));
+              const int e = block_exponent(amax, p.exp_min, p.exp_max);
+              const size_t idx = (size_t)(t0 + t) * ly.N + col;
+              if (t0 + t < p.M && col < ly.N && LQER_IN_BOUNDS(p.status, (size_t)p.M * ly.N + idx / 16, 1, ly.y_extent, 703)) {
+                yq[idx] = (uint8_t)quant_mantissa(v, e, p.a_bits);
+                if ((lane & 15) == 0) yq[(size_t)p.M * ly.N + idx / 16] = (uint8_t)(e + 127);
+              }
+            }
+          } else if (col < ly.N) {
+#pragma unroll
+            for (int t = 0; t < 16; ++t) {
+              const size_t idx = (size_t)(t0 + t) * ly.N + col;
+              const int size = p.y_type == kYBF16 ? 2 : 4;
+              if (t0 + t < p.M && LQER_IN_BOUNDS(p.status, idx * size, size, ly.y_extent, 701)) {
+                if (p.y_type == kYBF16) static_cast<uint16_t*>(ly.Y)[idx] = (uint16_t)bf16_rn(__uint_as_float(r[t]));
+                else static_cast<float*>(ly.Y)[idx] = __uint_as_float(r[t]);
               }
             }
           }
+          __syncwarp();
         }
       }
       tc_fence_before();
@@ -308,49 +373,91 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     // ------------------------------------------------------------------ converters
     const int c = threadIdx.x - 6 * 32;          // 0..767
     const int group = c >> 8, col = c & 255;     // stage group; weight column of the 256-column stage
-    const int half = col >> 7, nl = col & 127;   // its 128-column packed tile, and the column within it
-    const int sw = col & 7;
-    uint32_t chunk[8];                           // the row's eight 16-byte chunks after the 128-byte swizzle
-#pragma unroll
-    for (int i = 0; i < 8; ++i) chunk[i] = (uint32_t)(col * 128 + ((i ^ sw) << 4));
-    // the CTA's items one after the other; their K stages form one sequence of which this group takes every third
-    int item = cta, s = group;                   // s: offset into the current item's stages; normalised below
-    Item cur;
-    cur.layer = 0; cur.tile = 0; cur.chunk = 0; cur.s_lo = 0; cur.s_hi = 0;
-    if (item < num_items) cur = item_of(p, item);
+    const int half = col >> 7;                   // its 128-column packed tile; the column within it is the thread's lane of
+    const int nl = (warp & 3) * 32 + lane;       // tensor memory: a warp writes the lanes of its number mod 4
+    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    // the CTA's items one after the other; their slabs form one sequence of which this group takes every third
+    uint32_t it_no = 0, batch_no = 0;
     bool ok = true;
-    for (uint32_t it_no = group; item < num_items && ok; it_no += CONVERTER_GROUPS, s += CONVERTER_GROUPS) {
-      while (item < num_items && s >= cur.s_hi - cur.s_lo) {
-        s -= cur.s_hi - cur.s_lo;
-        item += num_ctas;
-        if (item < num_items) cur = item_of(p, item);
-      }
-      if (item >= num_items) break;
-      const Layer& ly = p.L[cur.layer];
-      const int stage = cur.s_lo + s;
-      const int pk = it_no % PK_SLOTS;
-      const bool has_w = 2 * cur.tile + half < ly.n_tiles;
-      if (!mbar_wait(w_full(pk), (it_no / PK_SLOTS) & 1, abort_flag)) { ok = false; break; }
-      if (!mbar_wait(cv_free(group), ((it_no / CV_SLOTS) & 1) ^ 1, abort_flag)) { ok = false; break; }
-      const uint8_t* pkt = pk_base + pk * C::PK_SLOT_BYTES + C::X_TILE_BYTES + half * kWTileBytes;
-      uint8_t* bt = cv_base + group * CV_TILE_BYTES;
-      if (!has_w) {                                // columns beyond N: a zero operand row
-        const int nchunks = stage < ly.k_slabs ? 8 : 4;
-        for (int i = 0; i < nchunks; ++i) *reinterpret_cast<uint4*>(bt + chunk[i]) = make_uint4(0u, 0u, 0u, 0u);
-      } else if (stage < ly.k_slabs) {
-        convert_column(pkt, nl, p.w_bits, bt, chunk);
-      } else {
-        const int nb = min(2, ly.r_blocks - (stage - ly.k_slabs) * 2);
-        for (int rb = 0; rb < nb; ++rb) {
-          const uint4 w = *reinterpret_cast<const uint4*>(pkt + (rb * kTileN + nl) * 16);
-          const float scale = pow2f((int)pkt[4096 + rb * kTileN + nl] - 127 - p.lr_shift);
-          *reinterpret_cast<uint4*>(bt + chunk[rb * 2]) = convert_i8x8(w.x, w.y, scale);
-          *reinterpret_cast<uint4*>(bt + chunk[rb * 2 + 1]) = convert_i8x8(w.z, w.w, scale);
+    const int w_tile = w_tile_bytes(p.w_bits);
+    for (int item = cta; item < num_items && ok; item += num_ctas) {
+      const Item it = item_of(p, item);
+      const int k_slabs = p.L[it.layer].k_slabs, r_blocks = p.L[it.layer].r_blocks;
+      const bool has_w = 2 * it.tile + half < p.L[it.layer].n_tiles;
+      for (int s0 = it.s_lo; s0 < it.s_hi && ok; ++batch_no) {
+        const int e = batch_end(s0, it.s_hi, k_slabs), pk = batch_no % PK_SLOTS;
+        // (also where none of the batch's slabs is this group's: a group must not get a pass ahead of a slot's barrier)
+        if (!mbar_wait(w_full(pk), (batch_no / PK_SLOTS) & 1, abort_flag)) { ok = false; break; }
+        const uint8_t* pkh = pk_base + pk * C::PK_SLOT_BYTES + C::X_BYTES + half * W_HALF_BYTES;
+        for (int st = s0; st < e; st += STEP, ++it_no) {
+          if (it_no % CONVERTER_GROUPS != (uint32_t)group) continue;
+          if (!mbar_wait(cv_free(group), ((it_no / CV_SLOTS) & 1) ^ 1, abort_flag)) { ok = false; break; }
+          tc_fence_after();                            // the MMAs that read the slot before have finished
+          if (has_w)                                   // (a missing half multiplies what its lanes happen to hold: nobody reads it)
+            for (int s = st; s < min(st + STEP, e); ++s) {
+              const uint32_t dst = tmem_base + lane_base + C::CV_COL0 + (group * STEP + s - st) * CV_COLS + half * 32;
+              uint4 o[4];
+              const uint8_t* pkt = pkh + (s - s0) * w_tile;
+              if (s >= k_slabs) {
+                // 64 ranks: four blocks of 16
+                const int rb0 = (s - s0) * 4, nb = min(4, r_blocks - (s - k_slabs) * 4);
+      #pragma unroll
+                for (int hp = 0; hp < 2; ++hp) {
+      #pragma unroll
+                  for (int rb = 0; rb < 2; ++rb) {
+                    o[2 * rb] = make_uint4(0u, 0u, 0u, 0u);
+                    o[2 * rb + 1] = o[2 * rb];
+                    if (2 * hp + rb < nb) {
+                      const uint4 w = *reinterpret_cast<const uint4*>(pkh + ((rb0 + 2 * hp + rb) * kTileN + nl) * 16);
+                      const float scale = pow2f((int)pkh[RANK_EXP_OFFSET + (rb0 + 2 * hp + rb) * kTileN + nl] - 127 - p.lr_shift);
+                      o[2 * rb] = convert_i8x8(w.x, w.y, scale);
+                      o[2 * rb + 1] = convert_i8x8(w.z, w.w, scale);
+                    }
+                  }
+                  tmem_st16(dst + 16 * hp, o[0], o[1], o[2], o[3]);
+                }
+              } else if (p.w_bits == 2) {
+                const uint4 wv = *reinterpret_cast<const uint4*>(pkt + nl * 16);
+                const uint32_t eb = *reinterpret_cast<const uint32_t*>(pkt + 2048 + nl * 4);
+                uint32_t s2, c2;
+                w_scales2(eb & 0xFFu, s2, c2);
+                convert_word2(wv.x, s2, c2, o[0], o[1]);
+                w_scales2((eb >> 8) & 0xFFu, s2, c2);
+                convert_word2(wv.y, s2, c2, o[2], o[3]);
+                tmem_st16(dst, o[0], o[1], o[2], o[3]);
+                w_scales2((eb >> 16) & 0xFFu, s2, c2);
+                convert_word2(wv.z, s2, c2, o[0], o[1]);
+                w_scales2(eb >> 24, s2, c2);
+                convert_word2(wv.w, s2, c2, o[2], o[3]);
+                tmem_st16(dst + 16, o[0], o[1], o[2], o[3]);
+              } else {
+                const uint4 wa = *reinterpret_cast<const uint4*>(pkt + nl * 16);
+                const uint4 wb = *reinterpret_cast<const uint4*>(pkt + (kTileN + nl) * 16);
+                const uint32_t eb = *reinterpret_cast<const uint32_t*>(pkt + kWTileNibbleBytes + nl * 4);
+                uint32_t s2, c2;
+                w_scales(eb & 0xFFu, s2, c2);
+                o[0] = convert_word(wa.x, s2, c2);
+                o[1] = convert_word(wa.y, s2, c2);
+                w_scales((eb >> 8) & 0xFFu, s2, c2);
+                o[2] = convert_word(wa.z, s2, c2);
+                o[3] = convert_word(wa.w, s2, c2);
+                tmem_st16(dst, o[0], o[1], o[2], o[3]);
+                w_scales((eb >> 16) & 0xFFu, s2, c2);
+                o[0] = convert_word(wb.x, s2, c2);
+                o[1] = convert_word(wb.y, s2, c2);
+                w_scales(eb >> 24, s2, c2);
+                o[2] = convert_word(wb.z, s2, c2);
+                o[3] = convert_word(wb.w, s2, c2);
+                tmem_st16(dst + 16, o[0], o[1], o[2], o[3]);
+              }
+            }
+          tmem_st_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(cv_ready(group));
         }
+        s0 = e;
       }
-      fence_proxy_async_smem();        // generic-proxy writes -> visible to the MMA's async proxy
-      __syncwarp();
-      if (lane == 0) mbar_arrive(cv_ready(group));
     }
   }
 
@@ -391,12 +498,12 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-template <int MT, int PK_SLOTS>
-static cudaError_t launch_mt(const TensorMaps& tmaps, const Params& p, int ctas, cudaStream_t s) {
-  using C = Cfg<MT, PK_SLOTS>;
+template <int NT>
+static cudaError_t launch_nt(const TensorMaps& tmaps, const Params& p, int ctas, cudaStream_t s) {
+  using C = Cfg<NT>;
   static OncePerDevice once;
   cudaError_t e = once.run([] {
-    return cudaFuncSetAttribute(gemm_small_kernel<MT, PK_SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+    return cudaFuncSetAttribute(gemm_small_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
   });
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -410,7 +517,7 @@ static cudaError_t launch_mt(const TensorMaps& tmaps, const Params& p, int ctas,
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   LaunchScope scope(kFamDecode, s);
-  return cudaLaunchKernelEx(&cfg, gemm_small_kernel<MT, PK_SLOTS>, tmaps, p);
+  return cudaLaunchKernelEx(&cfg, gemm_small_kernel<NT>, tmaps, p);
 }
 
 }  // namespace sg
@@ -425,26 +532,23 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
   const bool use_mma = !tensor_memory_form && small_takes_mma(*layers[0].meta, M);
   EncodeTiledFn enc = use_mma ? nullptr : encode_fn();
   if (enc == nullptr && !use_mma) return cudaErrorNotSupported;
-  const int MT = M <= 64 ? 64 : 128;
-  const int x_rows = (M + 7) / 8 * 8;
+  const int x_rows = (M + 15) / 16 * 16;
   TensorMaps tmaps;
   Params p;
   int item_begin = 0;
   // K chunks per tile.  A layer alone is cut as its shape says (small_gemm_chunks: enough work items for every SM).
-  // Layers that share a launch bring many tiles between them, and every chunk costs a pass of partial sums through
-  // L2, so they are cut less: just enough for about two work items per SM in all, never more than alone (the scratch
-  // is sized for that; finer cuts that would even out the last round of items were measured and lose more in
-  // epilogues than they gain).  The sums of a tile are then grouped differently, so a layer's result in a shared launch
-  // may differ from its result alone in the last bits; it is the same whenever the same layers share a launch.
+  // Layers that share a launch bring many tiles between them; they are cut by the time model below, never finer than alone
+  // (the scratch is sized for that).  The sums of a tile are then grouped differently, so a layer's result in a shared
+  // launch may differ from its result alone in the last bits; it is the same whenever the same layers share a launch.
   const int sms = sm_count();
   if (sms < 1) return cudaErrorInvalidDevice;
-  int total_tiles = 0;
-  for (int i = 0; i < n; ++i) total_tiles += small_gemm_col_tiles(*layers[i].meta);
-  int group_chunks = (2 * 148 + total_tiles - 1) / total_tiles;            // about two work items per SM in all
-  if (use_mma && n > 1) {
-    // The register-operand kernel runs two CTAs per SM, an item each at a time, and an item costs about ten slabs' worth
-    // of time beside its own slabs (activation copy, rank term, partial sums): the cut that makes (rounds of items over
-    // 2 x 148 CTAs) x (slabs per item + 10) smallest, a function of the shapes alone like the rule above.
+  int group_chunks = 1;
+  if (n > 1) {
+    // The cut that makes (rounds of items over the SMs) x (slabs per item + what an item costs beside its slabs) smallest,
+    // a function of the shapes alone.  This file's kernel runs one CTA per SM and an item's partial sums cost it about four
+    // slabs' worth of time; the register-operand kernel runs two CTAs per SM, an item each at a time, and an item costs it
+    // about ten (activation copy, rank term, partial sums).
+    const int ctas = use_mma ? 2 * 148 : 148, extra = use_mma ? 10 : 4;
     long best = -1;
     for (int c = 1; c <= 16; ++c) {
       long items = 0, len = 0;
@@ -454,7 +558,7 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
         items += (long)small_gemm_col_tiles(m) * ci;
         len = std::max(len, (long)(m.k_slabs + ci - 1) / ci);
       }
-      const long cost = ((items + 2 * 148 - 1) / (2 * 148)) * (len + 10);
+      const long cost = ((items + ctas - 1) / ctas) * (len + extra);
       if (best < 0 || cost < best) { best = cost; group_chunks = c; }
     }
   }
@@ -462,12 +566,14 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
     const SmallGemmLayer& src = layers[i < n ? i : 0];
     const PackedMeta& m = *src.meta;
     if (m.lr_bits != layers[0].meta->lr_bits || m.w_bits != layers[0].meta->w_bits) return cudaErrorInvalidValue;
-    const cuuint64_t dims[2] = {(cuuint64_t)xcat_cols(m), (cuuint64_t)M};
-    const cuuint64_t strides[1] = {(cuuint64_t)xcat_cols(m) * 2};
-    const cuuint32_t box[2] = {BK, (cuuint32_t)x_rows};
-    const cuuint32_t estr[2] = {1, 1};
+    // [slab][row][64 columns]; the last slab of T_q may reach past the end of a row (its columns beyond k_pad are never
+    // multiplied) and, in the last row, up to 96 bytes past Xcat, where the layer's partial sums of T lie
+    const cuuint64_t dims[3] = {64, (cuuint64_t)M, (cuuint64_t)(m.k_slabs + frag_rank_slabs(m))};
+    const cuuint64_t strides[2] = {(cuuint64_t)xcat_cols(m) * 2, 128};
+    const cuuint32_t box[3] = {BK, (cuuint32_t)x_rows, BATCH};
+    const cuuint32_t estr[3] = {1, 1, 1};
     if (!use_mma &&
-        enc(&tmaps.m[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(src.xcat), dims, strides, box, estr,
+        enc(&tmaps.m[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(src.xcat), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
@@ -486,7 +592,7 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
     ly.counters = src.counters;
     ly.N = m.N; ly.K64 = m.K64;
     ly.n_tiles = m.n_tiles; ly.k_slabs = m.k_slabs; ly.r_blocks = m.r_blocks;
-    ly.spt = m.k_slabs + (m.r_blocks + 1) / 2;
+    ly.spt = m.k_slabs + (use_mma ? (m.r_blocks + 1) / 2 : frag_rank_slabs(m));
     int want = small_gemm_chunks(m);
     if (n > 1 && group_chunks < want) want = group_chunks;
     ly.chunk_stages = (m.k_slabs + want - 1) / want;
@@ -510,7 +616,7 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
   p.stall = take_stall(kFamDecode) ? 1 : 0;
   if (use_mma) return launch_gemm_mma(p, s);
   const int ctas = p.num_items < sms ? p.num_items : sms;
-  return MT == 64 ? launch_mt<64, 6>(tmaps, p, ctas, s) : launch_mt<128, 3>(tmaps, p, ctas, s);
+  return M <= 32 ? launch_nt<32>(tmaps, p, ctas, s) : M <= 64 ? launch_nt<64>(tmaps, p, ctas, s) : launch_nt<128>(tmaps, p, ctas, s);
 }
 
 }  // namespace lqer

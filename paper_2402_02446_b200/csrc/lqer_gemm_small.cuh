@@ -37,7 +37,7 @@ struct Params {
   int y_type;                  // kYF32; kYBF16 (round to nearest even); kYMXINT8 (blocks of 16 along N, format below)
   int a_bits, exp_min, exp_max;// activation format, for an MXINT8 Y
   int w_bits;                  // mantissa bits of W_q: 4 or 2 (one value for all layers of a launch)
-  int x_rows;                  // rows of an activation tile that TMA fills: M rounded up to 8 (the rest stay zero)
+  int x_rows;                  // rows of an activation tile: M rounded up to 16 (those beyond M arrive as zeros)
   long long wait_limit;
   int epoch;                   // register-operand kernel: the value the prologue's flags take in this call
   int* exit_count;             // ... and a zeroed counter of the CTAs that have left (the last one clears the flags)
