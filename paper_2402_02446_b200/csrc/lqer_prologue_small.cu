@@ -2,10 +2,11 @@
 // small high-precision product X A_k), built for latency: a decode step of a few tokens is a chain of short
 // kernels, so this one spreads even 16 rows over many CTAs and has no wait in it.
 //
-//   grid = row groups (16 rows of X each) x K ranges (up to 16 per row group)
+//   grid = row groups (16 rows of X each) x K ranges (up to 16 per row group) x shares of a range (a cluster)
 //   CTA (r, g):  X[16 rows, K range] fp32/bf16 -> MXINT8 -> exact bf16 values into Xcat[:, K range]
 //                partial T = X_q A_q over its K range: one int8 mma.sync (m16n8k16, exact int32) per
 //                (16-block, 8 rank columns), scaled by 2^(e_x + e_a) and summed in fp64
+//                -> the cluster adds its shares up through distributed shared memory, in rank order
 //                -> slot (r, g) of the scratch; then it counts itself in.
 //   The CTA that arrives LAST for a row group (no one waits for anyone) adds the slots in range order,
 //   re-quantises T along the rank and appends T_q to Xcat[:, K64 : K64 + k_pad].
@@ -48,6 +49,7 @@ struct Params {
   int a_bits, lr_bits, exp_min, exp_max;
   int frag;                   // Xcat in the fragment order of the register-operand GEMM (M <= 16), with its flags
   int epoch;                  // value the flags take in this launch
+  int shares;                 // CTAs (a cluster) that share a K range: a power of two up to 8
 };
 
 // Byte offset of (row, column c of slab s) in the fragment order; plane: bytes of one plane.
@@ -57,19 +59,41 @@ __device__ __forceinline__ size_t frag_offset(int row, int slab, int c, size_t p
 }
 
 // TPW: rank tiles (8 columns) a warp owns: 1 for ranks up to 64, 2 up to 128, 4 up to 256.
+// The kernel is a chain of memory latencies, so a round requests as much as the registers hold: the A_q words of UB blocks
+// (those of a CTA's first blocks before it waits for the kernel before, on which they do not depend) and eight quads
+// of X per thread.  With four blocks and four quads a round it took 15 - 29 us at K = 5120 - 13824 and ranks 32 and 64, of
+// which 5 - 10 us were rounds of A_q.
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// A double at the same shared-memory offset in another CTA of the cluster.
+__device__ __forceinline__ double ld_dsmem(const double* local, uint32_t cta) {
+  uint32_t remote;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(cta));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(remote) : "memory");
+  return v;
+}
+
 template <int TPW>
-__global__ void __launch_bounds__(kThreads, TPW == 1 ? 3 : TPW == 2 ? 2 : 1) prologue_small_kernel(const __grid_constant__ Params p) {
+__global__ void __launch_bounds__(kThreads, TPW == 4 ? 1 : 2) prologue_small_kernel(const __grid_constant__ Params p) {
   __shared__ __align__(16) uint8_t s_xq[kRows * kXqStride];
   __shared__ int8_t s_xe[kRows][kStepCols / 16];
   __shared__ double s_part[kWarps][kRows * 8];        // warps that share a rank tile meet here (TPW == 1)
   __shared__ int s_last;
+  extern __shared__ double s_t[];                     // [16][k_pad]: this CTA's share of the range's partial sums
 
   int layer = 0;
 #pragma unroll
   for (int i = 1; i < kMaxLayers; ++i)
     if (i < p.n && (int)blockIdx.x >= p.L[i].cta_begin) layer = i;
   const Layer& ly = p.L[layer];
-  const int bid = (int)blockIdx.x - ly.cta_begin;
+  const int shares = p.shares, share = (int)cluster_rank();
+  const int bid = ((int)blockIdx.x - ly.cta_begin) / shares;
   const int rgroup = bid / ly.ranges, range = bid % ly.ranges;
   const int row0 = rgroup * kRows;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -77,7 +101,8 @@ __global__ void __launch_bounds__(kThreads, TPW == 1 ? 3 : TPW == 2 ? 2 : 1) pro
   const int M = p.M, K = ly.K, k_pad = ly.k_pad;
   const size_t ldx = (size_t)ly.K64 + (size_t)k_pad;
   const int KB64 = ly.K64 / 16, kblocks = K / 16;
-  const int kb_lo = (int)((long long)range * KB64 / ly.ranges), kb_hi = (int)((long long)(range + 1) * KB64 / ly.ranges);
+  const int kr0 = (int)((long long)range * KB64 / ly.ranges), kr1 = (int)((long long)(range + 1) * KB64 / ly.ranges);
+  const int kb_lo = kr0 + share * (kr1 - kr0) / shares, kb_hi = kr0 + (share + 1) * (kr1 - kr0) / shares;
   const uint8_t* a_exp = ly.asec + (size_t)kblocks * k_pad * 16;
   const int NT = k_pad / 8;                              // 8-column rank tiles
   const int WPN = NT >= kWarps ? 1 : kWarps / NT;        // warps that share one rank tile (they split the blocks)
@@ -85,6 +110,25 @@ __global__ void __launch_bounds__(kThreads, TPW == 1 ? 3 : TPW == 2 ? 2 : 1) pro
   const size_t plane = (size_t)(ly.K64 / 64 + (k_pad + 63) / 64) * 256;      // fragment order: bytes of one plane
   const bool active = has_rank && (NT >= kWarps || warp < NT * WPN);
   const int bias = -127 - (p.a_bits - 2) - (p.lr_bits - 2);   // exponent bytes carry +127
+  constexpr int UB = TPW == 1 ? 16 : TPW == 2 ? 8 : 4;
+  const int b_first = NT >= kWarps ? 0 : warp / NT;
+  const int b_step = NT >= kWarps ? 1 : WPN;
+  const int nt0 = NT >= kWarps ? warp : warp % NT;
+  uint32_t bw[UB][TPW], ew[UB][TPW];
+  // A_q words of blocks b, b + b_step, .. of the step that begins with block kb0 and has nreal real ones
+  auto load_a = [&](int kb0, int bq, int nreal) {
+#pragma unroll
+    for (int u = 0; u < UB; ++u) {
+      const int b = bq + u * b_step;
+      const size_t kb = (size_t)(kb0 + b);
+#pragma unroll
+      for (int i = 0; i < TPW; ++i) {
+        const int nt = min(nt0 + kWarps * i, NT - 1);
+        bw[u][i] = b < nreal ? __ldg(reinterpret_cast<const uint32_t*>(ly.asec + (kb * k_pad + nt * 8 + g) * 16 + tig * 4)) : 0u;
+        ew[u][i] = b < nreal ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(a_exp + kb * k_pad + nt * 8 + tig * 2)) : 0u;
+      }
+    }
+  };
 
   // The kernel after this one (the GEMM) may start at once: it only prefetches weights before its own wait.
   // This CTA's share of A_q depends on no earlier kernel: on its way to L2 while the kernel before drains.
@@ -97,6 +141,7 @@ __global__ void __launch_bounds__(kThreads, TPW == 1 ? 3 : TPW == 2 ? 2 : 1) pro
     for (int o = tid * 128; o < mant; o += kThreads * 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(gm + o));
     for (int o = tid * 128; o < ex; o += kThreads * 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(ge + o));
   }
+  if (active) load_a(kb_lo, b_first, min(min(kStepCols / 16, kb_hi - kb_lo), kblocks - kb_lo));
   // X and the workspace may still be in use by the kernel before: wait for it.
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -111,11 +156,10 @@ __global__ void __launch_bounds__(kThreads, TPW == 1 ? 3 : TPW == 2 ? 2 : 1) pro
     // ---- quantise 16 rows x (nblk * 16) columns: bf16 to Xcat, int8 + exponents to shared memory
     const int quads_per_row = nblk * 4;
     const int n_quads = kRows * quads_per_row;                             // a multiple of 64
-    for (int f0 = 0; f0 < n_quads; f0 += 4 * kThreads) {                  // whole warps: the block maximum is a shuffle
-      // four loads per thread in flight, then the arithmetic: a kernel this short is a chain of memory latencies
-      float4 v[4];
+    for (int f0 = 0; f0 < n_quads; f0 += 8 * kThreads) {                  // whole warps: the block maximum is a shuffle
+      float4 v[8];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < 8; ++u) {
         const int f = f0 + u * kThreads + tid;
         const bool live = f < n_quads;
         const int r = live ? f / quads_per_row : 0, c4 = live ? f % quads_per_row : 0;
@@ -124,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, TPW == 1 ? 3 : TPW == 2 ? 2 : 1) pro
         if (live && row < M && col < K) v[u] = load_x_quad(ly.X, p.x_type, M, K, row, col, p.a_bits, p.exp_min, p.exp_max);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < 8; ++u) {
         const int f = f0 + u * kThreads + tid;
         if (f0 + u * kThreads >= n_quads) break;                           // uniform over the CTA
         const bool live = f < n_quads;
@@ -153,33 +197,18 @@ __global__ void __launch_bounds__(kThreads, TPW == 1 ? 3 : TPW == 2 ? 2 : 1) pro
     const bool last_step = kb0 + kStepCols / 16 >= kb_hi;
     if (p.frag && last_step) __threadfence();          // this CTA's share of X_q before its arrival
     __syncthreads();
-    if (p.frag && last_step && tid == 0 && atomicAdd(ly.counts + kCountXq, 1) == ly.ranges - 1) {
+    if (p.frag && last_step && tid == 0 && atomicAdd(ly.counts + kCountXq, 1) == ly.ranges * shares - 1) {
       ly.counts[kCountXq] = 0;                         // zero again for the next call
       __threadfence();                                 // every CTA's share before the flag
       atomicExch(ly.flags, p.epoch);
     }
     // ---- partial T over these blocks (blocks beyond K are padding: zero mantissas, no A_q rows)
     if (active) {
-      const int b_first = NT >= kWarps ? 0 : warp / NT;
-      const int b_step = NT >= kWarps ? 1 : WPN;
-      const int nt0 = NT >= kWarps ? warp : warp % NT;
       const int nreal = min(nblk, kblocks - kb0);
-      // four blocks per round: their A_q words are requested together, then the MMAs run
-      for (int bq = b_first; bq < nreal; bq += 4 * b_step) {
-        uint32_t bw[4][TPW], ew[4][TPW];
+      for (int bq = b_first; bq < nreal; bq += UB * b_step) {
+        if (kb0 != kb_lo || bq != b_first) load_a(kb0, bq, nreal);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int b = bq + u * b_step;
-          const size_t kb = (size_t)(kb0 + (b < nreal ? b : bq));
-#pragma unroll
-          for (int i = 0; i < TPW; ++i) {
-            const int nt = min(nt0 + kWarps * i, NT - 1);
-            bw[u][i] = __ldg(reinterpret_cast<const uint32_t*>(ly.asec + (kb * k_pad + nt * 8 + g) * 16 + tig * 4));
-            ew[u][i] = __ldg(reinterpret_cast<const uint16_t*>(a_exp + kb * k_pad + nt * 8 + tig * 2));
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < UB; ++u) {
           const int b = bq + u * b_step;
           if (b < nreal) {
             const uint32_t a0 = *reinterpret_cast<const uint32_t*>(&s_xq[g * kXqStride + b * 16 + tig * 4]);
@@ -205,17 +234,15 @@ __global__ void __launch_bounds__(kThreads, TPW == 1 ? 3 : TPW == 2 ? 2 : 1) pro
   }
   if (!has_rank) return;
 
-  // ---- this CTA's partial sums -> its slot: the warps that share a rank tile add up in warp order
-  double* slot = ly.slots + ((size_t)rgroup * ly.ranges + range) * kRows * k_pad;
-  if (!LQER_IN_BOUNDS(p.status, (size_t)(slot - ly.slots) * 8, (size_t)kRows * k_pad * 8, ly.slots_extent, 312)) return;
+  // ---- this CTA's partial sums: the warps that share a rank tile add up in warp order
   if (NT >= kWarps) {
     if (active) {
 #pragma unroll
       for (int i = 0; i < TPW; ++i) {
         const int nt = warp + kWarps * i;
         if (nt < NT) {
-          *reinterpret_cast<double2*>(slot + g * k_pad + nt * 8 + tig * 2) = make_double2(acc[i][0], acc[i][1]);
-          *reinterpret_cast<double2*>(slot + (g + 8) * k_pad + nt * 8 + tig * 2) = make_double2(acc[i][2], acc[i][3]);
+          *reinterpret_cast<double2*>(s_t + g * k_pad + nt * 8 + tig * 2) = make_double2(acc[i][0], acc[i][1]);
+          *reinterpret_cast<double2*>(s_t + (g + 8) * k_pad + nt * 8 + tig * 2) = make_double2(acc[i][2], acc[i][3]);
         }
       }
     }
@@ -232,12 +259,30 @@ __global__ void __launch_bounds__(kThreads, TPW == 1 ? 3 : TPW == 2 ? 2 : 1) pro
       const int r = o / k_pad, j = o % k_pad, nt = j >> 3;
       double t = 0.0;
       for (int w = 0; w < WPN; ++w) t += s_part[w * NT + nt][r * 8 + (j & 7)];
-      slot[r * k_pad + j] = t;
+      s_t[r * k_pad + j] = t;
     }
   }
+  // ---- the range's slot: each CTA of the cluster adds up its part of the elements over the shares, in rank order
+  cluster_arrive();
+  cluster_wait();
+  double* slot = ly.slots + ((size_t)rgroup * ly.ranges + range) * kRows * k_pad;
+  const int n_slot = kRows * k_pad / shares;              // (a power of two divides 16 k_pad)
+  if (LQER_IN_BOUNDS(p.status, (size_t)(slot - ly.slots) * 8, (size_t)kRows * k_pad * 8, ly.slots_extent, 312)) {
+    for (int o = share * n_slot + tid; o < (share + 1) * n_slot; o += kThreads) {
+      double part[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) part[c] = c < shares ? ld_dsmem(s_t + o, (uint32_t)c) : 0.0;
+      double t = part[0];
+#pragma unroll
+      for (int c = 1; c < 8; ++c) t += part[c];
+      slot[o] = t;
+    }
+  }
+  cluster_arrive();                                  // nobody leaves while its shares may still be read (waited for at the exits)
   __threadfence();                                   // the slot before the count
   __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(ly.counts + rgroup, 1) == ly.ranges - 1) ? 1 : 0;
+  if (tid == 0) s_last = (atomicAdd(ly.counts + rgroup, 1) == ly.ranges * shares - 1) ? 1 : 0;
+  cluster_wait();
   __syncthreads();
   if (s_last == 0) return;
 
@@ -303,6 +348,16 @@ cudaError_t launch_prologue_small(const SmallPrologueLayer* layers, int n, int M
   p.status = st;
   p.a_bits = m0.a_bits; p.lr_bits = m0.lr_bits; p.exp_min = m0.exp_min; p.exp_max = m0.exp_max;
   const int rgroups = (M + kRows - 1) / kRows;
+  // A CTA's chain (its columns of X, then its blocks of A_q) is as long as its range, and 16 ranges leave most SMs without
+  // one at few rows: a range is shared by a cluster, up to 200 CTAs in the launch (384 take longer than 192), down to two
+  // blocks a CTA.  16 rows, K = 13824, rank 64: each of the two parts took 9 us with one CTA per range; the call with its
+  // GEMM 46 us, with eight 34.  A function of the shapes alone.
+  int all = 0;
+  for (int i = 0; i < n; ++i) all += rgroups * prologue_small_ranges(*layers[i].meta, M);
+  p.shares = 8;
+  while (p.shares > 1 && all * p.shares > 200) p.shares >>= 1;
+  for (int i = 0; i < n; ++i)
+    while (p.shares > 1 && layers[i].meta->K64 / 16 < 2 * prologue_small_ranges(*layers[i].meta, M) * p.shares) p.shares >>= 1;
   int begin = 0, max_kpad = 0;
   for (int i = 0; i < kMaxLayers; ++i) {
     const SmallPrologueLayer& src = layers[i < n ? i : 0];
@@ -323,20 +378,30 @@ cudaError_t launch_prologue_small(const SmallPrologueLayer* layers, int n, int M
     ly.ranges = prologue_small_ranges(m, M);
     ly.cta_begin = begin;
     if (i < n) {
-      begin += rgroups * ly.ranges;
+      begin += rgroups * ly.ranges * p.shares;
       if (m.k_pad > max_kpad) max_kpad = m.k_pad;
     }
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(begin);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = kRows * max_kpad * 8;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = p.shares; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
+  static OncePerDevice once;
+  const cudaError_t e = once.run([] {                    // 25 KB of static shared memory + up to 32 KB of partial sums
+    cudaError_t r = cudaFuncSetAttribute(prologue_small_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRows * 256 * 8);
+    if (r == cudaSuccess) r = cudaFuncSetAttribute(prologue_small_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRows * 256 * 8);
+    if (r == cudaSuccess) r = cudaFuncSetAttribute(prologue_small_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRows * 256 * 8);
+    return r;
+  });
+  if (e != cudaSuccess) return e;
   LaunchScope scope(kFamPrologue, s);
   if (max_kpad <= 64) return cudaLaunchKernelEx(&cfg, prologue_small_kernel<1>, p);
   if (max_kpad <= 128) return cudaLaunchKernelEx(&cfg, prologue_small_kernel<2>, p);
