@@ -301,47 +301,51 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
       if (!mbar_wait<true>(acc_full(acc), (tile_it / C::ACCS) & 1, abort_flag)) { ok = false; break; }
       tc_fence_after();
       const bool direct = ly.chunks == 1;
+      const int Nl = ly.N, M = p.M, y_type = p.y_type;
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         const int ccol = h * 128 + q * 32 + lane, col = it.tile * BN + ccol;
-        if (it.tile * BN + h * 128 >= ly.N) break;
-        const size_t pbase = (size_t)(it.tile * ly.chunks + it.chunk) * p.M * BN + ccol;
+        if (it.tile * BN + h * 128 >= Nl) break;
+        // where token 0 of this column goes, and the step from token to token, in bytes (an address per store worked out from
+        // the parameters made the 64-token bf16 epilogue 11 us long)
+        const int size = direct && y_type == kYBF16 ? 2 : direct && y_type == kYMXINT8 ? 1 : 4;
+        const size_t step = (size_t)(direct ? Nl : BN) * size;
+        uint8_t* dst = direct ? static_cast<uint8_t*>(ly.Y) + (size_t)col * size
+                              : reinterpret_cast<uint8_t*>(ly.partials + (size_t)(it.tile * ly.chunks + it.chunk) * M * BN + ccol);
+        [[maybe_unused]] const uint8_t* base = direct ? static_cast<const uint8_t*>(ly.Y) : reinterpret_cast<const uint8_t*>(ly.partials);
+        [[maybe_unused]] const size_t extent = direct ? ly.y_extent : ly.partial_extent;
+        uint8_t* dst_e = static_cast<uint8_t*>(ly.Y) + (size_t)M * Nl + col / 16;      // MXINT8: the exponent bytes
+        const size_t step_e = (size_t)Nl / 16;
 #pragma unroll 1
-        for (int t0 = 0; t0 < p.M; t0 += 16) {
+        for (int t0 = 0; t0 < M; t0 += 16) {
           uint32_t r[16];
           tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + acc * 2 * NT + h * NT + t0, r);
           tmem_ld_wait();
-          if (!direct) {
-#pragma unroll
-            for (int t = 0; t < 16; ++t) {
-              const size_t idx = pbase + (size_t)(t0 + t) * BN;
-              if (t0 + t < p.M && LQER_IN_BOUNDS(p.status, idx * 4, 4, ly.partial_extent, 704)) ly.partials[idx] = __uint_as_float(r[t]);
-            }
-          } else if (p.y_type == kYMXINT8) {
+          if (direct && y_type == kYMXINT8) {
             // sixteen lanes hold a 16-block of a token's row (N is a multiple of 16 here)
-            uint8_t* yq = static_cast<uint8_t*>(ly.Y);
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
+            for (int t = 0; t < 16; ++t, dst += step, dst_e += step_e) {
               const float v = __uint_as_float(r[t]);
               float amax = fmaxf(fabsf(v), 0.0f);            // (a NaN counts as zero)
 #pragma unroll
               for (int d = 1; d < 16; d <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, d));
               const int e = block_exponent(amax, p.exp_min, p.exp_max);
-              const size_t idx = (size_t)(t0 + t) * ly.N + col;
-              if (t0 + t < p.M && col < ly.N && LQER_IN_BOUNDS(p.status, (size_t)p.M * ly.N + idx / 16, 1, ly.y_extent, 703)) {
-                yq[idx] = (uint8_t)quant_mantissa(v, e, p.a_bits);
-                if ((lane & 15) == 0) yq[(size_t)p.M * ly.N + idx / 16] = (uint8_t)(e + 127);
+              if (t0 + t < M && col < Nl && LQER_IN_BOUNDS(p.status, dst_e - base, 1, extent, 703)) {
+                *dst = (uint8_t)quant_mantissa(v, e, p.a_bits);
+                if ((lane & 15) == 0) *dst_e = (uint8_t)(e + 127);
               }
             }
-          } else if (col < ly.N) {
+          } else if (!direct || col < Nl) {
+            const int left = M - t0;
+            if (size == 2) {
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
-              const size_t idx = (size_t)(t0 + t) * ly.N + col;
-              const int size = p.y_type == kYBF16 ? 2 : 4;
-              if (t0 + t < p.M && LQER_IN_BOUNDS(p.status, idx * size, size, ly.y_extent, 701)) {
-                if (p.y_type == kYBF16) static_cast<uint16_t*>(ly.Y)[idx] = (uint16_t)bf16_rn(__uint_as_float(r[t]));
-                else static_cast<float*>(ly.Y)[idx] = __uint_as_float(r[t]);
-              }
+              for (int t = 0; t < 16; ++t, dst += step)
+                if (t < left && LQER_IN_BOUNDS(p.status, dst - base, 2, extent, 701))
+                  *reinterpret_cast<uint16_t*>(dst) = (uint16_t)bf16_rn(__uint_as_float(r[t]));
+            } else {
+#pragma unroll
+              for (int t = 0; t < 16; ++t, dst += step)
+                if (t < left && LQER_IN_BOUNDS(p.status, dst - base, 4, extent, 704)) *reinterpret_cast<uint32_t*>(dst) = r[t];
             }
           }
           __syncwarp();

@@ -156,24 +156,30 @@ __global__ void __launch_bounds__(kThreads, TPW == 4 ? 1 : 2) prologue_small_ker
     // ---- quantise 16 rows x (nblk * 16) columns: bf16 to Xcat, int8 + exponents to shared memory
     const int quads_per_row = nblk * 4;
     const int n_quads = kRows * quads_per_row;                             // a multiple of 64
+    const int r_step = kThreads / quads_per_row, c_step = kThreads % quads_per_row;   // from quad to quad of a thread
+    int r_ld = tid / quads_per_row, c_ld = tid % quads_per_row, r_st = r_ld, c_st = c_ld;
+    auto advance = [&](int& r, int& c) {
+      r += r_step;
+      c += c_step;
+      if (c >= quads_per_row) { c -= quads_per_row; ++r; }
+    };
     for (int f0 = 0; f0 < n_quads; f0 += 8 * kThreads) {                  // whole warps: the block maximum is a shuffle
       float4 v[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int f = f0 + u * kThreads + tid;
-        const bool live = f < n_quads;
-        const int r = live ? f / quads_per_row : 0, c4 = live ? f % quads_per_row : 0;
-        const int col = kb0 * 16 + c4 * 4, row = row0 + r;
+        if (f0 + u * kThreads >= n_quads) break;                           // uniform over the CTA
+        const int col = kb0 * 16 + c_ld * 4, row = row0 + r_ld;
         v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (live && row < M && col < K) v[u] = load_x_quad(ly.X, p.x_type, M, K, row, col, p.a_bits, p.exp_min, p.exp_max);
+        if (r_ld < kRows && row < M && col < K) v[u] = load_x_quad(ly.X, p.x_type, M, K, row, col, p.a_bits, p.exp_min, p.exp_max);
+        advance(r_ld, c_ld);
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int f = f0 + u * kThreads + tid;
-        if (f0 + u * kThreads >= n_quads) break;                           // uniform over the CTA
-        const bool live = f < n_quads;
-        const int r = live ? f / quads_per_row : 0, c4 = live ? f % quads_per_row : 0;
+        if (f0 + u * kThreads >= n_quads) break;
+        const bool live = r_st < kRows;                                    // (n_quads is 16 rows of quads_per_row)
+        const int r = live ? r_st : 0, c4 = c_st;
         const int col = kb0 * 16 + c4 * 4, row = row0 + r;
+        advance(r_st, c_st);
         int e;
         uint32_t m8;
         uint2 bf;
