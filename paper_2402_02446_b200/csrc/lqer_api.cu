@@ -336,6 +336,7 @@ static int prefill_run(const lqer_call_t* calls, int first, int n_calls, int lim
 // the same M <= kSmallMaxM, the same formats, any shapes, none of them served by the column-owner decode kernel; at most
 // `limit`, only as many as the workspace has slices for, and tile counters for.
 constexpr size_t kGroupRowCountOffset = 256 + 32768 * 4 + 16 * 256 * 8;   // the row-tile counter area at its highest position
+static_assert(kGroupRowCountOffset + 16 * kRowCounters * 4 <= kPersistMaxBytes, "row-group counters of a launch");
 static int small_run(const lqer_call_t* calls, int first, int n_calls, int limit, size_t workspace_bytes, bool cols_ok,
                      PackedMeta* metas, size_t* need) {
   const int M = calls[first].M;
@@ -368,7 +369,7 @@ static lqer_status_t run_small_group(const lqer_call_t* calls, int n, const Pack
     off += small_slice_bytes(metas[g], calls[0].M);
     tile_counts[g] = reinterpret_cast<int*>(wsb + kStatusBytes) + tiles;
     tiles += metas[g].n_tiles;
-    row_counts[g] = reinterpret_cast<int*>(wsb + kGroupRowCountOffset) + 8 * g;
+    row_counts[g] = reinterpret_cast<int*>(wsb + kGroupRowCountOffset) + kRowCounters * g;
   }
   return run_small(calls, metas, n, slices, tile_counts, row_counts, static_cast<DeviceStatus*>(workspace), io, nullptr,
                    nullptr, false, s) == cudaSuccess ? LQER_OK : LQER_ERR_CUDA;

@@ -525,7 +525,7 @@ struct SmallPrologueLayer {
   const PackedMeta* meta;
   void* xcat;                 // bf16 [M, K64 + k_pad], or the fragment order below
   double* slots;              // prologue_small_slot_bytes of scratch
-  int* counts;                // one zeroed counter per group of 16 rows (eight ints; in fragment order counts[kCountXq] too)
+  int* counts;                // kRowCounters zeroed ints: eight per group of 16 rows (in fragment order two more, below)
   int8_t* Tm;                 // optional exports of T_q (may be null)
   uint8_t* Te;
   int* flags;                 // fragment order: the layer's two flags (below)
@@ -542,7 +542,8 @@ int prologue_small_max_layers();
 // An epoch is a number that no earlier launch on this workspace used, so a flag left by the call before never
 // passes for this call's, whenever the two overlap; the GEMM's last CTA clears the flags when it leaves (a counter
 // behind them counts its CTAs out), which is what a replayed graph, whose epoch repeats, relies on.
-constexpr int kCountXq = 1;
+constexpr int kRowCounters = 64;                   // of a layer in a small-batch launch (16 layers: the last 4 KB of the head)
+constexpr int kCountXq = 8, kCountTq = 9;          // up to 16 rows: behind the one row group's
 constexpr int kFlagAreaOffset = 64;                 // status area bytes [64, 64 + 16 layers * 8), then the exit counter
 inline int frag_rank_slabs(const PackedMeta& m) { return (m.k_pad + 63) / 64; }
 inline size_t frag_bytes(const PackedMeta& m) { return (size_t)8 * (m.k_slabs + frag_rank_slabs(m)) * 256; }

@@ -8,8 +8,8 @@
 //                (16-block, 8 rank columns), scaled by 2^(e_x + e_a) and summed in fp64
 //                -> the cluster adds its shares up through distributed shared memory, in rank order
 //                -> slot (r, g) of the scratch; then it counts itself in.
-//   The CTA that arrives LAST for a row group (no one waits for anyone) adds the slots in range order,
-//   re-quantises T along the rank and appends T_q to Xcat[:, K64 : K64 + k_pad].
+//   The CTA that arrives LAST for its share of a row group's elements (no one waits for anyone) adds the slots in range
+//   order, re-quantises T along the rank and appends T_q to Xcat[:, K64 : K64 + k_pad].
 // The results equal the other prologues' bit for bit: the block products are exact integers, the fp64 sums
 // are exact unless a row's block exponents spread over more than about 30 binades, and the order of the
 // additions is fixed by the ranges, which depend on the shape alone.
@@ -30,7 +30,7 @@ struct Layer {
   const uint8_t* asec;        // A_q section of the packed buffer
   uint16_t* xcat;             // [M, K64 + k_pad] bf16
   double* slots;              // [row group][range][16][k_pad] partial sums of T
-  int* counts;                // [row group] arrivals, zero between calls
+  int* counts;                // [row group][8 shares] arrivals, zero between calls
   int* flags;                 // fragment order: X_q ready, T_q ready (each takes the launch's epoch)
   int8_t* Tm;                 // optional exports of T_q
   uint8_t* Te;
@@ -287,16 +287,16 @@ __global__ void __launch_bounds__(kThreads, TPW == 4 ? 1 : 2) prologue_small_ker
   cluster_arrive();                                  // nobody leaves while its shares may still be read (waited for at the exits)
   __threadfence();                                   // the slot before the count
   __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(ly.counts + rgroup, 1) == ly.ranges * shares - 1) ? 1 : 0;
+  if (tid == 0) s_last = (atomicAdd(ly.counts + rgroup * 8 + share, 1) == ly.ranges - 1) ? 1 : 0;
   cluster_wait();
   __syncthreads();
   if (s_last == 0) return;
 
-  // ---- the last CTA of the row group: T = sum of the ranges (range order) -> MXINT8 along the rank -> Xcat
+  // ---- the last CTA of the row group with this share of the elements (whole rows): T = sum of the ranges (range order) -> MXINT8 along the rank -> Xcat
   __threadfence();
   const double* slots0 = ly.slots + (size_t)rgroup * ly.ranges * kRows * k_pad;
   const int n_out = kRows * k_pad;                   // a multiple of 32: 16 adjacent lanes hold one block
-  for (int o = tid; o < n_out; o += kThreads) {
+  for (int o = share * n_slot + tid; o < (share + 1) * n_slot; o += kThreads) {
     const int r = o / k_pad, j = o % k_pad;
     double part[16];                                 // at most 16 ranges: all loads in flight, then the sum in range order
 #pragma unroll
@@ -324,16 +324,20 @@ __global__ void __launch_bounds__(kThreads, TPW == 4 ? 1 : 2) prologue_small_ker
   if (p.frag) {
     // rank indices between k_pad and the end of the last rank slab: zeros (the GEMM multiplies them with zero weights)
     const int pad = ((k_pad + 63) / 64) * 64 - k_pad;
-    for (int o = tid; o < kRows * pad; o += kThreads) {
+    for (int o = tid; share == 0 && o < kRows * pad; o += kThreads) {
       const int r = o / pad, j = k_pad + o % pad;
       const size_t off = frag_offset(r, ly.K64 / 64 + (j >> 6), j & 63, plane);
       if (LQER_IN_BOUNDS(p.status, off, 2, ly.xcat_extent, 314)) *reinterpret_cast<uint16_t*>(reinterpret_cast<uint8_t*>(ly.xcat) + off) = 0;
     }
     __threadfence();                                 // T_q before its flag
     __syncthreads();
-    if (tid == 0) atomicExch(ly.flags + 1, p.epoch);
+    if (tid == 0 && (shares == 1 || atomicAdd(ly.counts + kCountTq, 1) == shares - 1)) {
+      ly.counts[kCountTq] = 0;
+      __threadfence();                               // every share before the flag
+      atomicExch(ly.flags + 1, p.epoch);
+    }
   }
-  if (tid == 0) ly.counts[rgroup] = 0;               // zero again for the next call
+  if (tid == 0) ly.counts[rgroup * 8 + share] = 0;   // zero again for the next call
 }
 
 }  // namespace psm
