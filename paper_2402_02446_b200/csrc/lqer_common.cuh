@@ -491,6 +491,7 @@ struct DigitCall {
 // 26.7 / 22.4; K = 11008: rank 80 at 129 rows 31.3 / 23.3, rank 256 at 4096 rows 464 / 141.
 inline bool prologue_digits_applies(const PackedMeta& m) { return m.k_pad > 64; }
 constexpr long long kDigitMinWork = 150LL * 1000 * 1000;
+constexpr long long kDigitMinShared = 500LL * 1000 * 1000;      // layers of any rank on one activation
 inline long long prologue_work(const PackedMeta& m, int M) { return (long long)M * m.K * m.k_pad; }
 size_t prologue_digits_scratch_bytes(const PackedMeta& m, int M);
 cudaError_t launch_prologue_digits(const DigitCall* calls, int n, int M, int x_type, void* scratch, GemmActs* places, int8_t* Tm,

@@ -93,6 +93,30 @@ def test_layers_that_share_an_activation_equal_single_calls(x_type):
         Pg.release()
 
 
+def test_low_ranks_on_one_activation():
+    # ranks up to 64 take the digit planes where large layers share an activation; single calls the fp64-scaled prologue
+    M, K = 1100, 4112
+    specs = [gen.LayerSpec(f"low{i}", M=M, K=K, N=264, k=k, calib_rows=32, outlier_frac=0.01, outlier_scale=50.0, seed=980 + i)
+             for i, k in enumerate((32, 40, 64))]
+    layers = []
+    for s in specs:
+        W, (A, B) = gen.make_weight(s), gen.make_random_factors(s)
+        layers.append((olqer.prepare_weights(W, A, B), L.prepare_weights(_t(W), _t(A), _t(B))))
+    X = gen.make_activations(specs[0])
+    X[5::7] = _spread(X[5::7], 1, 9, 3)
+    x = _t(X)
+    Ys = [torch.full((M, s.N), float("nan"), device=DEV) for s in specs]
+    calls = L.make_calls([(x, Pg, y) for (_, Pg), y in zip(layers, Ys)])
+    ws = torch.zeros(L.batched_workspace_bytes(calls), dtype=torch.uint8, device=DEV)
+    L.linear_batched(calls, ws)
+    assert L.poll_status(ws) == 0
+    rows = np.arange(0, M, 53)
+    for (P, Pg), y in zip(layers, Ys):
+        assert torch.equal(L.linear(x, Pg, ws), y)
+        assert worst_ratio(y.cpu().numpy()[rows], olqer.forward(X[rows], P)) <= 1.0
+        Pg.release()
+
+
 def test_a_workspace_without_room_for_the_planes_is_taken_as_before():
     spec = gen.LayerSpec("tight", M=300, K=4112, N=264, k=128, calib_rows=32, outlier_frac=0.01, outlier_scale=20.0, seed=970)
     A, B = gen.make_random_factors(spec)
