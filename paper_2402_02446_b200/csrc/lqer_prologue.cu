@@ -129,12 +129,10 @@ __global__ void __launch_bounds__(kThreads, TPW == 1 ? 3 : 2) prologue_kernel(co
     }
   };
 
-  // The first panel of A_q depends on no earlier kernel; X and the workspace may still be in use by the one before.  The GEMM
-  // behind this kernel may set up meanwhile (it waits before it reads Xcat).  (201 rows, K = 4112: 2 us of the call.)
-  if (crank < steps && has_rank) load_panel(crank, 0);
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (crank < steps) load_x(crank);
+  if (crank < steps) {
+    load_x(crank);
+    if (has_rank) load_panel(crank, 0);
+  }
   cp_async_commit();
 
   int buf = 0;
@@ -264,13 +262,11 @@ static cudaError_t launch_prologue_pb(const void* X, int x_type, int M, const Pa
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = s;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = 1;
   LaunchScope scope(kFamPrologue, s);
   return cudaLaunchKernelEx(&cfg, prologue_kernel<PB, TPW>, X, x_type, M, m, asec, xc, Tm, Te, st);
 }
