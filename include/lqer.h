@@ -313,6 +313,12 @@ lqer_status_t lqer_inject_stall(int kernel_family);
  * returns LQER_ERR_CONFIG. */
 lqer_status_t lqer_debug_bounds_shrink(long long bytes);
 
+/* Test hook of the checked build (host, process wide): in the launches of the tensor-memory small-batch GEMM that follow, a
+ * group of warps that has nothing to convert in a batch of weights looks at that batch `cycles` SM clock cycles late (0 ..
+ * 1e7; 0 restores), so that a wait that relied on its being in time would run out.  The ordinary build returns
+ * LQER_ERR_CONFIG. */
+lqer_status_t lqer_debug_converter_lag(long long cycles);
+
 /* Number of kernels launched by the library in this process so far (host). */
 unsigned long long lqer_launch_count(void);
 

@@ -71,6 +71,7 @@ def lib() -> C.CDLL:
             "lqer_set_wait_limit_cycles": (i, [C.c_longlong]),
             "lqer_inject_stall": (i, [i]),
             "lqer_debug_bounds_shrink": (i, [C.c_longlong]),
+            "lqer_debug_converter_lag": (i, [C.c_longlong]),
             "lqer_prepare_weights": (i, [vp, vp, vp, i, i, i, cfgp, vp, sz, vp]),
             "lqer_factor_sketch_columns": (i, [i, i, i, C.POINTER(i)]),
             "lqer_prepare_workspace_bytes": (i, [i, i, i, C.POINTER(sz)]),
@@ -430,6 +431,12 @@ def debug_bounds_shrink(nbytes: int) -> None:
     """Test hook of the checked build: the declared extent of every Y shrinks by nbytes for the launches that follow, so the
     bounds checks at the end of Y fire (their stores are skipped); 0 restores.  The ordinary build refuses."""
     _check(lib().lqer_debug_bounds_shrink(nbytes), "lqer_debug_bounds_shrink")
+
+
+def debug_converter_lag(cycles: int) -> None:
+    """Test hook of the checked build: converter warps of the tensor-memory small-batch GEMM that sit a batch of weights out look at
+    it that many SM clock cycles late; 0 restores.  The ordinary build refuses."""
+    _check(lib().lqer_debug_converter_lag(cycles), "lqer_debug_converter_lag")
 
 
 def launch_count() -> int:

@@ -49,6 +49,8 @@ static std::atomic<int> g_stall_family{-1};
 long long wait_limit_cycles() { return g_wait_limit.load(std::memory_order_relaxed); }
 static std::atomic<size_t> g_y_shrink{0};                      // checked build only: see lqer_debug_bounds_shrink
 size_t debug_y_shrink() { return g_y_shrink.load(std::memory_order_relaxed); }
+static std::atomic<long long> g_converter_lag{0};               // checked build only: see lqer_debug_converter_lag
+long long debug_converter_lag() { return g_converter_lag.load(std::memory_order_relaxed); }
 
 bool take_stall(int family) {
   int want = family;
@@ -1162,6 +1164,13 @@ lqer_status_t lqer_debug_bounds_shrink(long long bytes) {
   if (!kDebugBounds) return LQER_ERR_CONFIG;          // the ordinary build has no checks to trip
   if (bytes < 0 || bytes > (1LL << 40)) return LQER_ERR_CONFIG;
   g_y_shrink.store((size_t)bytes);
+  return LQER_OK;
+}
+
+lqer_status_t lqer_debug_converter_lag(long long cycles) {
+  if (!kDebugBounds) return LQER_ERR_CONFIG;
+  if (cycles < 0 || cycles > 10000000) return LQER_ERR_CONFIG;
+  g_converter_lag.store(cycles);
   return LQER_OK;
 }
 

@@ -385,6 +385,8 @@ constexpr bool kDebugBounds = false;
 #endif
 // Test hook of the checked build (lqer_debug_bounds_shrink): bytes taken off the declared extent of Y at the next launches.
 size_t debug_y_shrink();
+// Test hook of the checked build (lqer_debug_converter_lag), in SM clock cycles.
+long long debug_converter_lag();
 
 // ----------------------------------------------------------------------------
 // Per-device host state

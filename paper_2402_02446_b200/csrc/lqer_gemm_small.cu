@@ -44,6 +44,10 @@ constexpr int W_HALF_BYTES = BATCH * kWTileBytes;
 constexpr int CONVERTER_GROUPS = 3;
 constexpr int WARPS_PER_GROUP = 8;
 constexpr int NUM_THREADS = (6 + CONVERTER_GROUPS * WARPS_PER_GROUP) * 32;
+// A PK slot is free once the MMAs that read its activations have finished AND every converter warp is past it.  A group may own
+// no step of a batch, but it looks at every batch's barrier by parity, so it must not be a pass ahead of it (it waits for
+// each one) nor a pass behind: without its arrival here the slot could be filled again before the group has looked.
+constexpr int PK_FREE_ARRIVALS = 1 + CONVERTER_GROUPS * WARPS_PER_GROUP;
 
 __device__ __forceinline__ void epilogue_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
@@ -128,7 +132,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
   const int num_items = p.num_items;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < PK_SLOTS; ++s) { mbar_init(w_full(s), 1); mbar_init(x_full(s), 1); mbar_init(pk_free(s), 1); }
+    for (int s = 0; s < PK_SLOTS; ++s) { mbar_init(w_full(s), 1); mbar_init(x_full(s), 1); mbar_init(pk_free(s), PK_FREE_ARRIVALS); }
     for (int s = 0; s < CV_SLOTS; ++s) { mbar_init(cv_ready(s), WARPS_PER_GROUP); mbar_init(cv_free(s), 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(acc_full(a), 1); mbar_init(acc_empty(a), 4); }
     abort_flag->abort = 0;
@@ -390,7 +394,15 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
       const bool has_w = 2 * it.tile + half < p.L[it.layer].n_tiles;
       for (int s0 = it.s_lo; s0 < it.s_hi && ok; ++batch_no) {
         const int e = batch_end(s0, it.s_hi, k_slabs), pk = batch_no % PK_SLOTS;
-        // (also where none of the batch's slabs is this group's: a group must not get a pass ahead of a slot's barrier)
+        if (kDebugBounds && p.lag > 0) {                 // test hook: a group without a step in this batch comes late
+          bool mine = false;
+          for (int st = s0, n = it_no; st < e; st += STEP, ++n) mine = mine || n % CONVERTER_GROUPS == group;
+          if (!mine) {
+            const long long t0 = clock64();
+            while (clock64() - t0 < p.lag) { }
+          }
+        }
+        // also where none of the batch's steps is this group's: see PK_FREE_ARRIVALS
         if (!mbar_wait(w_full(pk), (batch_no / PK_SLOTS) & 1, abort_flag)) { ok = false; break; }
         const uint8_t* pkh = pk_base + pk * C::PK_SLOT_BYTES + C::X_BYTES + half * W_HALF_BYTES;
         for (int st = s0; st < e; st += STEP, ++it_no) {
@@ -460,6 +472,8 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
           __syncwarp();
           if (lane == 0) mbar_arrive(cv_ready(group));
         }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(pk_free(pk));
         s0 = e;
       }
     }
@@ -615,6 +629,7 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
   p.x_rows = x_rows;
   p.w_bits = layers[0].meta->w_bits;
   p.wait_limit = wait_limit_cycles();
+  p.lag = debug_converter_lag();
   p.epoch = epoch;
   p.exit_count = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(st) + kFlagAreaOffset + 2 * MAX_LAYERS * 4);
   p.stall = take_stall(kFamDecode) ? 1 : 0;

@@ -38,6 +38,7 @@ struct Params {
   int a_bits, exp_min, exp_max;// activation format, for an MXINT8 Y
   int w_bits;                  // mantissa bits of W_q: 4 or 2 (one value for all layers of a launch)
   int x_rows;                  // rows of an activation tile: M rounded up to 16 (those beyond M arrive as zeros)
+  long long lag;               // checked build, test hook: see lqer_debug_converter_lag
   long long wait_limit;
   int epoch;                   // register-operand kernel: the value the prologue's flags take in this call
   int* exit_count;             // ... and a zeroed counter of the CTAs that have left (the last one clears the flags)

@@ -75,9 +75,40 @@ def test_a_short_extent_is_reported_and_nothing_beyond_it_is_written():
     assert r.returncode == 0 and "checked-build-ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
 
 
+def test_converter_warps_that_come_late_to_a_batch_lose_nothing():
+    # three tiles per CTA, a tile being a batch of four slabs, one of one and one of two rank slabs: groups of converter
+    # warps sit batches out in every ring (four, three and two slots).  They look at those batches some 50 us late, long
+    # after the slot could have been filled again: the result must be the undelayed one, and no wait may run out.
+    code = textwrap.dedent("""
+        import torch
+        import paper_2402_02446_b200 as L
+        dev = "cuda:0"
+        K, N, k = 320, 3 * 148 * 256, 72
+        g = torch.Generator(device=dev); g.manual_seed(7)
+        draw = lambda *s: torch.randn(s, generator=g, device=dev)
+        Pg = L.prepare_weights(draw(K, N) * 0.02, draw(K, k) / K ** 0.5, draw(k, N) * 0.01)
+        for M in (20, 64, 100):
+            X = draw(M, K)
+            ws = L.new_workspace(M, Pg)
+            Y = L.linear(X, Pg, ws).clone()
+            assert L.poll_status(ws) == 0
+            L.debug_converter_lag(100_000)
+            try:
+                late = L.linear(X, Pg, ws)
+                assert L.poll_status(ws) == 0, M
+            finally:
+                L.debug_converter_lag(0)
+            assert torch.equal(late, Y), M
+        print("late-converters-ok")
+    """)
+    r = _run(["-c", code])
+    assert r.returncode == 0 and "late-converters-ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
+
+
 def test_the_ordinary_build_has_no_such_hook():
     import paper_2402_02446_b200 as L
     from paper_2402_02446_b200 import binding
     if binding.DEBUG_BOUNDS:
         pytest.skip("this process runs the checked build")
     assert L.lib().lqer_debug_bounds_shrink(16) == binding.STATUS_NAMES.index("LQER_ERR_CONFIG")
+    assert L.lib().lqer_debug_converter_lag(16) == binding.STATUS_NAMES.index("LQER_ERR_CONFIG")
