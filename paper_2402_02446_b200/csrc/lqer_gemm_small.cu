@@ -8,8 +8,9 @@
 // touch shared memory.  An MMA of K = 16 then takes 17 cycles at N = 16, 19 at 32, 32 at 64, 64 at 128 (measured; with
 // the operand in shared memory 39 at N = 16, and 128 with the tokens on the 64- or 128-row side against 256 weight
 // columns).  A CTA streams packed weight tiles exactly once into a ring of some 200 KB, in batches of four slabs of 64 K:
-// one bulk copy for each 128-column half of the tile and one TMA load for the four [N, 64] activation tiles (every copy
-// costs its issuing thread and the copy engine a hundred cycles and more, so a slab at a time held the ring back).
+// one bulk copy for each 128-column half of the tile and a TMA load for each of the four [N, 64] activation tiles (every
+// copy costs its issuing thread and the copy engine a hundred cycles and more, so a slab of weights at a time held the ring
+// back).
 // What bounds it is the stream of weights and, close behind, the instructions that expand them (1.8 per weight).
 //
 // Work items are (layer, 256-column tile, K chunk).  The chunks of a tile are fixed by the shape alone (so a
@@ -86,16 +87,9 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint4& a, const 
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z) : "memory");
-}
-
 struct TensorMaps {
-  CUtensorMap m[MAX_LAYERS];   // Xcat of each layer, bf16 [M, K64 + k_pad], as [slab][row][64]: box 4 x x_rows x 64
+  CUtensorMap m[MAX_LAYERS];   // Xcat of each layer, bf16 [M, K64 + k_pad], box x_rows x 64
 };
-
 
 // The batch that starts with slab s: up to BATCH slabs of weights, or two slabs of B_q (8-bit mantissas: eight blocks of 16
 // ranks, 16 KB, then their exponent bytes).
@@ -120,7 +114,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
 
   const uint32_t bar0 = smem_u32(bars);
   auto w_full = [&](int s) { return bar0 + 8u * s; };                       // packed weights of a PK slot have landed
-  auto x_full = [&](int s) { return bar0 + 8u * (PK_SLOTS + s); };          // its activation tile has landed
+  auto x_full = [&](int s) { return bar0 + 8u * (PK_SLOTS + s); };          // its activation tiles have landed
   auto pk_free = [&](int s) { return bar0 + 8u * (2 * PK_SLOTS + s); };
   auto cv_ready = [&](int s) { return bar0 + 8u * (3 * PK_SLOTS + s); };
   auto cv_free = [&](int s) { return bar0 + 8u * (3 * PK_SLOTS + CV_SLOTS + s); };
@@ -155,7 +149,10 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
       // then does the producer wait for the kernel before (the prologue that writes Xcat) and request the
       // activation tiles of those batches.  They land on a barrier of their own (x_full, used once per slot); later
       // ones share the weights' barrier, so that the MMA warp has one barrier to watch.
-      const uint32_t x_bytes = (uint32_t)BATCH * p.x_rows * 128u;   // (slabs and rows beyond the matrix arrive as zeros)
+      const uint32_t x_tile = (uint32_t)p.x_rows * 128u;       // bytes of a slab's activations (rows beyond M arrive as zeros)
+      auto load_x = [&](const CUtensorMap* map, int s, int e, uint32_t slot, uint32_t bar) {
+        for (; s < e; ++s, slot += x_tile) tma_load_2d(slot, map, s * BK, 0, bar);
+      };
       int npend = 0;                                           // batches requested without their activations: the first ones
       bool waited = false;
       auto flush = [&]() {
@@ -164,9 +161,11 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
         for (int i = cta, q = 0; q < npend; i += num_ctas) {
           const Item it = item_of(p, i);
           const int k_slabs = p.L[it.layer].k_slabs;
-          for (int s = it.s_lo; s < it.s_hi && q < npend; s = batch_end(s, it.s_hi, k_slabs), ++q) {
-            mbar_expect_tx(x_full(q), x_bytes);
-            tma_load_3d(smem_u32(pk_base + q * C::PK_SLOT_BYTES), &tmaps.m[it.layer], 0, 0, s, x_full(q));
+          for (int s = it.s_lo; s < it.s_hi && q < npend; ++q) {
+            const int e = batch_end(s, it.s_hi, k_slabs);
+            mbar_expect_tx(x_full(q), (e - s) * x_tile);
+            load_x(&tmaps.m[it.layer], s, e, smem_u32(pk_base + q * C::PK_SLOT_BYTES), x_full(q));
+            s = e;
           }
         }
       };
@@ -186,26 +185,26 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
           if (!waited && npend == PK_SLOTS) flush();
           if (!mbar_wait<true>(pk_free(pk), ph ^ 1, abort_flag)) { ok = false; break; }
           const uint32_t slot = smem_u32(pk_base + pk * C::PK_SLOT_BYTES), dst = slot + C::X_BYTES;
-          const uint32_t bar = w_full(pk);
+          const uint32_t bar = w_full(pk), x_bytes = waited ? (uint32_t)(e - s) * x_tile : 0u;
           if (s < k_slabs) {
             const size_t off = ((size_t)nt0 * k_slabs + s) * w_tile, half = (size_t)k_slabs * w_tile;
             const uint32_t bytes = (uint32_t)(e - s) * w_tile;
             if (!LQER_IN_BOUNDS(p.status, off + (n_half - 1) * half, bytes, ly.w_extent, 705)) { ok = false; break; }
-            mbar_expect_tx(bar, n_half * bytes + (waited ? x_bytes : 0u));
+            mbar_expect_tx(bar, n_half * bytes + x_bytes);
             bulk_load(dst, ly.wsec + off, bytes, bar);
             if (n_half > 1) bulk_load(dst + W_HALF_BYTES, ly.wsec + off + half, bytes, bar);
           } else {
             const int rb0 = (s - k_slabs) * 4, nb = min((e - s) * 4, r_blocks - rb0);
             if (!LQER_IN_BOUNDS(p.status, (size_t)(nt0 + n_half - 1) * b_tile_stride + (size_t)r_blocks * kTileN * 16 + rb0 * kTileN,
                                 nb * kTileN, ly.b_extent, 706)) { ok = false; break; }
-            mbar_expect_tx(bar, n_half * nb * (kTileN * 17) + (waited ? x_bytes : 0u));
+            mbar_expect_tx(bar, n_half * nb * (kTileN * 17) + x_bytes);
             for (int h = 0; h < n_half; ++h) {
               const uint8_t* tile = ly.bsec + (size_t)(nt0 + h) * b_tile_stride;
               bulk_load(dst + h * W_HALF_BYTES, tile + (size_t)rb0 * kTileN * 16, nb * kTileN * 16, bar);
               bulk_load(dst + h * W_HALF_BYTES + RANK_EXP_OFFSET, tile + (size_t)r_blocks * kTileN * 16 + rb0 * kTileN, nb * kTileN, bar);
             }
           }
-          if (waited) tma_load_3d(slot, &tmaps.m[it.layer], 0, 0, s, bar);
+          if (waited) load_x(&tmaps.m[it.layer], s, e, slot, bar);
           else ++npend;
           if (++pk == PK_SLOTS) { pk = 0; ph ^= 1; }
           s = e;
@@ -584,14 +583,12 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
     const SmallGemmLayer& src = layers[i < n ? i : 0];
     const PackedMeta& m = *src.meta;
     if (m.lr_bits != layers[0].meta->lr_bits || m.w_bits != layers[0].meta->w_bits) return cudaErrorInvalidValue;
-    // [slab][row][64 columns]; the last slab of T_q may reach past the end of a row (its columns beyond k_pad are never
-    // multiplied) and, in the last row, up to 96 bytes past Xcat, where the layer's partial sums of T lie
-    const cuuint64_t dims[3] = {64, (cuuint64_t)M, (cuuint64_t)(m.k_slabs + frag_rank_slabs(m))};
-    const cuuint64_t strides[2] = {(cuuint64_t)xcat_cols(m) * 2, 128};
-    const cuuint32_t box[3] = {BK, (cuuint32_t)x_rows, BATCH};
-    const cuuint32_t estr[3] = {1, 1, 1};
+    const cuuint64_t dims[2] = {(cuuint64_t)xcat_cols(m), (cuuint64_t)M};
+    const cuuint64_t strides[1] = {(cuuint64_t)xcat_cols(m) * 2};
+    const cuuint32_t box[2] = {BK, (cuuint32_t)x_rows};
+    const cuuint32_t estr[2] = {1, 1};
     if (!use_mma &&
-        enc(&tmaps.m[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(src.xcat), dims, strides, box, estr,
+        enc(&tmaps.m[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(src.xcat), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
