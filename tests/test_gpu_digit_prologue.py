@@ -68,6 +68,43 @@ def test_t_is_exact_inside_and_outside_the_windows(M, K, k, wide):
     Pg.release()
 
 
+# a row's blocks lie in windows of nine exponents below its largest or above its smallest (three of them, two above 32768 K)
+# or below those: block exponents at both edges of every window, in every block, in two blocks of a panel, in the last only
+@pytest.mark.parametrize("M,K,k,a_bits", [(140, 1040, 80, 8), (257, 4112, 136, 6), (129, 32784, 72, 8), (1030, 512, 256, 8)])
+def test_windows_beyond_the_first(M, K, k, a_bits):
+    N, g = 264, np.random.default_rng(K)
+    spec = gen.LayerSpec("windows", M=M, K=K, N=N, k=k, calib_rows=32, outlier_frac=0.0, outlier_scale=1.0, seed=930 + k)
+    W = gen.make_weight(spec)
+    A, B = gen.make_random_factors(spec)
+    A[:16 * (K // 32)] *= 2.0 ** -10                         # columns with blocks outside theirs
+    X = g.uniform(1.0, 2.0, (M, K)).astype(np.float32) * g.choice((-1.0, 1.0), (M, K)).astype(np.float32)
+    e = np.zeros((M, K // 16))
+    for r in range(M):
+        low = (8, 9, 17, 18, 26, 27, 35, 50)[r % 8]
+        kind = r // 8 % 4
+        if kind == 0: e[r] = -g.integers(0, low + 1, K // 16)
+        elif kind == 1: e[r, 9:11] = -low if r % 3 else low
+        elif kind == 2: e[r, -1] = low if r % 3 else -low
+        else: e[r] = -g.choice((0, 8, 9, 17, 18, 26, 27, 44), K // 16)
+    X *= np.exp2(e).repeat(16, axis=1).astype(np.float32)
+    cfg = L.default_config()
+    cfg.a_bits = a_bits
+    P, Pg = olqer.prepare_weights(W, A, B), L.prepare_weights(_t(W), _t(A), _t(B), cfg)
+    ref = olqer.forward(X, P, a_bits=a_bits)
+    ws = L.new_workspace(M, Pg)
+    L.set_path(binding.PATH_TENSOR_PROLOGUE)
+    try:
+        Tm, Te = L.project_lowrank(_t(X), Pg, ws)
+        Y = L.linear(_t(X), Pg, ws).cpu().numpy()
+    finally:
+        L.set_path(binding.PATH_AUTO)
+    assert L.poll_status(ws) == 0
+    assert np.array_equal(Te.cpu().numpy(), exp_bytes(ref.Te))
+    assert np.array_equal(Tm.cpu().numpy(), ref.Tm)
+    assert worst_ratio(Y, ref) <= 1.0
+    Pg.release()
+
+
 @pytest.mark.parametrize("x_type", ["f32", "bf16", "mxint8"])
 def test_layers_that_share_an_activation_equal_single_calls(x_type):
     # three calls on one X, one on another, ranks of two widths: one group; each result is the single call's, bit for bit
