@@ -268,7 +268,7 @@ static lqer_status_t run_linear(const void* X, int M, const void* packed, void* 
   const bool small = takes_small_path(path, M);
   // Paths 1 and 3 keep the mma.sync prologue, as does a workspace without room for the digit planes.
   const bool digits = !small && path != 1 && path != 3 && prologue_digits_applies(m) &&
-                      (path == 6 || prologue_work(m, M) >= kDigitMinWork) && workspace_bytes >= call_bytes_wanted(m, M, small);
+                      (path == 6 || prologue_digits_pays(m, M)) && workspace_bytes >= call_bytes_wanted(m, M, small);
   if (project_only && !small && !digits) path = 3;
   // Paths 1 and 3 keep the SIMT-style prologue at every batch size; the others take the tensor-core one where it fits.
   const bool tc_prologue = path != 1 && path != 3 && prologue_tc_fits(m, M, X, path == 6);

@@ -486,15 +486,25 @@ struct DigitCall {
   const void* packed;
   const PackedMeta* meta;
 };
-// It serves ranks above 64 (below, launch_prologue_tc), from this much work M K k_pad on, summed over the layers of a call:
-// three launches take some 20 us whatever the shape.  Measured, launch_prologue against this, K = 4096: rank 80 at 512 rows
-// 18.9 / 19.5 us, at 768 rows 33.2 / 21.4; rank 256 at 129 rows 25.2 / 25.0, at 512 rows 31.3 / 26.2, at 4096 rows 187 / 68;
-// K = 1024: rank 80 at 1024 rows 17.0 / 19.8, at 2048 rows 23.0 / 20.3; rank 256 at 512 rows 16.5 / 20.7, at 768 rows
-// 26.7 / 22.4; K = 11008: rank 80 at 129 rows 31.3 / 23.3, rank 256 at 4096 rows 464 / 141.
+// It serves ranks above 64 (below, launch_prologue_tc; groups of any rank on one activation: run_prefill_group) where its
+// three launches, some 20 us together whatever the shape, pay.  launch_prologue's clusters of eight CTAs hold 16 rows each and
+// fill the SMs once up to 592 rows: up to there a layer has to be wide (K k_pad), beyond, the work M K k_pad counts.  Both
+// sides measured, call with its GEMM, launch_prologue / this, us:
+//   512 rows: 5120 x 5120 rank 128 (K k_pad 6.6e5) 65 / 70, 4096 x 4096 rank 128 (5.2e5) 53 / 59, rank 256 (1.05e6) 65 / 62,
+//             11008 x 4096 rank 80 (8.8e5) 104 / 97;
+//   160 rows: 5120 x 5120 rank 128 48 / 54, 4096 x 4096 rank 256 49 / 48, 11008 x 4096 rank 80 63 / 57;
+//   640 rows: 1024 x 1024 rank 128 (work 8.4e7) 34 / 39, rank 256 (1.7e8) 44 / 41, 4096 x 4096 rank 80 (2.1e8) 65 / 56;
+//   1024 rows: 1024 x 1024 rank 128 (1.3e8) 37 / 40; 2048 rows: rank 80 (1.7e8) 40 / 38, 4096 x 4096 rank 256 (2.1e9) 167 / 111.
+// Several layers in one call pay launch_prologue each: they count by their work together (two 1024 x 1024 layers of rank 256,
+// 300 rows, 1.6e8: 46 / 50; 512 rows, 2.7e8: 48 / 41; seven of rank 80, 300 rows, 1.7e8: 85 / 40).
 inline bool prologue_digits_applies(const PackedMeta& m) { return m.k_pad > 64; }
-constexpr long long kDigitMinWork = 150LL * 1000 * 1000;
+constexpr long long kDigitMinWidth = 800LL * 1000;
+constexpr long long kDigitMinWork = 160LL * 1000 * 1000;
 constexpr long long kDigitMinShared = 500LL * 1000 * 1000;      // layers of any rank on one activation
 inline long long prologue_work(const PackedMeta& m, int M) { return (long long)M * m.K * m.k_pad; }
+inline bool prologue_digits_pays(const PackedMeta& m, int M) {
+  return M <= 592 ? (long long)m.K * m.k_pad >= kDigitMinWidth : prologue_work(m, M) >= kDigitMinWork;
+}
 size_t prologue_digits_scratch_bytes(const PackedMeta& m, int M);
 cudaError_t launch_prologue_digits(const DigitCall* calls, int n, int M, int x_type, void* scratch, GemmActs* places, int8_t* Tm,
                                    uint8_t* Te, DeviceStatus* st, cudaStream_t s);
