@@ -307,11 +307,28 @@ static lqer_status_t run_linear(const void* X, int M, const void* packed, void* 
   return err == cudaSuccess ? LQER_OK : LQER_ERR_CUDA;
 }
 
-// Scratch one layer of a grouped prefill launch needs: its own Xcat and its own prologue scratch (layers of rank above 64
-// that share an X take less together).
-static size_t group_slice_bytes(const PackedMeta& m, int M) { return xcat_bytes(m, M) + prologue_scratch(m, M); }
+// Scratch one layer of a grouped prefill launch is taken with: its own Xcat and the fp64 prologue's partial sums.
+static size_t group_slice_bytes(const PackedMeta& m, int M) { return xcat_bytes(m, M) + align_up(prologue_tc_scratch_bytes(m, M), 256); }
+// What a group takes on the digit planes, 0 where it does not go there: they serve groups of ranks above 64, and groups of any
+// rank on ONE activation from kDigitMinShared on: its quantisation is then shared too (2048 rows of 4096 columns, rank 32:
+// three layers 196 -> 180 us with their GEMM, two layers of 11008 columns 291 -> 278 us).
+static size_t group_digit_bytes(const lqer_call_t* calls, const PackedMeta* metas, int n) {
+  const int M = calls[0].M;
+  bool high = n > 1, one_x = n > 1;
+  long long work = 0;
+  DigitCall dc[8];
+  for (int g = 0; g < n; ++g) {
+    high = high && prologue_digits_applies(metas[g]);
+    one_x = one_x && metas[g].k_pad > 0 && calls[g].X != nullptr && calls[g].X == calls[0].X && metas[g].K == metas[0].K;
+    work += prologue_work(metas[g], M);
+    dc[g] = DigitCall{calls[g].X, calls[g].packed, &metas[g]};
+  }
+  const bool takes = (high && work >= kDigitMinWork) || (one_x && work >= kDigitMinShared);
+  return takes ? prologue_digits_group_bytes(dc, n, M) : 0;
+}
 // Consecutive prefill calls from `first` on that may share a GEMM launch with it (auto path only): the same M > 256,
-// the same formats, any shapes; at most `limit`, and only as many as the workspace has slices for.
+// the same formats, any shapes; at most `limit`, and only as many as the workspace has slices for (or, if at least two fit it
+// that way, room for the digit planes).  *need: what all of them would like.
 static bool same_formats(const PackedMeta& a, const PackedMeta& b) {
   return a.w_bits == b.w_bits && a.a_bits == b.a_bits && a.lr_bits == b.lr_bits && a.exp_min == b.exp_min &&
          a.exp_max == b.exp_max && a.block == b.block;
@@ -319,8 +336,8 @@ static bool same_formats(const PackedMeta& a, const PackedMeta& b) {
 static int prefill_run(const lqer_call_t* calls, int first, int n_calls, int limit, size_t workspace_bytes,
                        PackedMeta* metas, size_t* need) {
   const int M = calls[first].M;
-  size_t head = 0, slices = 0;
-  int n = 0;
+  size_t head = 0, slices = 0, digits = 0;
+  int n = 0, n_digits = 0;
   while (first + n < n_calls && n < limit) {
     PackedMeta m;
     if (calls[first + n].M != M || lookup(calls[first + n].packed, m) != LQER_OK) break;
@@ -330,9 +347,11 @@ static int prefill_run(const lqer_call_t* calls, int first, int n_calls, int lim
     if (n > 0 && h + sl > workspace_bytes) break;
     metas[n] = m; head = h; slices = sl;
     ++n;
+    digits = group_digit_bytes(calls + first, metas, n);
+    if (digits > 0 && digits <= workspace_bytes && head <= workspace_bytes - digits) n_digits = n;
   }
-  if (need != nullptr) *need = head + slices;
-  return n;
+  if (need != nullptr) *need = head + std::max(slices, digits);
+  return digits > 0 && n_digits > 1 ? n_digits : n;
 }
 // Consecutive small-batch calls from `first` on that may share the two launches of the small-batch path (auto path only):
 // the same M <= kSmallMaxM, the same formats, any shapes, none of them served by the column-owner decode kernel; at most
@@ -448,19 +467,8 @@ static lqer_status_t run_prefill_group(const lqer_call_t* calls, int n, const Pa
   GemmActs acts[8];
   const void* packed[8];
   void* Ys[8];
-  // The digit planes serve groups of ranks above 64, and groups of any rank on ONE activation from kDigitMinShared on: its
-  // quantisation is then shared too (2048 rows of 4096 columns, rank 32: three layers 207 -> 187 us with their GEMM, two
-  // layers of 11008 columns 296 -> 283 us).
-  bool high = n > 1, one_x = n > 1;
-  long long work = 0;
-  size_t need = 0;
-  for (int g = 0; g < n; ++g) {
-    high = high && prologue_digits_applies(metas[g]);
-    one_x = one_x && metas[g].k_pad > 0 && calls[g].X == calls[0].X && metas[g].K == metas[0].K;
-    work += prologue_work(metas[g], M);
-    need += xcat_bytes(metas[g], M) + align_up(prologue_digits_scratch_bytes(metas[g], M), 256);
-  }
-  if (((high && work >= kDigitMinWork) || (one_x && work >= kDigitMinShared)) && head + need <= workspace_bytes) {
+  const size_t digits = group_digit_bytes(calls, metas, n);
+  if (digits > 0 && head + digits <= workspace_bytes) {
     DigitCall dc[8];
     for (int g = 0; g < n; ++g) {
       dc[g] = DigitCall{calls[g].X, calls[g].packed, &metas[g]};

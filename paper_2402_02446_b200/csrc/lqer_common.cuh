@@ -476,10 +476,10 @@ struct GemmActs {
   int ld, t_col;
 };
 inline GemmActs plain_acts(void* xcat, const PackedMeta& m) { return GemmActs{xcat, (int)xcat_cols(m), m.K64}; }
-// The prologue with the projection as one integer contraction over all of K on the int8 tensor cores, for ranks above 64:
+// The prologue with the projection as one integer contraction over all of K on the int8 tensor cores (any rank but zero):
 // three launches for up to kDigitMaxLayers layers with one M and one set of formats, any shapes; layers with the same X
-// share its quantisation.  `scratch`: at most the sum over the layers of their Xcat bytes and
-// prologue_digits_scratch_bytes (each rounded up to 256); places[g] says where layer g's activations are.
+// share its quantisation.  `scratch`: prologue_digits_group_bytes, Xcat included (for one call its Xcat, rounded up to 256,
+// and prologue_digits_scratch_bytes); places[g] says where layer g's activations are.
 constexpr int kDigitMaxLayers = 8, kDigitMaxUnits = 8;
 struct DigitCall {
   const void* X;
@@ -506,6 +506,7 @@ inline bool prologue_digits_pays(const PackedMeta& m, int M) {
   return M <= 592 ? (long long)m.K * m.k_pad >= kDigitMinWidth : prologue_work(m, M) >= kDigitMinWork;
 }
 size_t prologue_digits_scratch_bytes(const PackedMeta& m, int M);
+size_t prologue_digits_group_bytes(const DigitCall* calls, int n, int M);
 cudaError_t launch_prologue_digits(const DigitCall* calls, int n, int M, int x_type, void* scratch, GemmActs* places, int8_t* Tm,
                                    uint8_t* Te, DeviceStatus* st, cudaStream_t s);
 cudaError_t launch_gemm_simt(const void* xcat, int M, const PackedMeta& m, const void* packed, float* Y,

@@ -731,8 +731,27 @@ static size_t digit_unit_scratch(int K64, int ktot, int M) {
          align256((size_t)M * words * 4) + align256((size_t)ktot * words * 4) + align256(panels * 2 * PANEL * ktot) +
          align256(rt * ktot * ROWS * 8);
 }
-// A group of layers needs at most the sum of this over its layers, whichever of them share an X.
 size_t prologue_digits_scratch_bytes(const PackedMeta& m, int M) { return digit_unit_scratch(m.K64, m.k_pad, M); }
+// The unit of each call: calls that multiply the same X share one (an X that is not known yet is nobody else's).
+static int digit_units(const DigitCall* calls, int n, int* unit_at) {
+  int units = 0, first[kDigitMaxLayers];
+  for (int g = 0; g < n; ++g) {
+    int q = 0;
+    while (q < units && !(calls[g].X != nullptr && calls[first[q]].X == calls[g].X && calls[first[q]].meta->K == calls[g].meta->K)) ++q;
+    if (q == units) first[units++] = g;
+    unit_at[g] = q;
+  }
+  return units;
+}
+size_t prologue_digits_group_bytes(const DigitCall* calls, int n, int M) {
+  using namespace pdg;
+  int unit_at[kDigitMaxLayers], ktot[kDigitMaxUnits] = {}, K64[kDigitMaxUnits] = {};
+  const int units = digit_units(calls, n, unit_at);
+  for (int g = 0; g < n; ++g) { ktot[unit_at[g]] += calls[g].meta->k_pad; K64[unit_at[g]] = calls[g].meta->K64; }
+  size_t bytes = 0;
+  for (int q = 0; q < units; ++q) bytes += align256((size_t)M * (K64[q] + ktot[q]) * 2) + digit_unit_scratch(K64[q], ktot[q], M);
+  return bytes;
+}
 
 cudaError_t launch_prologue_digits(const DigitCall* calls, int n, int M, int x_type, void* scratch, GemmActs* places, int8_t* Tm,
                                    uint8_t* Te, DeviceStatus* st, cudaStream_t s) {
@@ -749,14 +768,12 @@ cudaError_t launch_prologue_digits(const DigitCall* calls, int n, int M, int x_t
   p.wait_limit = wait_limit_cycles();
   // layers that multiply the same X share its quantised values
   int unit_at[kDigitMaxLayers];
+  digit_units(calls, n, unit_at);
   for (int g = 0; g < n; ++g) {
     const PackedMeta& m = *calls[g].meta;
     if (m.k_pad == 0) return cudaErrorInvalidValue;
-    int q = 0;
-    while (q < p.n && !(p.U[q].X == calls[g].X && p.U[q].K == m.K)) ++q;
-    unit_at[g] = q;
-    Unit& u = p.U[q];
-    if (q == p.n) {
+    Unit& u = p.U[unit_at[g]];
+    if (unit_at[g] == p.n) {
       ++p.n;
       u.X = calls[g].X; u.K = m.K; u.K64 = m.K64;
       u.panels = (m.K64 + PANEL - 1) / PANEL;

@@ -166,3 +166,31 @@ def test_a_workspace_without_room_for_the_planes_is_taken_as_before():
     with pytest.raises(binding.LqerError):
         L.linear(X, Pg, ws[: least - 256])
     Pg.release()
+
+
+# ranks whose own prologue needs less scratch than the planes: 48 (none at all), 32 at many row tiles, 16 at a long K; and
+# layers on activations of their own, whose planes need more than two slices have
+@pytest.mark.parametrize("M,K,k,shared", [(2048, 4096, 48, True), (8192, 4096, 32, True), (4096, 5120, 16, True), (1030, 2048, 128, False)])
+def test_the_advised_workspace_has_room_for_the_planes(M, K, k, shared):
+    N = 256
+    specs = [gen.LayerSpec(f"room{i}", M=M, K=K, N=N, k=k, calib_rows=32, outlier_frac=0.01, outlier_scale=20.0, seed=990 + i) for i in range(2)]
+    packs = [L.prepare_weights(_t(gen.make_weight(s)), *map(_t, gen.make_random_factors(s))) for s in specs]
+    Xs = [torch.randn((M, K), generator=torch.Generator(device=DEV).manual_seed(k + i), device=DEV) for i in range(2)]
+    Xs[1] = Xs[0] if shared else Xs[1]
+    Ys = [torch.full((M, N), float("nan"), device=DEV) for _ in specs]
+    calls = L.make_calls(list(zip(Xs, packs, Ys)))
+    single = [L.linear(x, P, L.new_workspace(M, P)) for x, P in zip(Xs, packs)]
+
+    def launches(nbytes):
+        ws = torch.zeros(nbytes, dtype=torch.uint8, device=DEV)
+        before = L.launch_count()
+        L.linear_batched(calls, ws)
+        n = L.launch_count() - before
+        assert L.poll_status(ws) == 0
+        assert all(torch.equal(y, s) for y, s in zip(Ys, single))
+        return n
+    assert launches(L.batched_workspace_bytes(calls)) == 4       # three for the planes, one GEMM
+    if not shared:                                               # two bare Xcats: taken, as before there were planes
+        assert launches(168192 + 2 * M * (K + k) * 2) == 3
+    for P in packs:
+        P.release()
