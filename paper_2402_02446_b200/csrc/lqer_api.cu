@@ -186,7 +186,7 @@ static size_t call_bytes(const PackedMeta& m, int M, bool small) {
          (small ? small_bytes(m, M)
                 : xcat_bytes(m, M) + align_up(prologue_tc_scratch_bytes(m, M), 256) + gemm_splitk_bytes(m, M));
 }
-// What it asks for.
+// What it makes use of if it is there.
 static size_t call_bytes_wanted(const PackedMeta& m, int M, bool small) {
   if (small) return call_bytes(m, M, small);
   return align_up(persist_bytes(m), 256) + xcat_bytes(m, M) + prologue_scratch(m, M) + gemm_splitk_bytes(m, M);
@@ -631,7 +631,7 @@ lqer_status_t lqer_call_workspace_bytes(int M, int K, int N, int k, const lqer_c
   if (M <= 0 || M > (1 << 24)) return LQER_ERR_SHAPE;
   PackedMeta m;
   fill_meta(m, K, N, k, *cfg);
-  *bytes = call_bytes_wanted(m, M, M <= kSmallMaxM);
+  *bytes = call_bytes(m, M, M <= kSmallMaxM);
   return LQER_OK;
 }
 

@@ -137,3 +137,13 @@ def test_static_scratch_limits_follow_the_call_need():
     # decode-sized calls fit for every K up to 131072, and whatever N
     assert L.call_workspace_bytes(16, 131072, 4096, 256) <= binding.STATIC_SCRATCH_BYTES
     assert L.call_workspace_bytes(16, 4096, 1 << 22, 256) <= binding.STATIC_SCRATCH_BYTES
+
+
+def test_call_workspace_is_the_least_a_call_is_taken_with_at_every_rank():
+    # above rank 64 a larger workspace makes the call faster, but [X_q | T_q] behind the head is all it has to have: that is
+    # what lqer_linear_static compares with its limit (rank 128, K = 4096: up to 973 rows)
+    for M, K, k in ((768, 4096, 128), (973, 4096, 128), (300, 4112, 200)):
+        k_pad, k64 = (k + 15) // 16 * 16, (K + 63) // 64 * 64
+        assert L.call_workspace_bytes(M, K, 4096, k) == 168192 + (M * (k64 + k_pad) * 2 + 255) // 256 * 256
+        assert L.workspace_bytes(M, K, 4096, k) > L.call_workspace_bytes(M, K, 4096, k)
+    assert L.call_workspace_bytes(973, 4096, 4096, 128) <= binding.STATIC_SCRATCH_BYTES

@@ -91,3 +91,19 @@ def test_static_scratch_boundary_on_a_4096_layer_and_no_allocation():
         assert torch.cuda.memory_allocated() == held0 and free1 >= free0      # nothing was allocated, by torch or by the library
         assert torch.equal(Y, Y_ref), M
     P.release()
+
+
+def test_static_scratch_takes_a_rank_above_64_up_to_the_call_need():
+    # rank 128, K = 4096: 973 rows are the last whose [X_q | T_q] fits behind the head
+    spec = gen.LayerSpec("static_r128", M=974, K=4096, N=256, k=128, calib_rows=32, outlier_frac=0.01, outlier_scale=20.0, seed=95)
+    P = _layer(spec)
+    Xall = torch.from_numpy(gen.make_activations(spec)).to(DEV)
+    ws = L.new_workspace(spec.M, P)
+    for M, fits in ((768, True), (973, True), (974, False)):
+        assert (L.call_workspace_bytes(M, spec.K, spec.N, spec.k) <= binding.STATIC_SCRATCH_BYTES) == fits
+        X, Y = Xall[:M].contiguous(), torch.full((M, spec.N), float("nan"), dtype=torch.float32, device=DEV)
+        st = L.lib().lqer_linear_static(X.data_ptr(), M, P.ptr, Y.data_ptr(), None)
+        assert st == (0 if fits else binding.STATUS_NAMES.index("LQER_ERR_STATIC_SCRATCH"))
+        if fits:
+            assert torch.equal(Y, L.linear(X, P, ws)), M
+    P.release()
