@@ -93,6 +93,11 @@ struct Params {
   int stall;                                      // test hook: the last panel's A digits are withheld
 };
 
+// Checked build: whether n elements from p[at] on lie in an array of `total` of them (all of a unit's arrays are scratch).
+template <class T>
+__device__ __forceinline__ bool inside(const Params& p, const T*, size_t at, size_t n, size_t total, int site) {
+  return LQER_IN_BOUNDS(p.status, at * sizeof(T), n * sizeof(T), total * sizeof(T), site);
+}
 __device__ __forceinline__ const Unit& unit_of(const Params& p, int index, int Unit::* first) {
   int u = 0;
   for (int i = 1; i < p.n; ++i)
@@ -192,13 +197,14 @@ __device__ __forceinline__ void a_digits(const Params& p, const Unit& u, int par
   }
   const int col = la.col0 + c;
   if (share == 0) {
-    if (lane == 0) { u.colinfo[col] = info[0]; u.colinfo[col + 1] = info[1]; }
+    if (lane == 0 && inside(p, u.colinfo, col, 2, u.ktot, 333)) { u.colinfo[col] = info[0]; u.colinfo[col + 1] = info[1]; }
     for (int j = 0; j < 2; ++j)
       if ((info[j] >> 16) != 0)
         for (int b0 = 0; b0 < kb; b0 += 32) {
           const int b = b0 + lane;
           const unsigned out = __ballot_sync(0xFFFFFFFFu, b < kb && outside(aexp[(size_t)b * kp + c + j], (info[j] & 0xFFFF) - 1024) && !zero(b, j));
-          if (lane == 0) u.colout[(size_t)(col + j) * u.far_words + (b0 >> 5)] = out;
+          const size_t at = (size_t)(col + j) * u.far_words + (b0 >> 5);
+          if (lane == 0 && inside(p, u.colout, at, 1, (size_t)u.ktot * u.far_words, 334)) u.colout[at] = out;
         }
   }
   int c0 = 0, nt = 0;
@@ -242,6 +248,7 @@ __device__ __forceinline__ void a_digits(const Params& p, const Unit& u, int par
           lo = make_uint4(o[0], o[1], o[2], o[3]);
         }
         uint8_t* at = tile + (n + j) * PANEL + (((b & 7) ^ ((n + j) & 7)) << 4);
+        if (!inside(p, u.planes, at - u.planes, nt * PANEL + 16, (size_t)u.panels * 2 * PANEL * u.ktot, 335)) continue;
         *reinterpret_cast<uint4*>(at) = hi;
         *reinterpret_cast<uint4*>(at + nt * PANEL) = lo;
       }
@@ -285,6 +292,7 @@ __device__ __forceinline__ void quantise_row(const Params& p, const Unit& u, int
     // the sums start at zero: any share of them will do (the last row takes those of the last row tile's missing rows too)
     const int rows_here = row == p.M - 1 ? u.row_tiles * ROWS - row : 1;
     unsigned long long* acc = u.tacc + (size_t)row * u.ktot;
+    if (inside(p, u.tacc, (size_t)row * u.ktot, (size_t)rows_here * u.ktot, (size_t)u.row_tiles * u.ktot * ROWS, 336))
     for (int i = part * 32 + lane; i < rows_here * u.ktot; i += p.warps_per_row * 32) acc[i] = 0ull;
   }
   const QuantConsts qc = quant_consts(p.a_bits, p.exp_min, p.exp_max);
@@ -316,14 +324,15 @@ __device__ __forceinline__ void quantise_row(const Params& p, const Unit& u, int
         *reinterpret_cast<uint4*>(xrow + b * 16) = x0;
         *reinterpret_cast<uint4*>(xrow + b * 16 + 8) = x1;
       }
-      erow[b] = (uint8_t)eb;
+      if (inside(p, u.ebytes, (size_t)row * u.ep + b, 1, (size_t)p.M * u.ep, 337)) erow[b] = (uint8_t)eb;
     }
   }
   mx = __reduce_max_sync(0xFFFFFFFFu, mx);
   mn = __reduce_min_sync(0xFFFFFFFFu, mn);
   sum = __reduce_add_sync(0xFFFFFFFFu, sum);
   n = __reduce_add_sync(0xFFFFFFFFu, n);
-  if (lane == 0) u.rowparts[(size_t)row * kParts + part] = (uint32_t)(mx | mn << 8 | (n > 0 ? sum / n : 0) << 16);
+  if (lane == 0 && inside(p, u.rowparts, (size_t)row * kParts + part, 1, (size_t)p.M * kParts, 338))
+    u.rowparts[(size_t)row * kParts + part] = (uint32_t)(mx | mn << 8 | (n > 0 ? sum / n : 0) << 16);
 }
 
 // Bound by reading X and writing Xcat; no warp waits for another.
@@ -554,6 +563,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) project_kernel(const __grid_co
           const int st = i % STAGES;
           if (p.stall != 0 && pn0 + q == u.panels - 1) { ok = false; break; }
           if (!mbar_wait<true>(empty(st), (uint32_t)((i / STAGES) & 1) ^ 1u, ws)) { ok = false; break; }
+          if (!inside(p, u.planes, img - u.planes + (size_t)(pn0 + q) * bytes, bytes, (size_t)u.panels * 2 * PANEL * u.ktot, 342)) { ok = false; break; }
           mbar_expect_tx(full(st), bytes);
           bulk_load(smem_u32(smem + st * STAGE_BYTES + 2 * X_PLANE), img + (size_t)(pn0 + q) * bytes, bytes, full(st));
         }
@@ -613,7 +623,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) project_kernel(const __grid_co
         dir = up ? 1 : -1;
         if (q4 == 0) {
           s_windows[r] = more | (up ? 256 : 0);
-          if (live && sp == 0) u.rowinfo[row] = ((up ? first : first - more * (kWindow + 1)) - 127 + 1024) | (all > more ? 1 << 16 : 0);
+          if (live && sp == 0 && inside(p, u.rowinfo, row, 1, p.M, 339))
+            u.rowinfo[row] = ((up ? first : first - more * (kWindow + 1)) - 127 + 1024) | (all > more ? 1 << 16 : 0);
         }
         unsigned far = sp == 0 && ct == 0 ? __ballot_sync(0xFFFFFFFFu, live && all > more) : 0u;
         while (far != 0) {                                             // a row at a time, all lanes
@@ -623,7 +634,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) project_kernel(const __grid_co
           for (int b0 = 0; b0 < u.K / 16; b0 += 32) {
             const int e = b0 + lane < u.K / 16 ? (int)u.ebytes[(size_t)frow * u.ep + b0 + lane] : 0;
             const unsigned low = __ballot_sync(0xFFFFFFFFu, e != 0 && ftop - e >= u.windows * (kWindow + 1));
-            if (lane == 0) u.rowfar[(size_t)frow * u.far_words + (b0 >> 5)] = low;
+            const size_t at = (size_t)frow * u.far_words + (b0 >> 5);
+            if (lane == 0 && inside(p, u.rowfar, at, 1, (size_t)p.M * u.far_words, 340)) u.rowfar[at] = low;
           }
         }
       }
@@ -690,6 +702,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) project_kernel(const __grid_co
             for (int j = 0; j < 16; ++j) {
               const long long v = ((long long)(int)hh[j] * 65536 + (long long)(int)mid[j] * 256 + (long long)(int)ll[j]) * unit;
               unsigned long long* at = acc + (size_t)(cb + j) * ROWS;
+              if (!inside(p, u.tacc, at - u.tacc, 1, (size_t)u.row_tiles * u.ktot * ROWS, 341)) continue;
               if (u.splits > 1) atomicAdd(at, (unsigned long long)v);
               else *at = (unsigned long long)v + (w > 0 ? *at : 0ull);
             }

@@ -28,7 +28,7 @@ def test_small_parity_cases_pass_under_the_checked_build():
     # launches, bf16 and MXINT8 boundaries; each test polls the status word, so a bounds report fails it
     r = _run(["-m", "pytest", "-x", "-q", "-m", "gpu",
               "tests/test_gpu_parity.py", "tests/test_gpu_bf16_io.py", "tests/test_gpu_mxint8_io.py", "tests/test_gpu_w2.py",
-              "tests/test_gpu_small_mma.py",
+              "tests/test_gpu_small_mma.py", "tests/test_gpu_small_batches.py", "tests/test_gpu_digit_prologue.py",
               "-k", "not full and not stack and not sweep and not round"])
     assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
     assert " passed" in r.stdout

@@ -40,6 +40,7 @@ CASES = [
     ("small_gemm_ring", FAM_DECODE, binding.PATH_AUTO, 9, 1024, 640, 40),
     ("small_mma_flags", FAM_DECODE, binding.PATH_SMALL, 9, 1024, 640, 40),      # the polls of the prologue's flags
     ("prologue_tc_row_tile", FAM_PROLOGUE, binding.PATH_TENSOR_PROLOGUE, 300, 1024, 640, 32),
+    ("digit_prologue_ring", FAM_PROLOGUE, binding.PATH_TENSOR_PROLOGUE, 300, 1040, 640, 136),   # several K ranges: one of them stalls
     ("gemm_pair_ring", FAM_GEMM, binding.PATH_AUTO, 300, 1024, 640, 40),
 ]
 
