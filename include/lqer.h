@@ -172,7 +172,7 @@ lqer_status_t lqer_project_lowrank(const float* X, int M, const void* packed, in
 /* The layer (Section 3.1 last display, Section 3.2 last display):
  *   Y[M,N] = X_q W_q + q(X_q A_q) B_q,  fp32 accumulation of exactly represented products.
  * M <= 4 runs a fused decode kernel whose CTAs own output columns; M <= 128 a latency-oriented
- * prologue and a tensor-core GEMM that streams the weights once against a 64- or 128-row token tile;
+ * prologue and a tensor-core GEMM that streams the weights once, 128 columns of them per MMA against all tokens;
  * larger M the activation prologue and the tensor-core GEMM over 256 x 256 tiles of the concatenated
  * contraction [X_q | T_q] . [W_q ; B_q].
  * lqer_linear uses the default stream. */
@@ -248,8 +248,9 @@ lqer_status_t lqer_linear_static(const float* X, int M, const void* packed, floa
  *    GEMM over the work items of all of them, under the same condition on the workspace.
  * In the first two cases a result does not depend on the sharing, bit for bit.  In the third the
  * contraction of a tile is cut into fewer K chunks when layers share a launch, so a result may
- * differ from the single call's in its last bits (both within the layer's tolerance); it is
- * reproducible for the same sequence of calls. */
+ * differ from the single call's in its last bits (both within the layer's tolerance); the fp64 sums
+ * of X A_k are grouped differently too, which shows only where a row's block exponents spread over
+ * more than about 30 binades.  A result is reproducible for the same sequence of calls. */
 lqer_status_t lqer_batched_workspace_bytes(const lqer_call_t* calls, int n_calls, size_t* bytes);
 lqer_status_t lqer_linear_batched(const lqer_call_t* calls, int n_calls,
                                   void* workspace, size_t workspace_bytes, void* stream);
@@ -289,8 +290,8 @@ lqer_status_t lqer_poll_status(const void* workspace, void* stream, lqer_status_
  * GEMM with the prologue chosen as in 0, 5 small prologue + small-batch GEMM for every M <= 128 (the register-operand
  * kernel up to 16 rows - which paths 0 and 2 use only where several calls share its launches - and
  * the tensor-memory kernel otherwise), 6 as 4 with the
- * tcgen05 activation prologue at every batch size (ranks up to 64; by default it serves M >= 1024,
- * and paths 1 and 3 never use it), 7 as 5 with the tensor-memory kernel at every M <= 128.  Host only, process wide. */
+ * tcgen05 activation prologues at every batch size (ranks up to 64: by default M >= 1024; above, the
+ * integer contraction, by default where it pays; paths 1 and 3 use neither), 7 as 5 with the tensor-memory kernel at every M <= 128.  Host only, process wide. */
 lqer_status_t lqer_set_path(int path);
 
 /* Test hooks for the device-side error path (host only, process wide; the paper has no counterpart: this is a

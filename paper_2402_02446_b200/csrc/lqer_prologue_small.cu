@@ -10,9 +10,10 @@
 //                -> slot (r, g) of the scratch; then it counts itself in.
 //   The CTA that arrives LAST for its share of a row group's elements (no one waits for anyone) adds the slots in range
 //   order, re-quantises T along the rank and appends T_q to Xcat[:, K64 : K64 + k_pad].
-// The results equal the other prologues' bit for bit: the block products are exact integers, the fp64 sums
-// are exact unless a row's block exponents spread over more than about 30 binades, and the order of the
-// additions is fixed by the ranges, which depend on the shape alone.
+// The results equal the other prologues' bit for bit: the block products are exact integers, and the fp64 sums
+// are exact unless a row's block exponents spread over more than about 30 binades.  The order of the additions is fixed by
+// the ranges, which depend on the shape alone, and by the shares, which depend on all layers of the launch: beyond that
+// spread a T may differ in its 53rd bit between a call alone and in company (and T_q where that bit decides a rounding).
 #include "lqer_common.cuh"
 
 namespace lqer {
@@ -58,11 +59,6 @@ __device__ __forceinline__ size_t frag_offset(int row, int slab, int c, size_t p
          (c & 1) * 2;
 }
 
-// TPW: rank tiles (8 columns) a warp owns: 1 for ranks up to 64, 2 up to 128, 4 up to 256.
-// The kernel is a chain of memory latencies, so a round requests as much as the registers hold: the A_q words of UB blocks
-// (those of a CTA's first blocks before it waits for the kernel before, on which they do not depend) and eight quads
-// of X per thread.  With four blocks and four quads a round it took 15 - 29 us at K = 5120 - 13824 and ranks 32 and 64, of
-// which 5 - 10 us were rounds of A_q.
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -79,6 +75,11 @@ __device__ __forceinline__ double ld_dsmem(const double* local, uint32_t cta) {
   return v;
 }
 
+// TPW: rank tiles (8 columns) a warp owns: 1 for ranks up to 64, 2 up to 128, 4 up to 256.
+// The kernel is a chain of memory latencies, so a round requests as much as the registers hold: the A_q words of UB blocks
+// (those of a CTA's first blocks before it waits for the kernel before, on which they do not depend) and eight quads
+// of X per thread.  With four blocks and four quads a round it took 15 - 29 us at K = 5120 - 13824 and ranks 32 and 64, of
+// which 5 - 10 us were rounds of A_q.
 template <int TPW>
 __global__ void __launch_bounds__(kThreads, TPW == 4 ? 1 : 2) prologue_small_kernel(const __grid_constant__ Params p) {
   __shared__ __align__(16) uint8_t s_xq[kRows * kXqStride];

@@ -70,3 +70,27 @@ def test_layers_of_one_launch(M):
     for s, (P, Pg), x, y in zip(specs, layers, Xs, Ys):
         assert worst_ratio(y.cpu().numpy(), olqer.forward(x.cpu().numpy(), P)) <= 1.0, s.name
         Pg.release()
+
+
+def test_wide_exponents_alone_and_in_company():
+    # block exponents over 50 binades: the fp64 sums of T round, and a launch of several layers groups them differently (the
+    # cluster that shares a K range depends on all of its layers); both stay within the tolerance
+    M = 20
+    specs = [gen.LayerSpec(f"wide{i}", M=M, K=K, N=264, k=40, calib_rows=32, outlier_frac=0.0, outlier_scale=1.0, seed=1400 + i)
+             for i, K in enumerate((4096, 1024, 4096, 2112))]
+    layers = [_layer(s, 4) for s in specs]
+    g = np.random.default_rng(5)
+    Xs = [(gen.make_activations(s) * np.exp2(g.integers(-40, 11, (M, s.K // 16))).repeat(16, axis=1)).astype(np.float32) for s in specs]
+    Ys = [torch.full((M, s.N), float("nan"), device=DEV) for s in specs]
+    xs = [_t(x) for x in Xs]
+    calls = L.make_calls([(x, lay[1], y) for x, lay, y in zip(xs, layers, Ys)])
+    ws = torch.zeros(L.batched_workspace_bytes(calls), dtype=torch.uint8, device=DEV)
+    L.linear_batched(calls, ws)
+    assert L.poll_status(ws) == 0
+    for (P, Pg), X, x, y in zip(layers, Xs, xs, Ys):
+        ref = olqer.forward(X, P)
+        assert worst_ratio(y.cpu().numpy(), ref) <= 1.0
+        assert worst_ratio(L.linear(x, Pg, ws).cpu().numpy(), ref) <= 1.0
+        Tm, Te = L.project_lowrank(x, Pg, ws)
+        assert np.array_equal(Tm.cpu().numpy(), ref.Tm) and np.array_equal(Te.cpu().numpy(), exp_bytes(ref.Te))
+        Pg.release()
