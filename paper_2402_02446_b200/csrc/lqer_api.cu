@@ -240,10 +240,11 @@ static cudaError_t run_small(const lqer_call_t* calls, const PackedMeta* metas, 
   // a number for the flags of this pair of launches that no earlier pair on any workspace used (never zero)
   static std::atomic<unsigned> epochs{0};
   const int epoch = (int)(epochs.fetch_add(1) & 0x3FFFFFFFu) + 1;
-  // the register-operand GEMM reads the activations in fragment order and follows the prologue's flags
-  // (a call on its own is a chain of latencies that the tensor-memory kernel gets through sooner: measured 23.6 against
-  // 26.6 us on a 4096 x 4096 layer; the register-operand kernel serves launches that several layers share, and single
-  // calls where path 5 is forced)
+  // The register-operand GEMM reads the activations in fragment order and follows the prologue's flags.  It serves launches that
+  // several layers share: 4096 x 4096, rank 32, 16 rows, us per layer, tensor-memory / register-operand: 2 layers 12.2 / 12.4,
+  // 4 layers 8.2 / 7.6, 6 layers 7.2 / 6.0, 16 layers 4.7 / 4.0 (8 rows: 11.9 / 12.1, 7.8 / 7.4, 6.3 / 5.9, 4.7 / 4.0).  A call on its
+  // own takes either in the same time (16 rows 21.7 / 21.7, 5 rows 20.6 / 20.9) and keeps the tensor-memory kernel; path 5
+  // forces the other.
   const int path = g_path.load();
   const bool tmem_form = path == 7 || ((path == 0 || path == 2) && n == 1);
   const bool frag = !project_only && !tmem_form && small_takes_mma(metas[0], M);
@@ -396,9 +397,11 @@ static lqer_status_t run_small_group(const lqer_call_t* calls, int n, const Pack
                    nullptr, false, s) == cudaSuccess ? LQER_OK : LQER_ERR_CUDA;
 }
 // Three or four rows in many layers at once: the register-operand GEMM's launches take less per layer than the
-// column-owner kernel's (measured on 4096 x 4096 layers: from 6 layers on at 4 rows, 5.7 against 6.9 us, and from 12 on
-// at 3 rows, 4.4 against 4.6 us; with fewer layers the column-owner kernel's shorter chain wins).  The length of such
-// a run from calls[first] on, or 0.
+// column-owner kernel's.  Measured on 4096 x 4096 layers of rank 32, us per layer, column-owner / register-operand: 4 rows,
+// 2 layers 12.4 / 11.9, 4 layers 8.5 / 7.3, 6 layers 7.2 / 5.8, 16 layers 5.2 / 4.0; 3 rows, 2 layers 10.7 / 12.1, 4 layers
+// 7.3 / 7.3, 6 layers 6.1 / 5.8, 12 layers 4.5 / 4.5, 16 layers 4.3 / 3.9.  (The lines, 6 and 12 layers, were drawn for an
+// earlier small prologue; with the present one the two sides meet at 2 layers for 4 rows and at 4 to 6 for 3.)  The length
+// of such a run from calls[first] on, or 0.
 static int many_small_rows(const lqer_call_t* calls, int first, int n_calls, size_t workspace_bytes, const PackedMeta& m0,
                            PackedMeta* metas, size_t* need) {
   const int M = calls[first].M;

@@ -122,9 +122,9 @@ inline size_t prologue_tc_scratch_bytes(const PackedMeta& m, int M) {
   if (!prologue_tc_rank_ok(m) || (M + 127) / 128 > kPrologueRowTiles) return 0;
   return (size_t)((M + 127) / 128) * prologue_tc_splits(m, M) * 128 * m.k_pad * 8;
 }
-// Small batches (up to kSmallMaxM rows): the prologue for few rows and the GEMM with the tokens on the MMA's M side
-// (padded to 64 or 128 rows) and 256 weight columns on its N side.
-// Everything below depends on the shape alone, never on the device or on what else shares a launch.
+// Small batches (up to kSmallMaxM rows): the prologue for few rows and the GEMM with 128 weight columns on the MMA's M side
+// and the tokens (rounded up to 16) on its N side.  The cuts below depend on the shape alone; layers that share a launch may
+// be cut less finely (launch_gemm_small, launch_prologue_small).
 constexpr int kSmallMaxM = 128;
 // K ranges per group of 16 rows in the small prologue (each a CTA; the last to arrive adds them up in range order).
 inline int prologue_small_ranges(const PackedMeta& m, int M) {
@@ -563,8 +563,8 @@ inline int frag_rank_slabs(const PackedMeta& m) { return (m.k_pad + 63) / 64; }
 inline size_t frag_bytes(const PackedMeta& m) { return (size_t)8 * (m.k_slabs + frag_rank_slabs(m)) * 256; }
 cudaError_t launch_prologue_small(const SmallPrologueLayer* layers, int n, int M, int x_type, bool frag_order, int epoch,
                                   DeviceStatus* st, cudaStream_t s);
-// The small-batch GEMM (tokens on the M side of a 64- or 128-row MMA, 256 weight columns on its N side); up to
-// gemm_small_max_layers() layers with one M per launch.
+// The small-batch GEMM (the weights are the MMA's 128-row operand, the tokens its narrow one); up to gemm_small_max_layers()
+// layers with one M per launch.
 struct SmallGemmLayer {
   const void* xcat;
   const void* packed;

@@ -1,9 +1,9 @@
 // Small-batch form of the layer's contraction for up to 16 tokens (paper Section 3.1 / 3.2:
 // Y = [X_q | T_q] . [W_q ; B_q]; Section 2.1: with this few tokens the layer is bound by the bytes of its weights).
 //
-// The tcgen05 form of the small-batch GEMM converts every packed weight tile to bf16 in shared memory (32 KB written
-// and read again per 9 KB of packed weights), and that traffic, not DRAM, sets its pace.  Here the weights never
-// touch shared memory: a lane loads 16 bytes of one column straight from the packed tile into registers, turns its
+// The tcgen05 form of the small-batch GEMM brings every packed weight tile through shared memory and hands the converted
+// weights over to the tensor core in tensor memory, with a barrier for each step; layers that share a launch are through
+// sooner without either.  Here the weights never touch shared memory: a lane loads 16 bytes of one column straight from the packed tile into registers, turns its
 // nibbles (or crumbs, with 2-bit weights) into the exact bf16 values m * 2^e there (one fma.rn.bf16x2 per pair) and feeds them to
 //     D[16 tokens, 8 columns] += A[16, 16 K] . B[16 K, 8]           (mma.sync m16n8k16, bf16 -> fp32)
 // as the B fragment.  The products are exact and the sums are fp32, as in the tensor-memory kernels.

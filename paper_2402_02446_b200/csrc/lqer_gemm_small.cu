@@ -605,7 +605,7 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
     ly.w_extent = m.off_b - m.off_w; ly.b_extent = m.off_a - m.off_b;
     ly.partials = src.partials;
     ly.counters = src.counters;
-    ly.N = m.N; ly.K64 = m.K64;
+    ly.N = m.N;
     ly.n_tiles = m.n_tiles; ly.k_slabs = m.k_slabs; ly.r_blocks = m.r_blocks;
     ly.spt = m.k_slabs + (use_mma ? (m.r_blocks + 1) / 2 : frag_rank_slabs(m));
     int want = small_gemm_chunks(m);

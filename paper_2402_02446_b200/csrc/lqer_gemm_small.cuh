@@ -20,7 +20,7 @@ struct Layer {
   int* counters;               // [tile] arrivals, zero between calls
   size_t y_extent, partial_extent;   // bytes behind Y and behind partials, for the checked build
   size_t w_extent, b_extent;         // bytes of the packed W and B sections
-  int N, K64, n_tiles, k_slabs, r_blocks;
+  int N, n_tiles, k_slabs, r_blocks;
   int plane;                   // bytes of a plane
   int spt;                     // K stages per tile: k_slabs + rank stages
   int chunks, chunk_stages;    // K chunks per tile; weight stages per chunk (the last chunk also takes the rank stages)

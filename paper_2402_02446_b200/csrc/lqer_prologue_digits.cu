@@ -1,4 +1,4 @@
-// Activation prologue of larger batches with ranks above 64 (paper Section 4.1: X_q in MXINT8, blocks [1,16]; Section 3.1:
+// Activation prologue of larger batches with ranks above 64, or of several layers on one activation (paper Section 4.1: X_q in MXINT8, blocks [1,16]; Section 3.1:
 // the small high-precision product T = X_q A_k), in three launches:
 //   quantise_kernel  X -> Xcat[:, 0:K64] (the exact bf16 values of X_q), one exponent byte per 16-block, and per row the
 //                    range of its exponents; A_q -> digit planes (below);
