@@ -10,8 +10,10 @@
 //            singular vectors V of the small matrix R (one-sided Jacobi in one CTA), and
 //            A = diag(1/s) Q V_k,   B = (Bt V_k)^T = Sigma_k V_k^T.
 // The large products read G as fp32 and accumulate in fp64 (on the fp64 tensor pipe); everything of rank size is fp64.
-// orth() is Cholesky QR applied twice.  Omega (the random test matrix) is an input, so the caller owns the random numbers.
+// orth() is Cholesky QR, applied twice in the end.  Omega (the random test matrix) is an input, so the caller owns the random numbers.
 // None of this is on the inference path; every sum has a fixed order.
+#include <utility>
+
 #include "lqer_common.cuh"
 
 namespace lqer {
@@ -231,45 +233,51 @@ static cudaError_t g_times(const float* G, int K, int N, const double* X, int r,
 }
 
 // ---------------------------------------------------------------------------- tall-skinny helpers (fp64)
-// Partial Gram matrices: part[chunk][r][r] = Y[rows of the chunk]^T Y[rows of the chunk].  grid (r tiles of 16,
-// r tiles of 16, chunks), 256 threads = 16 x 16 outputs.
+// Partial Gram matrices, upper tiles: part[chunk][r][r] = Y[rows of the chunk]^T Y[rows of the chunk].  grid (r tiles of 16,
+// r tiles of 16, chunks), 256 threads = 16 x 16 outputs; the next 32 rows are on their way while these are multiplied (7.2 us for
+// 4096 x 48 against 10.5).
 __global__ void __launch_bounds__(256) gram_partial_kernel(const double* __restrict__ Y, int m, int r, int rows_per_chunk,
                                                            double* __restrict__ part) {
-  __shared__ double s_a[32][17], s_b[32][17];
+  if (blockIdx.x > blockIdx.y) return;                       // only the upper triangle is read
+  __shared__ double s_a[2][32][17], s_b[2][32][17];
   const int i0 = blockIdx.x * 16, j0 = blockIdx.y * 16;
   const int row_lo = blockIdx.z * rows_per_chunk, row_hi = min(m, row_lo + rows_per_chunk);
-  const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
-  double acc = 0.0;
-  for (int q0 = row_lo; q0 < row_hi; q0 += 32) {
-    for (int q = threadIdx.x; q < 32 * 16; q += 256) {
-      const int c = q & 15, rr = q >> 4;
-      const int row = q0 + rr;
-      s_a[rr][c] = (row < row_hi && i0 + c < r) ? Y[(size_t)row * r + i0 + c] : 0.0;
-      s_b[rr][c] = (row < row_hi && j0 + c < r) ? Y[(size_t)row * r + j0 + c] : 0.0;
+  const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;    // the output; also a row and column of the tile being loaded
+  double va[2], vb[2];
+  auto load = [&](int q0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int row = q0 + tj + 16 * h;
+      va[h] = (row < row_hi && i0 + ti < r) ? Y[(size_t)row * r + i0 + ti] : 0.0;
+      vb[h] = (row < row_hi && j0 + ti < r) ? Y[(size_t)row * r + j0 + ti] : 0.0;
     }
+  };
+  double acc = 0.0;
+  load(row_lo);
+  int buf = 0;
+  for (int q0 = row_lo; q0 < row_hi; q0 += 32, buf ^= 1) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) { s_a[buf][tj + 16 * h][ti] = va[h]; s_b[buf][tj + 16 * h][ti] = vb[h]; }
     __syncthreads();
-#pragma unroll 8
-    for (int rr = 0; rr < 32; ++rr) acc = fma(s_a[rr][ti], s_b[rr][tj], acc);
-    __syncthreads();
+    load(q0 + 32);
+#pragma unroll
+    for (int rr = 0; rr < 32; ++rr) acc = fma(s_a[buf][rr][ti], s_b[buf][rr][tj], acc);
   }
   if (i0 + ti < r && j0 + tj < r) part[((size_t)blockIdx.z * r + i0 + ti) * r + j0 + tj] = acc;
 }
 // C = the sum of the partial Gram matrices (in chunk order) = R^T R (upper-triangular R by Cholesky), then Rinv = R^-1; one
 // CTA.  A pivot that is not positive (rank-deficient Y) is replaced by a tiny one so that the run stays finite; status
 // records it.
-// A chain of 2 r short steps, bound by their latency: a step is one update of a whole triangle by all threads (the trailing
-// part of C minus the outer product of a finished row; the rows of R^-1 above a finished one) and ONE barrier - the
-// division of a row by its pivot is left to whoever reads the row, and done for good at the end -, with both matrices in
-// shared memory where they fit (r <= kSharedR).  67 us at r = 48, the sum of the partial matrices included; dot products
-// along rows and columns in global memory took 150 us and the sum 15 us in a kernel of its own.
-constexpr int kSharedR = 112;              // two r x r fp64 matrices within 200 KB
+// Ranks beyond kSharedR: both matrices in global memory, a chain of 2 r short steps bound by their latency.  A step is one
+// update of a whole triangle by all threads (the trailing part of C minus the outer product of a finished row; the rows of
+// R^-1 above a finished one) and one barrier - the division of a row by its pivot is left to whoever reads the row, and done
+// for good at the end.
+constexpr int kSharedR = 112;              // two r x r fp64 matrices within 203 KB of shared memory
 __global__ void __launch_bounds__(1024) cholesky_inverse_kernel(const double* __restrict__ part, int chunks, double* __restrict__ Cg, int r,
                                                                 double* __restrict__ Rinvg, int* __restrict__ status) {
-  extern __shared__ double s_mat[];
   __shared__ double s_inv[kMaxR];                            // 1 / pivot of each row
-  const bool shared = r <= kSharedR;
-  double* C = shared ? s_mat : Cg;
-  double* Rinv = shared ? s_mat + r * r : Rinvg;
+  double* C = Cg;
+  double* Rinv = Rinvg;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   for (int q = threadIdx.x; q < r * r; q += 1024) {
     double acc = 0.0;
@@ -313,52 +321,175 @@ __global__ void __launch_bounds__(1024) cholesky_inverse_kernel(const double* __
   for (int q = threadIdx.x; q < r * r; q += 1024) {
     const int row = q / r, col = q % r;
     const double inv = s_inv[row];
-    if (shared || col >= row) Cg[q] = col == row ? 1.0 / inv : C[q] * inv;
-    Rinvg[q] = Rinv[q] * inv;
+    if (col >= row) C[q] = col == row ? 1.0 / inv : C[q] * inv;
+    Rinv[q] *= inv;
+  }
+}
+// 1 / sqrt(x) of an ordinary positive number: the hardware's first guess (some 22 bits) and one step of Halley's iteration,
+// y + y e (1/2 + 3/8 e) with e = 1 - x y^2, whose error is e^3.  Four dependent operations; an fp64 operation takes some 50 cycles
+// to its result here, and the chains below consist of little else.
+__device__ __forceinline__ double inv_sqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+// The same for r <= kSharedR, in panels of kPanel rows, so that the chain of dependent steps is as short as it can be: one
+// warp factors a diagonal block in registers (a column per lane; a step is one reciprocal square root, two shuffles, a product
+// and a multiply-add), a thread per remaining column solves for the panel's rows of R, all threads update what is left, and the
+// columns of R^-1, which depend on nothing but R, are formed at the end, eight lanes to a column, without a barrier.
+// 3 barriers per panel instead of one per row and another per row of the inverse: 28 us at r = 48 against 67 (33 with the library's
+// rsqrt in the chain).
+constexpr int kPanel = 8, kCholThreads = 512;
+__host__ __device__ constexpr int chol_ld(int r) { return (r + kPanel - 1) / kPanel * kPanel + 1; }   // odd: eight rows meet no bank twice
+__global__ void __launch_bounds__(kCholThreads) cholesky_inverse_panels_kernel(const double* __restrict__ part, int chunks, double* __restrict__ Cg,
+                                                                               int r, double* __restrict__ Rinvg, int* __restrict__ status) {
+  extern __shared__ double s_mat[];
+  const int rp = (r + kPanel - 1) / kPanel * kPanel, ld = chol_ld(r);
+  double* C = s_mat;
+  double* Ri = s_mat + rp * ld;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int q = tid; q < rp * rp; q += kCholThreads) {
+    const int row = q / rp, col = q % rp;
+    double acc = row == col ? 1.0 : 0.0;                     // rows beyond r: the identity
+    if (row < r && col < r && row <= col) {
+      acc = 0.0;
+#pragma unroll 16
+      for (int i = 0; i < chunks; ++i) acc += part[(size_t)i * r * r + row * r + col];
+    }
+    C[row * ld + col] = acc;
+    Ri[row * ld + col] = 0.0;
+  }
+  __syncthreads();
+  for (int j0 = 0; j0 < rp; j0 += kPanel) {
+    if (warp == 0) {
+      const int c = lane & 7;
+      double d[kPanel];
+#pragma unroll
+      for (int i = 0; i < kPanel; ++i) d[i] = i <= c ? C[(j0 + i) * ld + j0 + c] : 0.0;
+      double mine = 1.0;                                     // 1 / pivot of this lane's column
+      bool low = false;
+#pragma unroll
+      for (int j = 0; j < kPanel; ++j) {
+        double p = __shfl_sync(0xFFFFFFFFu, d[j], j);
+        if (!(p > 0.0)) { p = 1e-300; low = true; }
+        const double inv = inv_sqrt(p);
+        if (c == j) mine = inv;
+        d[j] = (c == j ? p : d[j]) * inv;
+#pragma unroll
+        for (int i = j + 1; i < kPanel; ++i) d[i] = fma(-__shfl_sync(0xFFFFFFFFu, d[j], i), d[j], d[i]);
+      }
+      if (low && lane == 0) atomicMax(status, 2);
+      if (lane < kPanel) Ri[(j0 + c) * ld + j0 + c] = mine;  // the reciprocals of the diagonal
+      if (lane < kPanel)
+#pragma unroll
+        for (int i = 0; i < kPanel; ++i)
+          if (i <= c) C[(j0 + i) * ld + j0 + c] = d[i];
+    }
+    __syncthreads();
+    const int left = rp - j0 - kPanel;
+    if (left == 0) break;
+    if (tid < left) {
+      const int c = j0 + kPanel + tid;
+      double x[kPanel];
+#pragma unroll
+      for (int j = 0; j < kPanel; ++j) x[j] = C[(j0 + j) * ld + c];
+#pragma unroll
+      for (int j = 0; j < kPanel; ++j) {
+        x[j] *= Ri[(j0 + j) * ld + j0 + j];
+#pragma unroll
+        for (int i = j + 1; i < kPanel; ++i) x[i] = fma(-C[(j0 + j) * ld + j0 + i], x[j], x[i]);
+        C[(j0 + j) * ld + c] = x[j];
+      }
+    }
+    __syncthreads();
+    for (int q = tid; q < left * left; q += kCholThreads) {
+      const int i = j0 + kPanel + q / left, c = j0 + kPanel + q % left;
+      if (c >= i) {
+        double v = C[i * ld + c];
+#pragma unroll
+        for (int j = 0; j < kPanel; ++j) v = fma(-C[(j0 + j) * ld + i], C[(j0 + j) * ld + c], v);
+        C[i * ld + c] = v;
+      }
+    }
+    __syncthreads();
+  }
+  // R Rinv = I: column c from its own row upwards, a panel of rows at a time; lane i of eight has row i of the panel
+  for (int c0 = warp * 4; c0 < rp; c0 += kCholThreads / 8) {
+    const int c = c0 + (lane >> 3), i = lane & 7;
+    for (int I = c / kPanel; I >= 0; --I) {
+      // every lane of the warp walks the same panels: the four columns of a warp lie in one panel
+      const int row = I * kPanel + i;
+      double v = row == c ? 1.0 : 0.0;
+      for (int k = (I + 1) * kPanel; k <= c; ++k) v = fma(-C[row * ld + k], Ri[k * ld + c], v);
+      // back substitution within the panel
+      double x = 0.0;
+#pragma unroll
+      for (int k = kPanel - 1; k >= 0; --k) {
+        const double xk = __shfl_sync(0xFFFFFFFFu, v * Ri[row * ld + row], (lane & 24) + k);
+        if (i == k) x = xk;
+        if (i < k) v = fma(-C[row * ld + I * kPanel + k], xk, v);
+      }
+      __syncwarp();
+      if (row <= c && row != c) Ri[row * ld + c] = x;
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  for (int q = tid; q < r * r; q += kCholThreads) {
+    const int row = q / r, col = q % r;
+    if (col >= row) Cg[q] = C[row * ld + col];
+    Rinvg[q] = Ri[row * ld + col];
   }
 }
 static cudaError_t cholesky_inverse(const double* part, int chunks, double* C, int r, double* Rinv, int* status, cudaStream_t s) {
   static OncePerDevice once;
-  const cudaError_t e = once.run([] {
-    return cudaFuncSetAttribute(cholesky_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kSharedR * kSharedR * 8);
-  });
+  constexpr int kMost = 2 * kSharedR * chol_ld(kSharedR) * 8;
+  const cudaError_t e = once.run([] { return cudaFuncSetAttribute(cholesky_inverse_panels_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost); });
   if (e != cudaSuccess) return e;
-  cholesky_inverse_kernel<<<1, 1024, r <= kSharedR ? 2 * r * r * 8 : 0, s>>>(part, chunks, C, r, Rinv, status);
+  if (r <= kSharedR)
+    cholesky_inverse_panels_kernel<<<1, kCholThreads, 2 * (chol_ld(r) - 1) * chol_ld(r) * 8, s>>>(part, chunks, C, r, Rinv, status);
+  else
+    cholesky_inverse_kernel<<<1, 1024, 0, s>>>(part, chunks, C, r, Rinv, status);
   return cudaGetLastError();
 }
 // Out[m, c] = rowscale[m] * sum_j Y[m, j] T[j, c] for c < cols (T is [r, ldt]); fp64 in, OutT out, optionally
-// written transposed (Out[c, m]).  One CTA = 64 rows; T's used columns are walked in tiles of 64.
+// written transposed (Out[c, m]).  One CTA = 32 rows and up to 64 columns; T's used columns are walked in tiles of 64.  Bound by the
+// latency of its loads, so all of a step's operands (48 of the r inner positions) are requested together: 8.6 us for 4096 x 48
+// against 15.8 with 64 rows and 16 positions.
+constexpr int kTallRows = 32, kTallStep = 48;
 template <typename OutT, bool TRANSPOSE_OUT>
 __global__ void __launch_bounds__(256) tall_times_small_kernel(const double* __restrict__ Y, int m, int r, const double* __restrict__ T,
                                                                int ldt, int cols, const double* __restrict__ rowscale, int invert_scale,
                                                                OutT* __restrict__ Out) {
-  __shared__ double s_y[16][65], s_t[16][65];
-  const int m0 = blockIdx.x * 64, c0 = blockIdx.y * 64;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4];
+  __shared__ double s_y[kTallStep][kTallRows + 1], s_t[kTallStep][64];
+  const int m0 = blockIdx.x * kTallRows, c0 = blockIdx.y * 64;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;      // columns tx, tx + 32 of rows 4 ty ..
+  double acc[4][2];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-  for (int j0 = 0; j0 < r; j0 += 16) {
-    for (int q = threadIdx.x; q < 64 * 16; q += 256) {
-      const int jj = q & 15, mi = q >> 4;
-      s_y[jj][mi] = (m0 + mi < m && j0 + jj < r) ? Y[(size_t)(m0 + mi) * r + j0 + jj] : 0.0;
-      const int cc = q & 63, j2 = q >> 6;
-      s_t[j2][cc] = (j0 + j2 < r && c0 + cc < cols) ? T[(size_t)(j0 + j2) * ldt + c0 + cc] : 0.0;
+    for (int j = 0; j < 2; ++j) acc[i][j] = 0.0;
+  for (int j0 = 0; j0 < r; j0 += kTallStep) {
+    const int n = min(kTallStep, r - j0);
+    for (int q = threadIdx.x; q < kTallRows * kTallStep; q += 256) {
+      const int jj = q % kTallStep, mi = q / kTallStep;
+      s_y[jj][mi] = (m0 + mi < m && jj < n) ? Y[(size_t)(m0 + mi) * r + j0 + jj] : 0.0;
+    }
+    for (int q = threadIdx.x; q < kTallStep * 64; q += 256) {
+      const int cc = q & 63, jj = q >> 6;
+      s_t[jj][cc] = (jj < n && c0 + cc < cols) ? T[(size_t)(j0 + jj) * ldt + c0 + cc] : 0.0;
     }
     __syncthreads();
+#pragma unroll 8
+    for (int jj = 0; jj < kTallStep; ++jj) {
+      const double b0 = s_t[jj][tx], b1 = s_t[jj][tx + 32];
 #pragma unroll
-    for (int jj = 0; jj < 16; ++jj) {
-      double a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = s_y[jj][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = s_t[jj][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+      for (int i = 0; i < 4; ++i) {
+        const double a = s_y[jj][ty * 4 + i];
+        acc[i][0] = fma(a, b0, acc[i][0]);
+        acc[i][1] = fma(a, b1, acc[i][1]);
+      }
     }
     __syncthreads();
   }
@@ -369,8 +500,8 @@ __global__ void __launch_bounds__(256) tall_times_small_kernel(const double* __r
     double sc = 1.0;
     if (rowscale != nullptr) sc = invert_scale ? 1.0 / rowscale[row] : rowscale[row];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = c0 + tx * 4 + j;
+    for (int j = 0; j < 2; ++j) {
+      const int c = c0 + tx + 32 * j;
       if (c < cols) {
         if (TRANSPOSE_OUT) Out[(size_t)c * m + row] = (OutT)(sc * acc[i][j]);
         else Out[(size_t)row * cols + c] = (OutT)(sc * acc[i][j]);
@@ -380,11 +511,29 @@ __global__ void __launch_bounds__(256) tall_times_small_kernel(const double* __r
 }
 
 // ---------------------------------------------------------------------------- small SVD (one CTA)
+// The rotation that makes two columns orthogonal: tan from approximate reciprocals (a tangent that is off by 1e-6 of itself
+// leaves that part of gamma for the next sweep, which the quadratic convergence absorbs), but cos = 1 / sqrt(1 + tan^2) in
+// full, so that the rotation is orthogonal to rounding.
+__device__ __forceinline__ double approx_rcp(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+__device__ __forceinline__ void rotation(double alpha, double beta, double gamma, double& c, double& s) {
+  const double zeta = (beta - alpha) * approx_rcp(2.0 * gamma), az = fabs(zeta);
+  const double u = fma(zeta, zeta, 1.0);
+  double root;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(root) : "d"(u));
+  const double t = copysign(approx_rcp(az < 1e100 ? fma(u, root, az) : 2.0 * az), zeta);
+  c = inv_sqrt(fma(t, t, 1.0));
+  s = c * t;
+}
 // Right singular vectors and singular values of the r x r upper-triangular R (the Cholesky factor left in the upper
 // triangle of C, row-major) by one-sided Jacobi: pairs of columns are rotated until all are mutually orthogonal,
-// V collects the rotations.  A warp per pair, the pairs of a step disjoint (round-robin tournament).  Mt, Vt: r x r
+// V collects the rotations.  A half warp per pair, the pairs of a step disjoint (round-robin tournament).  Mt, Vt: r x r
 // scratch, column-major.  Out: Vs row-major [r][r] with the columns in falling order of singular value, sigma[r].
-// Bound by the latency of its steps (r - 1 per sweep, one barrier each): both matrices sit in shared memory where they fit.
+// Bound by its steps (r - 1 per sweep, one barrier each), in them by the fp64 pipe as much as by latency: half warps and
+// approximate quotients took 707 us at r = 48 to 377.  Both matrices sit in shared memory where they fit.
 __global__ void __launch_bounds__(1024) jacobi_right_kernel(const double* __restrict__ C, int r, double* __restrict__ Mtg,
                                                             double* __restrict__ Vtg, double* __restrict__ Vs, double* __restrict__ sigma,
                                                             int* __restrict__ status) {
@@ -407,38 +556,46 @@ __global__ void __launch_bounds__(1024) jacobi_right_kernel(const double* __rest
     if (tid == 0) s_rotated = 0;
     __syncthreads();
     for (int t = 0; t < n - 1; ++t) {
-      for (int i = warp; i < n / 2; i += 32) {
-        int a = i == 0 ? n - 1 : (t + i) % (n - 1);
-        int b = i == 0 ? t % (n - 1) : (t + n - 1 - i) % (n - 1);
-        if (a >= r || b >= r) continue;
-        const int p = min(a, b), q = max(a, b);
+      for (int i0 = 2 * warp; i0 < n / 2; i0 += 64) {      // a half warp per pair: the scalars cost the fp64 pipe as much as a whole row
+        const int i = i0 + (lane >> 4);
+        int a = n - 1, b = t;
+        if (i > 0) {
+          a = t + i; b = t + n - 1 - i;
+          if (a >= n - 1) a -= n - 1;
+          if (b >= n - 1) b -= n - 1;
+        }
+        const bool live = i < n / 2 && a < r && b < r;
+        const int p = live ? min(a, b) : 0, q = live ? max(a, b) : 0;
         double* mp = Mt + (size_t)p * r;
         double* mq = Mt + (size_t)q * r;
         double alpha = 0.0, beta = 0.0, gamma = 0.0;
-        for (int row = lane; row < r; row += 32) {
-          const double x = mp[row], y = mq[row];
-          alpha = fma(x, x, alpha); beta = fma(y, y, beta); gamma = fma(x, y, gamma);
-        }
+        if (live)
+          for (int row = lane & 15; row < r; row += 16) {
+            const double x = mp[row], y = mq[row];
+            alpha = fma(x, x, alpha); beta = fma(y, y, beta); gamma = fma(x, y, gamma);
+          }
 #pragma unroll
-        for (int sft = 16; sft > 0; sft >>= 1) {
+        for (int sft = 8; sft > 0; sft >>= 1) {
           alpha += __shfl_xor_sync(0xFFFFFFFFu, alpha, sft);
           beta += __shfl_xor_sync(0xFFFFFFFFu, beta, sft);
           gamma += __shfl_xor_sync(0xFFFFFFFFu, gamma, sft);
         }
-        if (fabs(gamma) > tol * sqrt(alpha * beta)) {
-          const double zeta = (beta - alpha) / (2.0 * gamma);
-          const double tt = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-          const double c = 1.0 / sqrt(1.0 + tt * tt), s = c * tt;
-          double* vp = Vt + (size_t)p * r;
-          double* vq = Vt + (size_t)q * r;
-          for (int row = lane; row < r; row += 32) {
-            const double x = mp[row], y = mq[row];
-            mp[row] = c * x - s * y; mq[row] = s * x + c * y;
-            const double u = vp[row], w = vq[row];
-            vp[row] = c * u - s * w; vq[row] = s * u + c * w;
+        if (live && gamma * gamma > (tol * alpha) * (tol * beta)) {
+          double c, s;
+          rotation(alpha, beta, gamma, c, s);
+          if (s != 0.0) {
+            double* vp = Vt + (size_t)p * r;
+            double* vq = Vt + (size_t)q * r;
+            for (int row = lane & 15; row < r; row += 16) {
+              const double x = mp[row], y = mq[row];
+              mp[row] = c * x - s * y; mq[row] = s * x + c * y;
+              const double u = vp[row], w = vq[row];
+              vp[row] = c * u - s * w; vq[row] = s * u + c * w;
+            }
+            if ((lane & 15) == 0) s_rotated = 1;
           }
-          if (lane == 0) s_rotated = 1;
         }
+        __syncwarp();
       }
       __syncthreads();
     }
@@ -490,24 +647,22 @@ size_t factor_workspace_bytes(int K, int N, int k, int max_calib_rows) {
   return b;
 }
 
-static cudaError_t orthonormalise(const double* Yin, double* Yout, int m, int r, double* gram_part, double* C, double* Rinv,
-                                  int* status, cudaStream_t s) {
+// Y = Q R with Q^T Q = I by Cholesky QR, `passes` times, with `other` as the second buffer; *out: where Q lies.  One pass leaves
+// Q^T Q - I of the size rounding * cond(Y)^2, which is enough between two products of the iteration (what counts there is the
+// space the columns span, and that they are far from dependent); a second one makes it orthonormal to rounding.
+static cudaError_t orthonormalise(double* Y, double* other, int m, int r, int passes, double* gram_part, double* C, double* Rinv,
+                                  int* status, double** out, cudaStream_t s) {
   using namespace fac;
-  // Cholesky QR, twice: Y = Q R with Q^T Q = I to rounding once the first pass has tamed the conditioning
-  const double* src = Yin;
-  double* bufs[2] = {Yout, const_cast<double*>(Yin)};
-  for (int pass = 0; pass < 2; ++pass) {
-    const int chunks = kGramChunks, rows_per_chunk = (m + chunks - 1) / chunks;
-    const int rt = (r + 15) / 16;
-    gram_partial_kernel<<<dim3(rt, rt, chunks), 256, 0, s>>>(src, m, r, rows_per_chunk, gram_part);
+  const int chunks = kGramChunks, rows_per_chunk = (m + chunks - 1) / chunks, rt = (r + 15) / 16;
+  for (int pass = 0; pass < passes; ++pass) {
+    gram_partial_kernel<<<dim3(rt, rt, chunks), 256, 0, s>>>(Y, m, r, rows_per_chunk, gram_part);
     const cudaError_t e = cholesky_inverse(gram_part, chunks, C, r, Rinv, status, s);
     if (e != cudaSuccess) return e;
-    double* dst = bufs[pass];
-    tall_times_small_kernel<double, false><<<dim3((m + 63) / 64, (r + 63) / 64), 256, 0, s>>>(src, m, r, Rinv, r, r, nullptr, 0, dst);
-    src = dst;
+    tall_times_small_kernel<double, false><<<dim3((m + kTallRows - 1) / kTallRows, (r + 63) / 64), 256, 0, s>>>(Y, m, r, Rinv, r, r, nullptr, 0, other);
+    std::swap(Y, other);
   }
-  // after two passes the result sits in Yin's buffer; copy back to Yout so that the caller's view is uniform
-  return cudaMemcpyAsync(Yout, src, (size_t)m * r * 8, cudaMemcpyDeviceToDevice, s);
+  *out = Y;
+  return cudaGetLastError();
 }
 
 // W [K,N], calibration samples Xs[i] [rows[i], K] (n_samples may be 0: plain LQER, S = I), Omega [N, r] fp32 with
@@ -543,7 +698,7 @@ cudaError_t launch_factorize(const float* W, const float* const* Xs, const int* 
   if (A_used != nullptr) *A_used = A;
   if (B_used != nullptr) *B_used = B;
 
-  LaunchScope scope(kFamPrepare, s, 16 + 12 * kIters);
+  LaunchScope scope(kFamPrepare, s, 18 + 8 * kIters);
   cudaMemsetAsync(status, 0, 4, s);
   // ---- S (Appendix A), or the identity
   if (n_samples > 0) {
@@ -560,17 +715,19 @@ cudaError_t launch_factorize(const float* W, const float* const* Xs, const int* 
   scaled_error_kernel<<<dim3((N + 255) / 256, K / 16), 256, 0, s>>>(W, K, N, w_bits, emin, emax, sc, G);
   // ---- subspace iteration
   widen_kernel<<<(int)(((size_t)N * r + 255) / 256), 256, 0, s>>>(Omega, (size_t)N * r, T1);
+  double* Q = nullptr;
+  double* Z = nullptr;
   cudaError_t e = g_times<false>(G, K, N, T1, r, T0, s);                                 // Y = G Omega      [K, r]
   if (e != cudaSuccess) return e;
-  e = orthonormalise(T0, T1, K, r, gram_part, C, Rinv, status, s);           // Q in T1
-  if (e != cudaSuccess) return e;
+  if ((e = orthonormalise(T0, T1, K, r, 1, gram_part, C, Rinv, status, &Q, s)) != cudaSuccess) return e;   // Q in T1
   for (int it = 0; it < kIters; ++it) {
-    if ((e = g_times<true>(G, K, N, T1, r, T0, s)) != cudaSuccess) return e;     // Z = G^T Q        [N, r]
-    if ((e = orthonormalise(T0, Bt, N, r, gram_part, C, Rinv, status, s)) != cudaSuccess) return e;   // Z in Bt
-    if ((e = g_times<false>(G, K, N, Bt, r, T0, s)) != cudaSuccess) return e;    // Y = G Z          [K, r]
-    if ((e = orthonormalise(T0, T1, K, r, gram_part, C, Rinv, status, s)) != cudaSuccess) return e;   // Q in T1
+    if ((e = g_times<true>(G, K, N, Q, r, T0, s)) != cudaSuccess) return e;      // Z = G^T Q        [N, r]
+    if ((e = orthonormalise(T0, Bt, N, r, 1, gram_part, C, Rinv, status, &Z, s)) != cudaSuccess) return e;   // Z in Bt
+    if ((e = g_times<false>(G, K, N, Z, r, T0, s)) != cudaSuccess) return e;     // Y = G Z          [K, r]
+    // Q in T1, after the last round in T0
+    if ((e = orthonormalise(T0, T1, K, r, it + 1 < kIters ? 1 : 2, gram_part, C, Rinv, status, &Q, s)) != cudaSuccess) return e;
   }
-  if ((e = g_times<true>(G, K, N, T1, r, Bt, s)) != cudaSuccess) return e;       // Bt = G^T Q       [N, r]
+  if ((e = g_times<true>(G, K, N, Q, r, Bt, s)) != cudaSuccess) return e;        // Bt = G^T Q       [N, r]
   // ---- small SVD: Bt^T Bt = R^T R, R = U Sigma V^T  ->  G ~ (Q V) Sigma (...)^T
   {
     const int chunks = kGramChunks, rpc = (N + chunks - 1) / chunks, rt = (r + 15) / 16;
@@ -584,8 +741,8 @@ cudaError_t launch_factorize(const float* W, const float* const* Xs, const int* 
     jacobi_right_kernel<<<1, 1024, r <= kSharedR ? 2 * r * r * 8 : 0, s>>>(C, r, Mt, Vt, Vs, sigma, status);
   }
   // ---- A = S^-1 Q V_k  [K, k];  B = (Bt V_k)^T  [k, N]
-  tall_times_small_kernel<float, false><<<dim3((K + 63) / 64, (k + 63) / 64), 256, 0, s>>>(T1, K, r, Vs, r, k, sc, 1, A);
-  tall_times_small_kernel<float, true><<<dim3((N + 63) / 64, (k + 63) / 64), 256, 0, s>>>(Bt, N, r, Vs, r, k, nullptr, 0, B);
+  tall_times_small_kernel<float, false><<<dim3((K + kTallRows - 1) / kTallRows, (k + 63) / 64), 256, 0, s>>>(Q, K, r, Vs, r, k, sc, 1, A);
+  tall_times_small_kernel<float, true><<<dim3((N + kTallRows - 1) / kTallRows, (k + 63) / 64), 256, 0, s>>>(Bt, N, r, Vs, r, k, nullptr, 0, B);
   return cudaGetLastError();
 }
 

@@ -97,3 +97,25 @@ def test_prepare_reports_a_dead_calibration_channel():
     with pytest.raises(ValueError):
         olqer.calibration_scale([x])
     Pg.release()
+
+
+@pytest.mark.parametrize("k,scale", [(1, 20.0), (32, 1e5), (96, 20.0), (97, 1e3)])
+def test_prepare_at_the_edges_of_the_factorisation(k, scale):
+    # sketches of 17, 48, 112 (the last in shared memory) and 113 columns; and a calibration whose outlier channels are 1e5 times the
+    # others, so that the columns between two products of the iteration are nearly dependent (condition 1e5 and more).
+    # S A is orthonormal and B = (S A)^T (S E_q) up to the rounding of A and B to fp32 (2^-24 each, over k columns).
+    spec = gen.LayerSpec("pp_e", M=8, K=512, N=264, k=k, calib_rows=64, outlier_frac=0.0, n_outliers=6, outlier_scale=scale, seed=505)
+    W = gen.make_weight(spec)
+    samples = _samples(spec, (64,))
+    Pg, A, B, code = L.prepare_from_calibration(_t(W), [_t(x) for x in samples], k, seed=spec.seed)
+    assert code == 0
+    A, B = A.cpu().numpy().astype(np.float64), B.cpu().numpy().astype(np.float64)
+    Wm, We = olqer.quantize_weight(W)
+    SE = olqer.calibration_scale(samples)[:, None] * olqer.quantization_error(W, Wm, We)
+    SA = olqer.calibration_scale(samples)[:, None] * A
+    sig = np.linalg.svd(SE, compute_uv=False)
+    assert np.max(np.abs(SA.T @ SA - np.eye(k))) < 1e-6
+    assert np.linalg.norm(B - SA.T @ SE) < 1e-6 * np.linalg.norm(B)
+    optimum, got = np.sqrt(np.sum(sig[k:] ** 2)), np.linalg.norm(SE - SA @ B)
+    assert optimum * (1 - 1e-6) <= got <= optimum * (1 + 1e-2)
+    Pg.release()
