@@ -113,13 +113,13 @@ __host__ __device__ inline int t_subsets(int k_pad) {
 
 struct Formats { int a_bits, lr_bits, exp_min, exp_max, x_type, w_bits; };
 
-// X -> MXINT8 for the whole contraction, by all threads of the CTA: per row the mantissas in the byte order the nibbles
+// X -> MXINT8 for the columns [c_lo, c_lo + n_cols) of the contraction (multiples of 64), by all threads of the CTA: per row the mantissas in the byte order the nibbles
 // unpack to ({0,4,1,5}, {2,6,3,7} within each 8), the block scales 2^(e_x - 6) and the dp4a seeds (bits of
 // 1.5 * 2^23, minus sum(x) of the block times the offset of the stored weights: 8 for nibbles, 1 for crumbs).
-__device__ __forceinline__ void quantize_x_rows(const void* X, int M, int K, int K64, const Formats& f, uint8_t* xm,
+__device__ __forceinline__ void quantize_x_rows(const void* X, int M, int K, int c_lo, int n_cols, const Formats& f, uint8_t* xm,
                                                 float* xsc, int* xof) {
-  const int tid = threadIdx.x, KB = K64 / 16;
-  const int per_row = K64 / 4, total = M * per_row;             // float4 items: (row, quarter-block)
+  const int tid = threadIdx.x, KB = n_cols / 16;
+  const int per_row = n_cols / 4, total = M * per_row;             // float4 items: (row, quarter-block)
   constexpr int U = 4;                                             // loads in flight per thread
   for (int base = 0; base < total; base += kThreads * U) {
     float4 v[U];
@@ -128,7 +128,7 @@ __device__ __forceinline__ void quantize_x_rows(const void* X, int M, int K, int
       const int item = base + u * kThreads + tid;
       const int row = item / per_row, c4 = item % per_row;
       v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (item < total && c4 * 4 < K) v[u] = load_x_quad(X, f.x_type, M, K, row, c4 * 4, f.a_bits, f.exp_min, f.exp_max);
+      if (item < total && c_lo + c4 * 4 < K) v[u] = load_x_quad(X, f.x_type, M, K, row, c_lo + c4 * 4, f.a_bits, f.exp_min, f.exp_max);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -146,7 +146,7 @@ __device__ __forceinline__ void quantize_x_rows(const void* X, int M, int K, int
       sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
       sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 2);
       if (valid) {
-        *reinterpret_cast<uint32_t*>(xm + (size_t)row * K64 + c4 * 4) = perm;
+        *reinterpret_cast<uint32_t*>(xm + (size_t)row * n_cols + c4 * 4) = perm;
         if ((c4 & 3) == 0) {
           xsc[row * KB + (c4 >> 2)] = pow2f(e - (f.a_bits - 2));
           xof[row * KB + (c4 >> 2)] = kIntMagicBits - (f.w_bits == 2 ? 1 : 8) * sum;
@@ -161,10 +161,10 @@ __device__ __forceinline__ void quantize_x_rows(const void* X, int M, int K, int
 // exponents of one row spread over more than about 30 binades, and the order of the additions is fixed in any case.
 // Leaves tsub[t_subsets(k_pad)][kMaxM][k_pad]; the caller adds the subsets in order after a barrier.
 template <int MT, int UNROLL, bool STAGED>
-__device__ __forceinline__ void t_partial(const uint8_t* asec, int K, int K64, int k_pad, int kb_lo, int kb_hi, int M,
+__device__ __forceinline__ void t_partial(const uint8_t* asec, int K, int kb0, int n_cols, int k_pad, int kb_lo, int kb_hi, int M,
                                           const Formats& f, const uint8_t* xm, const float* xsc, double* tsub) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int KBr = K / 16, KB = K64 / 16;
+  const int KBr = K / 16, KB = n_cols / 16;                    // xm, xsc hold the blocks [kb0, kb0 + KB)
   const int NT = (k_pad + 31) / 32;                            // tiles of 32 rank columns, a lane each
   const uint8_t* a_exp = asec + (size_t)KBr * k_pad * 16;
   const int bias = -127 - (f.lr_bits - 2);                        // exponent bytes carry +127
@@ -189,12 +189,12 @@ __device__ __forceinline__ void t_partial(const uint8_t* asec, int K, int K64, i
         for (int r = 0; r < MT; ++r) {
           if (r < M) {
             // the X mantissas are stored as {0,4,1,5}, {2,6,3,7} within each 8: back to the order of A_q
-            const uint4 x = *reinterpret_cast<const uint4*>(xm + (size_t)r * K64 + kb * 16);
+            const uint4 x = *reinterpret_cast<const uint4*>(xm + (size_t)r * n_cols + (kb - kb0) * 16);
             int sm = __dp4a((int)__byte_perm(x.x, x.y, 0x6420), (int)a.x, 0);
             sm = __dp4a((int)__byte_perm(x.x, x.y, 0x7531), (int)a.y, sm);
             sm = __dp4a((int)__byte_perm(x.z, x.w, 0x6420), (int)a.z, sm);
             sm = __dp4a((int)__byte_perm(x.z, x.w, 0x7531), (int)a.w, sm);
-            tacc[r] = fma((double)sm, (double)xsc[r * KB + kb] * sa, tacc[r]);
+            tacc[r] = fma((double)sm, (double)xsc[r * KB + kb - kb0] * sa, tacc[r]);
           }
         }
       }
@@ -232,51 +232,98 @@ struct PreCall {
   int M, K, K64, k_pad;
   Formats f;
 };
+constexpr int kPreShare = 8;    // CTAs (a cluster) to a call, at most
 struct PreParams {
   PreCall c[kPreMaxCalls];
+  int share;                    // CTAs to a call in this launch
+  int off_tsub;                 // shared memory: where the sums of T begin
   int order;                    // ChainOrder, as for the decode kernel
 };
 __host__ __device__ inline size_t pre_x_bytes(int M, int K64) { return (size_t)M * K64 + (size_t)M * (K64 / 16) * 8; }
 __host__ __device__ inline size_t pre_t_bytes(int k_pad) { return (size_t)kMaxM * 16 * 4 + (size_t)kMaxM * (k_pad > 0 ? k_pad : 16); }
 
+// A call is worked on by a cluster: its CTAs take a range of K each (their part of X and of A_q), and the first adds their
+// sums of T up in CTA order through distributed shared memory.  Bound by the latency of fetching A_q, 139 to 374 KB a call at
+// rank 32, which one SM alone asks for in many rounds.
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ double ld_dsmem(const double* local, uint32_t cta) {
+  uint32_t remote;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(cta));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(remote) : "memory");
+  return v;
+}
 template <int MT>
-__global__ void __launch_bounds__(kThreads, 1) decode_pre_kernel(const __grid_constant__ PreParams p) {
+__global__ void __launch_bounds__(kThreads, 2) decode_pre_kernel(const __grid_constant__ PreParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
-  const PreCall& c = p.c[blockIdx.x];
-  const int M = c.M, KB = c.K64 / 16, tid = threadIdx.x;
-  uint8_t* xm = smem;
-  float* xsc = reinterpret_cast<float*>(xm + (size_t)M * c.K64);
-  int* xof = reinterpret_cast<int*>(xsc + (size_t)M * KB);
-  float* tqs = reinterpret_cast<float*>(xof + (size_t)M * KB);
+  const PreCall& c = p.c[(int)blockIdx.x / p.share];
+  const int rank = (int)cluster_rank(), slabs = c.K64 / 64;
+  const int c_lo = 64 * (rank * slabs / p.share), c_hi = 64 * ((rank + 1) * slabs / p.share), n_cols = c_hi - c_lo;
+  const int M = c.M, KB = c.K64 / 16, nb = n_cols / 16, tid = threadIdx.x;
+  const int subsets = t_subsets(c.k_pad), total = M * c.k_pad;
+  uint8_t* xm = smem;                                   // this range: [M][n_cols] mantissas, [M][nb] scales, [M][nb] seeds
+  float* xsc = reinterpret_cast<float*>(xm + (size_t)M * n_cols);
+  int* xof = reinterpret_cast<int*>(xsc + (size_t)M * nb);
+  float* tqs = reinterpret_cast<float*>(xof + (size_t)M * nb);
   int8_t* tq8 = reinterpret_cast<int8_t*>(tqs + kMaxM * 16);
-  const size_t out_bytes = pre_x_bytes(M, c.K64) + pre_t_bytes(c.k_pad);
-  double* tsub = reinterpret_cast<double*>(smem + ((out_bytes + 15) & ~(size_t)15));
+  double* tsub = reinterpret_cast<double*>(smem + p.off_tsub);
+  double* tsum = tsub + (size_t)subsets * kMaxM * c.k_pad;   // [M][k_pad]: the range's sums
+  uint8_t* out = c.out;
 
   if (p.order != kChainFirst) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (p.order != kChainLater) asm volatile("griddepcontrol.wait;" ::: "memory");   // X may be an earlier kernel's output
   if (p.order == kChainFirst) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-  quantize_x_rows(c.X, M, c.K, c.K64, c.f, xm, xsc, xof);
+  quantize_x_rows(c.X, M, c.K, c_lo, n_cols, c.f, xm, xsc, xof);
   for (int i = tid; i < (int)pre_t_bytes(c.k_pad) / 4; i += kThreads) reinterpret_cast<uint32_t*>(tqs)[i] = 0u;
   __syncthreads();
   if (c.k_pad > 0) {
-    t_partial<MT, 8, false>(c.asec, c.K, c.K64, c.k_pad, 0, c.K / 16, M, c.f, xm, xsc, tsub);   // the whole of K: many loads in flight
+    const int kb_lo = c_lo / 16, kb_hi = min(c_hi / 16, c.K / 16);
+    t_partial<MT, 8, false>(c.asec, c.K, kb_lo, n_cols, c.k_pad, kb_lo, kb_hi, M, c.f, xm, xsc, tsub);   // many loads in flight
     __syncthreads();
-    const int subsets = t_subsets(c.k_pad), total = M * c.k_pad;
+    for (int idx = tid; idx < total; idx += kThreads) {
+      const int row = idx / c.k_pad, col = idx % c.k_pad;
+      double v = 0.0;
+      for (int q = 0; q < subsets; ++q) v += tsub[((size_t)q * kMaxM + row) * c.k_pad + col];
+      tsum[idx] = v;
+    }
+  }
+  // X_q leaves while the cluster meets
+  for (int r = 0; r < M; ++r) {
+    for (int o = tid * 16; o < n_cols; o += kThreads * 16)
+      *reinterpret_cast<uint4*>(out + (size_t)r * c.K64 + c_lo + o) = *reinterpret_cast<const uint4*>(xm + (size_t)r * n_cols + o);
+    uint8_t* sc = out + (size_t)M * c.K64 + ((size_t)r * KB + c_lo / 16) * 4;
+    for (int o = tid * 16; o < nb * 4; o += kThreads * 16) {
+      *reinterpret_cast<uint4*>(sc + o) = *reinterpret_cast<const uint4*>(reinterpret_cast<uint8_t*>(xsc + r * nb) + o);
+      *reinterpret_cast<uint4*>(sc + (size_t)M * KB * 4 + o) = *reinterpret_cast<const uint4*>(reinterpret_cast<uint8_t*>(xof + r * nb) + o);
+    }
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (rank == 0) {
     for (int base = 0; base < total; base += kThreads) {
       const int idx = base + tid;
       const bool valid = idx < total;
       const int row = valid ? idx / c.k_pad : 0, col = valid ? idx % c.k_pad : 0;
-      double tv = 0.0;
-      if (valid)
-        for (int q = 0; q < subsets; ++q) tv += tsub[((size_t)q * kMaxM + row) * c.k_pad + col];
+      double part[kPreShare], tv = 0.0;
+#pragma unroll
+      for (int q = 0; q < kPreShare; ++q) part[q] = valid && q < p.share ? ld_dsmem(tsum + idx, (uint32_t)q) : 0.0;
+#pragma unroll
+      for (int q = 0; q < kPreShare; ++q) tv += part[q];
       store_tq(tv, valid, row, col, c.k_pad, c.f, tq8, tqs);
     }
     __syncthreads();
+    uint8_t* to = out + pre_x_bytes(M, c.K64);
+    for (int o = tid * 16; o < (int)pre_t_bytes(c.k_pad); o += kThreads * 16)
+      *reinterpret_cast<uint4*>(to + o) = *reinterpret_cast<const uint4*>(reinterpret_cast<uint8_t*>(tqs) + o);
   }
-  for (size_t o = (size_t)tid * 16; o < out_bytes; o += (size_t)kThreads * 16)
-    *reinterpret_cast<uint4*>(c.out + o) = *reinterpret_cast<const uint4*>(smem + o);
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // nobody leaves while its sums may still be read
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (p.order == kChainLater) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -401,7 +448,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cols_kernel(const __grid_c
     asm volatile("cp.async.commit_group;" ::: "memory");
     asm volatile("cp.async.wait_group 0;" ::: "memory");
   } else {
-    quantize_x_rows(X, M, ly.K, ly.K64, fmt, xm, xsc, xof);
+    quantize_x_rows(X, M, ly.K, 0, ly.K64, fmt, xm, xsc, xof);
   }
   __syncthreads();
 
@@ -411,9 +458,9 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cols_kernel(const __grid_c
     if (a_staged) {
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       __syncthreads();
-      t_partial<MT, 4, true>(a_stage, ly.K, ly.K64, ly.k_pad, kb_lo, kb_hi, M, fmt, xm, xsc, tsub);
+      t_partial<MT, 4, true>(a_stage, ly.K, 0, ly.K64, ly.k_pad, kb_lo, kb_hi, M, fmt, xm, xsc, tsub);
     } else {
-      t_partial<MT, 4, false>(asec, ly.K, ly.K64, ly.k_pad, kb_lo, kb_hi, M, fmt, xm, xsc, tsub);
+      t_partial<MT, 4, false>(asec, ly.K, 0, ly.K64, ly.k_pad, kb_lo, kb_hi, M, fmt, xm, xsc, tsub);
     }
     __syncthreads();
     if (t_local) {                                 // all of T is here: quantise it
@@ -862,7 +909,12 @@ cudaError_t launch_decode_pre(const lqer_call_t* calls, const PackedMeta* metas,
   if (n < 1 || n > kPreMaxCalls) return cudaErrorInvalidValue;
   PreParams p;
   p.order = order;
-  size_t smem = 0;
+  // as many CTAs to a call as fill the SMs about once, each with at least eight slabs
+  int slabs = metas[0].k_slabs;
+  for (int i = 1; i < n; ++i) slabs = std::min(slabs, (int)metas[i].k_slabs);
+  p.share = kPreShare;
+  while (p.share > 1 && (n * p.share > 300 || slabs < 8 * p.share)) p.share >>= 1;
+  size_t xt = 0, sums = 0;
   bool single = true;
   for (int i = 0; i < kPreMaxCalls; ++i) {
     const int g = i < n ? i : 0;
@@ -875,21 +927,24 @@ cudaError_t launch_decode_pre(const lqer_call_t* calls, const PackedMeta* metas,
     c.f = Formats{m.a_bits, m.lr_bits, m.exp_min, m.exp_max, x_type, m.w_bits};
     if (c.M < 1 || c.M > kMaxM) return cudaErrorInvalidValue;
     if (c.M > 1) single = false;
-    const size_t need = pre_x_bytes(c.M, c.K64) + pre_t_bytes(c.k_pad) + 16 +
-                        (size_t)t_subsets(c.k_pad) * kMaxM * c.k_pad * 8 + 128;
-    if (need > smem) smem = need;
+    xt = std::max(xt, pre_x_bytes(c.M, (m.k_slabs + p.share - 1) / p.share * 64) + pre_t_bytes(c.k_pad));
+    sums = std::max(sums, (size_t)(t_subsets(c.k_pad) + 1) * kMaxM * c.k_pad * 8);
   }
+  p.off_tsub = (int)((xt + 15) & ~(size_t)15);
+  const size_t smem = p.off_tsub + sums + 128;
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n);
+  cfg.gridDim = dim3(n * p.share);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = p.share; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   LaunchScope scope(kFamDecode, s);
   return single ? cudaLaunchKernelEx(&cfg, decode_pre_kernel<1>, p) : cudaLaunchKernelEx(&cfg, decode_pre_kernel<kMaxM>, p);
 }
