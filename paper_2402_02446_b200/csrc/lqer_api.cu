@@ -281,7 +281,10 @@ static lqer_status_t run_linear(const void* X, int M, const void* packed, void* 
   void* xcat = wsb + align_up(persist_bytes(m), 256);
   cudaError_t err;
   if (small) {
-    if (path != 5 && path != 7 && !project_only && decode_cols_fits(m, M)) {
+    if (path == 0 && !project_only && decode_cluster_takes(&m, 1, M, io.y_type)) {
+      const lqer_call_t one = {static_cast<const float*>(X), M, packed, static_cast<float*>(Y)};
+      err = launch_decode_cluster(&one, &m, 1, xcat, reinterpret_cast<int*>(wsb + kStatusBytes), dst, io.x_type, io.y_type, s);
+    } else if (path != 5 && path != 7 && !project_only && decode_cols_fits(m, M)) {
       err = launch_decode_cols(X, io.x_type, M, m, packed, Y, io.y_type, workspace, s);
     } else {
       const lqer_call_t one = {static_cast<const float*>(X), M, packed, static_cast<float*>(Y)};
@@ -809,6 +812,21 @@ lqer_status_t lqer_linear(const float* X, int M, const void* packed, float* Y, v
 
 }  // extern "C"
 
+// The calls from calls[first] on that go out as one launch of the cluster kernel: a run of two to decode_cluster_max_layers()
+// neighbours with one M and one set of formats (a longer run shares the launches of the other kernels), or 0.
+static int cluster_run(const lqer_call_t* calls, int first, int n_calls, size_t workspace_bytes, int y_type, PackedMeta* metas) {
+  const int M = calls[first].M;
+  size_t need = align_up(kPersistMaxBytes, 256);
+  int n = 0;
+  for (; first + n < n_calls && calls[first + n].M == M; ++n) {
+    PackedMeta m;
+    if (lookup(calls[first + n].packed, m) != LQER_OK || (n > 0 && !same_formats(metas[0], m))) break;
+    if (n == decode_cluster_max_layers()) return 0;
+    metas[n] = m;
+    need += decode_cluster_scratch_bytes(m);
+  }
+  return n > 1 && need <= workspace_bytes && decode_cluster_takes(metas, n, M, y_type) ? n : 0;
+}
 // The batched entry points: independent calls share launches where the path is left at 0.
 static lqer_status_t linear_batched(const lqer_call_t* calls, int n_calls, void* workspace, size_t workspace_bytes,
                                     void* stream, IoTypes io) {
@@ -847,8 +865,12 @@ static lqer_status_t linear_batched(const lqer_call_t* calls, int n_calls, void*
     // slice for each.
     int n = 1;
     PackedMeta m0, metas[16];
-    bool decode_group = false, small_group = false;
-    if (may_group && lookup(calls[i].packed, m0) == LQER_OK) {
+    bool decode_group = false, small_group = false, cluster_group = false;
+    const int clustered = may_group && !chain_open ? cluster_run(calls, i, n_calls, workspace_bytes, io.y_type, metas) : 0;
+    if (clustered > 1) {
+      n = clustered;
+      cluster_group = true;
+    } else if (may_group && lookup(calls[i].packed, m0) == LQER_OK) {
       const int many = cols_ok ? many_small_rows(calls, i, n_calls, workspace_bytes, m0, metas, nullptr) : 0;
       if (many > 0) {
         n = many;
@@ -871,7 +893,13 @@ static lqer_status_t linear_batched(const lqer_call_t* calls, int n_calls, void*
       lqer_status_t st = check_arch();
       if (st != LQER_OK) return st;
       if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return LQER_ERR_ALIGN;
-      if (decode_group) {
+      if (cluster_group) {
+        chain_open = false;
+        uint8_t* wsb = static_cast<uint8_t*>(workspace);
+        if (launch_decode_cluster(calls + i, metas, n, wsb + pre_base, reinterpret_cast<int*>(wsb + kStatusBytes), static_cast<DeviceStatus*>(workspace),
+                                  io.x_type, io.y_type, static_cast<cudaStream_t>(stream)) != cudaSuccess)
+          return LQER_ERR_CUDA;
+      } else if (decode_group) {
         cudaStream_t cs = static_cast<cudaStream_t>(stream);
         if (i >= pre_end) {
           std::vector<PackedMeta> pm;

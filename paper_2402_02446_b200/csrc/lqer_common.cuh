@@ -582,6 +582,14 @@ int gemm_small_max_layers();
 // would take the launch.
 cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_type, bool tensor_memory_form, int epoch,
                               DeviceStatus* st, cudaStream_t s);
+// The layer for 3 to 16 rows in one launch (lqer_decode_cluster.cu), up to decode_cluster_max_layers() independent layers with one M
+// and one set of formats.  scratch: decode_cluster_scratch_bytes per layer; counts: two zeroed counters per layer, zero again
+// when the call ends.
+int decode_cluster_max_layers();
+bool decode_cluster_takes(const PackedMeta* metas, int n, int M, int y_type);
+inline size_t decode_cluster_scratch_bytes(const PackedMeta& m) { return (size_t)(m.k_pad + 127) / 128 * 4096; }
+cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* metas, int n, void* scratch, int* counts, DeviceStatus* st,
+                                  int x_type, int y_type, cudaStream_t s);
 cudaError_t launch_decode_cols(const void* X, int x_type, int M, const PackedMeta& m, const void* packed, void* Y, int y_type,
                                void* workspace, cudaStream_t s);
 bool decode_cols_fits(const PackedMeta& m, int M);

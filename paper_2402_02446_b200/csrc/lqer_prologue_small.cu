@@ -14,10 +14,11 @@
 // are exact unless a row's block exponents spread over more than about 30 binades.  The order of the additions is fixed by
 // the ranges, which depend on the shape alone, and by the shares, which depend on all layers of the launch: beyond that
 // spread a T may differ in its 53rd bit between a call alone and in company (and T_q where that bit decides a rounding).
-#include "lqer_common.cuh"
+#include "lqer_mma_frag.cuh"
 
 namespace lqer {
 namespace psm {
+using mf::frag_offset;
 
 constexpr int kRows = 16;                 // rows per CTA = one MMA M tile
 constexpr int kThreads = 256;
@@ -52,12 +53,6 @@ struct Params {
   int epoch;                  // value the flags take in this launch
   int shares;                 // CTAs (a cluster) that share a K range: a power of two up to 8
 };
-
-// Byte offset of (row, column c of slab s) in the fragment order; plane: bytes of one plane.
-__device__ __forceinline__ size_t frag_offset(int row, int slab, int c, size_t plane) {
-  return (size_t)((c & 31) >> 2) * plane + (size_t)slab * 256 + (2 * (row & 7) + (c >> 5)) * 16 + (((c & 3) >> 1) * 2 + (row >> 3)) * 4 +
-         (c & 1) * 2;
-}
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;

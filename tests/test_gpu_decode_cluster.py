@@ -1,0 +1,104 @@
+"""Batches of 3 to 16 rows in one launch: a cluster of CTAs per range of columns, the contraction shared by its CTAs.
+
+Sizes sit at the edges of what the kernel cuts: contractions that give a CTA one slab, half a step or a ragged last block,
+column ranges of less than a warp's octets, of several rounds with a nearly empty last one (owners to whom nothing comes), ranks
+of no, one, several and sixteen blocks, and both sides of the eight-token tile.
+"""
+import numpy as np
+import pytest
+import torch
+
+import lqer_inputs as gen
+import paper_2402_02446_b200 as L
+from oracle import lqer as olqer
+from helpers import worst_ratio
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _t(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+
+
+def _layer(K, N, k, seed, w_bits=4):
+    spec = gen.LayerSpec("cluster", M=16, K=K, N=N, k=k, calib_rows=32, outlier_frac=0.01, outlier_scale=20.0, seed=seed)
+    W = gen.make_weight(spec)
+    A, B = gen.make_random_factors(spec) if k else (None, None)
+    cfg = L.default_config()
+    cfg.w_bits = w_bits
+    return spec, olqer.prepare_weights(W, A, B, w_bits=w_bits), L.prepare_weights(_t(W), *((_t(A), _t(B)) if k else (None, None)), cfg)
+
+
+SHAPES = [
+    # K, N, k, w_bits
+    (16, 8, 0, 4), (64, 24, 5, 4), (208, 264, 16, 4), (1024, 8704, 16, 4), (1040, 20008, 24, 4), (2112, 264, 72, 4),
+    (1152, 1032, 256, 4), (4112, 520, 40, 4), (1040, 648, 136, 2), (304, 4104, 20, 2),
+]
+
+
+@pytest.mark.parametrize("K,N,k,w_bits", SHAPES, ids=["x".join(map(str, s)) for s in SHAPES])
+def test_rows_3_to_16_against_the_oracle(K, N, k, w_bits):
+    spec, P, Pg = _layer(K, N, k, 901, w_bits)
+    X = gen.make_activations(spec, M=16)
+    for M in (3, 8, 9, 16):
+        ref = olqer.forward(X[:M], P, w_bits=w_bits)
+        Xg, ws = _t(X[:M]), L.new_workspace(M, Pg)
+        before = L.launch_count()
+        Y = L.linear(Xg, Pg, ws)
+        assert L.launch_count() - before == 1
+        again = L.linear(Xg, Pg, ws)                       # the counters are zero again
+        assert L.poll_status(ws) == 0
+        assert torch.equal(Y, again)
+        assert worst_ratio(Y.cpu().numpy(), ref) <= 1.0, M
+    Pg.release()
+
+
+@pytest.mark.parametrize("M", [3, 16])
+def test_types_at_the_boundary(M):
+    # bf16 X is the fp32 value it denotes; MXINT8 in and out agree with quantising outside
+    spec, P, Pg = _layer(1040, 1040, 40, 902)
+    X = _t(gen.make_activations(spec, M=M))
+    ws = L.new_workspace(M, Pg)
+    Xb = X.bfloat16()
+    y = L.linear_ex(Xb.float(), Pg, ws)
+    assert torch.equal(L.linear_ex(Xb, Pg, ws), y)
+    assert torch.equal(L.linear_ex(Xb, Pg, ws, out_dtype=torch.bfloat16), y.bfloat16())
+    cfg = L.default_config()
+    mx = L.to_mxint8(*L.quantize_activations(X, cfg))
+    y = L.linear(X, Pg, ws)
+    assert torch.equal(L.linear_ex(mx, Pg, ws, M=M), y)
+    got = L.linear_ex(mx, Pg, ws, out_dtype=L.MXINT8, M=M)
+    assert torch.equal(got, L.to_mxint8(*L.quantize_activations(y, cfg)))
+    assert L.poll_status(ws) == 0
+    Pg.release()
+
+
+@pytest.mark.parametrize("M", [4, 12])
+def test_groups_share_one_launch(M):
+    # two to four neighbours, of one shape and of several; also as replays of a captured graph on new activations
+    shapes = [(1040, 520, 40), (512, 1032, 0), (2112, 264, 72), (1040, 648, 256)]
+    layers = [_layer(*s, 903 + i) for i, s in enumerate(shapes)]
+    for pick in ((0, 0), (0, 3, 0), (0, 1, 2, 3)):
+        Xs = [_t(gen.make_activations(layers[j][0], M=M)) + 0.125 * i for i, j in enumerate(pick)]
+        Ys = [torch.full((M, layers[j][0].N), float("nan"), device=DEV) for j in pick]
+        calls = L.make_calls([(x, layers[j][2], y) for x, j, y in zip(Xs, pick, Ys)])
+        ws = torch.zeros(L.batched_workspace_bytes(calls), dtype=torch.uint8, device=DEV)
+        before = L.launch_count()
+        L.linear_batched(calls, ws)
+        assert L.launch_count() - before == 1
+        stream = torch.cuda.Stream()
+        stream.wait_stream(torch.cuda.current_stream())
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            L.linear_batched(calls, ws, stream=torch.cuda.current_stream())
+        for rep in range(3):
+            for x in Xs:
+                x.mul_(-1.5)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert L.poll_status(ws) == 0
+            for x, j, y in zip(Xs, pick, Ys):
+                assert worst_ratio(y.cpu().numpy(), olqer.forward(x.cpu().numpy(), layers[j][1])) <= 1.0, (pick, rep)
+    for l in layers:
+        l[2].release()
