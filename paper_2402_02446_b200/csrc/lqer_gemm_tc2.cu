@@ -1,18 +1,22 @@
 // CTA-pair form of the main GEMM (paper Section 3.1 / 3.2: Y = [X_q | T_q] . [W_q ; B_q]).
 //
-// Two CTAs on neighbouring SMs (a cluster of 2) share one 256 x 256 output tile.  CTA r holds
+// Two CTAs on neighbouring SMs (a cluster of 2) share one output tile of 256 rows and 2 H columns (H = 128; 96 or 64 where
+// that fills the last round of tiles better, see half_columns).  CTA r holds
 // token rows [128 r, 128 r + 128) of the tile (its own A operand and its own accumulator
-// lanes) and output columns [128 r, 128 r + 128) of the weight tile (its half of the B
+// lanes) and output columns [H r, H r + H) of the weight tile (its half of the B
 // operand).  Each CTA therefore fetches and converts only HALF of the 4-bit weights per
 // tensor-core stage, and reads half of B from its shared memory; tcgen05.mma.cta_group::2,
 // issued by CTA 0 alone, combines the halves.  Roles per CTA:
-//   warp 0      TMA producer (own activation tile + own packed weight half)
+//   warp 0      TMA producer (own activation tile)
 //   warp 1      tensor memory allocation; in CTA 0 also the MMA issuer
 //   warps 2-5   epilogue (tcgen05.ld of the finished accumulator, fp32 stores to Y)
 //   warps 6-29  converters in six groups; a group converts every sixth stage (one weight
 //               column = 64 weights per thread), so that its fixed per-stage latencies
-//               (barrier wait, shared-memory round trip, proxy fence) overlap the other groups
-// One ring of six stages; a stage holds the activation tile, the packed weight tile and the
+//               (barrier wait, shared-memory round trip, proxy fence) overlap the other groups.
+//               A thread's packed weights come straight from global memory into registers, a pass over the ring
+//               ahead.  (As bulk copies into the stage, which the converters then read, they held the ring back: 2048 rows
+//               of a 4096 / 11008 layer 698 us against 657, 4096 rows of 5120 x 13824 at rank 256 546 against 492.)
+// One ring of six stages; a stage holds the activation tile and the
 // converted weight tile, so each role waits on one barrier and signals one per stage:
 //   loaded[s]   (per CTA)  TMA bytes have landed          -> converters
 //   ready[s]    (in CTA 0) both CTAs' converters are done -> MMA issuer; implies both
@@ -33,14 +37,13 @@ namespace tc2 {
 using namespace tc;
 
 constexpr int BM = 128;                    // token rows per CTA (256 per pair)
-constexpr int BN = 256;                    // output columns per pair tile
-constexpr int BNH = 128;                   // columns converted by one CTA
+constexpr int BN = 256;                    // output columns per pair tile, at most: a launch takes 2 Params::half of them
+constexpr int BNH = 128;                   // columns converted by one CTA, at most
 constexpr int BK = 64;
 constexpr int STAGES = 6;
 constexpr int A_TILE_BYTES = BM * BK * 2;                     // 16384: activations (TMA, swizzled)
 constexpr int B_TILE_BYTES = BNH * BK * 2;                    // 16384: converted weights (swizzled)
-constexpr int PK_OFFSET = A_TILE_BYTES + B_TILE_BYTES;        // packed weight tile (4608) behind them
-constexpr int STAGE_BYTES = 37 * 1024;
+constexpr int STAGE_BYTES = A_TILE_BYTES + B_TILE_BYTES;
 constexpr int RANK_PER_STAGE = 32;
 constexpr int NUM_BARRIERS = 3 * STAGES + 4;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 256 + 1024;
@@ -50,7 +53,7 @@ constexpr int CONVERTER_GROUPS = 6;          // group g converts the stages with
                                              // the parity of its wait can never alias an older pass
 constexpr int WARPS_PER_GROUP = CONVERTER_WARPS / CONVERTER_GROUPS;
 constexpr int NUM_THREADS = (6 + CONVERTER_WARPS) * 32;
-static_assert(PK_OFFSET + kWTileBytes <= STAGE_BYTES && STAGE_BYTES % 1024 == 0, "stage layout");
+static_assert(STAGE_BYTES % 1024 == 0, "stage layout");
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
 static_assert(STAGES % CONVERTER_GROUPS == 0, "a converter group must revisit a ring slot exactly one pass later");
 
@@ -71,13 +74,14 @@ struct Layer {
   int slab0, slab_stride;      // a layer may be a K range of a real layer (split K): its first weight slab, and the
                                // real layer's slab count (the stride between column tiles of the packed weights)
   int spt;                     // K stages per tile: k_slabs + rank stages
-  int tile_begin;              // first tile of this layer in the launch's list (256 x 256 tiles, row tile fastest)
+  int tile_begin;              // first tile of this layer in the launch's list (256 rows x 2 half columns, row tile fastest)
 };
 
 struct Params {
   Layer L[MAX_GROUP];          // ordered by falling spt: the long tiles run first, the short ones fill the end
   int group;                   // layers in this launch
   int num_tiles;               // tiles of all layers
+  int half;                    // output columns of a tile per CTA: a multiple of 16 up to 128
   DeviceStatus* status;
   int M, m_tiles;              // row tiles of 256 (the same M for every layer)
   int lr_shift;
@@ -93,6 +97,17 @@ __device__ __forceinline__ uint32_t bf16x2_rn(uint32_t lo, uint32_t hi) {
   uint32_t d;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(__uint_as_float(hi)), "f"(__uint_as_float(lo)));
   return d;
+}
+
+__device__ __forceinline__ uint4 ld_weights16(const uint8_t* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_weights4(const uint8_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
 }
 
 __device__ __forceinline__ int layer_of(const Params& p, int t) {
@@ -149,49 +164,24 @@ gemm_tc2_kernel(const __grid_constant__ TensorMaps tmaps, const Params p) {
   const int num_tiles = p.num_tiles;
 
   if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer (own halves)
+    // ------------------------------------------------------------------ TMA producer (own rows)
     if (lane == 0) {
       int st = 0;
       uint32_t ph = 0;
       bool ok = true;
-      const uint32_t w_tile = (uint32_t)w_tile_bytes(p.w_bits);
       for (int t = pair; t < num_tiles && ok; t += num_pairs) {
         const int layer = layer_of(p, t), tl = t - p.L[layer].tile_begin;
-        const int mt = tl % p.m_tiles, nt = tl / p.m_tiles;
+        const int mt = tl % p.m_tiles;
         const CUtensorMap* tmap_x = &tmaps.m[layer];
-        const uint8_t* wsec = p.L[layer].wsec;
-        const uint8_t* bsec = p.L[layer].bsec;
-        const int k_slabs = p.L[layer].k_slabs, r_blocks = p.L[layer].r_blocks, t_col = p.L[layer].t_col;
-        const int stages_per_tile = p.L[layer].spt, n_tiles = p.L[layer].n_tiles;
-        const int slab0 = p.L[layer].slab0, slab_stride = p.L[layer].slab_stride;
-        const int b_tile_stride = r_blocks * kTileN * 17;
-        const int my_ntile = 2 * nt + (int)rank;
-        const bool has_w = my_ntile < n_tiles;
+        const int k_slabs = p.L[layer].k_slabs, t_col = p.L[layer].t_col, slab0 = p.L[layer].slab0;
+        const int stages_per_tile = p.L[layer].spt;
         const int row0 = mt * 2 * BM + (int)rank * BM;
         for (int s = 0; s < stages_per_tile; ++s) {
           if (p.stall != 0 && s == stages_per_tile - 1 && t + num_pairs >= num_tiles) { ok = false; break; }
           if (!mbar_wait<true>(freed(st), ph ^ 1, abort_flag)) { ok = false; break; }
-          const uint32_t a_dst = smem_u32(stage_base + st * STAGE_BYTES);
-          if (s < k_slabs) {
-            const size_t w_off = ((size_t)my_ntile * slab_stride + slab0 + s) * w_tile;
-            if (has_w && !LQER_IN_BOUNDS(p.status, w_off, w_tile, p.L[layer].w_extent, 605)) { ok = false; break; }
-            mbar_expect_tx(loaded(st), A_TILE_BYTES + (has_w ? w_tile : 0));
-            tma_load_2d(a_dst, tmap_x, (slab0 + s) * BK, row0, loaded(st));
-            if (has_w) bulk_load(a_dst + PK_OFFSET, wsec + w_off, w_tile, loaded(st));
-          } else {
-            const int rs = s - k_slabs;
-            const int rb0 = rs * 2, nb = min(2, r_blocks - rb0);
-            if (has_w && !LQER_IN_BOUNDS(p.status, (size_t)my_ntile * b_tile_stride + (size_t)r_blocks * kTileN * 16 + rb0 * kTileN,
-                                         nb * kTileN, p.L[layer].b_extent, 606)) { ok = false; break; }
-            mbar_expect_tx(loaded(st), A_TILE_BYTES + (has_w ? nb * (kTileN * 17) : 0));
-            tma_load_2d(a_dst, tmap_x, t_col + rs * RANK_PER_STAGE, row0, loaded(st));
-            if (has_w) {
-              const uint8_t* tile = bsec + (size_t)my_ntile * b_tile_stride;
-              bulk_load(a_dst + PK_OFFSET, tile + (size_t)rb0 * kTileN * 16, nb * kTileN * 16, loaded(st));
-              bulk_load(a_dst + PK_OFFSET + 4096, tile + (size_t)r_blocks * kTileN * 16 + rb0 * kTileN,
-                        nb * kTileN, loaded(st));
-            }
-          }
+          mbar_expect_tx(loaded(st), A_TILE_BYTES);
+          tma_load_2d(smem_u32(stage_base + st * STAGE_BYTES), tmap_x, s < k_slabs ? (slab0 + s) * BK : t_col + (s - k_slabs) * RANK_PER_STAGE,
+                      row0, loaded(st));
           if (++st == STAGES) { st = 0; ph ^= 1; }
         }
       }
@@ -204,7 +194,7 @@ gemm_tc2_kernel(const __grid_constant__ TensorMaps tmaps, const Params p) {
     if (rank == 0) {
       int st = 0;
       uint32_t ph = 0, tile_it = 0;
-      const uint32_t idesc = make_idesc(2 * BM, BN);
+      const uint32_t idesc = make_idesc(2 * BM, 2 * p.half);
       const uint64_t a_desc0 = make_desc(smem_u32(stage_base));
       const uint64_t b_desc0 = make_desc(smem_u32(stage_base + A_TILE_BYTES));
       bool ok = true;
@@ -244,7 +234,7 @@ gemm_tc2_kernel(const __grid_constant__ TensorMaps tmaps, const Params p) {
     }
   } else if (warp < 6) {
     // ------------------------------------------------------------------ epilogue (own 128 rows)
-    const int q = warp & 3;
+    const int q = warp & 3, width = 2 * p.half;
     uint32_t tile_it = 0;
     bool ok = true;
     for (int t = pair; t < num_tiles && ok; t += num_pairs, ++tile_it) {
@@ -255,16 +245,15 @@ gemm_tc2_kernel(const __grid_constant__ TensorMaps tmaps, const Params p) {
       if (!mbar_wait<true>(acc_full(acc), (tile_it >> 1) & 1, abort_flag)) { ok = false; break; }
       tc_fence_after();
       const int row = mt * 2 * BM + (int)rank * BM + q * 32 + lane;
-      const int ncols = min(BN, Nl - nt * BN);
-      const size_t yoff = (size_t)row * Nl + (size_t)nt * BN;
+      const int ncols = min(width, Nl - nt * width);
+      const size_t yoff = (size_t)row * Nl + (size_t)nt * width;
       float* yrow = static_cast<float*>(p.L[layer].Y) + yoff;
       uint16_t* yrow16 = static_cast<uint16_t*>(p.L[layer].Y) + yoff;
       // MXINT8 Y: mantissas [M, N], then exponent bytes [M, N / 16]; a thread holds whole 16-blocks of its row
       uint8_t* yq = static_cast<uint8_t*>(p.L[layer].Y) + yoff;
-      uint8_t* yqe = static_cast<uint8_t*>(p.L[layer].Y) + (size_t)p.M * Nl + ((size_t)row * Nl + (size_t)nt * BN) / 16;
+      uint8_t* yqe = static_cast<uint8_t*>(p.L[layer].Y) + (size_t)p.M * Nl + yoff / 16;
       const QuantConsts qc = quant_consts(p.a_bits, p.exp_min, p.exp_max);
-      for (int c = 0; c < BN; c += 32) {
-        if (c >= ncols) break;
+      for (int c = 0; c < ncols; c += 32) {
         uint32_t r[32];
         tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + acc * BN + c, r);
         tmem_ld_wait();
@@ -306,53 +295,85 @@ gemm_tc2_kernel(const __grid_constant__ TensorMaps tmaps, const Params p) {
     }
   } else {
     // ------------------------------------------------------------------ converters (own weight half)
+    // A thread takes its column's packed weights straight from global memory, for the group's next stage as soon as it has
+    // converted this one (six stages ahead: some 2000 cycles), so a tile may begin at any multiple of 16 columns.
     const int c = threadIdx.x - 6 * 32;          // 0..767
     const int group = c >> 7, nl = c & 127;      // stage group; weight column of the half tile
-    const int sw = nl & 7;
-    uint32_t chunk[8];                           // the row's eight 16-byte chunks after the 128-byte swizzle
-#pragma unroll
-    for (int i = 0; i < 8; ++i) chunk[i] = (uint32_t)(nl * 128 + ((i ^ sw) << 4));
+    const int half = p.half;
+    const bool mine = nl < half;
+    const uint32_t at = (uint32_t)(nl * 128 + ((nl & 7) << 4));   // the row's first 16-byte chunk after the 128-byte swizzle
     // the pair's tiles one after the other; their K stages form one sequence of which this group takes every sixth
-    int tile = pair, s = group;                  // s may run past the tile; normalised below
-    int stages_per_tile = 0, k_slabs = 0, r_blocks = 0;
+    int tile = pair, s = group;                  // s may run past the tile; normalised in next_stage
+    int stages_per_tile = 0, k_slabs = 0, r_blocks = 0, cl = 0;
     bool has_w = false;
+    const uint8_t* wcol = nullptr;               // this column's mantissas in the layer's first slab
+    const uint8_t* bcol = nullptr;               // this column's first rank block
+    const uint32_t w_tile = (uint32_t)w_tile_bytes(p.w_bits), mant = w_tile - kTileN * 4;
     auto enter_tile = [&]() {
       if (tile < num_tiles) {
-        const int layer = layer_of(p, tile);
-        stages_per_tile = p.L[layer].spt; k_slabs = p.L[layer].k_slabs; r_blocks = p.L[layer].r_blocks;
-        const int nt = (tile - p.L[layer].tile_begin) / p.m_tiles;
-        has_w = 2 * nt + (int)rank < p.L[layer].n_tiles;
+        const Layer& ly = p.L[layer_of(p, tile)];
+        stages_per_tile = ly.spt; k_slabs = ly.k_slabs; r_blocks = ly.r_blocks;
+        const int nt = (tile - ly.tile_begin) / p.m_tiles, col = (2 * nt + (int)rank) * half + nl;
+        has_w = mine && col < ly.n_tiles * kTileN;
+        cl = col & (kTileN - 1);
+        wcol = ly.wsec + ((size_t)(col >> 7) * ly.slab_stride + ly.slab0) * w_tile + cl * 16;
+        bcol = ly.bsec + (size_t)(col >> 7) * ((size_t)r_blocks * kTileN * 17) + cl * 16;
+        if (has_w && !LQER_IN_BOUNDS(p.status, (size_t)(wcol - ly.wsec) + (size_t)(k_slabs - 1) * w_tile + mant - cl * 12, 4, ly.w_extent, 605)) has_w = false;
+        if (has_w && r_blocks > 0 && !LQER_IN_BOUNDS(p.status, (size_t)(bcol - ly.bsec) - cl * 15 + (size_t)r_blocks * kTileN * 17 - kTileN, 1, ly.b_extent, 606))
+          has_w = false;
+      }
+    };
+    uint4 wa = make_uint4(0u, 0u, 0u, 0u), wb = wa;
+    uint32_t eb = 0;
+    auto next_stage = [&]() {                    // moves on to the group's next stage and requests its weights
+      while (tile < num_tiles && s >= stages_per_tile) { s -= stages_per_tile; tile += num_pairs; enter_tile(); }
+      if (tile >= num_tiles || !has_w) return;
+      if (s < k_slabs) {
+        const uint8_t* w = wcol + (size_t)s * w_tile;
+        wa = ld_weights16(w);
+        if (p.w_bits == 4) wb = ld_weights16(w + kTileN * 16);
+        eb = ld_weights4(w + mant - cl * 12);
+      } else {
+        const int rb = (s - k_slabs) * 2;
+        const uint8_t* e = bcol + (size_t)r_blocks * kTileN * 16 - cl * 15;
+        wa = ld_weights16(bcol + (size_t)rb * kTileN * 16);
+        eb = __ldg(e + rb * kTileN);
+        if (rb + 1 < r_blocks) {
+          wb = ld_weights16(bcol + (size_t)(rb + 1) * kTileN * 16);
+          eb |= (uint32_t)__ldg(e + (rb + 1) * kTileN) << 8;
+        }
       }
     };
     enter_tile();
+    next_stage();
     bool ok = true;
-    for (int it = group; tile < num_tiles && ok; it += CONVERTER_GROUPS, s += CONVERTER_GROUPS) {
-      while (tile < num_tiles && s >= stages_per_tile) { s -= stages_per_tile; tile += num_pairs; enter_tile(); }
-      if (tile >= num_tiles) break;
+    for (int it = group; tile < num_tiles && ok; it += CONVERTER_GROUPS) {
       const int st = it % STAGES;
       const uint32_t ph = (uint32_t)((it / STAGES) & 1);
       if (!mbar_wait(loaded(st), ph, abort_flag)) { ok = false; break; }
-      const uint8_t* pk = stage_base + st * STAGE_BYTES + PK_OFFSET;
       uint8_t* bt = stage_base + st * STAGE_BYTES + A_TILE_BYTES;
       if (s < k_slabs) {
         if (has_w) {
-          convert_column(pk, nl, p.w_bits, bt, chunk);
-        } else {                                 // columns beyond N: a zero operand half
+          convert_column(wa, wb, eb, p.w_bits, bt, at);
+        } else if (mine) {                       // columns beyond N: a zero operand
 #pragma unroll
-          for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4*>(bt + chunk[i]) = make_uint4(0u, 0u, 0u, 0u);
+          for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4*>(bt + (at ^ (uint32_t)(i << 4))) = make_uint4(0u, 0u, 0u, 0u);
         }
-      } else {
+      } else if (mine) {
         const int nb = min(2, r_blocks - (s - k_slabs) * 2);
-        for (int rb = 0; rb < nb; ++rb) {
-          uint4 o0 = make_uint4(0u, 0u, 0u, 0u), o1 = o0;
-          if (has_w) {
-            const uint4 w = *reinterpret_cast<const uint4*>(pk + (rb * kTileN + nl) * 16);
-            const float scale = pow2f((int)pk[4096 + rb * kTileN + nl] - 127 - p.lr_shift);
-            o0 = convert_i8x8(w.x, w.y, scale);
-            o1 = convert_i8x8(w.z, w.w, scale);
+#pragma unroll
+        for (int rb = 0; rb < 2; ++rb) {
+          if (rb < nb) {
+            uint4 o0 = make_uint4(0u, 0u, 0u, 0u), o1 = o0;
+            if (has_w) {
+              const uint4& w = rb == 0 ? wa : wb;
+              const float scale = pow2f((int)((eb >> (8 * rb)) & 0xFFu) - 127 - p.lr_shift);
+              o0 = convert_i8x8(w.x, w.y, scale);
+              o1 = convert_i8x8(w.z, w.w, scale);
+            }
+            *reinterpret_cast<uint4*>(bt + (at ^ (uint32_t)(rb << 5))) = o0;
+            *reinterpret_cast<uint4*>(bt + (at ^ (uint32_t)(rb << 5 | 16))) = o1;
           }
-          *reinterpret_cast<uint4*>(bt + chunk[rb * 2]) = o0;
-          *reinterpret_cast<uint4*>(bt + chunk[rb * 2 + 1]) = o1;
         }
       }
       fence_proxy_async_smem();        // generic-proxy writes -> visible to the MMA's async proxy
@@ -360,6 +381,8 @@ gemm_tc2_kernel(const __grid_constant__ TensorMaps tmaps, const Params p) {
       if (lane == 0) {
         if (rank == 0) mbar_arrive(ready(st)); else mbar_arrive_remote(ready(st), 0);
       }
+      s += CONVERTER_GROUPS;
+      next_stage();
     }
   }
 
@@ -398,6 +421,32 @@ static EncodeTiledFn encode_fn() {
 }  // namespace tc2
 
 namespace tc2 {
+
+// Columns per CTA of a tile.  A K stage of a tile takes 294 ns at 128, 260 at 96 and 214 at 64 (measured; 112 and 80 take what 128 and
+// 96 take), so 128 is the cheapest per column, but a launch takes as many rounds of tiles over the pairs as it takes: one whose
+// tiles do not fill the pairs, or whose last round is nearly empty, is better off with narrower ones.  us a call, 128 / 96 / 64:
+// 512 rows of 4096 x 4096 41.5 / 39.3 / 36.3, 201 rows of 4112 x 10992 45.3 / 41.5 / 54.6, 512 rows of three 4096 x 4096 in two rounds
+// instead of two longer ones.  The sums of an element run over K in one order whatever the width.
+static int half_columns(const PackedMeta* metas, const int* order, int n, int m_tiles) {
+  const int pairs = std::max(sm_count() / 2, 1);
+  static const int halves[3] = {128, 96, 64}, ns[3] = {294, 260, 214};
+  int best = 0;
+  long long least = -1;
+  for (int h = 0; h < 3; ++h) {
+    // a round is as long as its first tile: the tiles come by falling K
+    long long time = 0, tile = 0, next = 0;
+    for (int i = 0; i < n; ++i) {
+      const PackedMeta& m = metas[order[i]];
+      const long long end = tile + (long long)m_tiles * ((m.N + 2 * halves[h] - 1) / (2 * halves[h]));
+      const long long rounds = next < end ? (end - next + pairs - 1) / pairs : 0;
+      time += rounds * (m.k_slabs + (m.r_blocks + 1) / 2) * ns[h];
+      next += rounds * pairs;
+      tile = end;
+    }
+    if (least < 0 || time < least) { least = time; best = h; }
+  }
+  return halves[best];
+}
 
 static cudaError_t launch_params(const TensorMaps& tmaps, Params& p, cudaStream_t s) {
   static OncePerDevice once;
@@ -466,6 +515,7 @@ cudaError_t launch_gemm_tc2_splitk(const GemmActs& acts, int M, const PackedMeta
   Params p;
   p.m_tiles = (M + 2 * BM - 1) / (2 * BM);
   const uint8_t* base = static_cast<const uint8_t*>(packed);
+  p.half = BNH;
   const int per_layer = p.m_tiles * ((m.n_tiles + 1) / 2);
   // the last range (it carries the rank stages and is the longest) first
   for (int slot = 0; slot < MAX_GROUP; ++slot) {
@@ -528,6 +578,7 @@ cudaError_t launch_gemm_tc2_group(const GemmActs* acts, const void* const* packe
   TensorMaps tmaps;
   Params p;
   p.m_tiles = (M + 2 * BM - 1) / (2 * BM);
+  p.half = half_columns(metas, order, n, p.m_tiles);
   int tile_begin = 0;
   for (int slot = 0; slot < MAX_GROUP; ++slot) {
     const int g = order[slot < n ? slot : 0];
@@ -554,7 +605,7 @@ cudaError_t launch_gemm_tc2_group(const GemmActs* acts, const void* const* packe
     ly.slab0 = 0; ly.slab_stride = m.k_slabs;
     ly.spt = m.k_slabs + (m.r_blocks + 1) / 2;
     ly.tile_begin = tile_begin;
-    if (slot < n) tile_begin += p.m_tiles * ((m.n_tiles + 1) / 2);
+    if (slot < n) tile_begin += p.m_tiles * ((m.N + 2 * p.half - 1) / (2 * p.half));
   }
   p.group = n;
   p.num_tiles = tile_begin;

@@ -161,46 +161,29 @@ __device__ __forceinline__ void w_scales2(uint32_t eb, uint32_t& s2, uint32_t& c
   s2 = s | (s << 16);
   c2 = c | (c << 16);
 }
-// One weight column of a 64-K stage from its packed form (pk: the column's mantissas at mant_off + nl * 16 resp.
-// the two block pairs of the 4-bit layout, exponents at exp_off + nl * 4) into its eight swizzled 16-byte chunks.
-__device__ __forceinline__ void convert_column(const uint8_t* pk, int nl, int w_bits, uint8_t* bt, const uint32_t (&chunk)[8]) {
+// One weight column of a 64-K stage, in registers (wa, wb: the two block pairs of the 4-bit layout, or wa alone the 2-bit one; eb:
+// the four exponent bytes), into its eight swizzled 16-byte chunks: chunk i of the column lies at `at` with i in bits 4 to 6 (xor).
+__device__ __forceinline__ void convert_column(const uint4& wa, const uint4& wb, uint32_t eb, int w_bits, uint8_t* bt, uint32_t at) {
   uint32_t s2, c2;
+  auto put = [&](int i, const uint4& v) { *reinterpret_cast<uint4*>(bt + (at ^ (uint32_t)(i << 4))) = v; };
   if (w_bits == 2) {
-    const uint4 wv = *reinterpret_cast<const uint4*>(pk + nl * 16);
-    const uint32_t eb = *reinterpret_cast<const uint32_t*>(pk + 2048 + nl * 4);
-    uint4 lo, hi;
-    w_scales2(eb & 0xFFu, s2, c2);
-    convert_word2(wv.x, s2, c2, lo, hi);
-    *reinterpret_cast<uint4*>(bt + chunk[0]) = lo;
-    *reinterpret_cast<uint4*>(bt + chunk[1]) = hi;
-    w_scales2((eb >> 8) & 0xFFu, s2, c2);
-    convert_word2(wv.y, s2, c2, lo, hi);
-    *reinterpret_cast<uint4*>(bt + chunk[2]) = lo;
-    *reinterpret_cast<uint4*>(bt + chunk[3]) = hi;
-    w_scales2((eb >> 16) & 0xFFu, s2, c2);
-    convert_word2(wv.z, s2, c2, lo, hi);
-    *reinterpret_cast<uint4*>(bt + chunk[4]) = lo;
-    *reinterpret_cast<uint4*>(bt + chunk[5]) = hi;
-    w_scales2(eb >> 24, s2, c2);
-    convert_word2(wv.w, s2, c2, lo, hi);
-    *reinterpret_cast<uint4*>(bt + chunk[6]) = lo;
-    *reinterpret_cast<uint4*>(bt + chunk[7]) = hi;
+    const uint32_t w[4] = {wa.x, wa.y, wa.z, wa.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint4 lo, hi;
+      w_scales2((eb >> (8 * q)) & 0xFFu, s2, c2);
+      convert_word2(w[q], s2, c2, lo, hi);
+      put(2 * q, lo);
+      put(2 * q + 1, hi);
+    }
   } else {
-    const uint4 wa = *reinterpret_cast<const uint4*>(pk + nl * 16);
-    const uint4 wb = *reinterpret_cast<const uint4*>(pk + (kTileN + nl) * 16);
-    const uint32_t eb = *reinterpret_cast<const uint32_t*>(pk + kWTileNibbleBytes + nl * 4);
-    w_scales(eb & 0xFFu, s2, c2);
-    *reinterpret_cast<uint4*>(bt + chunk[0]) = convert_word(wa.x, s2, c2);
-    *reinterpret_cast<uint4*>(bt + chunk[1]) = convert_word(wa.y, s2, c2);
-    w_scales((eb >> 8) & 0xFFu, s2, c2);
-    *reinterpret_cast<uint4*>(bt + chunk[2]) = convert_word(wa.z, s2, c2);
-    *reinterpret_cast<uint4*>(bt + chunk[3]) = convert_word(wa.w, s2, c2);
-    w_scales((eb >> 16) & 0xFFu, s2, c2);
-    *reinterpret_cast<uint4*>(bt + chunk[4]) = convert_word(wb.x, s2, c2);
-    *reinterpret_cast<uint4*>(bt + chunk[5]) = convert_word(wb.y, s2, c2);
-    w_scales(eb >> 24, s2, c2);
-    *reinterpret_cast<uint4*>(bt + chunk[6]) = convert_word(wb.z, s2, c2);
-    *reinterpret_cast<uint4*>(bt + chunk[7]) = convert_word(wb.w, s2, c2);
+    const uint32_t w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      w_scales((eb >> (8 * q)) & 0xFFu, s2, c2);
+      put(2 * q, convert_word(w[2 * q], s2, c2));
+      put(2 * q + 1, convert_word(w[2 * q + 1], s2, c2));
+    }
   }
 }
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
