@@ -909,11 +909,13 @@ cudaError_t launch_decode_pre(const lqer_call_t* calls, const PackedMeta* metas,
   if (n < 1 || n > kPreMaxCalls) return cudaErrorInvalidValue;
   PreParams p;
   p.order = order;
-  // as many CTAs to a call as fill the SMs about once, each with at least eight slabs
+  // As many CTAs to a call as fill the SMs about once (two to an SM), each with at least two slabs.  Stacks of 2 to 6 decoder layers
+  // at 1 or 2 rows, us a pass, one CTA with all of A_q / at least eight slabs / two: hidden 2768 80.7 / 71.8 / 70.0, hidden 2672
+  // 96.7 / 88.6 / 85.1, hidden 5088 401 / 367 / 367, hidden 1216 35.5 / 37.2 / 32.7.
   int slabs = metas[0].k_slabs;
   for (int i = 1; i < n; ++i) slabs = std::min(slabs, (int)metas[i].k_slabs);
   p.share = kPreShare;
-  while (p.share > 1 && (n * p.share > 300 || slabs < 8 * p.share)) p.share >>= 1;
+  while (p.share > 1 && (n * p.share > 300 || slabs < 2 * p.share)) p.share >>= 1;
   size_t xt = 0, sums = 0;
   bool single = true;
   for (int i = 0; i < kPreMaxCalls; ++i) {
