@@ -750,16 +750,22 @@ static Plan plan(const PackedMeta* metas, int n, int M) {
 //   six of 4096 x 4096           4 rows 34.5 / 37.1    8 rows 35.2 / 37.8    16 rows 35.8 / 46.5
 // Up to eight rows one MMA multiplies sixteen weight columns with all tokens; from nine on it takes two, and the tensor pipe is
 // as busy as the conversion, so larger launches keep the kernels that share a prologue (11008 x 4096 alone, 16 rows: 29.9 / 32.4).
+// Three rows with ranks above 128 are level or worse in large launches (a 4064 / 10192 layer at rank 256 122.8 / 134.9, 4096 / 11008 126.6 /
+// 129.5; 2048 / 5632 87.3 / 62.3): the same line.
 // One and two rows keep the column-owner kernel (2 rows: 4096 x 4096 16.4 / 15.6, two of 4096 x 11008 26.0 / 30.3).
 constexpr int kClusterMaxLayers = 4;
-constexpr long long kClusterMaxWeights16 = 30000000;      // K N over the layers, from nine rows on
+constexpr long long kClusterMaxWeights = 30000000;        // K N over the layers, from nine rows on
 int decode_cluster_max_layers() { return kClusterMaxLayers; }
 bool decode_cluster_takes(const PackedMeta* metas, int n, int M, int y_type) {
   using namespace dcl;
   if (n < 1 || n > kClusterMaxLayers || M < 3 || M > kRows) return false;
   long long weights = 0;
-  for (int i = 0; i < n; ++i) weights += (long long)metas[i].K64 * metas[i].N;
-  if (M > 8 && weights > kClusterMaxWeights16) return false;
+  int k_pad = 0;
+  for (int i = 0; i < n; ++i) {
+    weights += (long long)metas[i].K64 * metas[i].N;
+    k_pad = std::max(k_pad, (int)metas[i].k_pad);
+  }
+  if ((M > 8 || (M == 3 && k_pad > 128)) && weights > kClusterMaxWeights) return false;
   const Plan q = plan(metas, n, M);
   if (q.smem > (size_t)kSmemOne) return false;
   return entry_of(metas[0].w_bits, M > 8 ? 2 : 1, y_type == kYMXINT8).resident(q.CS, q.two) >= n;
