@@ -42,8 +42,8 @@ M_DECODE, M_PREFILL = 1, 2048
 
 # DRAM traffic of one launch of the dominant kernel (dram__bytes_read.sum + dram__bytes_write.sum
 # from an ncu capture) per shape, valid only for the kernel sources whose hash is given.
-TRAFFIC = {"sources_sha256": "ce4bb4173fa372a7", "bytes_per_launch": 729.5e6,
-           "note": "638.3 MB measured on one launch of the seven linears of a decoder layer, scaled to the eight linears "
+TRAFFIC = {"sources_sha256": "35753370dcba349f", "bytes_per_launch": 814.7e6,
+           "note": "712.8 MB measured on a launch (mean of two) of the seven linears of a decoder layer, scaled to the eight linears "
                    "of a bench launch (profiles/gemm_tc2_kernel_7b_layer.md)"}
 DOMINANT_SOURCES = ["paper_2402_02446_b200/csrc/lqer_gemm_tc2.cu", "paper_2402_02446_b200/csrc/lqer_tc_ptx.cuh"]
 
@@ -60,9 +60,9 @@ def sources_hash(sources=None) -> str:
 # grows in proportion to the bytes a launch streams), valid for the sources whose hash is given.
 TRAFFIC_RATIO = {
     "decode": {"sources": ["paper_2402_02446_b200/csrc/lqer_decode_cols.cu", "paper_2402_02446_b200/csrc/lqer_common.cuh"],
-               "sha256": "a768b769609890b1", "ratio": 118.6 / 116.8, "note": "profiles/decode_cols_kernel_7b_layer.md"},
+               "sha256": "1347286dd44f615e", "ratio": 121.6 / 116.8, "note": "profiles/decode_cols_kernel_7b_layer.md"},
     "prologue": {"sources": ["paper_2402_02446_b200/csrc/lqer_prologue_tc.cu", "paper_2402_02446_b200/csrc/lqer_common.cuh"],
-                 "sha256": "6a0cf6e7e4090c5f", "ratio": 407.6 / 438.2, "note": "profiles/prologue_tc_kernel_7b_layer.md"},
+                 "sha256": "9cac3f6d92128f64", "ratio": 411.7 / 438.2, "note": "profiles/prologue_tc_kernel_7b_layer.md"},
 }
 
 

@@ -284,7 +284,7 @@ lqer_status_t lqer_workspace_init(void* workspace, size_t workspace_bytes, void*
 /* Read the device-side status word of `workspace` (synchronises `stream`). */
 lqer_status_t lqer_poll_status(const void* workspace, void* stream, lqer_status_t* device_status);
 
-/* Force a kernel path for tests: 0 auto, 1 plain CUDA-core reference kernel, 2 small-batch kernels
+/* Force a kernel path for tests: 0 auto (which also has a one-launch kernel for 3 to 16 rows that no other path runs), 1 plain CUDA-core reference kernel, 2 small-batch kernels
  * (column-owner kernel for M <= 4, small prologue + small-batch GEMM for M <= 128), 3 tensor-core GEMM behind the
  * activation prologue that runs the projection on int8 mma.sync (at every batch size), 4 tensor-core
  * GEMM with the prologue chosen as in 0, 5 small prologue + small-batch GEMM for every M <= 128 (the register-operand
