@@ -866,12 +866,15 @@ static lqer_status_t linear_batched(const lqer_call_t* calls, int n_calls, void*
     int n = 1;
     PackedMeta m0, metas[16];
     bool decode_group = false, small_group = false, cluster_group = false;
-    const int clustered = may_group && !chain_open ? cluster_run(calls, i, n_calls, workspace_bytes, io.y_type, metas) : 0;
+    // Inside a stretch whose activations lie ready behind the head, the calls that are left read them there: no kernel that
+    // has its own scratch in that place may run before the stretch ends.
+    const bool held = i < pre_end && !pre_off.empty();
+    const int clustered = may_group && !chain_open && !held ? cluster_run(calls, i, n_calls, workspace_bytes, io.y_type, metas) : 0;
     if (clustered > 1) {
       n = clustered;
       cluster_group = true;
     } else if (may_group && lookup(calls[i].packed, m0) == LQER_OK) {
-      const int many = cols_ok ? many_small_rows(calls, i, n_calls, workspace_bytes, m0, metas, nullptr) : 0;
+      const int many = cols_ok && !held ? many_small_rows(calls, i, n_calls, workspace_bytes, m0, metas, nullptr) : 0;
       if (many > 0) {
         n = many;
         small_group = true;
