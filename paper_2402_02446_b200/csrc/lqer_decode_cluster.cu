@@ -762,6 +762,7 @@ bool decode_cluster_takes(const PackedMeta* metas, int n, int M, int y_type) {
   long long weights = 0;
   int k_pad = 0;
   for (int i = 0; i < n; ++i) {
+    if (!w_offsets_fit(metas[i])) return false;
     weights += (long long)metas[i].K64 * metas[i].N;
     k_pad = std::max(k_pad, (int)metas[i].k_pad);
   }

@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cols_kernel(const __grid_c
   const int cg_lo = cgu * (cta * (ly.n_cg / cgu) / G), cg_hi = cgu * ((cta + 1) * (ly.n_cg / cgu) / G);
 
   // This lane's column of a round (the 32 columns from column group cg0 on) and slab j: global -> registers.  Byte
-  // offsets into the W section are kept per round (32 bits: the section is far below 4 GB).  Column groups past the
+  // offsets into the W section are kept per round (32 bits, see decode_cols_fits).  Column groups past the
   // CTA's range are clamped to its last one and slabs past K to the last slab: such loads stay inside the section
   // and what they return is never used (the sums of those slabs are skipped, those columns are not stored).
   const uint32_t lane_w = (uint32_t)((lane & 7) * 16);
@@ -740,8 +740,8 @@ static size_t cols_smem_bytes(const PackedMeta& m, int M) {
          (size_t)kMaxM * m.k_pad * 8 * t_subsets(m.k_pad) + kMaxM * 16 * 4 + (size_t)kMaxM * (m.k_pad > 0 ? m.k_pad : 16) + 256;
 }
 // The column-owner kernel serves M <= 4 (its dot products run on the raw nibbles or crumbs) as long as the quantised X of
-// the whole contraction fits in shared memory.
-bool decode_cols_fits(const PackedMeta& m, int M) { return M <= dcol::kMaxM && cols_smem_bytes(m, M) <= 200 * 1024; }
+// the whole contraction fits in shared memory and 32 bits hold an offset into its weights.
+bool decode_cols_fits(const PackedMeta& m, int M) { return M <= dcol::kMaxM && w_offsets_fit(m) && cols_smem_bytes(m, M) <= 200 * 1024; }
 
 cudaError_t launch_decode_cols(const void* X, int x_type, int M, const PackedMeta& m, const void* packed, void* Y, int y_type,
                                void* workspace, cudaStream_t s) {
