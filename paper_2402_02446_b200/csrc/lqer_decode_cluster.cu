@@ -191,11 +191,29 @@ __device__ __forceinline__ void mma_w(float (&d)[4], uint32_t a0, uint32_t a1, u
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 // 128 K of NP pairs of column octets: the octets of a pair are rows g and g + 8 of the MMA.  word(o, m): eight converted weights.
-// GLOBAL: the activations (T_q) come from global memory, and only the first `blocks` 16-blocks of the lane's two exist.
-template <int MT, int NP, bool GLOBAL = false, class Word>
+// RANK: the activations (T_q) come from global memory, and only the first `blocks` 16-blocks of the lane's two exist.
+// The MMAs of a step add up in chains of four (MT == 1; eight otherwise, for want of registers), and the chains' sums are added to
+// acc by fp32 additions: the accumulators of mma.sync cut off what does not fit, and one chain over a CTA's whole part of K was up to
+// 14 times as far off as the kernels that took these calls before (2-norm against 64 bits for 13824 K of one sign, block
+// exponents over a dozen binades: 4 rows 8.5e-7, column-owner kernel 6.2e-8, now 5.1e-8; 16 rows 8.5e-7, tensor-memory GEMM 8.9e-8,
+// now 5.0e-8).  Chains of eight for MT == 1 are at 1.0 to 1.7 times the column-owner kernel where the signs are mixed, of four at
+// 0.8 to 1.2.  us a call with one chain / these: 4096 x 4096, 4 rows 11.4 / 11.5, 16 rows 15.4 / 15.4.  The one or two rank steps of MT == 2
+// continue acc itself (with chains of their own, 16 rows of rank 256 took 24.6 us instead of 22.0: spilled registers).
+template <int MT, int NP, bool RANK = false, class Word>
 __device__ __forceinline__ void multiply_step(float (&acc)[kOcts / 2][MT][4], const uint8_t* x, uint32_t plane, Word&& word, int blocks = 2) {
+  constexpr bool kChains = !(RANK && MT == 2);
+  constexpr int kChain = MT == 1 ? 2 : 4;            // m per chain
+  float d[NP][MT][4];
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
+    if (kChains && m % kChain == 0) {
+#pragma unroll
+      for (int p = 0; p < NP; ++p)
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) d[p][i][q] = 0.f;
+    }
     uint4 w[2 * NP];
 #pragma unroll
     for (int o = 0; o < 2 * NP; ++o) w[o] = word(o, m);
@@ -205,12 +223,12 @@ __device__ __forceinline__ void multiply_step(float (&acc)[kOcts / 2][MT][4], co
       uint32_t b[2 * MT];
       if (MT == 1) {
         uint2 v = make_uint2(0u, 0u);
-        if (!GLOBAL) v = *reinterpret_cast<const uint2*>(at);
+        if (!RANK) v = *reinterpret_cast<const uint2*>(at);
         else if ((m >> 1) < blocks) v = __ldcg(reinterpret_cast<const uint2*>(at));
         b[0] = v.x; b[1] = v.y;
       } else {
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (!GLOBAL) v = *reinterpret_cast<const uint4*>(at);
+        if (!RANK) v = *reinterpret_cast<const uint4*>(at);
         else if ((m >> 1) < blocks) v = __ldcg(reinterpret_cast<const uint4*>(at));
         b[0] = v.x; b[2 * MT - 2] = v.y; b[1] = v.z; b[2 * MT - 1] = v.w;
       }
@@ -218,8 +236,16 @@ __device__ __forceinline__ void multiply_step(float (&acc)[kOcts / 2][MT][4], co
       for (int p = 0; p < NP; ++p)
 #pragma unroll
         for (int i = 0; i < MT; ++i)
-          mma_w(acc[p][i], h ? w[2 * p].z : w[2 * p].x, h ? w[2 * p + 1].z : w[2 * p + 1].x, h ? w[2 * p].w : w[2 * p].y,
+          mma_w(kChains ? d[p][i] : acc[p][i], h ? w[2 * p].z : w[2 * p].x, h ? w[2 * p + 1].z : w[2 * p + 1].x, h ? w[2 * p].w : w[2 * p].y,
                 h ? w[2 * p + 1].w : w[2 * p + 1].y, b[2 * i], b[2 * i + 1]);
+    }
+    if (kChains && m % kChain == kChain - 1) {
+#pragma unroll
+      for (int p = 0; p < NP; ++p)
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[p][i][q] += d[p][i][q];
     }
   }
 }

@@ -10,6 +10,7 @@ import torch
 
 import lqer_inputs as gen
 import paper_2402_02446_b200 as L
+from paper_2402_02446_b200 import binding
 from oracle import lqer as olqer
 from helpers import worst_ratio
 
@@ -51,6 +52,32 @@ def test_rows_3_to_16_against_the_oracle(K, N, k, w_bits):
         assert L.poll_status(ws) == 0
         assert torch.equal(Y, again)
         assert worst_ratio(Y.cpu().numpy(), ref) <= 1.0, M
+    Pg.release()
+
+
+@pytest.mark.parametrize("K,k", [(1040, 16), (13824, 64), (4096, 256)])
+@pytest.mark.parametrize("M", [3, 4, 8, 16])
+def test_rounded_sums_are_no_further_off_than_the_other_kernels(M, K, k):
+    # one sign and block exponents over a dozen binades: no fp32 sum is exact.  Against the column-owner kernel (up to four rows: dot
+    # products added by rounded fp32 operations) or the tensor-memory GEMM, both on path 2; half as much again is left for the
+    # draw of the inputs (the kernels' own ratios are 0.5 to 1.0).
+    spec = gen.LayerSpec("rounds", M=M, K=K, N=520, k=k, calib_rows=32, outlier_frac=0.01, outlier_scale=20.0, seed=904)
+    W = np.abs(gen.make_weight(spec))
+    A, B = gen.make_random_factors(spec)
+    P, Pg = olqer.prepare_weights(W, A, B), L.prepare_weights(_t(W), _t(A), _t(B))
+    X = np.abs(gen.make_activations(spec)) * np.exp2(np.random.default_rng(9).integers(-6, 7, size=(M, K // 16))).repeat(16, axis=1).astype(np.float32)
+    ref = olqer.forward(X, P)
+    ws = L.new_workspace(M, Pg)
+    error = {}
+    for path in (binding.PATH_AUTO, binding.PATH_DECODE):
+        L.set_path(path)
+        try:
+            y = L.linear(_t(X), Pg, ws).cpu().numpy().astype(np.float64)
+        finally:
+            L.set_path(binding.PATH_AUTO)
+        assert L.poll_status(ws) == 0
+        error[path] = np.linalg.norm(y - ref.Y) / np.linalg.norm(ref.Y)
+    assert 0.0 < error[binding.PATH_AUTO] <= 1.5 * error[binding.PATH_DECODE], error
     Pg.release()
 
 
