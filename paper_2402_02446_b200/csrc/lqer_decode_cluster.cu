@@ -671,7 +671,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_cluster_kernel(const __gri
 
 // Clusters of CS CTAs that the device holds at a time, with one or two CTAs to an SM (0 if the query fails).
 constexpr int kSmemTwo = 112 * 1024, kSmemOne = 220 * 1024;
-static cudaLaunchConfig_t launch_config(int CS, int clusters, size_t smem, cudaLaunchAttribute* attr, cudaStream_t s) {
+static cudaLaunchConfig_t launch_config(int CS, int clusters, size_t smem, bool cooperative, cudaLaunchAttribute* attr, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(clusters * CS);
   cfg.blockDim = dim3(kThreads);
@@ -681,8 +681,10 @@ static cudaLaunchConfig_t launch_config(int CS, int clusters, size_t smem, cudaL
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = CS; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  attr[2].id = cudaLaunchAttributeCooperative;
+  attr[2].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = cooperative ? 3 : 2;
   return cfg;
 }
 template <int WB, int MT, bool YQ, int D>
@@ -694,8 +696,8 @@ static int resident_clusters(int CS, bool two) {
   std::lock_guard<std::mutex> lock(mu);
   int& n = known[dev][CS == 8 ? 3 : CS == 4 ? 2 : CS == 2 ? 1 : 0][two ? 1 : 0];
   if (n == 0) {
-    cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = launch_config(CS, 1, two ? kSmemTwo : kSmemOne, attr, nullptr);
+    cudaLaunchAttribute attr[3];
+    const cudaLaunchConfig_t cfg = launch_config(CS, 1, two ? kSmemTwo : kSmemOne, false, attr, nullptr);
     if (cudaFuncSetAttribute(decode_cluster_kernel<WB, MT, YQ, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemOne) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, decode_cluster_kernel<WB, MT, YQ, D>, &cfg) != cudaSuccess)
       n = 0;
@@ -703,9 +705,9 @@ static int resident_clusters(int CS, bool two) {
   return n;
 }
 template <int WB, int MT, bool YQ, int D>
-static cudaError_t launch(const Params& p, int clusters, int CS, size_t smem, cudaStream_t s) {
-  cudaLaunchAttribute attr[2];
-  const cudaLaunchConfig_t cfg = launch_config(CS, clusters, smem, attr, s);
+static cudaError_t launch(const Params& p, int clusters, int CS, size_t smem, bool cooperative, cudaStream_t s) {
+  cudaLaunchAttribute attr[3];
+  const cudaLaunchConfig_t cfg = launch_config(CS, clusters, smem, cooperative, attr, s);
   LaunchScope scope(kFamDecode, s);
   return cudaLaunchKernelEx(&cfg, decode_cluster_kernel<WB, MT, YQ, D>, p, CS);
 }
@@ -713,13 +715,13 @@ static cudaError_t launch(const Params& p, int clusters, int CS, size_t smem, cu
 template <int WB, int MT, bool YQ>
 struct Instance {
   static int resident(int CS, bool two) { return two ? resident_clusters<WB, MT, YQ, 2>(CS, true) : resident_clusters<WB, MT, YQ, 4>(CS, false); }
-  static cudaError_t go(const Params& p, int clusters, int CS, bool two, size_t smem, cudaStream_t s) {
-    return two ? launch<WB, MT, YQ, 2>(p, clusters, CS, smem, s) : launch<WB, MT, YQ, 4>(p, clusters, CS, smem, s);
+  static cudaError_t go(const Params& p, int clusters, int CS, bool two, size_t smem, bool cooperative, cudaStream_t s) {
+    return two ? launch<WB, MT, YQ, 2>(p, clusters, CS, smem, cooperative, s) : launch<WB, MT, YQ, 4>(p, clusters, CS, smem, cooperative, s);
   }
 };
 struct Entry {
   int (*resident)(int, bool);
-  cudaError_t (*go)(const Params&, int, int, bool, size_t, cudaStream_t);
+  cudaError_t (*go)(const Params&, int, int, bool, size_t, bool, cudaStream_t);
 };
 template <int WB, int MT, bool YQ>
 static Entry entry() { return Entry{Instance<WB, MT, YQ>::resident, Instance<WB, MT, YQ>::go}; }
@@ -819,6 +821,14 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
   // places are left free: 4096 x 4096, 4 rows, 14.3 us with 32 of 33 clusters and 12.0 with 28; larger launches lose more by the
   // longer ranges of columns (two of 4096 x 11008: 35.5 with 28, 30.5 with 32, 34 with 33).
   int budget = kernel.resident(CS, q.two);
+  // The clusters that form a layer's T wait for one another, and all others of the layer, placed after them, wait for these.  A launch
+  // that runs beside others may get its places one by one, and until all of a layer's T clusters have theirs the ones that do
+  // cannot leave.  At most a quarter of the places go to such clusters, so that four launches on as many streams cannot hold
+  // each other up for good; where that would cost too much (one CTA to an SM: 13824 x 2048 of rank 256, 4 rows, 40.6 us instead of 21.8)
+  // the launch is a cooperative one, which is placed as a whole or not yet (some 1 us more).  With two CTAs to an SM the
+  // quarter costs nothing (rank 256, 4 rows: 4096 x 4096 14.4 / 14.3, 2048 x 5632 14.0 / 13.5; below rank 144 nothing changes).
+  const int most = std::max(budget / 4, 1);
+  bool cooperative = false;
   long long weights = 0;
   for (int i = 0; i < n; ++i) weights += (long long)metas[i].K64 * metas[i].N;
   if (q.two && budget >= 8) budget = weights <= 30000000 ? budget * 7 / 8 : budget / 4 * 4;
@@ -865,11 +875,13 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
     ly.tcount = counts + 2 * g;
     // each warp of an owner counts its 16-blocks of T in
     ly.t_expect = M * m.r_blocks;
-    ly.t_blocks = (m.r_blocks + clusters[g] - 1) / clusters[g];
+    const int formers = q.two ? std::min(clusters[g], most) : clusters[g];
+    ly.t_blocks = (m.r_blocks + formers - 1) / formers;
+    if (i < n && std::min(formers, (int)m.r_blocks) > most) cooperative = true;
     if (i < n) t_off += decode_cluster_scratch_bytes(m);
     if (i < n) begin += clusters[g];
   }
-  return kernel.go(p, total, CS, q.two, q.smem, s);
+  return kernel.go(p, total, CS, q.two, q.smem, cooperative, s);
 }
 
 }  // namespace lqer

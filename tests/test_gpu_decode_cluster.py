@@ -129,3 +129,34 @@ def test_groups_share_one_launch(M):
                 assert worst_ratio(y.cpu().numpy(), olqer.forward(x.cpu().numpy(), layers[j][1])) <= 1.0, (pick, rep)
     for l in layers:
         l[2].release()
+
+
+def test_streams_with_a_workspace_each():
+    # four streams of calls whose T comes from several clusters (one block of ranks each, two, and a launch placed as a whole),
+    # beside a stream that keeps the SMs busy: nobody waits for good, and every result is the lone call's
+    shapes = [(4096, 1032, 256), (4096, 1032, 64), (12288, 520, 256), (1040, 4104, 256)]
+    layers = [_layer(*s, 905 + i) for i, s in enumerate(shapes)]
+    rows = (3, 16, 8, 5)
+    Xs = [_t(gen.make_activations(l[0], M=m)) for l, m in zip(layers, rows)]
+    want = [L.linear(x, l[2], L.new_workspace(m, l[2])) for x, l, m in zip(Xs, layers, rows)]
+    for w, x, l in zip(want, Xs, layers):
+        assert worst_ratio(w.cpu().numpy(), olqer.forward(x.cpu().numpy(), l[1])) <= 1.0
+    streams = [torch.cuda.Stream(priority=-(i % 2)) for i in range(4)]
+    spaces = [[L.new_workspace(m, l[2]) for m, l in zip(rows, layers)] for _ in streams]
+    Ys = [[[torch.full_like(w, float("nan")) for w in want] for _ in range(12)] for _ in streams]
+    busy, a = torch.cuda.Stream(), torch.zeros((8192, 8192), device=DEV)
+    torch.cuda.synchronize()
+    for rep in range(12):
+        with torch.cuda.stream(busy):
+            torch.add(a, 1.0, out=a)
+        for i, s in enumerate(streams):
+            for j in range(4):
+                q = (i + j) % 4
+                L.linear(Xs[q], layers[q][2], spaces[i][q], Ys[i][rep][q], stream=s)
+    torch.cuda.synchronize()
+    for i in range(4):
+        assert all(L.poll_status(w) == 0 for w in spaces[i])
+        for got in Ys[i]:
+            assert all(torch.equal(y, w) for y, w in zip(got, want))
+    for l in layers:
+        l[2].release()
