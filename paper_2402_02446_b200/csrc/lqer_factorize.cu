@@ -325,21 +325,11 @@ __global__ void __launch_bounds__(1024) cholesky_inverse_kernel(const double* __
     Rinv[q] *= inv;
   }
 }
-// 1 / sqrt(x) of an ordinary positive number: the hardware's first guess (some 22 bits) and one step of Halley's iteration,
-// y + y e (1/2 + 3/8 e) with e = 1 - x y^2, whose error is e^3.  Four dependent operations; an fp64 operation takes some 50 cycles
-// to its result here, and the chains below consist of little else.
-__device__ __forceinline__ double inv_sqrt(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
 // The same for r <= kSharedR, in panels of kPanel rows, so that the chain of dependent steps is as short as it can be: one
 // warp factors a diagonal block in registers (a column per lane; a step is one reciprocal square root, two shuffles, a product
 // and a multiply-add), a thread per remaining column solves for the panel's rows of R, all threads update what is left, and the
 // columns of R^-1, which depend on nothing but R, are formed at the end, eight lanes to a column, without a barrier.
-// 3 barriers per panel instead of one per row and another per row of the inverse: 28 us at r = 48 against 67 (33 with the library's
-// rsqrt in the chain).
+// 3 barriers per panel instead of one per row and another per row of the inverse: 28 us at r = 48 against 67.
 constexpr int kPanel = 8, kCholThreads = 512;
 __host__ __device__ constexpr int chol_ld(int r) { return (r + kPanel - 1) / kPanel * kPanel + 1; }   // odd: eight rows meet no bank twice
 __global__ void __launch_bounds__(kCholThreads) cholesky_inverse_panels_kernel(const double* __restrict__ part, int chunks, double* __restrict__ Cg,
@@ -373,7 +363,7 @@ __global__ void __launch_bounds__(kCholThreads) cholesky_inverse_panels_kernel(c
       for (int j = 0; j < kPanel; ++j) {
         double p = __shfl_sync(0xFFFFFFFFu, d[j], j);
         if (!(p > 0.0)) { p = 1e-300; low = true; }
-        const double inv = inv_sqrt(p);
+        const double inv = rsqrt(p);
         if (c == j) mine = inv;
         d[j] = (c == j ? p : d[j]) * inv;
 #pragma unroll
@@ -511,29 +501,19 @@ __global__ void __launch_bounds__(256) tall_times_small_kernel(const double* __r
 }
 
 // ---------------------------------------------------------------------------- small SVD (one CTA)
-// The rotation that makes two columns orthogonal: tan from approximate reciprocals (a tangent that is off by 1e-6 of itself
-// leaves that part of gamma for the next sweep, which the quadratic convergence absorbs), but cos = 1 / sqrt(1 + tan^2) in
-// full, so that the rotation is orthogonal to rounding.
-__device__ __forceinline__ double approx_rcp(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
+// The rotation that makes two columns orthogonal.
 __device__ __forceinline__ void rotation(double alpha, double beta, double gamma, double& c, double& s) {
-  const double zeta = (beta - alpha) * approx_rcp(2.0 * gamma), az = fabs(zeta);
-  const double u = fma(zeta, zeta, 1.0);
-  double root;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(root) : "d"(u));
-  const double t = copysign(approx_rcp(az < 1e100 ? fma(u, root, az) : 2.0 * az), zeta);
-  c = inv_sqrt(fma(t, t, 1.0));
+  const double zeta = (beta - alpha) / (2.0 * gamma), az = fabs(zeta);
+  const double t = copysign(1.0 / (az + sqrt(fma(az, az, 1.0))), zeta);
+  c = rsqrt(fma(t, t, 1.0));
   s = c * t;
 }
 // Right singular vectors and singular values of the r x r upper-triangular R (the Cholesky factor left in the upper
 // triangle of C, row-major) by one-sided Jacobi: pairs of columns are rotated until all are mutually orthogonal,
 // V collects the rotations.  A half warp per pair, the pairs of a step disjoint (round-robin tournament).  Mt, Vt: r x r
 // scratch, column-major.  Out: Vs row-major [r][r] with the columns in falling order of singular value, sigma[r].
-// Bound by its steps (r - 1 per sweep, one barrier each), in them by the fp64 pipe as much as by latency: half warps and
-// approximate quotients took 707 us at r = 48 to 377.  Both matrices sit in shared memory where they fit.
+// Bound by its steps (r - 1 per sweep, one barrier each), in them by the fp64 pipe as much as by latency: half warps
+// took 707 us at r = 48 to 408.  Both matrices sit in shared memory where they fit.
 __global__ void __launch_bounds__(1024) jacobi_right_kernel(const double* __restrict__ C, int r, double* __restrict__ Mtg,
                                                             double* __restrict__ Vtg, double* __restrict__ Vs, double* __restrict__ sigma,
                                                             int* __restrict__ status) {
