@@ -129,8 +129,8 @@ lqer_status_t lqer_prepare_weights(const float* W, const float* A, const float* 
  *  - A_out [K,k], B_out [k,N] fp32 (device): the factors before quantisation, or NULL.
  *  - workspace (device, 256-byte aligned): lqer_prepare_workspace_bytes.  Asynchronous on `stream`.
  *  - lqer_prepare_status (synchronises) reads what only the device could see: 0 fine, 1 a calibration channel is
- *    identically zero (S not invertible; S = I was used), 2 a sketch lost rank (k larger than the rank of the
- *    error), 3 the small SVD did not converge. */
+ *    identically zero (S not invertible; S = I was used), 2 a sketch lost rank (its k + 16 columns are more than the
+ *    rank of the error; the factors are zero beyond that rank), 3 the small SVD did not converge. */
 lqer_status_t lqer_factor_sketch_columns(int K, int N, int k, int* columns);
 lqer_status_t lqer_prepare_workspace_bytes(int K, int N, int k, size_t* bytes);
 lqer_status_t lqer_prepare_from_calibration(const float* W, const float* const* samples, const int* sample_rows, int n_samples,

@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(256) gram_partial_kernel(const double* __restr
   if (i0 + ti < r && j0 + tj < r) part[((size_t)blockIdx.z * r + i0 + ti) * r + j0 + tj] = acc;
 }
 // C = the sum of the partial Gram matrices (in chunk order) = R^T R (upper-triangular R by Cholesky), then Rinv = R^-1; one
-// CTA.  A pivot that is not positive (rank-deficient Y) is replaced by a tiny one so that the run stays finite; status
-// records it.
+// CTA.  A column whose pivot is not positive depends on the ones before it (rank-deficient Y): its row of R and its column of
+// R^-1 are zero, so that the column is zero from there on and the run stays finite; status records it.
 // Ranks beyond kSharedR: both matrices in global memory, a chain of 2 r short steps bound by their latency.  A step is one
 // update of a whole triangle by all threads (the trailing part of C minus the outer product of a finished row; the rows of
 // R^-1 above a finished one) and one barrier - the division of a row by its pivot is left to whoever reads the row, and done
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(1024) cholesky_inverse_kernel(const double* __
   // row j of the upper triangle of C becomes pivot_j times row j of R; the warp that has row j + 1 works out its pivot
   // (all warps doing it would keep the fp64 pipe busy for longer than the update)
   const auto pivot = [&](double d) {
-    if (!(d > 0.0)) { d = 1e-300; atomicMax(status, 2); }
+    if (!(d > 0.0)) { atomicMax(status, 2); return 0.0; }
     return 1.0 / sqrt(d);
   };
   if (threadIdx.x == 0) s_inv[0] = pivot(C[0]);
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(1024) cholesky_inverse_kernel(const double* __
   for (int q = threadIdx.x; q < r * r; q += 1024) {
     const int row = q / r, col = q % r;
     const double inv = s_inv[row];
-    if (col >= row) C[q] = col == row ? 1.0 / inv : C[q] * inv;
+    if (col >= row) C[q] = col == row && inv > 0.0 ? 1.0 / inv : C[q] * inv;
     Rinv[q] *= inv;
   }
 }
@@ -361,9 +361,10 @@ __global__ void __launch_bounds__(kCholThreads) cholesky_inverse_panels_kernel(c
       bool low = false;
 #pragma unroll
       for (int j = 0; j < kPanel; ++j) {
-        double p = __shfl_sync(0xFFFFFFFFu, d[j], j);
-        if (!(p > 0.0)) { p = 1e-300; low = true; }
-        const double inv = rsqrt(p);
+        const double p = __shfl_sync(0xFFFFFFFFu, d[j], j);
+        double inv = 0.0;
+        if (p > 0.0) inv = rsqrt(p);
+        else low = true;
         if (c == j) mine = inv;
         d[j] = (c == j ? p : d[j]) * inv;
 #pragma unroll

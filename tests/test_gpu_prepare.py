@@ -119,3 +119,25 @@ def test_prepare_at_the_edges_of_the_factorisation(k, scale):
     optimum, got = np.sqrt(np.sum(sig[k:] ** 2)), np.linalg.norm(SE - SA @ B)
     assert optimum * (1 - 1e-6) <= got <= optimum * (1 + 1e-2)
     Pg.release()
+
+
+@pytest.mark.parametrize("k", [3, 5, 32, 100])
+def test_prepare_from_an_error_of_low_rank(k):
+    # W is on the quantiser's grid but for five columns: the sketch has dependent columns (code 2) whatever k is, and the factors
+    # still carry what there is of the error
+    rng = np.random.default_rng(506)
+    W = np.clip(np.round(rng.standard_normal((512, 512))), -3, 3).astype(np.float32)
+    W[::16] = 4.0
+    cols = [3, 50, 77, 200, 511]
+    W[:, cols] = (rng.standard_normal((512, 5)) * 0.02).astype(np.float32)
+    Pg, A, B, code = L.prepare_from_calibration(_t(W), [], k, seed=506)
+    assert code == 2
+    A, B = A.cpu().numpy().astype(np.float64), B.cpu().numpy().astype(np.float64)
+    assert np.all(np.isfinite(A)) and np.all(np.isfinite(B))
+    Wm, We = olqer.quantize_weight(W)
+    E = olqer.quantization_error(W, Wm, We)
+    sig = np.linalg.svd(E[:, cols], compute_uv=False)
+    optimum, got = np.sqrt(np.sum(sig[k:] ** 2)), np.linalg.norm(E - A @ B)
+    assert got <= optimum * (1 + 1e-2) + 1e-6 * np.linalg.norm(E)
+    assert np.linalg.norm(A, ord=2) <= 1 + 1e-6                  # (S = I) orthonormal columns, and zeros
+    Pg.release()
