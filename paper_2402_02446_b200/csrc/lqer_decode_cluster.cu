@@ -46,7 +46,7 @@ struct Layer {
   uint8_t* tq;                              // T_q on its way between clusters: eight planes (the layout of the activations)
   int* tcount;                              // arrivals, departures: zero between calls
   int t_blocks;                             // rank blocks of T that each of the layer's first clusters forms
-  int t_expect;                             // arrivals that make T_q whole
+  int t_expect;                             // arrivals that make T_q whole (one more under the test hook)
 };
 struct Params {
   Layer L[kMaxLayers];
@@ -57,7 +57,7 @@ struct Params {
   int slabs_max;                            // slabs of a CTA, rounded up to even: the extent of the activation planes
   int off_red[2], off_xq, off_xe, off_tpart, off_ring;   // offsets in shared memory (the planes of X_q come first)
   long long wait_limit;
-  int stall;                                // test hook: the sums of a round wait for bytes that never come
+  int stall;                                // test hook: the sums of the first round wait for bytes that never come (see also t_expect)
 };
 
 __device__ __forceinline__ uint32_t cta_rank() {
@@ -811,7 +811,8 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
   p.n = n; p.M = M; p.status = st; p.x_type = x_type; p.y_type = y_type;
   p.a_bits = metas[0].a_bits; p.lr_bits = metas[0].lr_bits; p.exp_min = metas[0].exp_min; p.exp_max = metas[0].exp_max;
   p.wait_limit = wait_limit_cycles();
-  p.stall = take_stall(kFamDecode) ? 1 : 0;
+  const bool stall = take_stall(kFamDecode);
+  p.stall = stall ? 1 : 0;
   p.slabs_max = q.slabs_max;
   p.off_red[0] = q.off_red[0]; p.off_red[1] = q.off_red[1];
   p.off_xq = q.off_xq; p.off_xe = q.off_xe; p.off_tpart = q.off_tpart; p.off_ring = q.off_ring;
@@ -874,7 +875,7 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
     ly.tq = static_cast<uint8_t*>(scratch) + t_off;
     ly.tcount = counts + 2 * g;
     // each warp of an owner counts its 16-blocks of T in
-    ly.t_expect = M * m.r_blocks;
+    ly.t_expect = M * m.r_blocks + (stall ? 1 : 0);
     const int formers = q.two ? std::min(clusters[g], most) : clusters[g];
     ly.t_blocks = (m.r_blocks + formers - 1) / formers;
     if (i < n && std::min(formers, (int)m.r_blocks) > most) cooperative = true;

@@ -29,6 +29,7 @@ def test_small_parity_cases_pass_under_the_checked_build():
     r = _run(["-m", "pytest", "-x", "-q", "-m", "gpu",
               "tests/test_gpu_parity.py", "tests/test_gpu_bf16_io.py", "tests/test_gpu_mxint8_io.py", "tests/test_gpu_w2.py",
               "tests/test_gpu_small_mma.py", "tests/test_gpu_small_batches.py", "tests/test_gpu_digit_prologue.py",
+              "tests/test_gpu_decode_cluster.py", "tests/test_gpu_pair_tiles.py", "tests/test_gpu_batched_mixed_rows.py",
               "-k", "not full and not stack and not sweep and not round"])
     assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
     assert " passed" in r.stdout
@@ -44,7 +45,7 @@ def test_a_short_extent_is_reported_and_nothing_beyond_it_is_written():
         E = binding.STATUS_NAMES.index
         dev = "cuda:0"
         t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)
-        for M, path in ((3, binding.PATH_AUTO), (9, binding.PATH_SMALL), (40, binding.PATH_AUTO), (300, binding.PATH_AUTO)):
+        for M, path in ((3, binding.PATH_AUTO), (3, binding.PATH_DECODE), (9, binding.PATH_SMALL), (40, binding.PATH_AUTO), (300, binding.PATH_AUTO)):
             spec = gen.LayerSpec("short", M=M, K=512, N=384, k=16, calib_rows=32, outlier_frac=0.01, outlier_scale=20.0, seed=501)
             W = gen.make_weight(spec); A, B = gen.make_random_factors(spec)
             Pg = L.prepare_weights(t(W), t(A), t(B))

@@ -30,6 +30,8 @@ def _t(a):
 
 def _layer(spec):
     W = gen.make_weight(spec)
+    if spec.k == 0:
+        return olqer.prepare_weights(W, None, None), L.prepare_weights(_t(W), None, None)
     A, B = gen.make_random_factors(spec)
     return olqer.prepare_weights(W, A, B), L.prepare_weights(_t(W), _t(A), _t(B))
 
@@ -37,7 +39,9 @@ def _layer(spec):
 CASES = [
     # (name, family, forced path, M, K, N, k)
     ("decode_cols_T_exchange", FAM_DECODE, binding.PATH_AUTO, 2, 2112, 264, 72),   # 132 K blocks x 3 rank tiles: T is exchanged
-    ("small_gemm_ring", FAM_DECODE, binding.PATH_AUTO, 9, 1024, 640, 40),
+    ("small_gemm_ring", FAM_DECODE, binding.PATH_SMALL_TMEM, 9, 1024, 640, 40),
+    ("decode_cluster_T_exchange", FAM_DECODE, binding.PATH_AUTO, 5, 1040, 20008, 40),   # T_q of other clusters, counters left behind
+    ("decode_cluster_sums", FAM_DECODE, binding.PATH_AUTO, 5, 1040, 20008, 0),          # no rank: the first of several rounds
     ("small_mma_flags", FAM_DECODE, binding.PATH_SMALL, 9, 1024, 640, 40),      # the polls of the prologue's flags
     ("prologue_tc_row_tile", FAM_PROLOGUE, binding.PATH_TENSOR_PROLOGUE, 300, 1024, 640, 32),
     ("digit_prologue_ring", FAM_PROLOGUE, binding.PATH_TENSOR_PROLOGUE, 300, 1040, 640, 136),   # several K ranges: one of them stalls

@@ -7,6 +7,7 @@ import torch
 
 import lqer_inputs as gen
 import paper_2402_02446_b200 as L
+from paper_2402_02446_b200 import binding
 from helpers import exp_bytes, worst_ratio
 from oracle import lqer as olqer
 
@@ -39,18 +40,23 @@ def test_token_counts_and_tile_edges(M, K, N, k):
     ref = olqer.forward(X, P, w_bits=w_bits)
     ws = L.new_workspace(M, Pg)
     ws[168192:] = 0xFF                                  # scratch holds NaN patterns: nothing unwritten may be read
-    for _ in range(2):
-        Y = L.linear(_t(X), Pg, ws)
-        assert L.poll_status(ws) == 0
-        assert worst_ratio(Y.cpu().numpy(), ref) <= 1.0
-    assert torch.equal(L.linear_ex(_t(X), Pg, ws, out_dtype=torch.bfloat16), Y.to(torch.bfloat16))
-    if k:
-        Tm, Te = L.project_lowrank(_t(X), Pg, ws)
-        assert np.array_equal(Tm.cpu().numpy(), ref.Tm) and np.array_equal(Te.cpu().numpy(), exp_bytes(ref.Te))
-    if N % 16 == 0:
-        m8, e8 = L.split_mxint8(L.linear_ex(_t(X), Pg, ws, out_dtype=L.MXINT8), M, N)
-        qm, qe = L.quantize_activations(Y)              # the codes of the same path's fp32 result
-        assert torch.equal(m8, qm) and torch.equal(e8, qe)
+    # up to 16 rows a lone call takes the cluster kernel by itself (test_gpu_decode_cluster.py)
+    L.set_path(binding.PATH_SMALL_TMEM if M <= 16 else binding.PATH_AUTO)
+    try:
+        for _ in range(2):
+            Y = L.linear(_t(X), Pg, ws)
+            assert L.poll_status(ws) == 0
+            assert worst_ratio(Y.cpu().numpy(), ref) <= 1.0
+        assert torch.equal(L.linear_ex(_t(X), Pg, ws, out_dtype=torch.bfloat16), Y.to(torch.bfloat16))
+        if k:
+            Tm, Te = L.project_lowrank(_t(X), Pg, ws)
+            assert np.array_equal(Tm.cpu().numpy(), ref.Tm) and np.array_equal(Te.cpu().numpy(), exp_bytes(ref.Te))
+        if N % 16 == 0:
+            m8, e8 = L.split_mxint8(L.linear_ex(_t(X), Pg, ws, out_dtype=L.MXINT8), M, N)
+            qm, qe = L.quantize_activations(Y)          # the codes of the same path's fp32 result
+            assert torch.equal(m8, qm) and torch.equal(e8, qe)
+    finally:
+        L.set_path(binding.PATH_AUTO)
     Pg.release()
 
 
