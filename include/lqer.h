@@ -100,7 +100,7 @@ lqer_status_t lqer_packed_bytes(int K, int N, int k, const lqer_config_t* cfg, s
 lqer_status_t lqer_workspace_bytes(int M_max, int K, int N, int k, const lqer_config_t* cfg, size_t* bytes);
 
 /* Size in bytes (host out) of the smallest workspace that one call with exactly M rows is taken with, on the path the
- * library picks for it (column-owner decode kernel up to 4 rows, small-batch kernels up to 128, prologue + GEMM above):
+ * library picks for it (decode and small-batch kernels up to 128 rows, prologue + GEMM above):
  * never more than lqer_workspace_bytes(M_max, ...) for any M_max >= M.  This is the figure lqer_linear_static holds against
  * LQER_STATIC_SCRATCH_BYTES.  A call of more than 128 rows and a rank above 64 runs faster (up to 1.7 times) with a
  * workspace of lqer_workspace_bytes(M, ...), which has room for its projection as one integer contraction; the results are
@@ -171,10 +171,17 @@ lqer_status_t lqer_project_lowrank(const float* X, int M, const void* packed, in
 
 /* The layer (Section 3.1 last display, Section 3.2 last display):
  *   Y[M,N] = X_q W_q + q(X_q A_q) B_q,  fp32 accumulation of exactly represented products.
- * M <= 4 runs a fused decode kernel whose CTAs own output columns; M <= 128 a latency-oriented
- * prologue and a tensor-core GEMM that streams the weights once, 128 columns of them per MMA against all tokens;
- * larger M the activation prologue and the tensor-core GEMM over 256 x 256 tiles of the concatenated
- * contraction [X_q | T_q] . [W_q ; B_q].
+ * One or two rows run a fused decode kernel whose CTAs own output columns.  Three to sixteen rows run one kernel in which
+ * clusters of CTAs own columns and share the contraction, unless that is the slower way for the layer: up to eight rows it takes
+ * every layer whose activations fit its shared memory, from nine on (and at three with ranks above 128) layers of up to
+ * 3e7 weights.  What it leaves runs the decode kernel up to 4 rows, and up to 128 rows a latency-oriented
+ * prologue and a tensor-core GEMM that streams the weights once, 128 columns of them per MMA against all tokens.
+ * Larger M run the activation prologue and the tensor-core GEMM over tiles (256 rows x 256, 192 or 128 columns) of the
+ * concatenated contraction [X_q | T_q] . [W_q ; B_q].
+ * Kernels whose CTAs share T wait for CTAs of their own launch (every wait is bounded, see lqer_set_wait_limit_cycles), so
+ * such a launch counts on the SMs of the whole device: beside other work it waits for its places, and calls on several
+ * streams, a workspace each, take theirs in turn; in a context that is limited to a part of the SMs it may end in
+ * LQER_ERR_TIMEOUT.
  * lqer_linear uses the default stream. */
 lqer_status_t lqer_linear(const float* X, int M, const void* packed, float* Y,
                           void* workspace, size_t workspace_bytes);
@@ -225,7 +232,7 @@ lqer_status_t lqer_linear_batched_ex(const lqer_call_t* calls, int n_calls, lqer
  *    status area at its head is cleared at the start of every call.  Two calls that overlap on
  *    the GPU (different streams without an ordering between them) race on the array and give
  *    undefined results: keep calls of this entry point on one stream, or order them.
- *  - Device-side conditions (a bounded wait that ran out) cannot be polled for this variant;
+ *  - Device-side conditions (a bounded wait that ran out, see lqer_linear) cannot be polled for this variant;
  *    use lqer_linear_stream with a workspace where that matters. */
 #define LQER_STATIC_SCRATCH_BYTES (8u << 20)
 lqer_status_t lqer_linear_static(const float* X, int M, const void* packed, float* Y, void* stream);
@@ -234,7 +241,9 @@ lqer_status_t lqer_linear_static(const float* X, int M, const void* packed, floa
  * The workspace is reused by consecutive calls (stream order makes that safe) and must
  * fit the largest of them.  Independent means that no call reads what another call of the
  * same batch writes; the library uses that, with the path left at 0, to share launches:
- *  - up to 16 consecutive calls with one M <= 4 (any shapes with N >= 32, one set of formats)
+ *  - a run of two to four calls with one M from 3 to 16 (one set of formats) that the cluster kernel takes (see
+ *    lqer_linear; the line of 3e7 weights is drawn over all of them) runs as ONE launch of it;
+ *  - otherwise up to 16 consecutive calls with one M <= 4 (any shapes with N >= 32, one set of formats)
  *    run as ONE launch of the decode kernel that divides the SMs among them; consecutive such
  *    launches do not wait for one another, and a stretch of more than one launch first has the
  *    quantised activations and T_q of all its calls computed by one kernel, into the workspace;
@@ -243,14 +252,15 @@ lqer_status_t lqer_linear_static(const float* X, int M, const void* packed, floa
  *    all of them - if the workspace holds lqer_batched_workspace_bytes(calls, n_calls); with a
  *    smaller workspace (at least the largest lqer_workspace_bytes of the calls) fewer calls, or
  *    none, share a launch;
- *  - up to 16 consecutive calls with one M <= 128 that the decode kernel does not serve (any shapes,
- *    one set of formats) run as ONE launch of the small prologue and ONE launch of the small-batch
- *    GEMM over the work items of all of them, under the same condition on the workspace.
- * In the first two cases a result does not depend on the sharing, bit for bit.  In the third the
- * contraction of a tile is cut into fewer K chunks when layers share a launch, so a result may
- * differ from the single call's in its last bits (both within the layer's tolerance); the fp64 sums
- * of X A_k are grouped differently too, which shows only where a row's block exponents spread over
- * more than about 30 binades.  A result is reproducible for the same sequence of calls. */
+ *  - up to 16 consecutive calls with one M <= 128 that neither of these serves (any shapes, one set of formats; of four
+ *    rows from six calls on and of three from twelve also calls that they would serve) run as ONE launch of the small
+ *    prologue and ONE launch of the small-batch GEMM over the work items of all of them, under the same condition on
+ *    the workspace.
+ * With one or two rows and with more than 128 a result does not depend on the sharing, bit for bit.  From 3 to 128 rows the
+ * kernel and the cut of the contraction depend on the calls that share a launch, so where fp32 sums round a result may
+ * differ from the single call's in its last bits (both within the layer's tolerance).  The fp64 sums of X A_k may be grouped
+ * differently at any size, which shows only where a row's block exponents spread over more than about 30 binades.  A result
+ * is reproducible for the same sequence of calls. */
 lqer_status_t lqer_batched_workspace_bytes(const lqer_call_t* calls, int n_calls, size_t* bytes);
 lqer_status_t lqer_linear_batched(const lqer_call_t* calls, int n_calls,
                                   void* workspace, size_t workspace_bytes, void* stream);
@@ -284,7 +294,8 @@ lqer_status_t lqer_workspace_init(void* workspace, size_t workspace_bytes, void*
 /* Read the device-side status word of `workspace` (synchronises `stream`). */
 lqer_status_t lqer_poll_status(const void* workspace, void* stream, lqer_status_t* device_status);
 
-/* Force a kernel path for tests: 0 auto (which also has a one-launch kernel for 3 to 16 rows that no other path runs), 1 plain CUDA-core reference kernel, 2 small-batch kernels
+/* Force a kernel path for tests: 0 auto (which alone runs the cluster kernel for 3 to 16 rows), 1 plain CUDA-core
+ * reference kernel, 2 small-batch kernels
  * (column-owner kernel for M <= 4, small prologue + small-batch GEMM for M <= 128), 3 tensor-core GEMM behind the
  * activation prologue that runs the projection on int8 mma.sync (at every batch size), 4 tensor-core
  * GEMM with the prologue chosen as in 0, 5 small prologue + small-batch GEMM for every M <= 128 (the register-operand
@@ -299,7 +310,7 @@ lqer_status_t lqer_set_path(int path);
  * the kernel give up, write LQER_ERR_TIMEOUT to the status word and return, so the context stays usable.
  *  - lqer_set_wait_limit_cycles: the bound in SM clock cycles (default 4e9, about two seconds; 1e3 .. 2^40).
  *  - lqer_inject_stall(family): the next launch of that kernel family (numbering of lqer_kernel_times_t:
- *    3 activation prologue, 6 tensor-core GEMM pair kernel, 7 decode kernels) is told to expect one arrival
+ *    3 activation prologue, 6 tensor-core GEMM pair kernel, 7 decode and small-batch kernels) is told to expect one arrival
  *    more than will ever come (3, 7) or has its last stage of operands withheld (6), so that its waits run
  *    out; no memory is touched that an ordinary launch would not touch.  -1 disarms.  After such a launch
  *    the outputs are undefined and the workspace needs lqer_workspace_init before its next use. */

@@ -358,7 +358,8 @@ def test_batched_decode_groups_same_shape_calls(M):
     assert L.launch_count() - launches == 1            # seven layers with one M: one launch
     for x, (sp, P, Pg), yb in zip(Xs, layers, Yb):
         ys = L.linear(x, Pg, ws)
-        assert torch.equal(ys, yb), sp.name             # same arithmetic, same order: bit-identical
+        # one row: the same arithmetic in the same order; three: lone calls run another kernel, but these sums are exact
+        assert torch.equal(ys, yb), sp.name
         assert worst_ratio(yb.cpu().numpy(), olqer.forward(x.cpu().numpy(), P)) <= 1.0, sp.name
     for _, _, Pg in layers:
         Pg.release()
@@ -495,7 +496,7 @@ def test_linear_decode_full_size(M, ratio_log):
     X = gen.make_activations(spec)
     ref = olqer.forward(X, P)
     ws = L.new_workspace(M, Pg)
-    Y = L.linear(_t(X), Pg, ws).cpu().numpy()          # automatic path selection: the column-owner kernel (M <= 4) or the small-batch kernels
+    Y = L.linear(_t(X), Pg, ws).cpu().numpy()          # automatic path selection: the column-owner kernel (M = 1) or the cluster kernel
     assert L.poll_status(ws) == 0
     assert ratio_log(spec.name, worst_ratio(Y, ref)) <= 1.0
     Pg.release()
