@@ -400,11 +400,10 @@ static lqer_status_t run_small_group(const lqer_call_t* calls, int n, const Pack
                    nullptr, false, s) == cudaSuccess ? LQER_OK : LQER_ERR_CUDA;
 }
 // Three or four rows in many layers at once: the register-operand GEMM's launches take less per layer than the
-// column-owner kernel's.  Measured on 4096 x 4096 layers of rank 32, us per layer, column-owner / register-operand: 4 rows,
-// 2 layers 12.4 / 11.9, 4 layers 8.5 / 7.3, 6 layers 7.2 / 5.8, 16 layers 5.2 / 4.0; 3 rows, 2 layers 10.7 / 12.1, 4 layers
-// 7.3 / 7.3, 6 layers 6.1 / 5.8, 12 layers 4.5 / 4.5, 16 layers 4.3 / 3.9.  (The lines, 6 and 12 layers, were drawn for an
-// earlier small prologue; with the present one the two sides meet at 2 layers for 4 rows and at 4 to 6 for 3.)  The length
-// of such a run from calls[first] on, or 0.
+// column-owner kernel's (runs of up to four layers take neither, see decode_cluster_takes).  Measured on 4096 x 4096 layers of
+// rank 32, us per layer, column-owner / register-operand: 4 rows, 6 layers 7.2 / 5.8, 16 layers 5.2 / 4.0; 3 rows, 6 layers
+// 6.1 / 5.8, 12 layers 4.5 / 4.5, 16 layers 4.3 / 3.9.  (The lines, 6 and 12 layers, were drawn for an earlier small prologue and
+// lie on the safe side of the present one.)  The length of such a run from calls[first] on, or 0.
 static int many_small_rows(const lqer_call_t* calls, int first, int n_calls, size_t workspace_bytes, const PackedMeta& m0,
                            PackedMeta* metas, size_t* need) {
   const int M = calls[first].M;
@@ -852,7 +851,7 @@ static lqer_status_t linear_batched(const lqer_call_t* calls, int n_calls, void*
   // in turn), so a launch need not wait for the one before it, as long as that one had a CTA on every SM.
   bool chain_open = false;
   int chain_set = 0;
-  // The quantised activations and T_q of a stretch of several decode launches are computed ahead, one CTA per call, if
+  // The quantised activations and T_q of a stretch of several decode launches are computed ahead, by a cluster of CTAs per call, if
   // the workspace has room for them behind its head: the decode launches then stream weights from their first
   // instruction.
   const size_t pre_base = align_up(kPersistMaxBytes, 256);
@@ -860,8 +859,8 @@ static lqer_status_t linear_batched(const lqer_call_t* calls, int n_calls, void*
   std::vector<size_t> pre_off;                  // its offsets behind pre_base; empty: nothing computed ahead
   for (int i = 0; i < n_calls;) {
     // The calls are independent, so consecutive calls of one shape (the q, k, v projections of a layer, or its gate
-    // and up projections) share launches: decode calls one launch of the column-owner kernel (a slot of the workspace per
-    // layer for the partial sums of T), prefill calls one GEMM launch after their prologues, if the workspace has a
+    // and up projections) share launches: decode calls one launch of the cluster kernel or of the column-owner kernel (a slot of
+    // the workspace per layer for the partial sums of T), prefill calls one GEMM launch after their prologues, if the workspace has a
     // slice for each.
     int n = 1;
     PackedMeta m0, metas[16];

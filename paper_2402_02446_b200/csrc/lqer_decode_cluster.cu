@@ -2,15 +2,17 @@
 // tokens per step make it memory bound on its weights).
 //
 // A cluster of CS CTAs (8 where the contraction has 16 slabs of 64) owns a range of output columns; its CTAs share the
-// contraction: CTA q takes the slabs [q k_slabs / CS, (q + 1) k_slabs / CS).  So a CTA quantises only its part of X, and
-// everything the parts have to exchange stays in the cluster's shared memory:
-//   - T = X_q A_q: each CTA multiplies its part (int8 mma.sync per 16-block, exact, scaled and summed in fp64), stores its
-//     partial sums into the CTA that owns the row (st.async, counted in bytes on the owner's mbarrier); the owner adds
-//     them in CTA order, re-quantises along the rank and stores T_q into every CTA of the cluster.  All clusters of a
-//     layer form the same T: that costs a microsecond of arithmetic at rank 64 and saves the trip through global memory.
+// contraction: CTA q takes the slabs [q k_slabs / CS, (q + 1) k_slabs / CS).  So a CTA quantises only its part of X.  What the
+// parts have to exchange:
 //   - Y: the warps of a CTA own column octets, a round of them at a time, over the CTA's slabs.  Warp w's sums of a round go
-//     to CTA w mod CS, which adds them in CTA order and writes Y once.
-// Nothing waits for another cluster and there is no scratch in global memory.
+//     to CTA w mod CS (st.async, counted in bytes on that CTA's mbarrier), which adds them in CTA order and writes Y once.
+//   - T = X_q A_q: the first clusters of a layer form it, one or a few rank blocks each.  Each CTA multiplies its part (int8
+//     mma.sync per 16-block, exact, scaled and summed in fp64) and stores its partial sums into the CTA of its cluster that owns
+//     the row; the owner adds them in CTA order, re-quantises along the rank, writes T_q to scratch in global memory and counts its
+//     blocks in.  Every cluster of the layer waits for the count (bounded) before its first rank term, the last thing of its
+//     first round; the last warp to have read T_q zeroes the counters for the next call.
+// So a cluster waits for other clusters of its launch.  The launch has no more of them than the device holds at a time, those
+// that form T come first, and launch_decode_cluster says what keeps launches on several streams from holding each other up.
 //
 // The weights take the register-operand form (lqer_mma_frag.cuh): a lane loads the 16 bytes which the packed tile stores
 // for one column and block pair, here through its own slots of a ring in shared memory (cp.async; a lane reads back only
@@ -30,7 +32,7 @@ using tc::smem_u32;
 
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
-constexpr int kMaxLayers = 16;
+constexpr int kMaxLayers = 4;                // layers of a launch, at most
 constexpr int kOcts = 4;                    // column octets a warp owns in a round, at most
 constexpr int kRows = 16;
 
@@ -78,9 +80,6 @@ __device__ __forceinline__ void st_async(uint32_t addr, double a, double b, uint
 }
 __device__ __forceinline__ void st_async(uint32_t addr, float a, float b, uint32_t bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void st_async(uint32_t addr, uint32_t a, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(a), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -489,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_cluster_kernel(const __gri
       }
     }
   }
-  // the rows this CTA owns: sum in CTA order, MXINT8 along the rank, out to all clusters of the layer
+  // the rows this CTA owns: sum in CTA order, MXINT8 along the rank, out to scratch for all clusters of the layer
   auto reduce_t = [&]() -> bool {
     const int total = own_rows * t_cols;
     if (warp * 32 >= total) return true;
@@ -781,12 +780,11 @@ static Plan plan(const PackedMeta* metas, int n, int M) {
 // Three rows with ranks above 128 are level or worse in large launches (a 4064 / 10192 layer at rank 256 122.8 / 134.9, 4096 / 11008 126.6 /
 // 129.5; 2048 / 5632 87.3 / 62.3): the same line.
 // One and two rows keep the column-owner kernel (2 rows: 4096 x 4096 16.4 / 15.6, two of 4096 x 11008 26.0 / 30.3).
-constexpr int kClusterMaxLayers = 4;
-constexpr long long kClusterMaxWeights = 30000000;        // K N over the layers, from nine rows on
-int decode_cluster_max_layers() { return kClusterMaxLayers; }
+constexpr long long kClusterMaxWeights = 30000000;        // K N over the layers, from nine rows on and at three with ranks above 128
+int decode_cluster_max_layers() { return dcl::kMaxLayers; }
 bool decode_cluster_takes(const PackedMeta* metas, int n, int M, int y_type) {
   using namespace dcl;
-  if (n < 1 || n > kClusterMaxLayers || M < 3 || M > kRows) return false;
+  if (n < 1 || n > kMaxLayers || M < 3 || M > kRows) return false;
   long long weights = 0;
   int k_pad = 0;
   for (int i = 0; i < n; ++i) {
@@ -818,7 +816,7 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
   p.off_xq = q.off_xq; p.off_xe = q.off_xe; p.off_tpart = q.off_tpart; p.off_ring = q.off_ring;
   const bool yq = y_type == kYMXINT8;
   const Entry kernel = entry_of(metas[0].w_bits, M > 8 ? 2 : 1, yq);
-  // All clusters of a launch are resident together (some wait for the T_q of others).  With two CTAs to an SM the last few
+  // No more clusters than the device holds at a time (they wait for the T_q of others).  With two CTAs to an SM the last few
   // places are left free: 4096 x 4096, 4 rows, 14.3 us with 32 of 33 clusters and 12.0 with 28; larger launches lose more by the
   // longer ranges of columns (two of 4096 x 11008: 35.5 with 28, 30.5 with 32, 34 with 33).
   int budget = kernel.resident(CS, q.two);
@@ -830,9 +828,10 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
   // quarter costs nothing (rank 256, 4 rows: 4096 x 4096 14.4 / 14.3, 2048 x 5632 14.0 / 13.5; below rank 144 nothing changes).
   const int most = std::max(budget / 4, 1);
   bool cooperative = false;
+  constexpr long long kFewWeights = 30000000;
   long long weights = 0;
   for (int i = 0; i < n; ++i) weights += (long long)metas[i].K64 * metas[i].N;
-  if (q.two && budget >= 8) budget = weights <= 30000000 ? budget * 7 / 8 : budget / 4 * 4;
+  if (q.two && budget >= 8) budget = weights <= kFewWeights ? budget * 7 / 8 : budget / 4 * 4;
   if (budget < n) return cudaErrorInvalidConfiguration;
   // clusters per layer: each has one, the others go one by one where the time (column octets x steps of K) is longest, as long
   // as every warp of a cluster has an octet
@@ -874,7 +873,7 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
     ly.clusters = clusters[g];
     ly.tq = static_cast<uint8_t*>(scratch) + t_off;
     ly.tcount = counts + 2 * g;
-    // each warp of an owner counts its 16-blocks of T in
+    // the warps of an owner count their 16-blocks of T in
     ly.t_expect = M * m.r_blocks + (stall ? 1 : 0);
     const int formers = q.two ? std::min(clusters[g], most) : clusters[g];
     ly.t_blocks = (m.r_blocks + formers - 1) / formers;

@@ -893,7 +893,7 @@ cudaError_t launch_decode_cols_group(const lqer_call_t* calls, const PackedMeta*
 
 int decode_pre_max_calls() { return dcol::kPreMaxCalls; }
 
-// X_q and T_q of n independent decode calls (M <= 4 each, every layer fitting decode_cols_fits), one CTA per call, into
+// X_q and T_q of n independent decode calls (M <= 4 each, every layer fitting decode_cols_fits), a cluster of CTAs per call, into
 // outs[i] (decode_pre_bytes each, 256-byte aligned).
 cudaError_t launch_decode_pre(const lqer_call_t* calls, const PackedMeta* metas, uint8_t* const* outs, int n, int order,
                               int x_type, cudaStream_t s) {
