@@ -361,12 +361,11 @@ __global__ void __launch_bounds__(kCholThreads) cholesky_inverse_panels_kernel(c
       bool low = false;
 #pragma unroll
       for (int j = 0; j < kPanel; ++j) {
-        const double p = __shfl_sync(0xFFFFFFFFu, d[j], j);
-        double inv = 0.0;
-        if (p > 0.0) inv = rsqrt(p);
-        else low = true;
+        double p = __shfl_sync(0xFFFFFFFFu, d[j], j);
+        if (!(p > 0.0)) { p = __longlong_as_double(0x7FF0000000000000LL); low = true; }   // infinity: a reciprocal root of zero
+        const double inv = rsqrt(p);
         if (c == j) mine = inv;
-        d[j] = (c == j ? p : d[j]) * inv;
+        d[j] *= inv;
 #pragma unroll
         for (int i = j + 1; i < kPanel; ++i) d[i] = fma(-__shfl_sync(0xFFFFFFFFu, d[j], i), d[j], d[i]);
       }
