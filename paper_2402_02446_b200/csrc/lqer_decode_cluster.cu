@@ -825,7 +825,7 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
   // cannot leave.  At most a quarter of the places go to such clusters, so that four launches on as many streams cannot hold
   // each other up for good; where that would cost too much (one CTA to an SM: 13824 x 2048 of rank 256, 4 rows, 40.6 us instead of 21.8)
   // the launch is a cooperative one, which is placed as a whole or not yet (some 1 us more).  With two CTAs to an SM the
-  // quarter costs nothing (rank 256, 4 rows: 4096 x 4096 14.4 / 14.3, 2048 x 5632 14.0 / 13.5; below rank 144 nothing changes).
+  // quarter costs nothing (rank 256, 4 rows: 4096 x 4096 14.4 / 14.3, 2048 x 5632 14.0 / 13.5; up to rank 128 nothing changes).
   const int most = std::max(budget / 4, 1);
   bool cooperative = false;
   constexpr long long kFewWeights = 30000000;

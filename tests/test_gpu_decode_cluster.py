@@ -160,3 +160,22 @@ def test_streams_with_a_workspace_each():
             assert all(torch.equal(y, w) for y, w in zip(got, want))
     for l in layers:
         l[2].release()
+
+
+def test_replays_of_a_launch_placed_as_a_whole():
+    # long K and a high rank: one CTA to an SM and more T clusters than a quarter of the places (a cooperative launch), captured
+    spec, P, Pg = _layer(12288, 520, 256, 909)
+    x, y, ws = torch.zeros((8, spec.K), device=DEV), torch.zeros((8, spec.N), device=DEV), L.new_workspace(8, Pg)
+    L.linear(x, Pg, ws, y)
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=stream):
+        L.linear(x, Pg, ws, y, stream=torch.cuda.current_stream())
+    for rep in range(3):
+        X = gen.make_activations(spec, M=8) * np.float32(1 + rep)
+        x.copy_(_t(X))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert L.poll_status(ws) == 0
+        assert worst_ratio(y.cpu().numpy(), olqer.forward(X, P)) <= 1.0, rep
+    Pg.release()
