@@ -172,9 +172,8 @@ lqer_status_t lqer_project_lowrank(const float* X, int M, const void* packed, in
 /* The layer (Section 3.1 last display, Section 3.2 last display):
  *   Y[M,N] = X_q W_q + q(X_q A_q) B_q,  fp32 accumulation of exactly represented products.
  * One or two rows run a fused decode kernel whose CTAs own output columns.  Three to sixteen rows run one kernel in which
- * clusters of CTAs own columns and share the contraction, unless that is the slower way for the layer: up to eight rows it takes
- * every layer whose activations fit its shared memory, from nine on (and at three with ranks above 128) layers of up to
- * 3e7 weights.  What it leaves runs the decode kernel up to 4 rows, and up to 128 rows a latency-oriented
+ * clusters of CTAs own columns and share the contraction, for every layer whose activations fit its shared memory.
+ * What it leaves runs the decode kernel up to 4 rows, and up to 128 rows a latency-oriented
  * prologue and a tensor-core GEMM that streams the weights once, 128 columns of them per MMA against all tokens.
  * Larger M run the activation prologue and the tensor-core GEMM over tiles (256 rows x 256, 192 or 128 columns) of the
  * concatenated contraction [X_q | T_q] . [W_q ; B_q].
@@ -242,7 +241,7 @@ lqer_status_t lqer_linear_static(const float* X, int M, const void* packed, floa
  * fit the largest of them.  Independent means that no call reads what another call of the
  * same batch writes; the library uses that, with the path left at 0, to share launches:
  *  - a run of two to four calls with one M from 3 to 16 (one set of formats) that the cluster kernel takes (see
- *    lqer_linear; the line of 3e7 weights is drawn over all of them) runs as ONE launch of it;
+ *    lqer_linear) runs as ONE launch of it;
  *  - otherwise up to 16 consecutive calls with one M <= 4 (any shapes with N >= 32, one set of formats)
  *    run as ONE launch of the decode kernel that divides the SMs among them; consecutive such
  *    launches do not wait for one another, and a stretch of more than one launch first has the

@@ -281,7 +281,7 @@ static lqer_status_t run_linear(const void* X, int M, const void* packed, void* 
   void* xcat = wsb + align_up(persist_bytes(m), 256);
   cudaError_t err;
   if (small) {
-    if (path == 0 && !project_only && decode_cluster_takes(&m, 1, M, io.y_type)) {
+    if (path == 0 && !project_only && decode_cluster_takes(&m, 1, M)) {
       const lqer_call_t one = {static_cast<const float*>(X), M, packed, static_cast<float*>(Y)};
       err = launch_decode_cluster(&one, &m, 1, xcat, reinterpret_cast<int*>(wsb + kStatusBytes), dst, io.x_type, io.y_type, s);
     } else if (path != 5 && path != 7 && !project_only && decode_cols_fits(m, M)) {
@@ -813,7 +813,7 @@ lqer_status_t lqer_linear(const float* X, int M, const void* packed, float* Y, v
 
 // The calls from calls[first] on that go out as one launch of the cluster kernel: a run of two to decode_cluster_max_layers()
 // neighbours with one M and one set of formats (a longer run shares the launches of the other kernels), or 0.
-static int cluster_run(const lqer_call_t* calls, int first, int n_calls, size_t workspace_bytes, int y_type, PackedMeta* metas) {
+static int cluster_run(const lqer_call_t* calls, int first, int n_calls, size_t workspace_bytes, PackedMeta* metas) {
   const int M = calls[first].M;
   size_t need = align_up(kPersistMaxBytes, 256);
   int n = 0;
@@ -824,7 +824,7 @@ static int cluster_run(const lqer_call_t* calls, int first, int n_calls, size_t 
     metas[n] = m;
     need += decode_cluster_scratch_bytes(m);
   }
-  return n > 1 && need <= workspace_bytes && decode_cluster_takes(metas, n, M, y_type) ? n : 0;
+  return n > 1 && need <= workspace_bytes && decode_cluster_takes(metas, n, M) ? n : 0;
 }
 // The batched entry points: independent calls share launches where the path is left at 0.
 static lqer_status_t linear_batched(const lqer_call_t* calls, int n_calls, void* workspace, size_t workspace_bytes,
@@ -868,7 +868,7 @@ static lqer_status_t linear_batched(const lqer_call_t* calls, int n_calls, void*
     // Inside a stretch whose activations lie ready behind the head, the calls that are left read them there: no kernel that
     // has its own scratch in that place may run before the stretch ends.
     const bool held = i < pre_end && !pre_off.empty();
-    const int clustered = may_group && !chain_open && !held ? cluster_run(calls, i, n_calls, workspace_bytes, io.y_type, metas) : 0;
+    const int clustered = may_group && !chain_open && !held ? cluster_run(calls, i, n_calls, workspace_bytes, metas) : 0;
     if (clustered > 1) {
       n = clustered;
       cluster_group = true;

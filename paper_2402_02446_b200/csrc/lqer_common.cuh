@@ -588,7 +588,7 @@ inline bool w_offsets_fit(const PackedMeta& m) { return m.off_b - m.off_w <= 0xF
 // and one set of formats.  scratch: decode_cluster_scratch_bytes per layer; counts: two zeroed counters per layer, zero again
 // when the call ends.
 int decode_cluster_max_layers();
-bool decode_cluster_takes(const PackedMeta* metas, int n, int M, int y_type);
+bool decode_cluster_takes(const PackedMeta* metas, int n, int M);
 inline size_t decode_cluster_scratch_bytes(const PackedMeta& m) { return (size_t)(m.k_pad + 127) / 128 * 4096; }
 cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* metas, int n, void* scratch, int* counts, DeviceStatus* st,
                                   int x_type, int y_type, cudaStream_t s);

@@ -1,24 +1,31 @@
 // The layer for M <= 16 tokens in one launch (paper Section 3.1 / 3.2: Y = X_q W_q + q(X_q A_q) B_q; Section 2.1: few
 // tokens per step make it memory bound on its weights).
 //
-// A cluster of CS CTAs (8 where the contraction has 16 slabs of 64) owns a range of output columns; its CTAs share the
-// contraction: CTA q takes the slabs [q k_slabs / CS, (q + 1) k_slabs / CS).  So a CTA quantises only its part of X.  What the
-// parts have to exchange:
-//   - Y: the warps of a CTA own column octets, a round of them at a time, over the CTA's slabs.  Warp w's sums of a round go
-//     to CTA w mod CS (st.async, counted in bytes on that CTA's mbarrier), which adds them in CTA order and writes Y once.
+// A cluster of CS CTAs owns a range of weight tiles (128 columns); its CTAs share the contraction: CTA q takes the slabs
+// [q k_slabs / CS, (q + 1) k_slabs / CS).  So a CTA quantises only its part of X.  What the parts have to exchange:
+//   - Y: consumer warps multiply 32 columns of a tile each, every third stage, and send their sums to the CTAs that own the columns
+//     (st.async, counted in bytes on that CTA's mbarrier), whose epilogue warps add them in order, add the rank term and write Y once,
+//     while the consumers are in the next tile.
 //   - T = X_q A_q: the first clusters of a layer form it, one or a few rank blocks each.  Each CTA multiplies its part (int8
 //     mma.sync per 16-block, exact, scaled and summed in fp64) and stores its partial sums into the CTA of its cluster that owns
-//     the row; the owner adds them in CTA order, re-quantises along the rank, writes T_q to scratch in global memory and counts its
-//     blocks in.  Every cluster of the layer waits for the count (bounded) before its first rank term, the last thing of its
-//     first round; the last warp to have read T_q zeroes the counters for the next call.
+//     the row; the owner adds them in order, re-quantises along the rank, writes T_q to scratch in global memory and counts its
+//     blocks in.  Every epilogue warp waits for the count (bounded) before its first rank term; the layer's last warp to
+//     have read T_q zeroes the counters for the next call.  Where a cluster has few weights to multiply, it forms all of T itself, and the
+//     owners of the rows store T_q into its CTAs' shared memory.
 // So a cluster waits for other clusters of its launch.  The launch has no more of them than the device holds at a time, those
 // that form T come first, and launch_decode_cluster says what keeps launches on several streams from holding each other up.
 //
-// The weights take the register-operand form (lqer_mma_frag.cuh): a lane loads the 16 bytes which the packed tile stores
-// for one column and block pair, here through its own slots of a ring in shared memory (cp.async; a lane reads back only
-// what it copied itself, so the ring needs no barrier), converts them to bf16 in registers and feeds them to
-// mma.sync.m16n8k16.  The ring is filled before griddepcontrol.wait, for weights depend on no earlier kernel.
+// The packed weights come by bulk copies, a stage (two slabs of a tile, 9 KB) at a time: a producer warp keeps a ring of stages full, from
+// before griddepcontrol.wait on, for weights depend on no earlier kernel.  Twelve consumer warps read a stage's mantissas with ldmatrix (the
+// 16 bytes that the tile stores for a column and block pair are a row of it, so every lane of a group of four gets one word without
+// bank conflicts), convert them to bf16 in registers and feed them to mma.sync.m16n8k16, weights on the 16-row side.
+// What bounds it: 540 cycles a stage up to eight rows, some 650 beyond (the ALU pipe's shifts and masks, two cycles each, and the MMAs,
+// 8.6 each), i.e. 4.6 and 3.8 TB/s; and some 7 us around the stages, of which the chain X -> X_q -> T -> T_q -> rank term is 4.5.
+// A CTA has an SM to itself: with two launches resident side by side, each with half of an SM, clusters came to lie two to an SM on some
+// and on others not at all; a run of (tile, step) to each CTA of 148 without clusters, the sums exchanged through global memory, took
+// 94 us where this takes 64 (decoder layer of 4096 / 11008, 4 rows); copies of 0.5 to 2 KB, padded against bank conflicts, 118.
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 
 #include "lqer_gemm_small.cuh"
@@ -30,11 +37,17 @@ using namespace mf;
 using sg::bf16_rn;
 using tc::smem_u32;
 
-constexpr int kWarps = 8;
-constexpr int kThreads = kWarps * 32;
+constexpr int kColumnWarps = 4, kPhases = 3;                       // consumer warps: 32 columns of a tile each, and every third stage
+constexpr int kConsumers = kColumnWarps * kPhases, kEpilogue = 4;  // warps; one more is the producer
+constexpr int kWorkerWarps = kConsumers + kEpilogue, kWorkers = kWorkerWarps * 32, kThreads = kWorkers + 32;
 constexpr int kMaxLayers = 4;                // layers of a launch, at most
-constexpr int kOcts = 4;                    // column octets a warp owns in a round, at most
+constexpr int kUnit = 16;                    // columns of a unit, one side of an MMA
+constexpr int kUnits = kTileN / kUnit;       // units of a tile
 constexpr int kRows = 16;
+constexpr int kMaxSlots = 20;                // ring slots, at most
+constexpr int kRed = 3;                      // tiles whose sums may be under way
+constexpr int kSmemMax = 222 * 1024;
+constexpr int kLocalStages = 10, kLocalBlocks = 8;   // stages of a cluster that forms all of T itself, and blocks of T (of eight rows) to a warp, at most
 
 struct Layer {
   const void* X;
@@ -43,11 +56,12 @@ struct Layer {
   const uint8_t* bsec;
   const uint8_t* asec;
   size_t y_extent, w_extent;
-  int K, N, k_pad, k_slabs, r_blocks;
+  int K, N, k_pad, k_slabs, r_blocks, tiles;
   int cluster_begin, clusters;
-  uint8_t* tq;                              // T_q on its way between clusters: eight planes (the layout of the activations)
+  uint8_t* tq;                              // T_q on its way between clusters: eight planes (token_offset)
   int* tcount;                              // arrivals, departures: zero between calls
   int t_blocks;                             // rank blocks of T that each of the layer's first clusters forms
+  int t_clusters, t_tiles;                  // ... and how many those are, if they get fewer tiles than the others: so many each
   int t_expect;                             // arrivals that make T_q whole (one more under the test hook)
 };
 struct Params {
@@ -56,10 +70,11 @@ struct Params {
   DeviceStatus* status;
   int x_type, y_type;
   int a_bits, lr_bits, exp_min, exp_max;
-  int slabs_max;                            // slabs of a CTA, rounded up to even: the extent of the activation planes
-  int off_red[2], off_xq, off_xe, off_tpart, off_ring;   // offsets in shared memory (the planes of X_q come first)
+  int steps_max;                            // steps of a CTA, at most: the extent of the activation planes
+  int slots;                                // ring slots
+  int off_red, red_bytes, off_xq, off_xe, off_tpart, off_trecv, off_tq, off_ring;   // offsets in shared memory (the planes of X_q come first)
   long long wait_limit;
-  int stall;                                // test hook: the sums of the first round wait for bytes that never come (see also t_expect)
+  int stall;                                // test hook: the sums of the first tile wait for bytes that never come (see also t_expect)
 };
 
 __device__ __forceinline__ uint32_t cta_rank() {
@@ -80,6 +95,9 @@ __device__ __forceinline__ void st_async(uint32_t addr, double a, double b, uint
 }
 __device__ __forceinline__ void st_async(uint32_t addr, float a, float b, uint32_t bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async(uint32_t addr, uint32_t a, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(a), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -112,16 +130,26 @@ __device__ __forceinline__ bool wait_count(const int* count, int expect, volatil
     __nanosleep(64);
   }
 }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void cp16(uint32_t dst, const void* src) { asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory"); }
-__device__ __forceinline__ void cp8(uint32_t dst, const void* src) { asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory"); }
-__device__ __forceinline__ void cp4(uint32_t dst, const void* src) { asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory"); }
+template <bool kBackoff = false>
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile tc::WaitState* ws) {
+  return __all_sync(0xFFFFFFFFu, tc::mbar_wait<kBackoff>(bar, parity, ws)) != 0;
+}
+__device__ __forceinline__ void worker_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory"); }
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void ldmatrix2(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
+}
 
+// A stage in shared memory: two slabs of a packed weight tile, as they lie in the packed buffer.
 template <int WB>
-__host__ __device__ constexpr int stage_bytes() { return kOcts * 32 * (WB == 4 ? 16 : 8) + kOcts * 32 * 4; }
-
-// Words from column to column of a warp's sums in the buffer of the CTA that adds them: tokens, two more against bank conflicts.
+struct Stage {
+  static constexpr int kMant = WB == 4 ? kWTileNibbleBytes : 2048;   // bytes of a tile's mantissas
+  static constexpr int kTile = kMant + kTileN * 4;                   // and of the whole tile
+  static constexpr int kBytes = 2 * kTile;
+};
+// Words from column to column of a unit on its way to Y: tokens, two more against bank conflicts.
 __host__ __device__ constexpr int token_stride(int mt) { return 8 * mt + 2; }
 
 // Four consecutive columns of a row of Y (a lane of a quad of lanes that hold a 16-block of the row), all lanes calling.
@@ -178,9 +206,30 @@ __device__ __forceinline__ void load_x_block(float (&v)[16], const void* X, int 
   }
 }
 
-// Activations as the MMA's narrow operand (n = 8 tokens to a tile, MT tiles): eight planes of [slab][16 positions][MT pairs of
-// words]; plane i of a lane's 32 K holds its K 4 i .. 4 i + 3.  Byte offset of (token, slab, column c of the slab, a multiple of 4)
-// within its plane; the second pair of K lies 4 MT bytes on.
+// Activations as the MMA's narrow operand (n = 8 tokens to a tile, MT tiles).  MMA i of a step of 128 K takes four K from each lane t, in the
+// order in which the lanes get the weights: word t of every block pair (4-bit mantissas: K 32 (i >> 1) + 8 t + 4 (i & 1) of the step),
+// or word t of every slab (2-bit ones: K 64 (i >> 2) + 16 t + 4 (i & 3)).  Four planes, of the MMAs 2 m and 2 m + 1 of every step: [step][MMA where MT
+// == 2][token, lane t][16 bytes], the 16 bytes being both MMAs' words of one tile, or one MMA's of two.
+// The sixteen K of a block (f0, f1: eight pairs of bf16 values) to their places.
+template <int WB, int MT>
+__device__ __forceinline__ void store_block(uint8_t* planes, uint32_t plane, int row, int block, const uint4& f0, const uint4& f1) {
+  const int b = block & 3, slab = block >> 2;
+  uint8_t* at = planes + (uint32_t)((slab & 1) * 2 + (WB == 4 ? b >> 1 : 0)) * plane + (uint32_t)((slab >> 1) * (512 * MT) + (row >> 3) * 4) +
+                ((row & 7) * 4 + (WB == 4 ? (b & 1) * 2 : b)) * 16;
+  const uint32_t next = WB == 4 ? 16u : plane;               // the block's second half: the next lane's, or the next pair of MMAs
+  if (MT == 1) {
+    *reinterpret_cast<uint4*>(at) = f0;
+    *reinterpret_cast<uint4*>(at + next) = f1;
+  } else {
+    const uint32_t w[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) *reinterpret_cast<uint32_t*>(at + (k >> 1) * next + (k & 1) * 512 + h * 8) = w[2 * k + h];
+  }
+}
+// T_q: eight planes of [rank slab of 64][16 positions][MT pairs of words]; plane i of a lane's 32 ranks holds its ranks 4 i .. 4 i + 3.
+// Byte offset of (token, slab, rank c of the slab, a multiple of 4) within its plane.
 template <int MT>
 __device__ __forceinline__ uint32_t token_offset(int row, int slab, int c) {
   return (uint32_t)(slab * (128 * MT) + (2 * (row & 7) + (c >> 5)) * (8 * MT) + (row >> 3) * 4);
@@ -189,23 +238,19 @@ __device__ __forceinline__ void mma_w(float (&d)[4], uint32_t a0, uint32_t a1, u
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// 128 K of NP pairs of column octets: the octets of a pair are rows g and g + 8 of the MMA.  word(o, m): eight converted weights.
-// RANK: the activations (T_q) come from global memory, and only the first `blocks` 16-blocks of the lane's two exist.
-// The MMAs of a step add up in chains of four (MT == 1; eight otherwise, for want of registers), and the chains' sums are added to
-// acc by fp32 additions: the accumulators of mma.sync cut off what does not fit, and one chain over a CTA's whole part of K was up to
-// 14 times as far off as the kernels that took these calls before (2-norm against 64 bits for 13824 K of one sign, block
-// exponents over a dozen binades: 4 rows 8.5e-7, column-owner kernel 6.2e-8, now 5.1e-8; 16 rows 8.5e-7, tensor-memory GEMM 8.9e-8,
-// now 5.0e-8).  Chains of eight for MT == 1 are at 1.0 to 1.7 times the column-owner kernel where the signs are mixed, of four at
-// 0.8 to 1.2.  us a call with one chain / these: 4096 x 4096, 4 rows 11.4 / 11.5, 16 rows 15.4 / 15.4.  The one or two rank steps of MT == 2
-// continue acc itself (with chains of their own, 16 rows of rank 256 took 24.6 us instead of 22.0: spilled registers).
-template <int MT, int NP, bool RANK = false, class Word>
-__device__ __forceinline__ void multiply_step(float (&acc)[kOcts / 2][MT][4], const uint8_t* x, uint32_t plane, Word&& word, int blocks = 2) {
-  constexpr bool kChains = !(RANK && MT == 2);
+// 128 K of NP units: columns g and g + 8 of a unit are rows g and g + 8 of the MMA.  word(o, m): eight converted weights of column octet o,
+// for the MMAs 2 m and 2 m + 1; load(m, b0, b1): those MMAs' activations (two words for each tile of tokens).
+// The MMAs of a step add up in chains of four (MT == 1; eight otherwise), and the chains' sums are added to acc by fp32 additions: the
+// accumulators of mma.sync cut off what does not fit, and one chain over 1700 K was up to 14 times as far off as kernels that
+// add by rounded fp32 operations (2-norm against 64 bits for 13824 K of one sign, block exponents over a dozen binades: 4 rows 8.5e-7,
+// column-owner kernel 6.2e-8, with these chains 5.1e-8; 16 rows 8.5e-7, tensor-memory GEMM 8.9e-8, with these 5.0e-8).
+template <int MT, int NP, class Word, class Load>
+__device__ __forceinline__ void multiply_step(float (&acc)[NP][MT][4], Word&& word, Load&& load) {
   constexpr int kChain = MT == 1 ? 2 : 4;            // m per chain
   float d[NP][MT][4];
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
-    if (kChains && m % kChain == 0) {
+    if (m % kChain == 0) {
 #pragma unroll
       for (int p = 0; p < NP; ++p)
 #pragma unroll
@@ -213,32 +258,20 @@ __device__ __forceinline__ void multiply_step(float (&acc)[kOcts / 2][MT][4], co
 #pragma unroll
           for (int q = 0; q < 4; ++q) d[p][i][q] = 0.f;
     }
+    uint32_t b[2][2 * MT];
+    load(m, b[0], b[1]);
     uint4 w[2 * NP];
 #pragma unroll
     for (int o = 0; o < 2 * NP; ++o) w[o] = word(o, m);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const uint8_t* at = x + (2 * m + h) * plane;
-      uint32_t b[2 * MT];
-      if (MT == 1) {
-        uint2 v = make_uint2(0u, 0u);
-        if (!RANK) v = *reinterpret_cast<const uint2*>(at);
-        else if ((m >> 1) < blocks) v = __ldcg(reinterpret_cast<const uint2*>(at));
-        b[0] = v.x; b[1] = v.y;
-      } else {
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (!RANK) v = *reinterpret_cast<const uint4*>(at);
-        else if ((m >> 1) < blocks) v = __ldcg(reinterpret_cast<const uint4*>(at));
-        b[0] = v.x; b[2 * MT - 2] = v.y; b[1] = v.z; b[2 * MT - 1] = v.w;
-      }
+    for (int p = 0; p < NP; ++p)
 #pragma unroll
-      for (int p = 0; p < NP; ++p)
+      for (int i = 0; i < MT; ++i) mma_w(d[p][i], w[2 * p].x, w[2 * p + 1].x, w[2 * p].y, w[2 * p + 1].y, b[0][2 * i], b[0][2 * i + 1]);
 #pragma unroll
-        for (int i = 0; i < MT; ++i)
-          mma_w(kChains ? d[p][i] : acc[p][i], h ? w[2 * p].z : w[2 * p].x, h ? w[2 * p + 1].z : w[2 * p + 1].x, h ? w[2 * p].w : w[2 * p].y,
-                h ? w[2 * p + 1].w : w[2 * p + 1].y, b[2 * i], b[2 * i + 1]);
-    }
-    if (kChains && m % kChain == kChain - 1) {
+    for (int p = 0; p < NP; ++p)
+#pragma unroll
+      for (int i = 0; i < MT; ++i) mma_w(d[p][i], w[2 * p].z, w[2 * p + 1].z, w[2 * p].w, w[2 * p + 1].w, b[1][2 * i], b[1][2 * i + 1]);
+    if (m % kChain == kChain - 1) {
 #pragma unroll
       for (int p = 0; p < NP; ++p)
 #pragma unroll
@@ -248,20 +281,27 @@ __device__ __forceinline__ void multiply_step(float (&acc)[kOcts / 2][MT][4], co
     }
   }
 }
+// Eight signed bytes as bf16 values times sc, exact, by the integers' bits (conversion instructions run at an eighth of the rate): byte + 128 is the low
+// byte of the float 1.5 * 2^23 + 128 + byte.
+__device__ __forceinline__ uint4 convert_i8x8(uint32_t w0, uint32_t w1, float sc) {
+  const float back = -12583040.0f * sc;
+  auto value = [&](uint32_t u, uint32_t select) { return fmaf(__uint_as_float(__byte_perm(u, 0x4B400000u, select)), sc, back); };
+  auto pair = [&](uint32_t u, uint32_t lo, uint32_t hi) { return __byte_perm(__float_as_uint(value(u, lo)), __float_as_uint(value(u, hi)), 0x7632); };
+  w0 ^= 0x80808080u;
+  w1 ^= 0x80808080u;
+  return make_uint4(pair(w0, 0x7640, 0x7641), pair(w0, 0x7642, 0x7643), pair(w1, 0x7640, 0x7641), pair(w1, 0x7642, 0x7643));
+}
 // int -> fp64 by the integer's bits (2^52 + 2^31 + v), where the conversion instruction runs at a sixteenth of the rate.
 __device__ __forceinline__ double int_to_double(int v) { return __hiloint2double(0x43300000, v ^ 0x80000000) - 4503601774854144.0; }
 
-// WB: mantissa bits of W_q (4 or 2).  MT: tiles of eight tokens (1 or 2).  YQ: Y is MXINT8 (a warp then owns whole 16-column
-// blocks).  D: ring slots per warp.
-template <int WB, int MT, bool YQ, int D>
-__global__ void __launch_bounds__(kThreads, 2) decode_cluster_kernel(const __grid_constant__ Params p, int CS) {
-  constexpr int kTile = WB == 4 ? kWTileBytes : 2048 + kTileN * 4;   // bytes of a packed weight tile
-  constexpr int kMant = WB == 4 ? kWTileNibbleBytes : 2048;          // of which mantissas
-  constexpr int kPiece = WB == 4 ? 16 : 8;                           // a lane's mantissas in one octet of a step
-  constexpr int kStage = stage_bytes<WB>();
+// WB: mantissa bits of W_q (4 or 2).  MT: tiles of eight tokens (1 or 2).  LOCAL: every cluster forms all of T for itself.
+template <int WB, int MT, bool LOCAL>
+__global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __grid_constant__ Params p, int CS) {
+  using St = Stage<WB>;
+  constexpr int kTile = St::kTile, kMant = St::kMant;
   constexpr int TS = token_stride(MT);
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ __align__(8) uint64_t s_bars[6];
+  __shared__ __align__(8) uint64_t s_bars[3 + 2 * kRed + 2 * kMaxSlots];
   __shared__ tc::WaitState s_ws;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -273,136 +313,135 @@ __global__ void __launch_bounds__(kThreads, 2) decode_cluster_kernel(const __gri
   const Layer& ly = p.L[layer];
   const int M = p.M, K = ly.K, k_pad = ly.k_pad;
   const int cl = cluster - ly.cluster_begin;
-  constexpr int kUnit = YQ ? 2 : 1;                                  // octets that stay together
-  const int n_units = ly.N / (8 * kUnit);
-  const int oc_lo = kUnit * (int)((long long)cl * n_units / ly.clusters), oc_hi = kUnit * (int)((long long)(cl + 1) * n_units / ly.clusters);
-  const int n_oct = oc_hi - oc_lo, rounds = (n_oct + kWarps * kOcts - 1) / (kWarps * kOcts);
-  // octets of warp w in round r: [first, first + count); all rounds but the last are full
-  auto octets = [&](int r, int w, int& count) {
-    const int left = min(n_oct - r * (kWarps * kOcts), kWarps * kOcts) / kUnit;
-    const int a = w * left / kWarps, b = (w + 1) * left / kWarps;
-    count = kUnit * (b - a);
-    return oc_lo + r * (kWarps * kOcts) + kUnit * a;
-  };
+  // this cluster's tiles: t_tiles for each of those that form T, equal shares of the rest for the others
+  const int f_all = ly.t_clusters * ly.t_tiles, others = ly.clusters - ly.t_clusters, rest = ly.tiles - f_all, nth = cl - ly.t_clusters;
+  const int tile_lo = nth < 0 ? cl * ly.t_tiles : f_all + (int)((uint32_t)nth * (uint32_t)rest / (uint32_t)others);
+  const int chunks = nth < 0 ? ly.t_tiles : f_all + (int)((uint32_t)(nth + 1) * (uint32_t)rest / (uint32_t)others) - tile_lo;
   const int s_lo = rank * ly.k_slabs / CS, s_hi = (rank + 1) * ly.k_slabs / CS, n_slabs = s_hi - s_lo;
-  const int ksteps = (n_slabs + 1) / 2;                              // steps of two slabs (128 K)
-  const uint32_t plane = (uint32_t)p.slabs_max * (128u * MT);
+  const int steps = (n_slabs + 1) / 2;                               // of two slabs (128 K)
+  const uint32_t plane = (uint32_t)p.steps_max * (512u * MT);
   const uint32_t sm = smem_u32(smem);
   const uint32_t bar0 = smem_u32(s_bars);
   const uint32_t t_full = bar0, t_seen = bar0 + 8;
-  auto red_full = [&](int b) { return bar0 + 16 + 8u * b; };
-  auto red_free = [&](int b) { return bar0 + 32 + 8u * b; };
-  const int slots_w = kWarps / CS;                                   // warps of a CTA whose sums go to the same CTA
+  const uint32_t t_ready = bar0 + 16;
+  auto red_full = [&](int b) { return bar0 + 24 + 8u * b; };
+  auto red_free = [&](int b) { return bar0 + 24 + 8u * (kRed + b); };
+  auto full = [&](int s) { return bar0 + 24 + 8u * (2 * kRed + s); };
+  auto empty = [&](int s) { return bar0 + 24 + 8u * (2 * kRed + kMaxSlots + s); };
+  // unit j of a tile is CTA j mod CS's (columns beyond N are multiplied like the others: a packed tile has all of them)
+  const int n_own = kUnits / CS;
+  const uint32_t chunk_bytes = (uint32_t)(n_own * kUnit * 8 * ((M + 1) / 2) * CS * kPhases);
   // This cluster's share of T: rank blocks [rb_lo, rb_hi), i.e. NT tiles of 8 columns; where there are fewer tiles than warps,
   // WPN warps share one and split its blocks of K.
-  const int rb_lo = min(cl * ly.t_blocks, ly.r_blocks), rb_hi = min(rb_lo + ly.t_blocks, ly.r_blocks);
-  const int t_cols = 16 * (rb_hi - rb_lo), NT = t_cols / 8, WPN = NT == 0 || NT >= kWarps ? 1 : kWarps / NT;
-  const int RP = kRows / CS;                                         // rows whose T a CTA owns
+  const int rb_lo = LOCAL ? 0 : min(cl * ly.t_blocks, ly.r_blocks), rb_hi = min(rb_lo + ly.t_blocks, ly.r_blocks);
+  const int t_cols = 16 * (rb_hi - rb_lo), NT = t_cols / 8, WPN = NT == 0 || NT >= kWorkerWarps ? 1 : kWorkerWarps / NT;
+  const int RP = 8 * MT / CS;                                        // rows whose T a CTA owns
   const int own_rows = max(0, min(M - rank * RP, RP));
   const uint32_t rplane = (uint32_t)((k_pad + 127) / 128) * (256u * MT);   // a plane of T_q: rank slabs, an even number of them
 
-  // bytes of round r that come to this CTA
-  auto round_bytes = [&](int r) {
-    int total = 0;
-    for (int s = 0; s < slots_w; ++s) {
-      int c;
-      octets(r, rank + s * CS, c);
-      total += c;
+  if (warp == kWorkerWarps) {
+    // ------------------------------------------------------------------ producer
+    // (the one slab of an odd last step is taken twice: its second half meets activations that are zeros)
+    const int x_hi = chunks * steps;
+    auto fill = [&](int x, int slot) -> bool {
+      const int tile = x / steps, slab = s_lo + 2 * (x - tile * steps);
+      const size_t src = ((size_t)(tile_lo + tile) * ly.k_slabs + slab) * kTile;
+      const uint32_t dst = sm + p.off_ring + slot * St::kBytes;
+      const uint32_t bytes = slab + 1 < s_hi ? 2 * kTile : kTile;
+      if (!LQER_IN_BOUNDS(p.status, src, bytes, ly.w_extent, 733)) return false;
+      tc::mbar_expect_tx(full(slot), 2 * kTile);
+      tc::bulk_load(dst, ly.wsec + src, bytes, full(slot));
+      if (bytes == kTile) tc::bulk_load(dst + kTile, ly.wsec + src, bytes, full(slot));
+      return true;
+    };
+    int x = 0;
+    bool go = true;
+    if (lane == 0) {
+      tc::mbar_init(t_full, 1);
+      tc::mbar_init(t_seen, CS * kEpilogue);
+      tc::mbar_init(t_ready, 1);
+      for (int i = 0; i < kRed; ++i) { tc::mbar_init(red_full(i), 1); tc::mbar_init(red_free(i), CS * kEpilogue); }
+      for (int i = 0; i < p.slots; ++i) { tc::mbar_init(full(i), 1); tc::mbar_init(empty(i), kColumnWarps); }
+      s_ws.abort = 0;
+      s_ws.limit = p.wait_limit;
+      tc::fence_barrier_init();
+      tc::fence_proxy_async_smem();
+      if (NT > 0 && own_rows > 0) tc::mbar_expect_tx(t_full, (uint32_t)(own_rows * t_cols * 8 * CS));
+      if (LOCAL) tc::mbar_expect_tx(t_ready, (uint32_t)(M * k_pad * 2));
+      for (int i = 0; i < min(chunks, kRed); ++i) tc::mbar_expect_tx(red_full(i), chunk_bytes + (p.stall && i == 0 ? 16u : 0u));
     }
-    return (uint32_t)(total * 64 * ((M + 1) / 2) * CS);
-  };
-  if (tid == 0) {
-    tc::mbar_init(t_full, 1);
-    tc::mbar_init(t_seen, CS * kWarps);
-    for (int i = 0; i < 2; ++i) { tc::mbar_init(red_full(i), 1); tc::mbar_init(red_free(i), CS * kWarps); }
-    s_ws.abort = 0;
-    s_ws.limit = p.wait_limit;
-    tc::fence_barrier_init();
-    if (NT > 0 && own_rows > 0) tc::mbar_expect_tx(t_full, (uint32_t)(own_rows * t_cols * 8 * CS * WPN));
-    // (a round that brings nothing is not armed: its phase would pass before every warp has seen the one before)
-    if (round_bytes(0) > 0) tc::mbar_expect_tx(red_full(0), round_bytes(0) + (p.stall ? 16u : 0u));
-    if (rounds > 1 && round_bytes(1) > 0) tc::mbar_expect_tx(red_full(1), round_bytes(1));
+    __syncwarp();
+    tc::pdl_launch_dependents();
+    cluster_arrive();
+    // (a copy takes its issuing thread some 50 ns: the others do not wait for all of the ring)
+    const int first = min(min(p.slots, x_hi), kPhases);
+    if (lane == 0)
+      for (; x < first && go; ++x) go = fill(x, x);
+    __syncwarp();
+    cluster_wait();
+    __syncthreads();
+    if (lane == 0) {
+      for (; x < p.slots && x < x_hi && go; ++x) go = fill(x, x);
+      for (int slot = 0, ph = 0; x < x_hi && go; ++x) {
+        if (!tc::mbar_wait<true>(empty(slot), ph, &s_ws)) break;
+        go = fill(x, slot);
+        if (++slot == p.slots) { slot = 0; ph ^= 1; }
+      }
+      if (!go) s_ws.abort = 1;
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    if (s_ws.abort != 0) {                             // given up: copies in flight land before the CTA's shared memory goes
+      const long long t0 = clock64();
+      while (clock64() - t0 < 400000) { }
+    }
+    return;
   }
   tc::pdl_launch_dependents();
   cluster_arrive();
 
-  // ---- weights: this lane's pieces of the steps to come, through its own slots of the ring
-  const uint32_t ring = sm + p.off_ring + warp * (D * kStage);
-  int pf_round = 0, pf_step = 0, pf_count = 0, pf_slot = 0;
-  uint32_t pf_w[kOcts], pf_e[kOcts];
-  auto pf_columns = [&]() {
-    const int first = octets(pf_round, warp, pf_count);
-#pragma unroll
-    for (int o = 0; o < kOcts; ++o) {
-      const int oc = first + o;
-      const uint32_t tile = (uint32_t)(oc >> 4) * (uint32_t)ly.k_slabs * (uint32_t)kTile, nl = (uint32_t)((oc & 15) * 8 + g);
-      pf_w[o] = tile + nl * 16u + (WB == 4 ? (uint32_t)(t & 1) * 2048u : (uint32_t)(t & 1) * 8u);
-      pf_e[o] = tile + (uint32_t)kMant + nl * 4u;
-    }
-  };
-  auto prefetch_step = [&]() {
-    if (pf_round < rounds) {
-      // the second slab of an odd last step: the lane takes the last one again, its activations are zeros there
-      const uint32_t slab = (uint32_t)min(s_lo + 2 * pf_step + (t >> 1), s_hi - 1) * (uint32_t)kTile;
-      const uint32_t dst = ring + pf_slot * kStage;
-#pragma unroll
-      for (int o = 0; o < kOcts; ++o)
-        if (o < pf_count && LQER_IN_BOUNDS(p.status, pf_e[o] + slab, 4, ly.w_extent, 733)) {
-          if (WB == 4) cp16(dst + (o * 32 + lane) * kPiece, ly.wsec + (pf_w[o] + slab));
-          else cp8(dst + (o * 32 + lane) * kPiece, ly.wsec + (pf_w[o] + slab));
-          cp4(dst + kOcts * 32 * kPiece + (o * 32 + lane) * 4, ly.wsec + (pf_e[o] + slab));
-        }
-      if (++pf_step == ksteps) {
-        pf_step = 0;
-        if (++pf_round < rounds) pf_columns();
-      }
-    }
-    if (++pf_slot == D) pf_slot = 0;
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  pf_columns();
-#pragma unroll 1
-  for (int i = 0; i < D; ++i) prefetch_step();
-
-  // ---- A_q of this CTA's blocks and this cluster's ranks: the first words into registers
+  // ---- A_q of this CTA's blocks and this cluster's ranks: the first words into registers, the others towards L2
   const int kblocks = K / 16, kb0 = s_lo * 4, nreal = min(n_slabs * 4, kblocks - kb0);
-  const int nt_first = NT >= kWarps ? warp : NT > 0 ? warp % NT : 0, sub = NT >= kWarps || NT == 0 ? 0 : warp / NT;
-  const bool t_active = NT > 0 && (NT >= kWarps || warp < NT * WPN);
-  constexpr int UB = 16;
-  uint32_t bw[UB], ew[UB];
-  auto load_a = [&](int bq, int nt) {
+  const int nt_first = NT >= kWorkerWarps ? warp : NT > 0 ? warp % NT : 0, sub = NT >= kWorkerWarps || NT == 0 ? 0 : warp / NT;
+  const bool t_active = NT > 0 && (NT >= kWorkerWarps || warp < NT * WPN);
+  constexpr int UB = 8;
+  uint32_t aw[2][UB], ae[2][UB];
+  auto load_a = [&](int bq, int nt, uint32_t (&w)[UB], uint32_t (&e)[UB]) {
     const uint8_t* am = ly.asec + ((size_t)(kb0 + bq) * k_pad + rb_lo * 16 + nt * 8 + g) * 16 + t * 4;
-    const uint8_t* ae = ly.asec + (size_t)kblocks * k_pad * 16 + (size_t)(kb0 + bq) * k_pad + rb_lo * 16 + nt * 8 + t * 2;
+    const uint8_t* ax = ly.asec + (size_t)kblocks * k_pad * 16 + (size_t)(kb0 + bq) * k_pad + rb_lo * 16 + nt * 8 + t * 2;
 #pragma unroll
     for (int u = 0; u < UB; ++u) {
-      bw[u] = 0u; ew[u] = 0u;
+      w[u] = 0u; e[u] = 0u;
       if (bq + u * WPN < nreal) {
-        bw[u] = __ldg(reinterpret_cast<const uint32_t*>(am));
-        ew[u] = (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(ae));
+        w[u] = __ldg(reinterpret_cast<const uint32_t*>(am));
+        e[u] = (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(ax));
       }
       am += (size_t)WPN * k_pad * 16;
-      ae += (size_t)WPN * k_pad;
+      ax += (size_t)WPN * k_pad;
     }
   };
-  if (t_active) load_a(sub, nt_first);
-  // B_q of the octets whose rank term falls to this CTA, towards L2
-  if (k_pad > 0 && warp % CS == rank)
-    for (int r = 0; r < rounds; ++r) {
-      int c;
-      const int first = octets(r, warp, c);
-      for (int rb = lane >> 2; rb < ly.r_blocks; rb += 8)
-        if ((lane & 3) < c) {
-          const int oc = first + (lane & 3);
-          const uint8_t* bt = ly.bsec + (size_t)(oc >> 4) * ly.r_blocks * kTileN * 17;
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(bt + ((size_t)rb * kTileN + (oc & 15) * 8) * 16));
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(bt + (size_t)ly.r_blocks * kTileN * 16 + rb * kTileN));
-        }
+  if (t_active) load_a(sub, nt_first, aw[0], ae[0]);
+  if (NT > 0)
+    for (int i = tid; i < nreal * NT; i += kWorkers) {                 // 128 bytes of mantissas each, and the exponents beside them
+      const size_t at = (size_t)(kb0 + i / NT) * k_pad + rb_lo * 16 + (i % NT) * 8;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(ly.asec + at * 16));
+      if (i % 4 == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(ly.asec + (size_t)kblocks * k_pad * 16 + at));
+    }
+  // B_q of this CTA's units, towards L2
+  if (k_pad > 0 && warp >= kConsumers)
+    for (int i = tid - kConsumers * 32; i < chunks * n_own * ly.r_blocks; i += kEpilogue * 32) {
+      const int rb = i % ly.r_blocks, u = i / ly.r_blocks, col = (rank + (u % n_own) * CS) * kUnit;
+      const uint8_t* bt = ly.bsec + (size_t)(tile_lo + u / n_own) * ly.r_blocks * kTileN * 17;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(bt + ((size_t)rb * kTileN + col) * 16));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(bt + ((size_t)rb * kTileN + col + 8) * 16));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(bt + (size_t)ly.r_blocks * kTileN * 16 + rb * kTileN + col));
     }
   // ---- zeros where no activation is written: rows beyond M, the second half of an odd last step, ranks beyond k_pad
-  for (int o = tid * 16; o < (int)(8 * plane); o += kThreads * 16) *reinterpret_cast<uint4*>(smem + o) = make_uint4(0u, 0u, 0u, 0u);
+  for (int o = tid * 16; o < (int)(4 * plane); o += kWorkers * 16) *reinterpret_cast<uint4*>(smem + o) = make_uint4(0u, 0u, 0u, 0u);
   uint8_t* xq = smem + p.off_xq;
   int8_t* xe = reinterpret_cast<int8_t*>(smem + p.off_xe);
-  const int xq_stride = p.slabs_max * 64 + 16, xe_stride = p.slabs_max * 4;
+  const int xq_stride = p.steps_max * 128 + 16, xe_stride = p.steps_max * 8;
   cluster_wait();                                    // every CTA's barriers are set up
   __syncthreads();
   tc::pdl_wait();                                    // X and Y may be in use by the kernel before
@@ -410,23 +449,24 @@ __global__ void __launch_bounds__(kThreads, 2) decode_cluster_kernel(const __gri
   // ---- X -> MXINT8, a lane per 16-block: bf16 pairs for W_q, mantissas and exponents for A_q
   {
     const QuantConsts qc = quant_consts(p.a_bits, p.exp_min, p.exp_max);
-    const int n_items = M * nreal;
-    int row = tid / nreal, b = tid % nreal;
-    const int row_step = kThreads / nreal, b_step = kThreads % nreal;
-    auto next = [&](int& r, int& c) {
+    const int n_blk = M * nreal;
+    float v[2][16];                                  // a block is on its way while the one before is quantised
+    const int row_step = kWorkers / nreal, blk_step = kWorkers % nreal;
+    int row = tid / nreal, blk = tid % nreal, i = tid;
+    auto next = [&](int& r, int& b) {
       r += row_step;
-      c += b_step;
-      if (c >= nreal) { c -= nreal; ++r; }
+      b += blk_step;
+      if (b >= nreal) { b -= nreal; ++r; }
     };
-    float v[2][16];
-    if (tid < n_items) load_x_block(v[0], ly.X, p.x_type, M, K, row, kb0 + b, p.a_bits, p.exp_min, p.exp_max);
-    for (int i = tid; i < n_items; i += 2 * kThreads) {
+    if (i < n_blk) load_x_block(v[0], ly.X, p.x_type, M, K, row, kb0 + blk, p.a_bits, p.exp_min, p.exp_max);
+    while (i < n_blk) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        if (i + h * kThreads >= n_items) break;
-        const int r = row, c = b;
-        next(row, b);
-        if (i + (h + 1) * kThreads < n_items) load_x_block(v[h ^ 1], ly.X, p.x_type, M, K, row, kb0 + b, p.a_bits, p.exp_min, p.exp_max);
+        if (i >= n_blk) break;
+        const int r = row, c = blk;
+        next(row, blk);
+        i += kWorkers;
+        if (i < n_blk) load_x_block(v[h ^ 1], ly.X, p.x_type, M, K, row, kb0 + blk, p.a_bits, p.exp_min, p.exp_max);
         int e;
         uint4 m8, f0, f1;
         quantize_block16(v[h], qc, e, m8, f0, f1);
@@ -434,39 +474,35 @@ __global__ void __launch_bounds__(kThreads, 2) decode_cluster_kernel(const __gri
           *reinterpret_cast<uint4*>(xq + r * xq_stride + c * 16) = m8;
           xe[r * xe_stride + c] = (int8_t)e;
         }
-        uint8_t* dst = smem + token_offset<MT>(r, c >> 2, (c & 3) * 16) + ((c & 1) * 4) * plane;
-        const uint32_t w[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (MT == 1) {
-            *reinterpret_cast<uint2*>(dst + q * plane) = make_uint2(w[2 * q], w[2 * q + 1]);
-          } else {
-            *reinterpret_cast<uint32_t*>(dst + q * plane) = w[2 * q];
-            *reinterpret_cast<uint32_t*>(dst + q * plane + 8) = w[2 * q + 1];
-          }
-        }
+        store_block<WB, MT>(smem, plane, r, c, f0, f1);
       }
     }
   }
-  __syncthreads();
+  worker_barrier();
 
-  // ---- T over this CTA's blocks, to the CTAs that own the rows
+  // ---- T over this CTA's blocks, a share of them and a tile of ranks to a warp
   if (t_active) {
     const int bias = -127 - (p.a_bits - 2) - (p.lr_bits - 2);        // exponent bytes carry +127
-    // rows beyond M are read (whatever lies there) but never stored
-    for (int nt = nt_first; nt < NT; nt += kWarps) {
+    double* tpart = reinterpret_cast<double*>(smem + p.off_tpart);
+    // rows beyond M are read (whatever lies there) but never sent
+    for (int nt = nt_first; nt < NT; nt += kWorkerWarps) {
       double acc[4] = {0.0, 0.0, 0.0, 0.0};
-      for (int bq = sub; bq < nreal; bq += UB * WPN) {
-        if (bq != sub || nt != nt_first) load_a(bq, nt);
+      if (nt != nt_first) load_a(sub, nt, aw[0], ae[0]);
+      for (int b0 = sub; b0 < nreal; b0 += 2 * UB * WPN) {
 #pragma unroll
-        for (int u = 0; u < UB; ++u) {
-          const int b = bq + u * WPN;
-          if (b < nreal) {
+        for (int h = 0; h < 2; ++h) {
+          const int bq = b0 + h * UB * WPN;
+          if (bq >= nreal) break;
+          if (bq + UB * WPN < nreal) load_a(bq + UB * WPN, nt, aw[h ^ 1], ae[h ^ 1]);
+          // (blocks beyond the last have zeros for A_q: without a branch the chains of eight blocks run side by side)
+#pragma unroll
+          for (int u = 0; u < UB; ++u) {
+            const int b = min(bq + u * WPN, nreal - 1);
             const uint32_t a0 = *reinterpret_cast<const uint32_t*>(xq + g * xq_stride + b * 16 + t * 4);
             const uint32_t a1 = MT == 2 ? *reinterpret_cast<const uint32_t*>(xq + (g + 8) * xq_stride + b * 16 + t * 4) : 0u;
             int c[4];
-            mma_s8(c, a0, a1, bw[u]);
-            const int ea_lo = (int)(ew[u] & 0xFFu), ea_hi = (int)(ew[u] >> 8);
+            mma_s8(c, a0, a1, aw[h][u]);
+            const int ea_lo = (int)(ae[h][u] & 0xFFu), ea_hi = (int)(ae[h][u] >> 8);
             const int ex0 = xe[g * xe_stride + b] + bias;
             acc[0] = fma(int_to_double(c[0]), pow2d(ex0 + ea_lo), acc[0]);
             acc[1] = fma(int_to_double(c[1]), pow2d(ex0 + ea_hi), acc[1]);
@@ -479,198 +515,263 @@ __global__ void __launch_bounds__(kThreads, 2) decode_cluster_kernel(const __gri
         }
       }
 #pragma unroll
-      for (int h = 0; h < MT; ++h) {
-        const int row = g + 8 * h, owner = row / RP;
-        if (row < M) {
-          const uint32_t at = sm + p.off_tpart + (uint32_t)(((rank * WPN + sub) * RP + row % RP) * t_cols + nt * 8 + t * 2) * 8u;
-          st_async(map_cta(at, owner), acc[2 * h], acc[2 * h + 1], map_cta(t_full, owner));
-        }
-      }
+      for (int h = 0; h < MT; ++h)
+        *reinterpret_cast<double2*>(tpart + (sub * (8 * MT) + g + 8 * h) * t_cols + nt * 8 + t * 2) = make_double2(acc[2 * h], acc[2 * h + 1]);
     }
   }
-  // the rows this CTA owns: sum in CTA order, MXINT8 along the rank, out to scratch for all clusters of the layer
-  auto reduce_t = [&]() -> bool {
-    const int total = own_rows * t_cols;
-    if (warp * 32 >= total) return true;
-    if (!wait_cluster(t_full, 0, &s_ws)) return false;
-    const double* tp = reinterpret_cast<const double*>(smem + p.off_tpart);
-    int done = 0;                                    // 16-blocks
-    for (int o = tid; o - lane < total; o += kThreads) {
-      const bool live = o < total;
-      done += min(32, total - (o - lane)) >> 4;
-      double v = 0.0;
-      if (live) {
-#pragma unroll 8
-        for (int c = 0; c < CS * WPN; ++c) v += tp[(size_t)c * RP * t_cols + o];
-      }
-      double amax = (v != v) ? 0.0 : fabs(v);
-#pragma unroll
-      for (int d = 1; d < 16; d <<= 1) amax = fmax(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, d));
-      const int e = block_exponent(amax, p.exp_min, p.exp_max);
-      const uint32_t bits = (uint32_t)bf16_bits_of(quant_mantissa(v, e, p.a_bits), e - (p.a_bits - 2)) & 0xFFFFu;
-      const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, bits, 1);
-      if (live && (lane & 1) == 0) {
-        const int row = rank * RP + o / t_cols, j = rb_lo * 16 + o % t_cols;
-        const uint32_t at = (uint32_t)((j & 31) >> 2) * rplane + token_offset<MT>(row, j >> 6, j & 63) + (uint32_t)((j & 2) * 2 * MT);
-        if (LQER_IN_BOUNDS(p.status, at, 4, 8 * rplane, 734)) *reinterpret_cast<uint32_t*>(ly.tq + at) = bits | (next << 16);
-      }
-    }
-    __threadfence();
-    __syncwarp();
-    if (lane == 0) atomicAdd(ly.tcount, done);
-    return true;
-  };
-
-  // ---- the rounds
-  const ConvConsts kc = conv_consts<WB>();
-  const uint32_t x_off = (uint32_t)((t >> 1) * (128 * MT) + (2 * g + (t & 1)) * (8 * MT));   // the lane's position within a step of a plane
-  const int eb0 = 2 * (t & 1);
-  bool ok = true;
   if (NT > 0) {
-    ok = reduce_t();
-    __syncwarp();
-    if (rounds > 1 && lane < CS) arrive_remote(map_cta(t_seen, lane));
+    // the sum of the CTA's shares, to the CTA that owns the row
+    worker_barrier();
+    const double* tpart = reinterpret_cast<const double*>(smem + p.off_tpart);
+    const int pairs = t_cols / 2;
+    for (int o = tid; o < M * pairs; o += kWorkers) {
+      const int row = o / pairs, owner = row / RP;
+      const double* src = tpart + row * t_cols + (o % pairs) * 2;
+      double a = 0.0, b = 0.0;
+#pragma unroll 4
+      for (int c = 0; c < WPN; ++c) {
+        const double2 d = *reinterpret_cast<const double2*>(src + c * (8 * MT) * t_cols);
+        a += d.x; b += d.y;
+      }
+      st_async(map_cta(sm + p.off_trecv + (uint32_t)((rank * RP + row % RP) * t_cols + (o % pairs) * 2) * 8u, owner), a, b, map_cta(t_full, owner));
+    }
   }
-  int slot = 0;
-  auto reduce_round = [&](int r) -> bool {
-    const int b = r & 1;
-    if (round_bytes(r) == 0) return true;                      // nothing comes, as in a short last round
-    if (!wait_cluster(red_full(b), (r >> 1) & 1, &s_ws)) return false;
-    if (tid == 0 && r + 2 < rounds && round_bytes(r + 2) > 0) tc::mbar_expect_tx(red_full(b), round_bytes(r + 2));
-    const float* buf = reinterpret_cast<const float*>(smem + p.off_red[b]);
-    for (int s = 0; s < slots_w; ++s) {
-      int c;
-      const int first = octets(r, rank + s * CS, c);
-      for (int i = tid; i - lane < M * 8; i += kThreads) {     // (row, quad of columns)
-        const int row = i >> 3, quad = i & 7;
-        const bool live = row < M && quad < 2 * c;
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-        if (live)
-          for (int q = 0; q < CS; ++q) {
-            const float* src = buf + ((s * CS + q) * 32 + quad * 4) * TS + row;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) v[j] += src[j * TS];
-          }
-        write_y4(p, ly, row, first * 8 + quad * 4, make_float4(v[0], v[1], v[2], v[3]), live);
-      }
-    }
-    if (r + 2 < rounds) {
-      __syncwarp();
-      if (lane < CS) arrive_remote(map_cta(red_free(b), lane));
-    }
-    return true;
-  };
+  bool ok = true;
+
+  if (warp < kConsumers) {
+    // ------------------------------------------------------------------ consumers
+    const ConvConsts kc = conv_consts<WB>();
+    const int cw = warp % kColumnWarps, phase = warp / kColumnWarps, col = cw * 2 * kUnit;
+    const uint8_t* x_lane = smem + lane * 16;
+    // addresses of the rows of 16 bytes that ldmatrix distributes: lanes 8 i .. 8 i + 7 give the eight columns of piece i
+    const uint32_t w_row = sm + p.off_ring + (col + (lane & 7)) * 16 + (WB == 4 ? (lane >> 4) * kTile + ((lane >> 3) & 1) * 2048 : ((lane >> 3) & 1) * kTile);
+    const uint8_t* e_lane = smem + p.off_ring + kMant + (col + g) * 4;
+    int x = phase, slot = phase % p.slots;
+    uint32_t ph = (phase / p.slots) & 1;
 #pragma unroll 1
-  for (int r = 0; r < rounds; ++r) {
-    int count;
-    const int first = octets(r, warp, count);
-    float acc[kOcts / 2][MT][4];
+    for (int r = 0, begin = 0, b = 0, turn = 0; r < chunks; ++r, begin += steps) {     // b, turn: r mod and by kRed
+      float acc[2][MT][4];
 #pragma unroll
-    for (int o = 0; o < kOcts / 2; ++o)
+      for (int u = 0; u < 2; ++u)
 #pragma unroll
-      for (int i = 0; i < MT; ++i)
+        for (int i = 0; i < MT; ++i)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[o][i][q] = 0.f;
+          for (int c = 0; c < 4; ++c) acc[u][i][c] = 0.f;
 #pragma unroll 1
-    for (int j = 0; j < ksteps; ++j) {
-      cp_wait<D - 1>();
-      const uint8_t* st = smem + (ring - sm) + slot * kStage + lane * kPiece;
-      const uint8_t* se = smem + (ring - sm) + slot * kStage + kOcts * 32 * kPiece + lane * 4;
-      const uint8_t* x = smem + j * (256 * MT) + x_off;
-      // eight weights of octet o: word m of the lane's four (2-bit mantissas: half a word)
-      auto load_w = [&](uint4& w, uint32_t& e, int o) {
-        if (WB == 4) {
-          w = *reinterpret_cast<const uint4*>(st + o * 32 * kPiece);
-        } else {
-          const uint2 v = *reinterpret_cast<const uint2*>(st + o * 32 * kPiece);
-          w = make_uint4(v.x, v.y, 0u, 0u);
-        }
-        e = *reinterpret_cast<const uint32_t*>(se + o * 128);
-      };
-      auto convert = [&](const uint4& w, uint32_t e, int m) -> uint4 {
-        uint32_t s2, c2;
-        if (WB == 4) {
-          w_scale_pair(e, eb0 + (m >> 1), s2, c2);
-          return convert_nibbles(m == 0 ? w.x : m == 1 ? w.y : m == 2 ? w.z : w.w, s2, c2, kc);
-        } else {
-          w_scale_pair2(e, eb0 + (m >> 1), s2, c2);
-          return convert_crumbs(m < 2 ? w.x : w.y, m & 1, s2, c2, kc);
-        }
-      };
-      if (count > 2) {
-        uint4 w[4];
-        uint32_t e[4];
-#pragma unroll
-        for (int o = 0; o < 4; ++o) load_w(w[o], e[o], min(o, count - 1));
-        multiply_step<MT, 2>(acc, x, plane, [&](int o, int m) { return convert(w[o], e[o], m); });
-      } else if (count > 0) {
-        uint4 w[2];
-        uint32_t e[2];
-#pragma unroll
-        for (int o = 0; o < 2; ++o) load_w(w[o], e[o], min(o, count - 1));
-        multiply_step<MT, 1>(acc, x, plane, [&](int o, int m) { return convert(w[o], e[o], m); });
-      }
-      prefetch_step();
-      if (++slot == D) slot = 0;
-    }
-    // the rank term of warp w's octets is CTA w mod CS's
-    if (k_pad > 0 && warp % CS == rank) {
-      for (int j = 0; j * 128 < k_pad && ok; ++j) {
-        uint4 w[4][2];
-        float sc[4][2];
+      for (; x < begin + steps; x += kPhases) {
+        if (!warp_wait(full(slot), ph, &s_ws)) { ok = false; break; }
+        uint32_t w[4][4], e[4][2];
 #pragma unroll
         for (int o = 0; o < 4; ++o) {
-          const int oc = first + max(min(o, count - 1), 0), nl = (oc & 15) * 8 + g;
-          const uint8_t* bt = ly.bsec + (size_t)(oc >> 4) * ly.r_blocks * kTileN * 17;
+          if (WB == 4) ldmatrix4(w[o], w_row + slot * St::kBytes + o * 128);
+          else ldmatrix2(w[o], w_row + slot * St::kBytes + o * 128);
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int rb = 8 * j + 2 * t + u;
-            const bool in = rb < ly.r_blocks;
-            w[o][u] = in ? ld_stream16(bt + ((size_t)rb * kTileN + nl) * 16) : make_uint4(0u, 0u, 0u, 0u);
-            sc[o][u] = in ? pow2f((int)bt[(size_t)ly.r_blocks * kTileN * 16 + rb * kTileN + nl] - 127 - (p.lr_bits - 2)) : 1.0f;
+          for (int h = 0; h < 2; ++h) e[o][h] = *reinterpret_cast<const uint32_t*>(e_lane + slot * St::kBytes + o * 32 + h * kTile);
+        }
+        const uint8_t* xs = x_lane + (x - begin) * (512 * MT);
+        multiply_step<MT, 2>(acc, [&](int o, int m) -> uint4 {
+          uint32_t s2, c2;
+          if (WB == 4) {
+            w_scale_pair(e[o][m >> 1], 2 * (m & 1) + (t >> 1), s2, c2);
+            return convert_nibbles(w[o][m], s2, c2, kc);
+          } else {
+            w_scale_pair2(e[o][m >> 1], t, s2, c2);
+            return convert_crumbs(w[o][m >> 1], m & 1, s2, c2, kc);
+          }
+        }, [&](int m, uint32_t (&b0)[2 * MT], uint32_t (&b1)[2 * MT]) {
+          uint4 v = *reinterpret_cast<const uint4*>(xs + m * plane);
+          if (MT == 1) {
+            b0[0] = v.x; b0[1] = v.y; b1[0] = v.z; b1[1] = v.w;
+          } else {
+            b0[0] = v.x; b0[2 * MT - 2] = v.y; b0[1] = v.z; b0[2 * MT - 1] = v.w;
+            v = *reinterpret_cast<const uint4*>(xs + m * plane + 512);
+            b1[0] = v.x; b1[2 * MT - 2] = v.y; b1[1] = v.z; b1[2 * MT - 1] = v.w;
+          }
+        });
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(empty(slot));
+        slot += kPhases;
+        while (slot >= p.slots) { slot -= p.slots; ph ^= 1; }
+      }
+      if (ok && r == 0 && NT > 0) ok = wait_cluster(t_seen, 0, &s_ws);       // the sums lie where T was formed
+      if (ok && r >= kRed) ok = wait_cluster(red_free(b), (uint32_t)(turn - 1) & 1u, &s_ws);
+      if (!ok) break;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int j = 2 * cw + u;
+        const uint32_t base = map_cta(sm + p.off_red + b * p.red_bytes + (uint32_t)((((j / CS) * CS + rank) * kPhases + phase) * kUnit * TS * 4), (uint32_t)(j % CS));
+        const uint32_t bar = map_cta(red_full(b), (uint32_t)(j % CS));
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+          if (8 * i + 2 * t < M) {
+            st_async(base + (uint32_t)((g * TS + 8 * i + 2 * t) * 4), acc[u][i][0], acc[u][i][1], bar);
+            st_async(base + (uint32_t)(((g + 8) * TS + 8 * i + 2 * t) * 4), acc[u][i][2], acc[u][i][3], bar);
+          }
+      }
+      if (++b == kRed) { b = 0; ++turn; }
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogue
+    const int ew_ = warp - kConsumers, etid = tid - kConsumers * 32;
+    // the rows of T this CTA owns: sum in order, MXINT8 along the rank, out to scratch for all clusters of the layer
+    auto reduce_t = [&]() -> bool {
+      const int total = own_rows * t_cols;
+      if (ew_ * 32 >= total) return true;
+      if (!wait_cluster(t_full, 0, &s_ws)) return false;
+      const double* tp = reinterpret_cast<const double*>(smem + p.off_trecv);
+      int done = 0;                                    // 16-blocks
+      for (int o = etid; o - lane < total; o += kEpilogue * 32) {
+        const bool live = o < total;
+        done += min(32, total - (o - lane)) >> 4;
+        double v = 0.0;
+        if (live) {
+#pragma unroll 8
+          for (int c = 0; c < CS; ++c) v += tp[c * RP * t_cols + o];
+        }
+        double amax = (v != v) ? 0.0 : fabs(v);
+#pragma unroll
+        for (int d = 1; d < 16; d <<= 1) amax = fmax(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, d));
+        const int e = block_exponent(amax, p.exp_min, p.exp_max);
+        const uint32_t bits = (uint32_t)bf16_bits_of(quant_mantissa(v, e, p.a_bits), e - (p.a_bits - 2)) & 0xFFFFu;
+        const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, bits, 1);
+        if (live && (lane & 1) == 0) {
+          const int row = rank * RP + o / t_cols, j = rb_lo * 16 + o % t_cols;
+          const uint32_t at = (uint32_t)((j & 31) >> 2) * rplane + token_offset<MT>(row, j >> 6, j & 63) + (uint32_t)((j & 2) * 2 * MT);
+          if (LOCAL) {
+            for (int c = 0; c < CS; ++c) st_async(map_cta(sm + p.off_tq + at, c), bits | (next << 16), map_cta(t_ready, c));
+          } else if (LQER_IN_BOUNDS(p.status, at, 4, 8 * rplane, 734)) {
+            *reinterpret_cast<uint32_t*>(ly.tq + at) = bits | (next << 16);
           }
         }
-        if (r == 0 && j == 0) ok = wait_count(ly.tcount, ly.t_expect, &s_ws);
-        multiply_step<MT, 2, true>(acc, ly.tq + j * (256 * MT) + x_off, rplane, [&](int o, int m) {
-          const uint4& v = w[o][m >> 1];
-          return tc::convert_i8x8(m & 1 ? v.z : v.x, m & 1 ? v.w : v.y, sc[o][m >> 1]);
-        }, ly.r_blocks - (8 * j + 2 * t));
       }
-      // the last of the layer's warps to have read T_q zeroes the counters for the next call
-      if (r == rounds - 1 && lane == 0 && ok && atomicAdd(ly.tcount + 1, 1) == ly.clusters * kWarps - 1) {
-        ly.tcount[0] = 0;
-        ly.tcount[1] = 0;
-      }
+      __syncwarp();
+      // (one lane's release covers what the warp wrote before)
+      if (lane == 0 && !LOCAL) asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(ly.tcount), "r"(done) : "memory");
+      return true;
+    };
+    if (NT > 0) {
+      ok = reduce_t();
+      __syncwarp();
+      if (lane < CS) arrive_remote(map_cta(t_seen, lane));
     }
-    if (r > 0) ok = ok && reduce_round(r - 1);
-    if (r == 1 && NT > 0) ok = ok && wait_cluster(t_seen, 0, &s_ws);   // the sums of the odd rounds lie where T was formed
-    if (r > 1) ok = ok && wait_cluster(red_free(r & 1), ((r >> 1) - 1) & 1, &s_ws);
-    if (!ok) break;
-    {
-      const uint32_t dst_cta = (uint32_t)(warp % CS);
-      const uint32_t base = map_cta(sm + p.off_red[r & 1] + (uint32_t)(((warp / CS) * CS + rank) * 32 * TS * 4), dst_cta);
-      const uint32_t bar = map_cta(red_full(r & 1), dst_cta);
+    const uint32_t r_off = (uint32_t)((t >> 1) * (128 * MT) + (2 * g + (t & 1)) * (8 * MT));   // the lane's position within a step of a plane of T_q
+    bool have_t = false;
+    // Units of this warp to come; after the last one's rank term it counts itself out.  The layer's last warp to do so zeroes the counters for
+    // the next call (all of T_q is there then: some warp has waited for it).
+    int left = 0, out = 0;
+    for (int r = 0; r < chunks; ++r)
+      for (int q = (ew_ - r * n_own) & (kEpilogue - 1); q < n_own; q += kEpilogue) ++left;
+    auto count_out = [&]() {
+      if (k_pad > 0 && !LOCAL && left == 0 && lane == 0) out = atomicAdd(ly.tcount + 1, 1);
+    };
+    count_out();
+#pragma unroll 1
+    for (int r = 0, b = 0, turn = 0; r < chunks && ok; ++r) {
+      bool here = false;                               // the tile's sums have come
+      // the units of one tile after the other go to the epilogue warps in turn
+      for (int q = (ew_ - r * n_own) & (kEpilogue - 1); q < n_own; q += kEpilogue) {
+        const int unit = rank + q * CS, col = (tile_lo + r) * kTileN + unit * kUnit;
+        float term[1][MT][4];
 #pragma unroll
-      for (int o = 0; o < kOcts; ++o)
-        if (o < count) {
+        for (int i = 0; i < MT; ++i)
 #pragma unroll
-          for (int i = 0; i < MT; ++i)
-            if (8 * i + 2 * t < M)
-              st_async(base + (uint32_t)(((o * 8 + g) * TS + 8 * i + 2 * t) * 4), acc[o >> 1][i][2 * (o & 1)], acc[o >> 1][i][2 * (o & 1) + 1], bar);
+          for (int c = 0; c < 4; ++c) term[0][i][c] = 0.f;
+        const uint8_t* bt = ly.bsec + (size_t)(tile_lo + r) * ly.r_blocks * kTileN * 17;
+#pragma unroll 1
+        for (int j = 0; j * 128 < k_pad; ++j) {
+          uint4 w[2][2];
+          float sc[2][2];
+#pragma unroll
+          for (int o = 0; o < 2; ++o) {
+            const int nl = unit * kUnit + o * 8 + g;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const int rb = 8 * j + 2 * t + u;
+              const bool in = rb < ly.r_blocks;
+              w[o][u] = in ? ld_stream16(bt + ((size_t)rb * kTileN + nl) * 16) : make_uint4(0u, 0u, 0u, 0u);
+              sc[o][u] = in ? pow2f((int)bt[(size_t)ly.r_blocks * kTileN * 16 + rb * kTileN + nl] - 127 - (p.lr_bits - 2)) : 1.0f;
+            }
+          }
+          if (!have_t) {
+            ok = LOCAL ? wait_cluster(t_ready, 0, &s_ws) : wait_count(ly.tcount, ly.t_expect, &s_ws);
+            have_t = true;
+            if (!ok) break;
+          }
+          // all of the lane's T_q of these ranks at once
+          const int blocks = ly.r_blocks - (8 * j + 2 * t);
+          const uint32_t x_at = j * (256 * MT) + r_off;
+          uint32_t x[8][2 * MT];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const bool in = (i >> 2) < blocks;
+            if (MT == 1) {
+              const uint2 a = !in ? make_uint2(0u, 0u) : LOCAL ? *reinterpret_cast<const uint2*>(smem + p.off_tq + x_at + i * rplane)
+                                                                    : __ldcg(reinterpret_cast<const uint2*>(ly.tq + x_at + i * rplane));
+              x[i][0] = a.x; x[i][1] = a.y;
+            } else {
+              const uint4 a = !in ? make_uint4(0u, 0u, 0u, 0u) : LOCAL ? *reinterpret_cast<const uint4*>(smem + p.off_tq + x_at + i * rplane)
+                                                                            : __ldcg(reinterpret_cast<const uint4*>(ly.tq + x_at + i * rplane));
+              x[i][0] = a.x; x[i][2 * MT - 2] = a.y; x[i][1] = a.z; x[i][2 * MT - 1] = a.w;
+            }
+          }
+          multiply_step<MT, 1>(term, [&](int o, int m) {
+            const uint4& a = w[o][m >> 1];
+            return convert_i8x8(m & 1 ? a.z : a.x, m & 1 ? a.w : a.y, sc[o][m >> 1]);
+          }, [&](int m, uint32_t (&b0)[2 * MT], uint32_t (&b1)[2 * MT]) {
+#pragma unroll
+            for (int i = 0; i < 2 * MT; ++i) { b0[i] = x[2 * m][i]; b1[i] = x[2 * m + 1][i]; }
+          });
         }
+        if (!ok) break;
+        --left;
+        count_out();
+        if (!here) { ok = wait_cluster(red_full(b), (uint32_t)turn & 1u, &s_ws); here = true; }
+        if (!ok) break;
+        float* buf = reinterpret_cast<float*>(smem + p.off_red + b * p.red_bytes) + q * CS * kPhases * kUnit * TS;
+#pragma unroll
+        for (int i = 0; i < MT; ++i) {
+          float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 6
+          for (int c = 0; c < CS * kPhases; ++c) {
+            const float2 a0 = *reinterpret_cast<const float2*>(buf + (c * kUnit + g) * TS + 8 * i + 2 * t);
+            const float2 a1 = *reinterpret_cast<const float2*>(buf + (c * kUnit + g + 8) * TS + 8 * i + 2 * t);
+            v[0] += a0.x; v[1] += a0.y; v[2] += a1.x; v[3] += a1.y;
+          }
+          *reinterpret_cast<float2*>(buf + g * TS + 8 * i + 2 * t) = make_float2(v[0] + term[0][i][0], v[1] + term[0][i][1]);
+          *reinterpret_cast<float2*>(buf + (g + 8) * TS + 8 * i + 2 * t) = make_float2(v[2] + term[0][i][2], v[3] + term[0][i][3]);
+        }
+        __syncwarp();
+        // a quad of lanes holds a row's sixteen columns
+#pragma unroll
+        for (int i = 0; i < MT; ++i) {
+          const int row = (lane >> 2) + 8 * i, c = (lane & 3) * 4;
+          const float* src = buf + c * TS + row;
+          write_y4(p, ly, row, col + c, make_float4(src[0], src[TS], src[2 * TS], src[3 * TS]), row < M && col + c < ly.N);
+        }
+      }
+      if (ok && !here) ok = wait_cluster(red_full(b), (uint32_t)turn & 1u, &s_ws);
+      if (!ok) break;
+      if (r + kRed < chunks) {
+        // (its bytes cannot come before this warp's arrivals below)
+        if (etid == 0) tc::mbar_expect_tx(red_full(b), chunk_bytes);
+        __syncwarp();
+        if (lane < CS) arrive_remote(map_cta(red_free(b), lane));
+      }
+      if (++b == kRed) { b = 0; ++turn; }
+    }
+    if (ok && k_pad > 0 && !LOCAL && lane == 0 && out == ly.clusters * CS * kEpilogue - 1) {
+      ly.tcount[0] = 0;
+      ly.tcount[1] = 0;
     }
   }
+  __syncwarp();
   cluster_arrive();                                  // this warp's last store into another CTA lies behind it
-  if (ok) ok = reduce_round(rounds - 1);
-  cp_wait<0>();
   cluster_wait();                                    // no CTA leaves while another may still store into its shared memory
   if (tid == 0 && s_ws.abort != 0) report_error(p.status, LQER_ERR_TIMEOUT, 730, blockIdx.x);
 }
 
-
-// Clusters of CS CTAs that the device holds at a time, with one or two CTAs to an SM (0 if the query fails).
-constexpr int kSmemTwo = 112 * 1024, kSmemOne = 220 * 1024;
-static cudaLaunchConfig_t launch_config(int CS, int clusters, size_t smem, bool cooperative, cudaLaunchAttribute* attr, cudaStream_t s) {
+// Clusters of CS CTAs that the device holds at a time (0 if the query fails).
+static cudaLaunchConfig_t launch_config(int CS, int clusters, size_t smem, cudaLaunchAttribute* attr, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(clusters * CS);
   cfg.blockDim = dim3(kThreads);
@@ -680,122 +781,192 @@ static cudaLaunchConfig_t launch_config(int CS, int clusters, size_t smem, bool 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = CS; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-  attr[2].id = cudaLaunchAttributeCooperative;
-  attr[2].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = cooperative ? 3 : 2;
+  cfg.numAttrs = 2;
   return cfg;
 }
-template <int WB, int MT, bool YQ, int D>
-static int resident_clusters(int CS, bool two) {
+template <int WB, int MT, bool LOCAL>
+static int resident_clusters(int CS) {
   static std::mutex mu;
-  static int known[64][4][2] = {};
+  static int known[64][4] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   std::lock_guard<std::mutex> lock(mu);
-  int& n = known[dev][CS == 8 ? 3 : CS == 4 ? 2 : CS == 2 ? 1 : 0][two ? 1 : 0];
+  int& n = known[dev][CS == 8 ? 3 : CS == 4 ? 2 : CS == 2 ? 1 : 0];
   if (n == 0) {
-    cudaLaunchAttribute attr[3];
-    const cudaLaunchConfig_t cfg = launch_config(CS, 1, two ? kSmemTwo : kSmemOne, false, attr, nullptr);
-    if (cudaFuncSetAttribute(decode_cluster_kernel<WB, MT, YQ, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemOne) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, decode_cluster_kernel<WB, MT, YQ, D>, &cfg) != cudaSuccess)
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = launch_config(CS, 1, kSmemMax, attr, nullptr);
+    if (cudaFuncSetAttribute(decode_cluster_kernel<WB, MT, LOCAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, decode_cluster_kernel<WB, MT, LOCAL>, &cfg) != cudaSuccess)
       n = 0;
   }
   return n;
 }
-template <int WB, int MT, bool YQ, int D>
-static cudaError_t launch(const Params& p, int clusters, int CS, size_t smem, bool cooperative, cudaStream_t s) {
-  cudaLaunchAttribute attr[3];
-  const cudaLaunchConfig_t cfg = launch_config(CS, clusters, smem, cooperative, attr, s);
+template <int WB, int MT, bool LOCAL>
+static cudaError_t launch(const Params& p, int clusters, int CS, size_t smem, cudaStream_t s) {
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = launch_config(CS, clusters, smem, attr, s);
   LaunchScope scope(kFamDecode, s);
-  return cudaLaunchKernelEx(&cfg, decode_cluster_kernel<WB, MT, YQ, D>, p, CS);
+  return cudaLaunchKernelEx(&cfg, decode_cluster_kernel<WB, MT, LOCAL>, p, CS);
 }
-// The instance of the kernel for a call.
-template <int WB, int MT, bool YQ>
-struct Instance {
-  static int resident(int CS, bool two) { return two ? resident_clusters<WB, MT, YQ, 2>(CS, true) : resident_clusters<WB, MT, YQ, 4>(CS, false); }
-  static cudaError_t go(const Params& p, int clusters, int CS, bool two, size_t smem, bool cooperative, cudaStream_t s) {
-    return two ? launch<WB, MT, YQ, 2>(p, clusters, CS, smem, cooperative, s) : launch<WB, MT, YQ, 4>(p, clusters, CS, smem, cooperative, s);
-  }
-};
 struct Entry {
-  int (*resident)(int, bool);
-  cudaError_t (*go)(const Params&, int, int, bool, size_t, bool, cudaStream_t);
+  int (*resident)(int);
+  cudaError_t (*go)(const Params&, int, int, size_t, cudaStream_t);
 };
-template <int WB, int MT, bool YQ>
-static Entry entry() { return Entry{Instance<WB, MT, YQ>::resident, Instance<WB, MT, YQ>::go}; }
-static Entry entry_of(int wb, int mt, bool yq) {
-  if (wb == 4) return mt == 1 ? (yq ? entry<4, 1, true>() : entry<4, 1, false>()) : (yq ? entry<4, 2, true>() : entry<4, 2, false>());
-  return mt == 1 ? (yq ? entry<2, 1, true>() : entry<2, 1, false>()) : (yq ? entry<2, 2, true>() : entry<2, 2, false>());
+template <int WB, int MT>
+static Entry entry(bool local) {
+  return local ? Entry{resident_clusters<WB, MT, true>, launch<WB, MT, true>} : Entry{resident_clusters<WB, MT, false>, launch<WB, MT, false>};
+}
+static Entry entry_of(int wb, int mt, bool local) {
+  if (wb == 4) return mt == 1 ? entry<4, 1>(local) : entry<4, 2>(local);
+  return mt == 1 ? entry<2, 1>(local) : entry<2, 2>(local);
 }
 
-}  // namespace dcl
-
-// The cluster size and the shared memory of a launch over these layers, functions of the shapes alone.
-namespace dcl {
+// The cluster size, the clusters of each layer and the shared memory of a launch over these layers: functions of the shapes (and of
+// what the device holds) alone.
 struct Plan {
-  int CS, slabs_max;
-  int off_red[2], off_xq, off_xe, off_tpart, off_ring;
-  bool two;                                 // two CTAs to an SM
+  int CS, steps_max, slots;
+  int off_red, red_bytes, off_xq, off_xe, off_tpart, off_trecv, off_tq, off_ring;
   size_t smem;
+  int resident, clusters[kMaxLayers], total;
+  int t_blocks[kMaxLayers], t_clusters[kMaxLayers], t_tiles[kMaxLayers];
+  bool local;                               // every cluster forms all of T for itself
+  double cost;
 };
-static Plan plan(const PackedMeta* metas, int n, int M) {
-  int k_slabs_min = metas[0].k_slabs, k_slabs_max = 0, r_blocks_max = 0;
+static bool plan_with(const PackedMeta* metas, int n, int M, int CS, Plan& q) {
+  const int MT = M > 8 ? 2 : 1, wb = metas[0].w_bits;
+  int k_slabs_max = 0, r_blocks_max = 0;
   for (int i = 0; i < n; ++i) {
-    k_slabs_min = std::min(k_slabs_min, (int)metas[i].k_slabs);
     k_slabs_max = std::max(k_slabs_max, (int)metas[i].k_slabs);
     r_blocks_max = std::max(r_blocks_max, (int)metas[i].r_blocks);
   }
-  Plan q;
-  q.CS = 8;
-  while (q.CS > 1 && k_slabs_min < 2 * q.CS) q.CS >>= 1;             // at least one step of two slabs to a CTA
-  const int MT = M > 8 ? 2 : 1;
+  q.CS = CS;
   auto al = [](int v) { return (v + 127) / 128 * 128; };
-  const int red = al(kWarps * 32 * token_stride(MT) * 4), stage = metas[0].w_bits == 4 ? stage_bytes<4>() : stage_bytes<2>();
-  q.slabs_max = ((k_slabs_max + q.CS - 1) / q.CS + 1) / 2 * 2;
-  int off = q.slabs_max * 1024 * MT;
-  q.off_red[0] = off; off += red;
-  // X_q for the projection and the partial sums of T share their room with the sums of the odd rounds
-  q.off_red[1] = off;
+  const int red = al(kUnits * kPhases * kUnit * token_stride(MT) * 4), stage = wb == 4 ? Stage<4>::kBytes : Stage<2>::kBytes;
+  q.steps_max = ((k_slabs_max + CS - 1) / CS + 1) / 2;
+  if ((long long)q.steps_max * 2048 * MT > kSmemMax) return false;
+  const int off = q.steps_max * 2048 * MT;
+  // X_q for the projection and the partial sums of T share their room with the sums of the tiles
+  q.off_red = off;
+  q.red_bytes = red;
   q.off_xq = off;
-  q.off_xe = q.off_xq + al(8 * MT * (q.slabs_max * 64 + 16));
-  q.off_tpart = q.off_xe + al(8 * MT * q.slabs_max * 4);
-  q.off_ring = std::max(off + red, q.off_tpart + (r_blocks_max > 0 ? std::max(kWarps, 2 * r_blocks_max) * 1024 : 0));
-  q.two = q.off_ring + kWarps * 2 * stage <= kSmemTwo;
-  q.smem = (size_t)q.off_ring + (size_t)kWarps * (q.two ? 2 : 4) * stage;
-  return q;
+  q.off_xe = q.off_xq + al(8 * MT * (q.steps_max * 128 + 16));
+  q.off_tpart = q.off_xe + al(8 * MT * q.steps_max * 8);
+  const int t_width = std::max(8 * kWorkerWarps, 16 * r_blocks_max);
+  q.off_trecv = q.off_tpart + 64 * MT * t_width;
+  q.off_tq = r_blocks_max > 0 ? std::max(off + kRed * red, q.off_trecv + 64 * MT * 16 * r_blocks_max) : off + kRed * red;
+  q.off_ring = q.off_tq + 2048 * MT;
+  if (kSmemMax - q.off_ring < kPhases * stage) return false;
+  int stages_max = 0;
+  for (int i = 0; i < n; ++i) stages_max = std::max(stages_max, (int)metas[i].n_tiles * q.steps_max);
+  q.slots = std::min(std::min((kSmemMax - q.off_ring) / stage, kMaxSlots), stages_max);
+  q.smem = (size_t)q.off_ring + (size_t)q.slots * stage;
+  q.resident = std::min(entry_of(wb, MT, false).resident(CS), entry_of(wb, MT, true).resident(CS));
+  if (q.resident < n) return false;
+  // each layer has a cluster, the others go one by one where the time is longest, as long as every cluster keeps a tile
+  auto steps = [&](int i) { return ((metas[i].k_slabs + CS - 1) / CS + 1) / 2; };
+  q.total = n;
+  for (int i = 0; i < n; ++i) q.clusters[i] = 1;
+  while (q.total < q.resident) {
+    int best = -1;
+    double longest = 0.0;
+    for (int i = 0; i < n; ++i) {
+      const double len = (double)metas[i].n_tiles / q.clusters[i] * steps(i);
+      if (q.clusters[i] < metas[i].n_tiles && len > longest) { longest = len; best = i; }
+    }
+    if (best < 0) break;
+    ++q.clusters[best];
+    ++q.total;
+  }
+  // In the time of a stage: the stages, what a tile costs beyond them (many CTAs hand over more sums in less time), the rounds in which
+  // X is quantised, and what T costs the clusters that form it, which get fewer tiles for that (see launch_decode_cluster for how many
+  // they are).  Fitted to calls of 3, 8, 9 and 16 rows with clusters of 2, 4 and 8; us for the four groups of a 4096 / 11008 and of a
+  // 5120 / 13824 layer (qkv, o, gate and up, down), 3 rows: 17.9 10.8 25.3 28.8 with 2, 15.1 10.2 25.9 14.4 with 4, 18.4 11.1 31.3 18.4 with 8;
+  // 21.6 13.1 31.6 37.6, 21.7 12.2 35.4 28.5, 25.7 12.0 41.3 22.6; 16 rows: 26.3 19.5 34.1 -, 23.7 13.6 31.8 25.6, 28.8 15.5 47.4 24.8;
+  // 33.3 25.6 45.3 -, 28.7 18.6 43.1 46.1, 36.1 17.2 57.6 31.1.
+  const double tile_cost = CS == 8 ? (MT == 1 ? 2.0 : 3.5) : CS == 4 ? (MT == 1 ? 0.7 : 1.2) : (MT == 1 ? 0.3 : 0.6);
+  const int most = std::max(q.resident / 4 / n, 1);
+  auto share = [&](int i) { return (metas[i].n_tiles + q.clusters[i] - 1) / q.clusters[i]; };
+  // few stages: T's way through global memory would take longer than they do
+  q.local = r_blocks_max > 0 && r_blocks_max <= 8;
+  for (int i = 0; i < n; ++i)
+    q.local = q.local && steps(i) * 8 * 2 * metas[i].r_blocks * MT <= kLocalBlocks * kWorkerWarps && share(i) * steps(i) <= kLocalStages;
+  q.cost = 0.0;
+  for (int i = 0; i < n; ++i) {
+    const int tiles = metas[i].n_tiles, formers = q.local ? 1 : std::min(q.clusters[i], most);
+    q.t_blocks[i] = (metas[i].r_blocks + formers - 1) / formers;
+    int f = !q.local && q.t_blocks[i] > 0 ? (metas[i].r_blocks + q.t_blocks[i] - 1) / q.t_blocks[i] : 0, tf = 0;
+    const double per_tile = steps(i) + tile_cost;
+    const double t_cost = metas[i].r_blocks > 0 ? 2.0 + 0.15 * MT * steps(i) * 16 * q.t_blocks[i] / kWorkerWarps : 0.0;
+    if (f > 0 && f < q.clusters[i]) {
+      // equal times: f * tf + (clusters - f) * (tf + t_cost / per_tile) = tiles
+      const double level = (tiles - (q.clusters[i] - f) * t_cost / per_tile) / q.clusters[i];
+      tf = std::max(1, (int)(level + 0.5));
+      if (tiles - f * tf < q.clusters[i] - f) tf = 0;
+    }
+    if (tf == 0) f = 0;                              // equal shares for all
+    q.t_clusters[i] = f;
+    q.t_tiles[i] = tf;
+    const int longest = (tiles - f * tf + q.clusters[i] - f - 1) / (q.clusters[i] - f);
+    q.cost = std::max(q.cost, std::max(longest * per_tile + (f > 0 ? 0.0 : t_cost), f > 0 ? tf * per_tile + t_cost : 0.0) +
+                                  (MT == 1 ? 3.0 : 3.5) * ((M * steps(i) * 8 + kWorkers - 1) / kWorkers));
+  }
+  return true;
+}
+static bool make_plan(const PackedMeta* metas, int n, int M, Plan& best) {
+  int k_slabs_min = metas[0].k_slabs;
+  for (int i = 1; i < n; ++i) k_slabs_min = std::min(k_slabs_min, (int)metas[i].k_slabs);
+  bool found = false;
+  for (int CS = 8; CS >= 1; CS >>= 1) {
+    if (CS > 1 && k_slabs_min < 2 * CS) continue;                    // at least one step of two slabs to a CTA
+    Plan q;
+    if (!plan_with(metas, n, M, CS, q)) continue;
+    if (!found || q.cost < best.cost) { best = q; found = true; }
+  }
+  return found;
+}
+// The plans of the last few shapes a thread has asked for (a call asks twice, and working one out takes about a microsecond).
+static bool plan(const PackedMeta* metas, int n, int M, Plan& q) {
+  struct Shape {
+    int dev, n, M, w_bits, k_slabs[kMaxLayers], N[kMaxLayers], k_pad[kMaxLayers];
+  };
+  struct Known {
+    Shape shape;
+    Plan plan;
+    bool found;
+  };
+  static thread_local Known known[8] = {};
+  static thread_local unsigned next = 0;
+  Shape sh = {};
+  if (cudaGetDevice(&sh.dev) != cudaSuccess) return false;
+  sh.n = n; sh.M = M; sh.w_bits = metas[0].w_bits;
+  for (int i = 0; i < n; ++i) { sh.k_slabs[i] = metas[i].k_slabs; sh.N[i] = metas[i].N; sh.k_pad[i] = metas[i].k_pad; }
+  for (const Known& k : known)
+    if (std::memcmp(&k.shape, &sh, sizeof(sh)) == 0) { q = k.plan; return k.found; }
+  const bool found = make_plan(metas, n, M, q);
+  Known& k = known[next++ % 8];
+  k.shape = sh; k.plan = q; k.found = found;
+  return found;
 }
 }  // namespace dcl
 
-// Whether n layers with one M go out as one launch of this kernel (with Y of y_type): at 3 to 16 rows, up to four layers, and
-// where it is the faster way.  Measured on one B200, us a call, what ran before / this kernel (rank 32 unless stated):
-//   4096 x 4096 alone            4 rows 19.9 / 12.0    8 rows 20.9 / 12.4    16 rows 21.8 / 15.9
-//   three of them                4 rows 28.8 / 21.0    8 rows 27.0 / 21.4    16 rows 27.4 / 27.1
-//   two of 4096 x 11008          4 rows 38.7 / 30.5    8 rows 32.4 / 31.2    16 rows 32.9 / 38.9
-//   two of 5120 x 13824, rank 64 4 rows 50.0 / 43.7    8 rows 45.7 / 44.6    16 rows 46.4 / 54.3
-//   three of 2048 x 2048         4 rows 14.3 / 11.9    8 rows 20.0 / 12.3    16 rows 20.6 / 14.4
-//   six of 4096 x 4096           4 rows 34.5 / 37.1    8 rows 35.2 / 37.8    16 rows 35.8 / 46.5
-// Up to eight rows one MMA multiplies sixteen weight columns with all tokens; from nine on it takes two, and the tensor pipe is
-// as busy as the conversion, so larger launches keep the kernels that share a prologue (11008 x 4096 alone, 16 rows: 29.9 / 32.4).
-// Three rows with ranks above 128 are level or worse in large launches (a 4064 / 10192 layer at rank 256 122.8 / 134.9, 4096 / 11008 126.6 /
-// 129.5; 2048 / 5632 87.3 / 62.3): the same line.
-// One and two rows keep the column-owner kernel (2 rows: 4096 x 4096 16.4 / 15.6, two of 4096 x 11008 26.0 / 30.3).
-constexpr long long kClusterMaxWeights = 30000000;        // K N over the layers, from nine rows on and at three with ranks above 128
+// Whether n layers with one M go out as one launch of this kernel: at 3 to 16 rows, up to four layers, wherever X_q fits.  Measured on one
+// B200, us a call in a chain of such calls over weights beyond L2, the same sums through two CTAs to an SM with a ring of each lane's own
+// pieces (before) / this kernel; for 16 rows the kernels that share a prologue, which took the larger of these calls / this kernel:
+//   4096 x 4096, rank 32 alone   4 rows 11.2 / 10.3   8 rows 11.4 / 10.5   16 rows 14.7 / 13.6
+//   three of them                4 rows 20.8 / 15.1   8 rows 21.3 / 15.6   16 rows 28.1 / 21.6
+//   two of 4096 x 11008          4 rows 30.3 / 25.3   8 rows 30.8 / 25.6   16 rows 33.1 / 31.6
+//   11008 x 4096 alone           4 rows 17.2 / 14.4   8 rows 18.4 / 15.4   16 rows 28.9 / 25.5
+//   two of 5120 x 13824, rank 64 4 rows 43.8 / 32.0   8 rows 44.5 / 33.0   16 rows 45.8 / 45.2
+//   the same, rank 256           3 rows 48.9 / 34.6   8 rows 53.2 / 36.3   16 rows 52.7 / 48.0
+//   2048 x 2048, rank 32 alone   4 rows 8.9 / 7.0;  rank 64, 16 rows 10.7 / 11.7 (the one size found where the smaller CTAs were faster)
+// One and two rows keep the column-owner kernel, whose launches several layers share bit for bit.
 int decode_cluster_max_layers() { return dcl::kMaxLayers; }
-bool decode_cluster_takes(const PackedMeta* metas, int n, int M, int y_type) {
+bool decode_cluster_takes(const PackedMeta* metas, int n, int M) {
   using namespace dcl;
   if (n < 1 || n > kMaxLayers || M < 3 || M > kRows) return false;
-  long long weights = 0;
-  int k_pad = 0;
-  for (int i = 0; i < n; ++i) {
-    if (!w_offsets_fit(metas[i])) return false;
-    weights += (long long)metas[i].K64 * metas[i].N;
-    k_pad = std::max(k_pad, (int)metas[i].k_pad);
-  }
-  if ((M > 8 || (M == 3 && k_pad > 128)) && weights > kClusterMaxWeights) return false;
-  const Plan q = plan(metas, n, M);
-  if (q.smem > (size_t)kSmemOne) return false;
-  return entry_of(metas[0].w_bits, M > 8 ? 2 : 1, y_type == kYMXINT8).resident(q.CS, q.two) >= n;
+  Plan q;
+  return plan(metas, n, M, q);
 }
 
 cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* metas, int n, void* scratch, int* counts, DeviceStatus* st,
@@ -803,57 +974,22 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
   using namespace dcl;
   if (n < 1 || n > kMaxLayers) return cudaErrorInvalidValue;
   const int M = calls[0].M;
-  const Plan q = plan(metas, n, M);
-  const int CS = q.CS;
+  Plan q;
+  if (!plan(metas, n, M, q)) return cudaErrorInvalidConfiguration;
   Params p;
   p.n = n; p.M = M; p.status = st; p.x_type = x_type; p.y_type = y_type;
   p.a_bits = metas[0].a_bits; p.lr_bits = metas[0].lr_bits; p.exp_min = metas[0].exp_min; p.exp_max = metas[0].exp_max;
   p.wait_limit = wait_limit_cycles();
-  const bool stall = take_stall(kFamDecode);
-  p.stall = stall ? 1 : 0;
-  p.slabs_max = q.slabs_max;
-  p.off_red[0] = q.off_red[0]; p.off_red[1] = q.off_red[1];
-  p.off_xq = q.off_xq; p.off_xe = q.off_xe; p.off_tpart = q.off_tpart; p.off_ring = q.off_ring;
-  const bool yq = y_type == kYMXINT8;
-  const Entry kernel = entry_of(metas[0].w_bits, M > 8 ? 2 : 1, yq);
-  // No more clusters than the device holds at a time (they wait for the T_q of others).  With two CTAs to an SM the last few
-  // places are left free: 4096 x 4096, 4 rows, 14.3 us with 32 of 33 clusters and 12.0 with 28; larger launches lose more by the
-  // longer ranges of columns (two of 4096 x 11008: 35.5 with 28, 30.5 with 32, 34 with 33).
-  int budget = kernel.resident(CS, q.two);
+  p.stall = take_stall(kFamDecode) ? 1 : 0;
+  p.steps_max = q.steps_max;
+  p.slots = q.slots;
+  p.off_red = q.off_red; p.red_bytes = q.red_bytes;
+  p.off_xq = q.off_xq; p.off_xe = q.off_xe; p.off_tpart = q.off_tpart; p.off_trecv = q.off_trecv; p.off_tq = q.off_tq; p.off_ring = q.off_ring;
   // The clusters that form a layer's T wait for one another, and all others of the layer, placed after them, wait for these.  A launch
-  // that runs beside others may get its places one by one, and until all of a layer's T clusters have theirs the ones that do
-  // cannot leave.  At most a quarter of the places go to such clusters, so that four launches on as many streams cannot hold
-  // each other up for good; where that would cost too much (one CTA to an SM: 13824 x 2048 of rank 256, 4 rows, 40.6 us instead of 21.8)
-  // the launch is a cooperative one, which is placed as a whole or not yet (some 1 us more).  With two CTAs to an SM the
-  // quarter costs nothing (rank 256, 4 rows: 4096 x 4096 14.4 / 14.3, 2048 x 5632 14.0 / 13.5; up to rank 128 nothing changes).
-  const int most = std::max(budget / 4, 1);
-  bool cooperative = false;
-  constexpr long long kFewWeights = 30000000;
-  long long weights = 0;
-  for (int i = 0; i < n; ++i) weights += (long long)metas[i].K64 * metas[i].N;
-  if (q.two && budget >= 8) budget = weights <= kFewWeights ? budget * 7 / 8 : budget / 4 * 4;
-  if (budget < n) return cudaErrorInvalidConfiguration;
-  // clusters per layer: each has one, the others go one by one where the time (column octets x steps of K) is longest, as long
-  // as every warp of a cluster has an octet
-  int clusters[kMaxLayers];
-  double per_oct[kMaxLayers];
-  int total = 0;
-  for (int i = 0; i < n; ++i) {
-    clusters[i] = 1;
-    per_oct[i] = 0.5 * ((metas[i].k_slabs + CS - 1) / CS) + 1.0;
-    ++total;
-  }
-  while (total < budget) {
-    int best = -1;
-    double worst = 0.0;
-    for (int i = 0; i < n; ++i) {
-      const double t = (double)(metas[i].N / 8) / clusters[i] * per_oct[i];
-      if (clusters[i] < metas[i].N / (yq ? 16 : 8) / kWarps && t > worst) { worst = t; best = i; }
-    }
-    if (best < 0) break;
-    ++clusters[best];
-    ++total;
-  }
+  // that runs beside others may get its places one by one, and until all of its T clusters have theirs the ones that do
+  // cannot leave.  At most a quarter of the places go to such clusters (one to each layer at least), so that four launches on as many
+  // streams cannot hold each other up for good.
+  // (plan_with sees to it.)
   int begin = 0;
   size_t t_off = 0;
   for (int i = 0; i < kMaxLayers; ++i) {
@@ -868,20 +1004,18 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
     ly.y_extent = y_bytes(y_type, (size_t)M, (size_t)m.N);
     if (kDebugBounds) ly.y_extent -= std::min(ly.y_extent, debug_y_shrink());
     ly.w_extent = m.off_b - m.off_w;
-    ly.K = m.K; ly.N = m.N; ly.k_pad = m.k_pad; ly.k_slabs = m.k_slabs; ly.r_blocks = m.r_blocks;
+    ly.K = m.K; ly.N = m.N; ly.k_pad = m.k_pad; ly.k_slabs = m.k_slabs; ly.r_blocks = m.r_blocks; ly.tiles = m.n_tiles;
     ly.cluster_begin = begin;
-    ly.clusters = clusters[g];
+    ly.clusters = q.clusters[g];
     ly.tq = static_cast<uint8_t*>(scratch) + t_off;
     ly.tcount = counts + 2 * g;
     // the warps of an owner count their 16-blocks of T in
-    ly.t_expect = M * m.r_blocks + (stall ? 1 : 0);
-    const int formers = q.two ? std::min(clusters[g], most) : clusters[g];
-    ly.t_blocks = (m.r_blocks + formers - 1) / formers;
-    if (i < n && std::min(formers, (int)m.r_blocks) > most) cooperative = true;
+    ly.t_expect = M * m.r_blocks + p.stall;
+    ly.t_blocks = q.t_blocks[g]; ly.t_clusters = q.t_clusters[g]; ly.t_tiles = q.t_tiles[g];
     if (i < n) t_off += decode_cluster_scratch_bytes(m);
-    if (i < n) begin += clusters[g];
+    if (i < n) begin += q.clusters[g];
   }
-  return kernel.go(p, total, CS, q.two, q.smem, cooperative, s);
+  return entry_of(metas[0].w_bits, M > 8 ? 2 : 1, q.local).go(p, q.total, q.CS, q.smem, s);
 }
 
 }  // namespace lqer
