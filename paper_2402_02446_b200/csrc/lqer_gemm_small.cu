@@ -15,13 +15,13 @@
 //
 // Work items are (layer, 256-column tile, K chunk).  The chunks of a tile are fixed by the shape alone (so a
 // result never depends on the number of SMs or on which layers share a launch); each chunk is summed from
-// zero in tensor memory and, if a tile has more than one, leaves its fp32 partial in scratch; the CTA whose
-// partial arrives last adds the chunks in chunk order and writes Y.  Nothing waits for another CTA.
+// zero in tensor memory and, if a tile has more than one, leaves its fp32 partial in scratch; the CTAs whose last chunk is of one
+// tile add its chunks up together, in chunk order, a share of the rows each (finish_tile).  None depends on another's help.
 // Roles per CTA:
 //   warp 0      producer: bulk copies of packed weight tiles (issued before the dependency wait: weights
 //               depend on no earlier kernel) and TMA loads of activation tiles (after it)
 //   warp 1      tensor memory allocation, MMA issue (the whole warp runs the loop, one elected lane issues)
-//   warps 2-5   epilogue (tcgen05.ld, Y or partial sums, the last-arriver reduction)
+//   warps 2-5   epilogue (tcgen05.ld, Y or partial sums)
 //   warps 6-29  converters in three groups of 256 threads (a weight column each); group g converts the steps
 //               with index = g (mod 3)
 // Two rings: PK slots hold a batch {four activation tiles, two halves of four packed weight tiles}, with a barrier for the
@@ -91,6 +91,155 @@ struct TensorMaps {
   CUtensorMap m[MAX_LAYERS];   // Xcat of each layer, bf16 [M, K64 + k_pad], box x_rows x 64
 };
 
+// A tile's counter: chunks that have arrived, shares of the rows that have been taken, CTAs that have left; and whether one of them
+// took a share and left before all chunks had arrived.
+constexpr int kTaken = 1 << 8, kLeft = 1 << 20, kGaveUp = (int)0x80000000u;
+__device__ __forceinline__ int arrived(int v) { return v & 0xFF; }
+__device__ __forceinline__ int taken(int v) { return (v >> 8) & 0xFFF; }
+__device__ __forceinline__ int left(int v) { return (v >> 20) & 0x7FF; }
+// Rows [lo, hi) of a tile from its chunks' partial sums, by `nthreads` threads (a multiple of 64): four columns to a thread.
+__device__ __forceinline__ void finish_rows(const Params& p, const Layer& ly, const Item& c, int lo, int hi, int tid, int nthreads) {
+  const int col0 = c.tile * BN, c4 = (tid & 63) * 4, step = nthreads >> 6;
+  const bool quad_ok = col0 + c4 < ly.N;                                   // N is a multiple of 8: the quad is whole
+  const size_t chunk_stride = (size_t)p.M * BN;
+  const float* p0 = ly.partials + (size_t)c.tile * ly.chunks * chunk_stride + c4;
+  for (int t0 = lo + (tid >> 6); t0 < hi; t0 += 2 * step) {
+    float4 v[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    for (int cb = 0; cb < ly.chunks; cb += 4) {
+      float4 t[2][4];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (cb + k < ly.chunks && t0 + u * step < hi)
+            t[u][k] = __ldcg(reinterpret_cast<const float4*>(p0 + (size_t)(cb + k) * chunk_stride + (size_t)(t0 + u * step) * BN));
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (cb + k < ly.chunks && t0 + u * step < hi) { v[u].x += t[u][k].x; v[u].y += t[u][k].y; v[u].z += t[u][k].z; v[u].w += t[u][k].w; }
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (t0 + u * step < hi) store_row_quad(p, ly, t0 + u * step, col0, c4, quad_ok, v[u]);
+  }
+}
+// Adds a tile's chunks up, by all threads of a CTA or by its epilogue.  A CTA takes a share of the rows as its last chunk arrives and
+// waits for the other chunks, but not for long: if it does so in vain, it says so and leaves.  The CTA whose chunk arrives last
+// knows by that which shares are taken and does the others, or all of the rows if one has left (what others do of them at the
+// same time is the same).  So none depends on another's progress.  The last one to leave puts the counter back to zero.
+// With the CTA of the last chunk alone, the sums of 64 rows and 7 chunks took 9 us, 4 now; 4096 x 4096, 20 / 64 / 128 tokens, the call
+// 22.3 / 29.2 / 40.8 us before and 20.1 / 25 / 29.5 now, 11008 x 4096 30.5 / 39.1 / 57.9 and 27.9 / 34 / 44.4.
+constexpr int kFinishWait = 40000;             // cycles
+// old: the counter before this CTA's chunk arrived.
+template <bool WHOLE_CTA>
+__device__ __forceinline__ void finish_tile(const Params& p, const Item& c, int old, int tid, int* flag) {
+  const Layer& ly = p.L[c.layer];
+  int* count = ly.counters + c.tile;
+  // shares of some 96 rows of partial sums; where that makes one of them, the CTA of the last chunk is through sooner than the first's
+  const int shares = min((p.M * ly.chunks + 95) / 96, ly.chunks), rows = (p.M + shares - 1) / shares, share = shares > 1 ? taken(old) : ly.chunks;
+  const bool last = arrived(old) == ly.chunks - 1;
+  bool ok = true;
+  if (WHOLE_CTA && !last && share < shares) {  // (an epilogue comes here with the last chunk only)
+    if (tid == 0) {
+      int v = *reinterpret_cast<volatile int*>(count);
+      for (const long long t0 = clock64(); arrived(v) != ly.chunks && clock64() - t0 < kFinishWait;) v = *reinterpret_cast<volatile int*>(count);
+      *flag = arrived(v) == ly.chunks || arrived(atomicOr(count, kGaveUp)) == ly.chunks ? 1 : 0;
+    }
+    __syncthreads();
+    ok = *flag != 0;
+  }
+  if (tid == 0 && left(atomicAdd(count, kLeft)) + 1 == ly.chunks) *count = 0;
+  __threadfence();
+  const int lo = last && (old < 0 || shares == 1) ? 0 : share * rows, hi = last ? p.M : min(p.M, (share + 1) * rows);
+  if (ok && lo < hi) finish_rows(p, ly, c, lo, hi, tid, WHOLE_CTA ? NUM_THREADS : 128);
+}
+__device__ __noinline__ void finish_by_epilogue(const Params& p, const Item c, int old, int tid) { finish_tile<false>(p, c, old, tid, nullptr); }
+
+// bf16_rn by the conversion instruction, which has one NaN for all.
+__device__ __forceinline__ uint16_t bf16_rn_cvt(uint32_t v) {
+  uint16_t h;
+  asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(h) : "f"(__uint_as_float(v)));
+  return (v & 0x7FFFFFFFu) > 0x7F800000u ? (uint16_t)((v >> 16) | 0x40u) : h;
+}
+// A finished chunk from its accumulator to Y or to the partial sums, by the epilogue's warps: warp q of them has a quarter of the
+// lanes; a lane holds a weight column, its columns are the tokens.  Each warp is alone on its scheduler by then and bound by its own
+// instructions, so bf16 is the conversion's (7 us for 64 tokens with bf16_rn, 4 now), and a partial sum's address is a constant away
+// from the one before.  (All 28 warps at the end took no less time.)
+template <int NT>
+__device__ __forceinline__ void store_chunk(const Params& p, const Item& c, uint32_t tmem_base, int acc, int q) {
+  const Layer& ly = p.L[c.layer];
+  const int lane = threadIdx.x & 31, M = p.M, Nl = ly.N, y_type = p.y_type;
+  const int halves = c.tile * BN + 128 < Nl ? 2 : 1;
+  const uint32_t t_base = tmem_base + ((uint32_t)(q * 32) << 16) + acc * 2 * NT;
+  if (ly.chunks > 1) {
+    float* dst0 = ly.partials + (size_t)(c.tile * ly.chunks + c.chunk) * M * BN + q * 32 + lane;
+#pragma unroll 1
+    for (int h = 0; h < halves; ++h) {
+      float* dst = dst0 + h * 128;
+#pragma unroll 1
+      for (int t0 = 0; t0 < M; t0 += 16, dst += 16 * BN) {
+        uint32_t r[16];
+        tmem_ld16(t_base + h * NT + t0, r);
+        tmem_ld_wait();
+        if (kDebugBounds && !LQER_IN_BOUNDS(p.status, (size_t)(dst - ly.partials) * 4, ((size_t)(min(16, M - t0) - 1) * BN + 1) * 4, ly.partial_extent, 704)) continue;
+        if (t0 + 16 <= M) {
+#pragma unroll
+          for (int t = 0; t < 16; ++t) dst[t * BN] = __uint_as_float(r[t]);
+        } else {
+#pragma unroll
+          for (int t = 0; t < 16; ++t)
+            if (t0 + t < M) dst[t * BN] = __uint_as_float(r[t]);
+        }
+      }
+    }
+    return;
+  }
+  [[maybe_unused]] const uint8_t* base = static_cast<const uint8_t*>(ly.Y);
+  [[maybe_unused]] const size_t extent = ly.y_extent;
+  const int size = y_type == kYBF16 ? 2 : y_type == kYMXINT8 ? 1 : 4;
+  const size_t step = (size_t)Nl * size, step_e = (size_t)Nl / 16;
+#pragma unroll 1
+  for (int h = 0; h < halves; ++h) {
+    const int col = c.tile * BN + h * 128 + q * 32 + lane;
+    uint8_t* dst = static_cast<uint8_t*>(ly.Y) + (size_t)col * size;
+    uint8_t* dst_e = static_cast<uint8_t*>(ly.Y) + (size_t)M * Nl + col / 16;            // MXINT8: the exponent bytes
+#pragma unroll 1
+    for (int t0 = 0; t0 < M; t0 += 16) {
+      uint32_t r[16];
+      tmem_ld16(t_base + h * NT + t0, r);
+      tmem_ld_wait();
+      const int rows = M - t0;
+      if (y_type == kYMXINT8) {
+        // sixteen lanes hold a 16-block of a token's row (N is a multiple of 16 here)
+#pragma unroll
+        for (int t = 0; t < 16; ++t, dst += step, dst_e += step_e) {
+          const float v = __uint_as_float(r[t]);
+          float amax = fmaxf(fabsf(v), 0.0f);            // (a NaN counts as zero)
+#pragma unroll
+          for (int d = 1; d < 16; d <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, d));
+          const int e = block_exponent(amax, p.exp_min, p.exp_max);
+          if (t < rows && col < Nl && LQER_IN_BOUNDS(p.status, dst_e - base, 1, extent, 703)) {
+            *dst = (uint8_t)quant_mantissa(v, e, p.a_bits);
+            if ((lane & 15) == 0) *dst_e = (uint8_t)(e + 127);
+          }
+        }
+      } else if (col < Nl) {
+        if (size == 2) {
+#pragma unroll
+          for (int t = 0; t < 16; ++t, dst += step)
+            if (t < rows && LQER_IN_BOUNDS(p.status, dst - base, 2, extent, 701)) *reinterpret_cast<uint16_t*>(dst) = bf16_rn_cvt(r[t]);
+        } else {
+#pragma unroll
+          for (int t = 0; t < 16; ++t, dst += step)
+            if (t < rows && LQER_IN_BOUNDS(p.status, dst - base, 4, extent, 704)) *reinterpret_cast<uint32_t*>(dst) = r[t];
+        }
+      }
+      __syncwarp();
+    }
+  }
+}
+
 // The batch that starts with slab s: up to BATCH slabs of weights, or two slabs of B_q (8-bit mantissas: eight blocks of 16
 // ranks, 16 KB, then their exponent bytes).
 __device__ __forceinline__ int batch_end(int s, int s_hi, int k_slabs) {
@@ -109,7 +258,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BARS);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::NUM_BARS);
   int* last_flag = reinterpret_cast<int*>(tmem_slot + 1);
-  int* deferred = reinterpret_cast<int*>(tmem_slot + 6);       // item whose chunks the whole CTA adds up at the end, or -1
+  int* at_end = reinterpret_cast<int*>(tmem_slot + 6);         // item whose chunks the whole CTA helps to add up at the end, or -1; its counter's old value
   volatile WaitState* abort_flag = reinterpret_cast<volatile WaitState*>(tmem_slot + 2);
 
   const uint32_t bar0 = smem_u32(bars);
@@ -131,7 +280,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     for (int a = 0; a < 2; ++a) { mbar_init(acc_full(a), 1); mbar_init(acc_empty(a), 4); }
     abort_flag->abort = 0;
     abort_flag->limit = p.wait_limit;
-    *deferred = -1;
+    at_end[0] = -1;
     fence_barrier_init();
     fence_proxy_async_smem();
   }
@@ -303,77 +452,31 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
       const int acc = tile_it % C::ACCS;
       if (!mbar_wait<true>(acc_full(acc), (tile_it / C::ACCS) & 1, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      const bool direct = ly.chunks == 1;
-      const int Nl = ly.N, M = p.M, y_type = p.y_type;
-#pragma unroll 1
-      for (int h = 0; h < 2; ++h) {
-        const int ccol = h * 128 + q * 32 + lane, col = it.tile * BN + ccol;
-        if (it.tile * BN + h * 128 >= Nl) break;
-        // where token 0 of this column goes, and the step from token to token, in bytes (an address per store worked out from
-        // the parameters made the 64-token bf16 epilogue 11 us long)
-        const int size = direct && y_type == kYBF16 ? 2 : direct && y_type == kYMXINT8 ? 1 : 4;
-        const size_t step = (size_t)(direct ? Nl : BN) * size;
-        uint8_t* dst = direct ? static_cast<uint8_t*>(ly.Y) + (size_t)col * size
-                              : reinterpret_cast<uint8_t*>(ly.partials + (size_t)(it.tile * ly.chunks + it.chunk) * M * BN + ccol);
-        [[maybe_unused]] const uint8_t* base = direct ? static_cast<const uint8_t*>(ly.Y) : reinterpret_cast<const uint8_t*>(ly.partials);
-        [[maybe_unused]] const size_t extent = direct ? ly.y_extent : ly.partial_extent;
-        uint8_t* dst_e = static_cast<uint8_t*>(ly.Y) + (size_t)M * Nl + col / 16;      // MXINT8: the exponent bytes
-        const size_t step_e = (size_t)Nl / 16;
-#pragma unroll 1
-        for (int t0 = 0; t0 < M; t0 += 16) {
-          uint32_t r[16];
-          tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + acc * 2 * NT + h * NT + t0, r);
-          tmem_ld_wait();
-          if (direct && y_type == kYMXINT8) {
-            // sixteen lanes hold a 16-block of a token's row (N is a multiple of 16 here)
-#pragma unroll
-            for (int t = 0; t < 16; ++t, dst += step, dst_e += step_e) {
-              const float v = __uint_as_float(r[t]);
-              float amax = fmaxf(fabsf(v), 0.0f);            // (a NaN counts as zero)
-#pragma unroll
-              for (int d = 1; d < 16; d <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, d));
-              const int e = block_exponent(amax, p.exp_min, p.exp_max);
-              if (t0 + t < M && col < Nl && LQER_IN_BOUNDS(p.status, dst_e - base, 1, extent, 703)) {
-                *dst = (uint8_t)quant_mantissa(v, e, p.a_bits);
-                if ((lane & 15) == 0) *dst_e = (uint8_t)(e + 127);
-              }
-            }
-          } else if (!direct || col < Nl) {
-            const int left = M - t0;
-            if (size == 2) {
-#pragma unroll
-              for (int t = 0; t < 16; ++t, dst += step)
-                if (t < left && LQER_IN_BOUNDS(p.status, dst - base, 2, extent, 701))
-                  *reinterpret_cast<uint16_t*>(dst) = (uint16_t)bf16_rn(__uint_as_float(r[t]));
-            } else {
-#pragma unroll
-              for (int t = 0; t < 16; ++t, dst += step)
-                if (t < left && LQER_IN_BOUNDS(p.status, dst - base, 4, extent, 704)) *reinterpret_cast<uint32_t*>(dst) = r[t];
-            }
-          }
-          __syncwarp();
-        }
-      }
+      store_chunk<NT>(p, it, tmem_base, acc, q);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty(acc));
-      if (!direct) {
-        // count this chunk in; whoever brings the last partial of the tile adds them all up, in chunk order
+      if (ly.chunks > 1) {
+        // count this chunk in; the CTA's last one is seen to by all of its threads at the end (every other role is about to fall
+        // idle), another one by the epilogue where it is the tile's last to arrive
         __threadfence();
         epilogue_barrier();
-        if (et == 0) *last_flag = (atomicAdd(ly.counters + it.tile, 1) == ly.chunks - 1) ? 1 : 0;
-        epilogue_barrier();
-        if (*last_flag != 0) {
-          if (i + num_ctas >= num_items) {
-            // the CTA's last item: every other role is about to fall idle, so the whole CTA adds the chunks up at the end
-            if (et == 0) *deferred = i;
-          } else {
-            __threadfence();
-            reduce_tile(p, ly, it.tile, et, 128);
-            if (et == 0) ly.counters[it.tile] = 0;    // zero again for the next call
+        if (i + num_ctas >= num_items) {
+          if (et == 0) {
+            at_end[0] = i;
+            at_end[1] = atomicAdd(ly.counters + it.tile, 1 + kTaken);
           }
+          break;
         }
-        epilogue_barrier();                         // last_flag may be rewritten only after everyone has read it
+        if (et == 0) {
+          const int old = atomicAdd(ly.counters + it.tile, 1);
+          *last_flag = old;
+          if (arrived(old) != ly.chunks - 1 && left(atomicAdd(ly.counters + it.tile, kLeft)) + 1 == ly.chunks) ly.counters[it.tile] = 0;
+        }
+        epilogue_barrier();
+        const int old = *last_flag;
+        epilogue_barrier();                         // everyone has read it
+        if (arrived(old) == ly.chunks - 1) finish_by_epilogue(p, it, old, et);
       }
     }
   } else {
@@ -480,12 +583,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
 
   // ------------------------------------------------------------------ teardown
   __syncthreads();                      // every role is done (or has given up): the flags below are final for this CTA
-  if (*deferred >= 0 && abort_flag->abort == 0) {
-    const Item it = item_of(p, *deferred);
-    __threadfence();
-    reduce_tile(p, p.L[it.layer], it.tile, threadIdx.x, NUM_THREADS);
-    if (threadIdx.x == 0) p.L[it.layer].counters[it.tile] = 0;     // zero again for the next call
-  }
+  if (at_end[0] >= 0 && abort_flag->abort == 0) finish_tile<true>(p, item_of(p, at_end[0]), at_end[1], threadIdx.x, last_flag);
   if (abort_flag->abort != 0) {
     const long long t0 = clock64();
     while (clock64() - t0 < 400000) { }
@@ -562,10 +660,13 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
   int group_chunks = 1;
   if (n > 1) {
     // The cut that makes (rounds of items over the SMs) x (slabs per item + what an item costs beside its slabs) smallest,
-    // a function of the shapes alone.  This file's kernel runs one CTA per SM and an item's partial sums cost it about four
-    // slabs' worth of time; the register-operand kernel runs two CTAs per SM, an item each at a time, and an item costs it
-    // about ten (activation copy, rank term, partial sums).
-    const int ctas = use_mma ? 2 * 148 : 148, extra = use_mma ? 10 : 4;
+    // a function of the shapes alone.  The register-operand kernel runs two CTAs per SM, an item each at a time, and an item costs
+    // it about ten slabs' worth of time (activation copy, rank term, partial sums).  This file's kernel runs one CTA per SM; in
+    // slabs' time (0.4 us) a tile in one piece costs it 4 + M / 8 (two- or four-byte stores of a column each), a chunk 5 + M / 20 and
+    // then 14 until the tile's chunks are added up, which keep the CTA from its next item.  (At four slabs for any item two layers of
+    // 4096 x 11008, 86 tiles, were cut into three chunks each, two rounds: 54 / 81 / 133 us with 32 / 64 / 128 tokens, 41 / 46 /
+    // 60 in one piece.)
+    const int ctas = use_mma ? 2 * 148 : 148;
     long best = -1;
     for (int c = 1; c <= 16; ++c) {
       long items = 0, len = 0;
@@ -575,7 +676,7 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
         items += (long)small_gemm_col_tiles(m) * ci;
         len = std::max(len, (long)(m.k_slabs + ci - 1) / ci);
       }
-      const long cost = ((items + ctas - 1) / ctas) * (len + extra);
+      const long cost = ((items + ctas - 1) / ctas) * (len + (use_mma ? 10 : c > 1 ? 19 + M / 20 : 4 + M / 8));
       if (best < 0 || cost < best) { best = cost; group_chunks = c; }
     }
   }

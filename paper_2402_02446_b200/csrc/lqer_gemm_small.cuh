@@ -1,5 +1,5 @@
 // What the two small-batch GEMM kernels share: the work items (layer, 256-column tile, K chunk), the parameters of a
-// launch, and the sum of a tile's chunks by the CTA whose partial arrives last (paper Section 3.1 / 3.2:
+// launch, and the sum of a tile's chunks (here by one CTA, the register-operand kernel's way) (paper Section 3.1 / 3.2:
 // Y = [X_q | T_q] . [W_q ; B_q] for few tokens; Section 2.1: the layer is memory bound on its weights there).
 #pragma once
 #include "lqer_common.cuh"
@@ -80,6 +80,24 @@ __device__ __forceinline__ void store_y4(void* Y, size_t idx, float4 v, int y_ty
     *reinterpret_cast<float4*>(static_cast<float*>(Y) + idx) = v;
 }
 
+// Columns col0 + c4 .. + 3 of token tk's row of Y.  MXINT8: four adjacent lanes hold a 16-block of the row, so a whole warp calls it.
+__device__ __forceinline__ void store_row_quad(const Params& p, const Layer& ly, int tk, int col0, int c4, bool quad_ok, float4 v) {
+  if (p.y_type == kYMXINT8) {
+    uint32_t m8;
+    uint2 unused;
+    int e;
+    quantize_quad(v, p.a_bits, p.exp_min, p.exp_max, e, m8, unused);
+    if (tk < p.M && quad_ok && LQER_IN_BOUNDS(p.status, (size_t)p.M * ly.N + ((size_t)tk * ly.N + col0 + c4) / 16, 1, ly.y_extent, 702)) {
+      uint8_t* yq = static_cast<uint8_t*>(ly.Y);
+      const size_t idx = (size_t)tk * ly.N + col0 + c4;
+      *reinterpret_cast<uint32_t*>(yq + idx) = m8;
+      if ((c4 & 15) == 0) yq[(size_t)p.M * ly.N + idx / 16] = (uint8_t)(e + 127);
+    }
+  } else if (tk < p.M && quad_ok) {
+    store_y4(ly.Y, (size_t)tk * ly.N + col0 + c4, v, p.y_type, p.status, ly.y_extent);
+  }
+}
+
 // Y of one 256-column tile = the sum of its chunks' partials, in chunk order (the same sum whoever computes it), by
 // `nthreads` threads (a multiple of 64): a thread per four columns, nthreads / 64 token rows per pass; the chunk loads
 // of four rows are in flight together.
@@ -108,24 +126,7 @@ __device__ __forceinline__ void reduce_tile(const Params& p, const Layer& ly, in
           if (cb + c < ly.chunks) { v[u].x += t[u][c].x; v[u].y += t[u][c].y; v[u].z += t[u][c].z; v[u].w += t[u][c].w; }
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int tk = t0 + rstep * u;
-      if (p.y_type == kYMXINT8) {
-        // four adjacent lanes hold a 16-block of the row (every lane of the warp takes part in the exchange)
-        uint32_t m8;
-        uint2 unused;
-        int e;
-        quantize_quad(v[u], p.a_bits, p.exp_min, p.exp_max, e, m8, unused);
-        if (tk < p.M && quad_ok && LQER_IN_BOUNDS(p.status, (size_t)p.M * ly.N + ((size_t)tk * ly.N + col0 + c4) / 16, 1, ly.y_extent, 702)) {
-          uint8_t* yq = static_cast<uint8_t*>(ly.Y);
-          const size_t idx = (size_t)tk * ly.N + col0 + c4;
-          *reinterpret_cast<uint32_t*>(yq + idx) = m8;
-          if ((c4 & 15) == 0) yq[(size_t)p.M * ly.N + idx / 16] = (uint8_t)(e + 127);
-        }
-      } else if (tk < p.M && quad_ok) {
-        store_y4(ly.Y, (size_t)tk * ly.N + col0 + c4, v[u], p.y_type, p.status, ly.y_extent);
-      }
-    }
+    for (int u = 0; u < 4; ++u) store_row_quad(p, ly, t0 + rstep * u, col0, c4, quad_ok, v[u]);
   }
 }
 
