@@ -21,7 +21,7 @@ namespace psm {
 using mf::frag_offset;
 
 constexpr int kRows = 16;                 // rows per CTA = one MMA M tile
-constexpr int kThreads = 256;
+constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kStepCols = 1024;           // columns of X a CTA quantises per step (shared-memory panel)
 constexpr int kXqStride = kStepCols + 16; // bytes per row of the int8 panel (+16: conflict-free fragment loads)
@@ -70,13 +70,15 @@ __device__ __forceinline__ double ld_dsmem(const double* local, uint32_t cta) {
   return v;
 }
 
-// TPW: rank tiles (8 columns) a warp owns: 1 for ranks up to 64, 2 up to 128, 4 up to 256.
-// The kernel is a chain of memory latencies, so a round requests as much as the registers hold: the A_q words of UB blocks
-// (those of a CTA's first blocks before it waits for the kernel before, on which they do not depend) and eight quads
-// of X per thread.  With four blocks and four quads a round it took 15 - 29 us at K = 5120 - 13824 and ranks 32 and 64, of
-// which 5 - 10 us were rounds of A_q.
+// TPW: rank tiles (8 columns) a warp owns: 1 for ranks up to 128, 2 up to 256.
+// The kernel is a chain of memory latencies and of short stretches of instructions that only a CTA's own warps can hide: sixteen of them,
+// two CTAs an SM, in 64 registers a thread, and with these a round requests the A_q words of UB blocks (those of a CTA's
+// first blocks before it waits for the kernel before, on which they do not depend) and eight quads of X per thread.  With eight
+// warps of 128 registers and 16 blocks a round it took 14 - 21 us at 64 rows, K = 5120 - 13824 and rank 32 (5 - 9 of them to
+// quantise, 2 - 5 for the products); the layer's four calls with their GEMMs 172 us, 159 now (4096 / 11008: 140 and 128; rank 256
+// 269 with the GEMM's cut of then, 210 now; with four quads of X a round 236).
 template <int TPW>
-__global__ void __launch_bounds__(kThreads, TPW == 4 ? 1 : 2) prologue_small_kernel(const __grid_constant__ Params p) {
+__global__ void __launch_bounds__(kThreads, 2) prologue_small_kernel(const __grid_constant__ Params p) {
   __shared__ __align__(16) uint8_t s_xq[kRows * kXqStride];
   __shared__ int8_t s_xe[kRows][kStepCols / 16];
   __shared__ double s_part[kWarps][kRows * 8];        // warps that share a rank tile meet here (TPW == 1)
@@ -106,7 +108,7 @@ __global__ void __launch_bounds__(kThreads, TPW == 4 ? 1 : 2) prologue_small_ker
   const size_t plane = (size_t)(ly.K64 / 64 + (k_pad + 63) / 64) * 256;      // fragment order: bytes of one plane
   const bool active = has_rank && (NT >= kWarps || warp < NT * WPN);
   const int bias = -127 - (p.a_bits - 2) - (p.lr_bits - 2);   // exponent bytes carry +127
-  constexpr int UB = TPW == 1 ? 16 : TPW == 2 ? 8 : 4;
+  constexpr int UB = TPW == 1 ? 8 : 4;
   const int b_first = NT >= kWarps ? 0 : warp / NT;
   const int b_step = NT >= kWarps ? 1 : WPN;
   const int nt0 = NT >= kWarps ? warp : warp % NT;
@@ -401,17 +403,14 @@ cudaError_t launch_prologue_small(const SmallPrologueLayer* layers, int n, int M
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   static OncePerDevice once;
-  const cudaError_t e = once.run([] {                    // 25 KB of static shared memory + up to 32 KB of partial sums
+  const cudaError_t e = once.run([] {                    // 34 KB of static shared memory + up to 32 KB of partial sums
     cudaError_t r = cudaFuncSetAttribute(prologue_small_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRows * 256 * 8);
     if (r == cudaSuccess) r = cudaFuncSetAttribute(prologue_small_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRows * 256 * 8);
-    if (r == cudaSuccess) r = cudaFuncSetAttribute(prologue_small_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRows * 256 * 8);
     return r;
   });
   if (e != cudaSuccess) return e;
   LaunchScope scope(kFamPrologue, s);
-  if (max_kpad <= 64) return cudaLaunchKernelEx(&cfg, prologue_small_kernel<1>, p);
-  if (max_kpad <= 128) return cudaLaunchKernelEx(&cfg, prologue_small_kernel<2>, p);
-  return cudaLaunchKernelEx(&cfg, prologue_small_kernel<4>, p);
+  return max_kpad <= 128 ? cudaLaunchKernelEx(&cfg, prologue_small_kernel<1>, p) : cudaLaunchKernelEx(&cfg, prologue_small_kernel<2>, p);
 }
 
 }  // namespace lqer
