@@ -357,13 +357,15 @@ cudaError_t launch_prologue_small(const SmallPrologueLayer* layers, int n, int M
   p.a_bits = m0.a_bits; p.lr_bits = m0.lr_bits; p.exp_min = m0.exp_min; p.exp_max = m0.exp_max;
   const int rgroups = (M + kRows - 1) / kRows;
   // A CTA's chain (its columns of X, then its blocks of A_q) is as long as its range, and 16 ranges leave most SMs without
-  // one at few rows: a range is shared by a cluster, up to 200 CTAs in the launch (384 take longer than 192), down to two
-  // blocks a CTA.  16 rows, K = 13824, rank 64: each of the two parts took 9 us with one CTA per range; the call with its
-  // GEMM 46 us, with eight 34.  A function of the shapes alone.
+  // one at few rows: a range is shared by a cluster, up to two CTAs an SM in the launch, down to two blocks a CTA; clusters of eight only up
+  // to 200 CTAs.  16 rows, K = 13824, rank 64: each of the two parts took 9 us with one CTA per range; the call with its
+  // GEMM 46 us, with eight 34.  Up to 200 / up to 296 CTAs in any clusters, us a call with its GEMM: 64 rows, 13824 x 5120, rank 64 39.8 / 35.9;
+  // 11008 x 4096, rank 256 51.7 / 39.9; 128 rows, 13824 x 5120 58.2 / 47.9; but 20 rows, 4096 x 4096, 128 CTAs in fours / 256 in
+  // eights 19.1 / 24.0, 11008 x 4096 26.8 / 31.3.  A function of the shapes alone.
   int all = 0;
   for (int i = 0; i < n; ++i) all += rgroups * prologue_small_ranges(*layers[i].meta, M);
   p.shares = 8;
-  while (p.shares > 1 && all * p.shares > 200) p.shares >>= 1;
+  while (p.shares > 1 && all * p.shares > (p.shares == 8 ? 200 : 296)) p.shares >>= 1;
   for (int i = 0; i < n; ++i)
     while (p.shares > 1 && layers[i].meta->K64 / 16 < 2 * prologue_small_ranges(*layers[i].meta, M) * p.shares) p.shares >>= 1;
   int begin = 0, max_kpad = 0;
