@@ -129,7 +129,7 @@ __device__ __forceinline__ void finish_rows(const Params& p, const Layer& ly, co
 // knows by that which shares are taken and does the others, or all of the rows if one has left (what others do of them at the
 // same time is the same).  So none depends on another's progress.  The last one to leave puts the counter back to zero.
 // With the CTA of the last chunk alone, the sums of 64 rows and 7 chunks took 9 us, 4 now; 4096 x 4096, 20 / 64 / 128 tokens, the call
-// 22.3 / 29.2 / 40.8 us before and 20.1 / 25 / 29.5 now, 11008 x 4096 30.5 / 39.1 / 57.9 and 27.9 / 34 / 44.4.
+// 22.3 / 29.2 / 40.8 us alone and 20.1 / 25 / 29.5 shared, 11008 x 4096 30.5 / 39.1 / 57.9 and 27.9 / 34 / 44.4.
 constexpr int kFinishWait = 40000;             // cycles
 // old: the counter before this CTA's chunk arrived.
 template <bool WHOLE_CTA>
