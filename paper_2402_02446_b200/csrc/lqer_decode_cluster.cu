@@ -30,6 +30,7 @@
 
 #include "lqer_gemm_small.cuh"
 #include "lqer_mma_frag.cuh"
+#include "lqer_ring.h"
 
 namespace lqer {
 namespace dcl {
@@ -44,7 +45,7 @@ constexpr int kMaxLayers = 4;                // layers of a launch, at most
 constexpr int kUnit = 16;                    // columns of a unit, one side of an MMA
 constexpr int kUnits = kTileN / kUnit;       // units of a tile
 constexpr int kRows = 16;
-constexpr int kMaxSlots = 20;                // ring slots, at most
+constexpr int kMaxSlots = 20;                // ring slots, at most (RingCursor: each phase has its own of them, a third if the ring is filled again)
 constexpr int kRed = 3;                      // tiles whose sums may be under way
 constexpr int kSmemMax = 222 * 1024;
 constexpr int kLocalStages = 10, kLocalBlocks = 8;   // stages of a cluster that forms all of T itself, and blocks of T (of eight rows) to a warp, at most
@@ -74,6 +75,7 @@ struct Params {
   int slots;                                // ring slots
   int off_red, red_bytes, off_xq, off_xe, off_tpart, off_trecv, off_tq, off_ring;   // offsets in shared memory (the planes of X_q come first)
   long long wait_limit;
+  long long lag;                            // checked build, test hook: see lqer_debug_converter_lag
   int stall;                                // test hook: the sums of the first tile wait for bytes that never come (see also t_expect)
 };
 
@@ -382,10 +384,20 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
     __syncthreads();
     if (lane == 0) {
       for (; x < p.slots && x < x_hi && go; ++x) go = fill(x, x);
-      for (int slot = 0, ph = 0; x < x_hi && go; ++x) {
-        if (!tc::mbar_wait<true>(empty(slot), ph, &s_ws)) break;
-        go = fill(x, slot);
-        if (++slot == p.slots) { slot = 0; ph ^= 1; }
+      RingWalk<kPhases> walk(x);
+      int held = -1, held_slot = 0;                    // checked build, test hook: a stage whose copy comes late (see lqer_debug_converter_lag)
+      for (; x < x_hi && go; ++x) {
+        const int slot = walk.turn[0].slot;
+        if (!tc::mbar_wait<true>(empty(slot), walk.turn[0].parity, &s_ws)) break;
+        if (kDebugBounds && p.lag > 0 && held < 0 && x % 5 == 4 && x + p.slots - kPhases < x_hi) { held = x; held_slot = slot; }
+        else go = fill(x, slot);
+        walk.next(p.slots);
+        if (kDebugBounds && held >= 0 && x >= held + p.slots - kPhases) {    // (until here no stage waits for this one)
+          const long long t0 = clock64();
+          while (clock64() - t0 < p.lag) { }
+          go = go && fill(held, held_slot);
+          held = -1;
+        }
       }
       if (!go) s_ws.abort = 1;
     }
@@ -546,8 +558,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
     // addresses of the rows of 16 bytes that ldmatrix distributes: lanes 8 i .. 8 i + 7 give the eight columns of piece i
     const uint32_t w_row = sm + p.off_ring + (col + (lane & 7)) * 16 + (WB == 4 ? (lane >> 4) * kTile + ((lane >> 3) & 1) * 2048 : ((lane >> 3) & 1) * kTile);
     const uint8_t* e_lane = smem + p.off_ring + kMant + (col + g) * 4;
-    int x = phase, slot = phase % p.slots;
-    uint32_t ph = (phase / p.slots) & 1;
+    int x = phase;
+    RingCursor at(phase);
 #pragma unroll 1
     for (int r = 0, begin = 0, b = 0, turn = 0; r < chunks; ++r, begin += steps) {     // b, turn: r mod and by kRed
       float acc[2][MT][4];
@@ -559,7 +571,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
           for (int c = 0; c < 4; ++c) acc[u][i][c] = 0.f;
 #pragma unroll 1
       for (; x < begin + steps; x += kPhases) {
-        if (!warp_wait(full(slot), ph, &s_ws)) { ok = false; break; }
+        const int slot = at.slot;
+        if (!warp_wait(full(slot), at.parity, &s_ws)) { ok = false; break; }
         uint32_t w[4][4], e[4][2];
 #pragma unroll
         for (int o = 0; o < 4; ++o) {
@@ -590,8 +603,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
         });
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(empty(slot));
-        slot += kPhases;
-        while (slot >= p.slots) { slot -= p.slots; ph ^= 1; }
+        at.next(kPhases, p.slots);
       }
       if (ok && r == 0 && NT > 0) ok = wait_cluster(t_seen, 0, &s_ws);       // the sums lie where T was formed
       if (ok && r >= kRed) ok = wait_cluster(red_free(b), (uint32_t)(turn - 1) & 1u, &s_ws);
@@ -981,6 +993,7 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
   p.a_bits = metas[0].a_bits; p.lr_bits = metas[0].lr_bits; p.exp_min = metas[0].exp_min; p.exp_max = metas[0].exp_max;
   p.wait_limit = wait_limit_cycles();
   p.stall = take_stall(kFamDecode) ? 1 : 0;
+  p.lag = debug_converter_lag();
   p.steps_max = q.steps_max;
   p.slots = q.slots;
   p.off_red = q.off_red; p.red_bytes = q.red_bytes;

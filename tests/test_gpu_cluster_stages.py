@@ -36,9 +36,36 @@ def test_cuts_against_the_oracle(K, N, k, w_bits):
     for M in (3, 8, 9, 16):
         ref = olqer.forward(X[:M], P, w_bits=w_bits)
         Xg, ws = _t(X[:M]), L.new_workspace(M, Pg)
+        before = L.launch_count()
         Y = L.linear(Xg, Pg, ws)
+        assert L.launch_count() - before == 1
         again = L.linear(Xg, Pg, ws)
         assert L.poll_status(ws) == 0
         assert torch.equal(Y, again)
         assert worst_ratio(Y.cpu().numpy(), ref) <= 1.0, M
+    Pg.release()
+
+
+# rings of 5, 4, 17 and 20 slots for 40 to 72 stages: filled many times over, and no multiple of the three consumers that take them in turn
+@pytest.mark.parametrize("M,K,N,k,w_bits", [(16, 11008, 11008, 32, 4), (16, 12288, 11008, 32, 4), (4, 4096, 20488, 32, 4), (8, 4096, 25096, 0, 2)])
+def test_rings_that_are_filled_again(M, K, N, k, w_bits):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(942)
+    draw = lambda *s: torch.randn(s, generator=g, device=DEV)
+    W, A, B, X = draw(K, N) * 0.02, draw(K, k) / K ** 0.5, draw(k, N) * 0.01, draw(M, K)
+    cfg = L.default_config()
+    cfg.w_bits = w_bits
+    Pg = L.prepare_weights(W, A if k else None, B if k else None, cfg)
+    cols = torch.cat([torch.arange(0, 72), torch.arange(N // 2 - 64, N // 2 + 64), torch.arange(N - 136, N)]).to(DEV)
+    h = lambda a: a.cpu().numpy()
+    P = olqer.prepare_weights(h(W[:, cols]), h(A) if k else None, h(B[:, cols]) if k else None, w_bits=w_bits)    # columns are independent
+    del W
+    ws = L.new_workspace(M, Pg)
+    before = L.launch_count()
+    Y = L.linear(X, Pg, ws)
+    assert L.launch_count() - before == 1
+    assert L.poll_status(ws) == 0
+    assert worst_ratio(h(Y[:, cols]), olqer.forward(h(X), P, w_bits=w_bits)) <= 1.0
+    for _ in range(4):
+        assert torch.equal(L.linear(X, Pg, ws), Y)
     Pg.release()

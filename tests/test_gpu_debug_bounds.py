@@ -106,6 +106,39 @@ def test_converter_warps_that_come_late_to_a_batch_lose_nothing():
     assert r.returncode == 0 and "late-converters-ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
 
 
+def test_weight_stages_that_land_late_lose_nothing():
+    # the cluster kernel's ring (rings of 5, 4, 17 and 20 slots): every fifth stage from the second round on lands some 10 us after the others that
+    # the ring has room for.  Whoever took the stage before it for its own would multiply that one's weights.
+    code = textwrap.dedent("""
+        import torch
+        import paper_2402_02446_b200 as L
+        dev = "cuda:0"
+        g = torch.Generator(device=dev); g.manual_seed(8)
+        draw = lambda *s: torch.randn(s, generator=g, device=dev)
+        for M, K, N, k, w_bits in ((16, 11008, 11008, 32, 4), (16, 12288, 11008, 32, 4), (4, 4096, 20488, 32, 4), (8, 4096, 25096, 0, 2)):
+            cfg = L.default_config(); cfg.w_bits = w_bits
+            A, B = (draw(K, k) / K ** 0.5, draw(k, N) * 0.01) if k else (None, None)
+            Pg = L.prepare_weights(draw(K, N) * 0.02, A, B, cfg)
+            X = draw(M, K)
+            ws = L.new_workspace(M, Pg)
+            Y = L.linear(X, Pg, ws).clone()
+            assert L.poll_status(ws) == 0
+            L.debug_converter_lag(20_000)
+            try:
+                before = L.launch_count()
+                late = L.linear(X, Pg, ws)
+                assert L.launch_count() - before == 1
+                assert L.poll_status(ws) == 0, (M, K)
+            finally:
+                L.debug_converter_lag(0)
+            assert torch.equal(late, Y), (M, K)
+            Pg.release()
+        print("late-stages-ok")
+    """)
+    r = _run(["-c", code])
+    assert r.returncode == 0 and "late-stages-ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
+
+
 def test_the_ordinary_build_has_no_such_hook():
     import paper_2402_02446_b200 as L
     from paper_2402_02446_b200 import binding
