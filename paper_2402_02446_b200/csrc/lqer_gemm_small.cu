@@ -13,10 +13,11 @@
 // back).
 // What bounds it is the stream of weights and, close behind, the instructions that expand them (1.8 per weight).
 //
-// Work items are (layer, 256-column tile, K chunk).  The chunks of a tile are fixed by the shape alone (so a
-// result never depends on the number of SMs or on which layers share a launch); each chunk is summed from
-// zero in tensor memory and, if a tile has more than one, leaves its fp32 partial in scratch; the CTAs whose last chunk is of one
-// tile add its chunks up together, in chunk order, a share of the rows each (finish_tile).  None depends on another's help.
+// Work items are (layer, 256-column tile, K chunk).  A layer alone is cut into chunks by its shape, layers that share a launch by
+// the shapes of all of them (launch_gemm_small), so a result does not depend on the number of SMs, but its last bits may on the layers
+// beside it.  Each chunk is summed from zero in tensor memory and, if a tile has more than one, leaves its fp32 partial in scratch;
+// the CTAs whose last chunk is of one tile add its chunks up together, in chunk order, a share of the rows each (finish_tile), and
+// none depends on another's help; or one CTA takes all chunks of a tile, one after the other, and adds them up (RUN).
 // Roles per CTA:
 //   warp 0      producer: bulk copies of packed weight tiles (issued before the dependency wait: weights
 //               depend on no earlier kernel) and TMA loads of activation tiles (after it)
@@ -132,29 +133,34 @@ __device__ __forceinline__ void finish_rows(const Params& p, const Layer& ly, co
 // 22.3 / 29.2 / 40.8 us alone and 20.1 / 25 / 29.5 shared, 11008 x 4096 30.5 / 39.1 / 57.9 and 27.9 / 34 / 44.4.
 constexpr int kFinishWait = 40000;             // cycles
 // old: the counter before this CTA's chunk arrived.
-template <bool WHOLE_CTA>
+template <bool WHOLE_CTA, bool RUN>
 __device__ __forceinline__ void finish_tile(const Params& p, const Item& c, int old, int tid, int* flag) {
   const Layer& ly = p.L[c.layer];
-  int* count = ly.counters + c.tile;
-  // shares of some 96 rows of partial sums; where that makes one of them, the CTA of the last chunk is through sooner than the first's
-  const int shares = min((p.M * ly.chunks + 95) / 96, ly.chunks), rows = (p.M + shares - 1) / shares, share = shares > 1 ? taken(old) : ly.chunks;
-  const bool last = arrived(old) == ly.chunks - 1;
-  bool ok = true;
-  if (WHOLE_CTA && !last && share < shares) {  // (an epilogue comes here with the last chunk only)
-    if (tid == 0) {
-      int v = *reinterpret_cast<volatile int*>(count);
-      for (const long long t0 = clock64(); arrived(v) != ly.chunks && clock64() - t0 < kFinishWait;) v = *reinterpret_cast<volatile int*>(count);
-      *flag = arrived(v) == ly.chunks || arrived(atomicOr(count, kGaveUp)) == ly.chunks ? 1 : 0;
+  int lo = 0, hi = p.M;
+  if (!RUN) {                                  // (otherwise all of the chunks were this CTA's)
+    int* count = ly.counters + c.tile;
+    // shares of some 96 rows of partial sums; where that makes one of them, the CTA of the last chunk is through sooner than the first's
+    const int shares = min((p.M * ly.chunks + 95) / 96, ly.chunks), rows = (p.M + shares - 1) / shares, share = shares > 1 ? taken(old) : ly.chunks;
+    const bool last = arrived(old) == ly.chunks - 1;
+    bool ok = true;
+    if (WHOLE_CTA && !last && share < shares) {  // (an epilogue comes here with the last chunk only)
+      if (tid == 0) {
+        int v = *reinterpret_cast<volatile int*>(count);
+        for (const long long t0 = clock64(); arrived(v) != ly.chunks && clock64() - t0 < kFinishWait;) v = *reinterpret_cast<volatile int*>(count);
+        *flag = arrived(v) == ly.chunks || arrived(atomicOr(count, kGaveUp)) == ly.chunks ? 1 : 0;
+      }
+      __syncthreads();
+      ok = *flag != 0;
     }
-    __syncthreads();
-    ok = *flag != 0;
+    if (tid == 0 && left(atomicAdd(count, kLeft)) + 1 == ly.chunks) *count = 0;
+    if (!last || (old >= 0 && shares > 1)) lo = share * rows;
+    if (!last) hi = ok ? min(p.M, (share + 1) * rows) : lo;
   }
-  if (tid == 0 && left(atomicAdd(count, kLeft)) + 1 == ly.chunks) *count = 0;
   __threadfence();
-  const int lo = last && (old < 0 || shares == 1) ? 0 : share * rows, hi = last ? p.M : min(p.M, (share + 1) * rows);
-  if (ok && lo < hi) finish_rows(p, ly, c, lo, hi, tid, WHOLE_CTA ? NUM_THREADS : 128);
+  finish_rows(p, ly, c, lo, hi, tid, WHOLE_CTA ? NUM_THREADS : 128);
 }
-__device__ __noinline__ void finish_by_epilogue(const Params& p, const Item c, int old, int tid) { finish_tile<false>(p, c, old, tid, nullptr); }
+template <bool RUN>
+__device__ __noinline__ void finish_by_epilogue(const Params& p, const Item c, int old, int tid) { finish_tile<false, RUN>(p, c, old, tid, nullptr); }
 
 // bf16_rn by the conversion instruction, which has one NaN for all.
 __device__ __forceinline__ uint16_t bf16_rn_cvt(uint32_t v) {
@@ -247,7 +253,7 @@ __device__ __forceinline__ int batch_end(int s, int s_hi, int k_slabs) {
 }
 constexpr int RANK_EXP_OFFSET = 8 * kTileN * 16;
 static_assert(RANK_EXP_OFFSET + 8 * kTileN <= W_HALF_BYTES, "two rank slabs");
-template <int NT>
+template <int NT, bool RUN>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constant__ Params p) {
   using C = Cfg<NT>;
@@ -307,7 +313,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
       auto flush = [&]() {
         pdl_wait();
         waited = true;
-        for (int i = cta, q = 0; q < npend; i += num_ctas) {
+        for (int i = first_item<RUN>(p, cta), q = 0; q < npend; i = next_item<RUN>(p, i, num_ctas)) {
           const Item it = item_of(p, i);
           const int k_slabs = p.L[it.layer].k_slabs;
           for (int s = it.s_lo; s < it.s_hi && q < npend; ++q) {
@@ -322,7 +328,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
       uint32_t ph = 0;
       bool ok = true;
       const uint32_t w_tile = (uint32_t)w_tile_bytes(p.w_bits);
-      for (int i = cta; i < num_items && ok; i += num_ctas) {
+      for (int i = first_item<RUN>(p, cta); i < num_items && ok; i = next_item<RUN>(p, i, num_ctas)) {
         const Item it = item_of(p, i);
         const Layer& ly = p.L[it.layer];
         const int k_slabs = ly.k_slabs, r_blocks = ly.r_blocks, b_tile_stride = r_blocks * kTileN * 17;
@@ -330,7 +336,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
         const int n_half = nt0 + 1 < ly.n_tiles ? 2 : 1;       // 128-column tiles of this 256-column tile that exist
         for (int s = it.s_lo; s < it.s_hi;) {
           const int e = batch_end(s, it.s_hi, k_slabs);
-          if (p.stall != 0 && e == it.s_hi && i + num_ctas >= num_items) { ok = false; break; }
+          if (p.stall != 0 && e == it.s_hi && next_item<RUN>(p, i, num_ctas) >= num_items) { ok = false; break; }
           if (!waited && npend == PK_SLOTS) flush();
           if (!mbar_wait<true>(pk_free(pk), ph ^ 1, abort_flag)) { ok = false; break; }
           const uint32_t slot = smem_u32(pk_base + pk * C::PK_SLOT_BYTES), dst = slot + C::X_BYTES;
@@ -375,7 +381,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     const uint32_t b_hi = (uint32_t)(desc0 >> 32), b_lo0 = (uint32_t)desc0;
     uint32_t cv = 0, cv_ph = 0, pk = 0, acc = 0, acc_ph = 1;
     bool first_pass = true, ok = true;
-    for (int i = cta; i < num_items && ok; i += num_ctas) {
+    for (int i = first_item<RUN>(p, cta); i < num_items && ok; i = next_item<RUN>(p, i, num_ctas)) {
       const Item it = item_of(p, i);
       const int k_slabs = p.L[it.layer].k_slabs, r_blocks = p.L[it.layer].r_blocks;
       ok = __all_sync(0xFFFFFFFFu, mbar_wait(acc_empty(acc), acc_ph, abort_flag)) != 0;
@@ -446,7 +452,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     uint32_t tile_it = 0;
     bool ok = true;
     pdl_wait();                                    // Y, the scratch and the counters may be in use by the kernel before
-    for (int i = cta; i < num_items && ok; i += num_ctas, ++tile_it) {
+    for (int i = first_item<RUN>(p, cta); i < num_items && ok; i = next_item<RUN>(p, i, num_ctas), ++tile_it) {
       const Item it = item_of(p, i);
       const Layer& ly = p.L[it.layer];
       const int acc = tile_it % C::ACCS;
@@ -459,15 +465,17 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
       if (ly.chunks > 1) {
         // count this chunk in; the CTA's last one is seen to by all of its threads at the end (every other role is about to fall
         // idle), another one by the epilogue where it is the tile's last to arrive
+        if (RUN && it.chunk + 1 < ly.chunks) continue;       // (the tile's other chunks are this CTA's too)
         __threadfence();
         epilogue_barrier();
-        if (i + num_ctas >= num_items) {
+        if (next_item<RUN>(p, i, num_ctas) >= num_items) {
           if (et == 0) {
             at_end[0] = i;
-            at_end[1] = atomicAdd(ly.counters + it.tile, 1 + kTaken);
+            at_end[1] = RUN ? 0 : atomicAdd(ly.counters + it.tile, 1 + kTaken);
           }
           break;
         }
+        if (RUN) { finish_by_epilogue<RUN>(p, it, 0, et); continue; }
         if (et == 0) {
           const int old = atomicAdd(ly.counters + it.tile, 1);
           *last_flag = old;
@@ -476,7 +484,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
         epilogue_barrier();
         const int old = *last_flag;
         epilogue_barrier();                         // everyone has read it
-        if (arrived(old) == ly.chunks - 1) finish_by_epilogue(p, it, old, et);
+        if (arrived(old) == ly.chunks - 1) finish_by_epilogue<RUN>(p, it, old, et);
       }
     }
   } else {
@@ -490,7 +498,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     uint32_t it_no = 0, batch_no = 0;
     bool ok = true;
     const int w_tile = w_tile_bytes(p.w_bits);
-    for (int item = cta; item < num_items && ok; item += num_ctas) {
+    for (int item = first_item<RUN>(p, cta); item < num_items && ok; item = next_item<RUN>(p, item, num_ctas)) {
       const Item it = item_of(p, item);
       const int k_slabs = p.L[it.layer].k_slabs, r_blocks = p.L[it.layer].r_blocks;
       const bool has_w = 2 * it.tile + half < p.L[it.layer].n_tiles;
@@ -583,7 +591,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
 
   // ------------------------------------------------------------------ teardown
   __syncthreads();                      // every role is done (or has given up): the flags below are final for this CTA
-  if (at_end[0] >= 0 && abort_flag->abort == 0) finish_tile<true>(p, item_of(p, at_end[0]), at_end[1], threadIdx.x, last_flag);
+  if (at_end[0] >= 0 && abort_flag->abort == 0) finish_tile<true, RUN>(p, item_of(p, at_end[0]), at_end[1], threadIdx.x, last_flag);
   if (abort_flag->abort != 0) {
     const long long t0 = clock64();
     while (clock64() - t0 < 400000) { }
@@ -613,12 +621,12 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-template <int NT>
+template <int NT, bool RUN>
 static cudaError_t launch_nt(const TensorMaps& tmaps, const Params& p, int ctas, cudaStream_t s) {
   using C = Cfg<NT>;
   static OncePerDevice once;
   cudaError_t e = once.run([] {
-    return cudaFuncSetAttribute(gemm_small_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+    return cudaFuncSetAttribute(gemm_small_kernel<NT, RUN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
   });
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -632,7 +640,7 @@ static cudaError_t launch_nt(const TensorMaps& tmaps, const Params& p, int ctas,
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   LaunchScope scope(kFamDecode, s);
-  return cudaLaunchKernelEx(&cfg, gemm_small_kernel<NT>, tmaps, p);
+  return cudaLaunchKernelEx(&cfg, gemm_small_kernel<NT, RUN>, tmaps, p);
 }
 
 }  // namespace sg
@@ -658,16 +666,24 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
   const int sms = sm_count();
   if (sms < 1) return cudaErrorInvalidDevice;
   int group_chunks = 1;
+  p.run = 1;
   if (n > 1) {
     // The cut that makes (rounds of items over the SMs) x (slabs per item + what an item costs beside its slabs) smallest,
     // a function of the shapes alone.  The register-operand kernel runs two CTAs per SM, an item each at a time, and an item costs
-    // it about ten slabs' worth of time (activation copy, rank term, partial sums).  This file's kernel runs one CTA per SM; in
-    // slabs' time (0.4 us) a tile in one piece costs it 4 + M / 8 (two- or four-byte stores of a column each), a chunk 5 + M / 20 and
-    // then 14 until the tile's chunks are added up, which keep the CTA from its next item.  (At four slabs for any item two layers of
-    // 4096 x 11008, 86 tiles, were cut into three chunks each, two rounds: 54 / 81 / 133 us with 32 / 64 / 128 tokens, 41 / 46 /
-    // 60 in one piece.)
-    const int ctas = use_mma ? 2 * 148 : 148;
-    long best = -1;
+    // it about ten slabs' worth of time (activation copy, rank term, partial sums); this file's kernel one, and four.
+    // The cut is also how long a chain of sums in tensor memory gets, and these cut off what does not fit: two layers of
+    // 4096 x 11008 in one piece instead of three chunks a tile are 7 times as far from 64 bits (one sign, block exponents over a dozen
+    // binades: 1.9e-6 and 2.7e-7), although that was the faster way.  So the time model below, which knows more of what an item
+    // costs, does not choose the cut, only who takes a tile's chunks.
+    const int ctas = use_mma ? 2 * 148 : 148, extra = use_mma ? 10 : 4;
+    long best = -1, best_rounds = 0, best_len = 0, tiles = 0, slabs = 0;
+    bool alike = true;                                       // one number of chunks for all layers
+    for (int i = 0; i < n; ++i) {
+      const PackedMeta& m = *layers[i].meta;
+      tiles += small_gemm_col_tiles(m);
+      slabs = std::max(slabs, (long)m.k_slabs);
+      alike = alike && m.k_slabs == layers[0].meta->k_slabs && small_gemm_chunks(m) == small_gemm_chunks(*layers[0].meta);
+    }
     for (int c = 1; c <= 16; ++c) {
       long items = 0, len = 0;
       for (int i = 0; i < n; ++i) {
@@ -676,9 +692,16 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
         items += (long)small_gemm_col_tiles(m) * ci;
         len = std::max(len, (long)(m.k_slabs + ci - 1) / ci);
       }
-      const long cost = ((items + ctas - 1) / ctas) * (len + (use_mma ? 10 : c > 1 ? 19 + M / 20 : 4 + M / 8));
-      if (best < 0 || cost < best) { best = cost; group_chunks = c; }
+      const long rounds = (items + ctas - 1) / ctas, cost = rounds * (len + extra);
+      if (best < 0 || cost < best) { best = cost; group_chunks = c; best_rounds = rounds; best_len = len; }
     }
+    // Several rounds of chunks though each tile could have an SM to itself: above 32 rows the rounds cost 2 M / 3 slabs' time (0.4 us) each beside
+    // their slabs (partial sums of every chunk, and of all CTAs at a time), a CTA that takes a tile's chunks one after the other 4 + M / 8
+    // and 3 + M / 17 for each chunk's partial sums.  Two layers of 4096 x 11008, us, apart / one after the other: 32 rows 46.8 / 46.0,
+    // 64 rows 64.3 / 51.9, 128 rows 103 / 70.5.  (The sums are the same, bit for bit.)
+    if (!use_mma && M > 32 && alike && group_chunks > 1 && best_rounds > 1 && tiles <= ctas &&
+        slabs + 4 + M / 8 + group_chunks * (3 + M / 17) < best_rounds * (best_len + 2 * M / 3))
+      p.run = 0;                                             // all of a tile's chunks: see below
   }
   for (int i = 0; i < MAX_LAYERS; ++i) {
     const SmallGemmLayer& src = layers[i < n ? i : 0];
@@ -718,6 +741,7 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
     if (i < n) item_begin += small_gemm_col_tiles(m) * ly.chunks;
   }
   p.n = n;
+  if (p.run == 0) p.run = p.L[0].chunks;
   p.num_items = item_begin;
   p.status = st;
   p.M = M;
@@ -732,8 +756,9 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
   p.exit_count = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(st) + kFlagAreaOffset + 2 * MAX_LAYERS * 4);
   p.stall = take_stall(kFamDecode) ? 1 : 0;
   if (use_mma) return launch_gemm_mma(p, s);
-  const int ctas = p.num_items < sms ? p.num_items : sms;
-  return M <= 32 ? launch_nt<32>(tmaps, p, ctas, s) : M <= 64 ? launch_nt<64>(tmaps, p, ctas, s) : launch_nt<128>(tmaps, p, ctas, s);
+  const int ctas = std::min(p.num_items / p.run, sms);
+  if (p.run > 1) return M <= 64 ? launch_nt<64, true>(tmaps, p, ctas, s) : launch_nt<128, true>(tmaps, p, ctas, s);
+  return M <= 32 ? launch_nt<32, false>(tmaps, p, ctas, s) : M <= 64 ? launch_nt<64, false>(tmaps, p, ctas, s) : launch_nt<128, false>(tmaps, p, ctas, s);
 }
 
 }  // namespace lqer

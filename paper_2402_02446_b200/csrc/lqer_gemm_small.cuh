@@ -31,6 +31,7 @@ struct Params {
   Layer L[MAX_LAYERS];
   int n;                       // layers in this launch
   int num_items;
+  int run;                     // neighbouring items that one CTA takes, one after the other: 1, or all chunks of a tile (RUN kernels)
   DeviceStatus* status;
   int M;
   int lr_shift;
@@ -62,6 +63,15 @@ __device__ __forceinline__ Item item_of(const Params& p, int i) {
   it.s_lo = it.chunk * ly.chunk_stages;
   it.s_hi = it.chunk == ly.chunks - 1 ? ly.spt : it.s_lo + ly.chunk_stages;
   return it;
+}
+
+// The items that a CTA takes: its first, and the one after item i.
+template <bool RUN>
+__device__ __forceinline__ int first_item(const Params& p, int cta) { return RUN ? cta * p.run : cta; }
+template <bool RUN>
+__device__ __forceinline__ int next_item(const Params& p, int i, int num_ctas) {
+  if (!RUN) return i + num_ctas;
+  return (i + 1) % p.run != 0 ? i + 1 : i + 1 + (num_ctas - 1) * p.run;
 }
 
 __device__ __forceinline__ uint32_t bf16_rn(float v) {

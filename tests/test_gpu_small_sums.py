@@ -1,5 +1,6 @@
 """The sum of a tile's K chunks in the small-batch GEMM (Section 3.1: Y = X_q W_q + T_q B_q), which the CTAs of its chunks share:
-few and many rows, up to 21 chunks, a missing 128-column half, and a launch whose CTAs have several chunks each."""
+few and many rows, up to 21 chunks, a missing 128-column half, a launch whose CTAs have several chunks each, and one whose CTAs have all
+chunks of a tile each; and how far layers that share a launch may be from 64 bits."""
 import numpy as np
 import pytest
 import torch
@@ -61,3 +62,71 @@ def test_ctas_with_several_chunks(M):
     for y in Ys[1:]:
         assert torch.equal(y, Ys[0])
     Pg.release()
+
+
+def _groups(K, N, k, n, g, one_sign=False):
+    draw = lambda *s: torch.randn(s, generator=g, device=DEV)
+    W, A, B = [], [], []
+    for _ in range(n):
+        w = draw(K, N) * 0.02
+        W.append(w.abs() if one_sign else w)
+        A.append(draw(K, k) / K ** 0.5)
+        B.append(draw(k, N) * 0.01)
+    return W, A, B, [L.prepare_weights(*f) for f in zip(W, A, B)]
+
+
+def _oracle(W, A, B, cols):
+    h = lambda a: a.cpu().numpy()
+    return olqer.prepare_weights(h(W[:, cols]), h(A), h(B[:, cols]))         # (columns are independent)
+
+
+# two layers of 76 tiles (the last with one half) and three chunks: 228 items where 76 CTAs can take a tile each; 33 rows up
+@pytest.mark.parametrize("M", [33, 64, 65, 128])
+def test_ctas_with_all_chunks_of_a_tile(M):
+    K, N, k = 4096, 9592, 40
+    g = torch.Generator(device=DEV)
+    g.manual_seed(1700 + M)
+    W, A, B, P = _groups(K, N, k, 2, g)
+    X = torch.randn((M, K), generator=g, device=DEV)
+    cols = torch.cat([torch.arange(0, 64), torch.arange(N - 136, N)]).to(DEV)
+    lone = [L.linear(X, p, L.new_workspace(M, p)) for p in P]
+    for y, w, a, b in zip(lone, W, A, B):
+        assert worst_ratio(y[:, cols].cpu().numpy(), olqer.forward(X.cpu().numpy(), _oracle(w, a, b, cols))) <= 1.0
+    for dtype in (torch.float32, torch.bfloat16):
+        Ys = [torch.full((M, N), float("nan"), device=DEV, dtype=dtype) for _ in P]
+        calls = L.make_calls([(X, p, y) for p, y in zip(P, Ys)], torch.float32, dtype)
+        ws = torch.zeros(L.batched_workspace_bytes(calls), dtype=torch.uint8, device=DEV)
+        ws[168192:] = 0xFF                              # scratch holds NaN patterns: nothing unwritten may be read
+        for _ in range(2):
+            before = L.launch_count()
+            L.linear_batched_ex(calls, ws, torch.float32, dtype)
+            assert L.poll_status(ws) == 0 and L.launch_count() - before == 2
+            # the layer alone has the same cut, one CTA to a chunk
+            assert all(torch.equal(y, z.to(dtype)) for y, z in zip(Ys, lone))
+    for p in P:
+        p.release()
+
+
+@pytest.mark.parametrize("K,N,n", [(4096, 11008, 2), (1024, 1024, 3), (1024, 2816, 2)])
+@pytest.mark.parametrize("M", [17, 64, 128])
+def test_shared_launches_are_no_further_off_than_the_layer_alone(M, K, N, n):
+    # one sign and block exponents over a dozen binades: no fp32 sum is exact, and the accumulators of tensor memory cut off what does not
+    # fit, so a longer chain is further off (4096 x 11008 in one piece 7 times).  Half as much again is left for the draw of the inputs.
+    g = torch.Generator(device=DEV)
+    g.manual_seed(1800 + M)
+    W, A, B, P = _groups(K, N, 32, n, g, one_sign=True)
+    X = torch.randn((M, K), generator=g, device=DEV).abs()
+    X = X * torch.exp2(torch.randint(-6, 7, (M, K // 16), generator=g, device=DEV).float()).repeat_interleave(16, 1)
+    cols = torch.arange(0, N, max(N // 192, 1)).to(DEV)
+    ref = olqer.forward(X.cpu().numpy(), _oracle(W[0], A[0], B[0], cols)).Y
+    error = lambda y: float(np.linalg.norm(y[:, cols].double().cpu().numpy() - ref) / np.linalg.norm(ref))
+    ws = L.new_workspace(M, P[0])
+    alone = error(L.linear(X, P[0], ws))
+    Ys = [torch.empty((M, N), device=DEV) for _ in P]
+    calls = L.make_calls([(X, p, y) for p, y in zip(P, Ys)])
+    ws = torch.zeros(L.batched_workspace_bytes(calls), dtype=torch.uint8, device=DEV)
+    L.linear_batched(calls, ws)
+    assert L.poll_status(ws) == 0
+    assert 0.0 < error(Ys[0]) <= 1.5 * alone, (error(Ys[0]), alone)
+    for p in P:
+        p.release()
