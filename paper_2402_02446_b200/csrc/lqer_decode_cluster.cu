@@ -9,11 +9,14 @@
 //   - T = X_q A_q: the first clusters of a layer form it, one or a few rank blocks each.  Each CTA multiplies its part (int8
 //     mma.sync per 16-block, exact, scaled and summed in fp64) and stores its partial sums into the CTA of its cluster that owns
 //     the row; the owner adds them in order, re-quantises along the rank, writes T_q to scratch in global memory and counts its
-//     blocks in.  Every epilogue warp waits for the count (bounded) before its first rank term; the layer's last warp to
-//     have read T_q zeroes the counters for the next call.  Where a cluster has few weights to multiply, it forms all of T itself, and the
-//     owners of the rows store T_q into its CTAs' shared memory.
-// So a cluster waits for other clusters of its launch.  The launch has no more of them than the device holds at a time, those
-// that form T come first, and launch_decode_cluster says what keeps launches on several streams from holding each other up.
+//     blocks in.  Every epilogue warp waits for the count before its first rank term, and where a CTA's wait in vain, another of its warps
+//     forms T_q by itself (form_t_alone).  The layer's last warp to have read T_q zeroes the counters for the next call.  Where a
+//     cluster has few weights to multiply, it forms all of T itself, and the owners of the rows store T_q into its CTAs' shared memory.
+// So a cluster waits for other clusters of its launch, which need not be there yet: launches on several streams get their places one by
+// one, and the clusters that form a layer's T cannot leave before all of it is there.  With form_t_alone nobody waits for a cluster that has no
+// place, and launches cannot hold each other up, however many there are.  (With one cluster for all of a layer's T nobody would either:
+// 4096 / 11008, 4 rows, rank 32 64 -> 68 us a layer, rank 128 68 -> 89, 3 rows, rank 256 78 -> 128; placed as a whole by a cooperative launch
+// 64 -> 72, 68 -> 75, 78 -> 86 and 3 us a launch on the host.)
 //
 // The packed weights come by bulk copies, a stage (two slabs of a tile, 9 KB) at a time: a producer warp keeps a ring of stages full, from
 // before griddepcontrol.wait on, for weights depend on no earlier kernel.  Twelve consumer warps read a stage's mantissas with ldmatrix (the
@@ -39,8 +42,8 @@ using sg::bf16_rn;
 using tc::smem_u32;
 
 constexpr int kColumnWarps = 4, kPhases = 3;                       // consumer warps: 32 columns of a tile each, and every third stage
-constexpr int kConsumers = kColumnWarps * kPhases, kEpilogue = 4;  // warps; one more is the producer
-constexpr int kWorkerWarps = kConsumers + kEpilogue, kWorkers = kWorkerWarps * 32, kThreads = kWorkers + 32;
+constexpr int kConsumers = kColumnWarps * kPhases, kEpilogue = 4;  // warps; one more is the producer, and one looks after T
+constexpr int kWorkerWarps = kConsumers + kEpilogue, kWorkers = kWorkerWarps * 32, kThreads = kWorkers + 64;
 constexpr int kMaxLayers = 4;                // layers of a launch, at most
 constexpr int kUnit = 16;                    // columns of a unit, one side of an MMA
 constexpr int kUnits = kTileN / kUnit;       // units of a tile
@@ -63,7 +66,7 @@ struct Layer {
   int* tcount;                              // arrivals, departures: zero between calls
   int t_blocks;                             // rank blocks of T that each of the layer's first clusters forms
   int t_clusters, t_tiles;                  // ... and how many those are, if they get fewer tiles than the others: so many each
-  int t_expect;                             // arrivals that make T_q whole (one more under the test hook)
+  int t_expect;                             // arrivals that make T_q whole (one more under the test hooks)
 };
 struct Params {
   Layer L[kMaxLayers];
@@ -119,18 +122,24 @@ __device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, vola
     }
   }
 }
-// The same for a counter in global memory that other clusters of the launch raise.
-__device__ __forceinline__ bool wait_count(const int* count, int expect, volatile tc::WaitState* ws) {
+__device__ __forceinline__ bool count_reached(const int* count, int expect) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+  return __all_sync(0xFFFFFFFFu, v >= expect) != 0;
+}
+// The same for a counter in global memory that other clusters of the launch raise, or for a warp of the CTA that has done their work.
+enum TState { kAwaited = 0, kHere, kFormed };    // T_q as a CTA knows it: not there, counted in by its clusters, formed by the CTA's own warp
+__device__ __forceinline__ bool wait_count(const int* count, int expect, volatile int* t_state, volatile tc::WaitState* ws) {
   const long long t0 = clock64();
-  for (;;) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
-    if (__all_sync(0xFFFFFFFFu, v >= expect)) return true;
+  while (!count_reached(count, expect)) {
+    if (__any_sync(0xFFFFFFFFu, *t_state == kFormed)) { __threadfence(); break; }
     bool give_up = ws->abort != 0;
     if (clock64() - t0 > ws->limit) { ws->abort = 1; give_up = true; }
     if (__any_sync(0xFFFFFFFFu, give_up)) return false;
     __nanosleep(64);
   }
+  if (*t_state == kAwaited) *t_state = kHere;
+  return true;
 }
 template <bool kBackoff = false>
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile tc::WaitState* ws) {
@@ -296,6 +305,71 @@ __device__ __forceinline__ uint4 convert_i8x8(uint32_t w0, uint32_t w1, float sc
 // int -> fp64 by the integer's bits (2^52 + 2^31 + v), where the conversion instruction runs at a sixteenth of the rate.
 __device__ __forceinline__ double int_to_double(int v) { return __hiloint2double(0x43300000, v ^ 0x80000000) - 4503601774854144.0; }
 
+// A 16-block of T in as many neighbouring lanes, as MXINT8 along the rank: the lane's value in bf16 and its neighbour's.
+__device__ __forceinline__ uint32_t quantize_t(const Params& p, double v) {
+  double amax = (v != v) ? 0.0 : fabs(v);
+#pragma unroll
+  for (int d = 1; d < 16; d <<= 1) amax = fmax(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, d));
+  const int e = block_exponent(amax, p.exp_min, p.exp_max);
+  const uint32_t bits = (uint32_t)bf16_bits_of(quant_mantissa(v, e, p.a_bits), e - (p.a_bits - 2)) & 0xFFFFu;
+  return bits | (__shfl_down_sync(0xFFFFFFFFu, bits, 1) << 16);
+}
+// Warps that share the tiles of T of a cluster with `cols` ranks.
+__device__ __forceinline__ int warps_per_tile(int cols) { return cols == 0 || cols / 8 >= kWorkerWarps ? 1 : kWorkerWarps / (cols / 8); }
+// The byte of T_q in scratch that ranks j and j + 1 (j even) of a row begin at.
+template <int MT>
+__device__ __forceinline__ uint32_t tq_offset(int row, int j, uint32_t rplane) {
+  return (uint32_t)((j & 31) >> 2) * rplane + token_offset<MT>(row, j >> 6, j & 63) + (uint32_t)((j & 2) * 2 * MT);
+}
+constexpr int kHelpWait = 200000;               // cycles (T takes some 10 us where its clusters run)
+// All of a layer's T_q by one warp, unless the clusters that are to form it do so meanwhile: the same sums in the same order, hence the
+// same bytes whoever writes them.  A lane has a rank of a row and walks K (0.5 us a block of 16): half a millisecond for 4 rows, rank 32 and
+// K = 4096, where waiting takes as long as other launches hold the places.
+template <int MT>
+__device__ __forceinline__ void form_t_alone(const Params& p, const Layer& ly, int CS, uint32_t rplane, const volatile int* t_state) {
+  const int lane = threadIdx.x & 31, total = p.M * ly.k_pad, kblocks = ly.K / 16;
+  const QuantConsts qc = quant_consts(p.a_bits, p.exp_min, p.exp_max);
+  const int bias = -127 - (p.a_bits - 2) - (p.lr_bits - 2);
+#pragma unroll 1
+  for (int o = lane; o - lane < total; o += 32) {
+    if (__any_sync(0xFFFFFFFFu, *t_state != kAwaited) || count_reached(ly.tcount, ly.t_expect)) return;
+    const bool live = o < total;
+    const int row = live ? o / ly.k_pad : 0, j = o % ly.k_pad, rb_lo = j / 16 / ly.t_blocks * ly.t_blocks;
+    const int share = warps_per_tile(16 * (min(rb_lo + ly.t_blocks, ly.r_blocks) - rb_lo));
+    double v = 0.0;
+#pragma unroll 1
+    for (int c = 0; c < CS; ++c) {
+      const int lo = c * ly.k_slabs / CS * 4, hi = min((c + 1) * ly.k_slabs / CS * 4, kblocks);
+      double sum = 0.0;
+#pragma unroll 1
+      for (int first = lo; first < lo + share; ++first) {
+        double acc = 0.0;
+#pragma unroll 1
+        for (int b = first; b < hi; b += share) {
+          float x[16];
+          int e;
+          uint4 m8, f0, f1;
+          load_x_block(x, ly.X, p.x_type, p.M, ly.K, row, b, p.a_bits, p.exp_min, p.exp_max);
+          quantize_block16(x, qc, e, m8, f0, f1);
+          const uint4 a = __ldg(reinterpret_cast<const uint4*>(ly.asec + ((size_t)b * ly.k_pad + j) * 16));
+          const int ea = __ldg(ly.asec + (size_t)kblocks * ly.k_pad * 16 + (size_t)b * ly.k_pad + j);
+          int dot = __dp4a((int)m8.x, (int)a.x, 0);
+          dot = __dp4a((int)m8.y, (int)a.y, dot);
+          dot = __dp4a((int)m8.z, (int)a.z, dot);
+          dot = __dp4a((int)m8.w, (int)a.w, dot);
+          acc = fma(int_to_double(dot), pow2d(e + bias + ea), acc);
+        }
+        sum += acc;
+      }
+      v += sum;
+    }
+    const uint32_t bits = quantize_t(p, live ? v : 0.0), at = tq_offset<MT>(row, j, rplane);
+    if (live && (lane & 1) == 0 && LQER_IN_BOUNDS(p.status, at, 4, 8 * rplane, 735)) *reinterpret_cast<uint32_t*>(ly.tq + at) = bits;
+  }
+  __threadfence();
+  __syncwarp();
+}
+
 // WB: mantissa bits of W_q (4 or 2).  MT: tiles of eight tokens (1 or 2).  LOCAL: every cluster forms all of T for itself.
 template <int WB, int MT, bool LOCAL>
 __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __grid_constant__ Params p, int CS) {
@@ -305,6 +379,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ __align__(8) uint64_t s_bars[3 + 2 * kRed + 2 * kMaxSlots];
   __shared__ tc::WaitState s_ws;
+  __shared__ volatile int s_t_state;                   // of TState
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int rank = (int)cta_rank(), cluster = (int)blockIdx.x / CS;
@@ -336,7 +411,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
   // This cluster's share of T: rank blocks [rb_lo, rb_hi), i.e. NT tiles of 8 columns; where there are fewer tiles than warps,
   // WPN warps share one and split its blocks of K.
   const int rb_lo = LOCAL ? 0 : min(cl * ly.t_blocks, ly.r_blocks), rb_hi = min(rb_lo + ly.t_blocks, ly.r_blocks);
-  const int t_cols = 16 * (rb_hi - rb_lo), NT = t_cols / 8, WPN = NT == 0 || NT >= kWorkerWarps ? 1 : kWorkerWarps / NT;
+  const int t_cols = 16 * (rb_hi - rb_lo), NT = t_cols / 8, WPN = warps_per_tile(t_cols);
   const int RP = 8 * MT / CS;                                        // rows whose T a CTA owns
   const int own_rows = max(0, min(M - rank * RP, RP));
   const uint32_t rplane = (uint32_t)((k_pad + 127) / 128) * (256u * MT);   // a plane of T_q: rank slabs, an even number of them
@@ -366,6 +441,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
       for (int i = 0; i < p.slots; ++i) { tc::mbar_init(full(i), 1); tc::mbar_init(empty(i), kColumnWarps); }
       s_ws.abort = 0;
       s_ws.limit = p.wait_limit;
+      s_t_state = kAwaited;
       tc::fence_barrier_init();
       tc::fence_proxy_async_smem();
       if (NT > 0 && own_rows > 0) tc::mbar_expect_tx(t_full, (uint32_t)(own_rows * t_cols * 8 * CS));
@@ -412,12 +488,33 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
   }
   tc::pdl_launch_dependents();
   cluster_arrive();
+  if (warp > kWorkerWarps) {
+    // ------------------------------------------------------------------ T where its clusters do not come
+    cluster_wait();
+    __syncthreads();
+    tc::pdl_wait();
+    if (!LOCAL && k_pad > 0) {
+      const long long t0 = clock64();
+      while (__all_sync(0xFFFFFFFFu, s_t_state == kAwaited && *(volatile int*)&s_ws.abort == 0)) {
+        if (__any_sync(0xFFFFFFFFu, clock64() - t0 > kHelpWait)) {
+          form_t_alone<MT>(p, ly, CS, rplane, &s_t_state);
+          s_t_state = kFormed;
+          break;
+        }
+        __nanosleep(500);
+      }
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    return;
+  }
 
   // ---- A_q of this CTA's blocks and this cluster's ranks: the first words into registers, the others towards L2
   const int kblocks = K / 16, kb0 = s_lo * 4, nreal = min(n_slabs * 4, kblocks - kb0);
   const int nt_first = NT >= kWorkerWarps ? warp : NT > 0 ? warp % NT : 0, sub = NT >= kWorkerWarps || NT == 0 ? 0 : warp / NT;
   const bool t_active = NT > 0 && (NT >= kWorkerWarps || warp < NT * WPN);
-  constexpr int UB = 8;
+  constexpr int UB = 6;                                                // words of each of the two in flight (with eight the registers spill)
   uint32_t aw[2][UB], ae[2][UB];
   auto load_a = [&](int bq, int nt, uint32_t (&w)[UB], uint32_t (&e)[UB]) {
     const uint8_t* am = ly.asec + ((size_t)(kb0 + bq) * k_pad + rb_lo * 16 + nt * 8 + g) * 16 + t * 4;
@@ -433,7 +530,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
       ax += (size_t)WPN * k_pad;
     }
   };
-  if (t_active) load_a(sub, nt_first, aw[0], ae[0]);
+  if (t_active) {
+    load_a(sub, nt_first, aw[0], ae[0]);
+    load_a(sub + UB * WPN, nt_first, aw[1], ae[1]);
+  }
   if (NT > 0)
     for (int i = tid; i < nreal * NT; i += kWorkers) {                 // 128 bytes of mantissas each, and the exponents beside them
       const size_t at = (size_t)(kb0 + i / NT) * k_pad + rb_lo * 16 + (i % NT) * 8;
@@ -499,14 +599,16 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
     // rows beyond M are read (whatever lies there) but never sent
     for (int nt = nt_first; nt < NT; nt += kWorkerWarps) {
       double acc[4] = {0.0, 0.0, 0.0, 0.0};
-      if (nt != nt_first) load_a(sub, nt, aw[0], ae[0]);
+      if (nt != nt_first) {
+        load_a(sub, nt, aw[0], ae[0]);
+        load_a(sub + UB * WPN, nt, aw[1], ae[1]);
+      }
       for (int b0 = sub; b0 < nreal; b0 += 2 * UB * WPN) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int bq = b0 + h * UB * WPN;
           if (bq >= nreal) break;
-          if (bq + UB * WPN < nreal) load_a(bq + UB * WPN, nt, aw[h ^ 1], ae[h ^ 1]);
-          // (blocks beyond the last have zeros for A_q: without a branch the chains of eight blocks run side by side)
+          // (blocks beyond the last have zeros for A_q: without a branch the chains of UB blocks run side by side)
 #pragma unroll
           for (int u = 0; u < UB; ++u) {
             const int b = min(bq + u * WPN, nreal - 1);
@@ -524,6 +626,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
               acc[3] = fma(int_to_double(c[3]), pow2d(ex1 + ea_hi), acc[3]);
             }
           }
+          if (bq + 2 * UB * WPN < nreal) load_a(bq + 2 * UB * WPN, nt, aw[h], ae[h]);
         }
       }
 #pragma unroll
@@ -640,19 +743,14 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
 #pragma unroll 8
           for (int c = 0; c < CS; ++c) v += tp[c * RP * t_cols + o];
         }
-        double amax = (v != v) ? 0.0 : fabs(v);
-#pragma unroll
-        for (int d = 1; d < 16; d <<= 1) amax = fmax(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, d));
-        const int e = block_exponent(amax, p.exp_min, p.exp_max);
-        const uint32_t bits = (uint32_t)bf16_bits_of(quant_mantissa(v, e, p.a_bits), e - (p.a_bits - 2)) & 0xFFFFu;
-        const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, bits, 1);
+        const uint32_t bits = quantize_t(p, v);
         if (live && (lane & 1) == 0) {
           const int row = rank * RP + o / t_cols, j = rb_lo * 16 + o % t_cols;
-          const uint32_t at = (uint32_t)((j & 31) >> 2) * rplane + token_offset<MT>(row, j >> 6, j & 63) + (uint32_t)((j & 2) * 2 * MT);
+          const uint32_t at = tq_offset<MT>(row, j, rplane);
           if (LOCAL) {
-            for (int c = 0; c < CS; ++c) st_async(map_cta(sm + p.off_tq + at, c), bits | (next << 16), map_cta(t_ready, c));
+            for (int c = 0; c < CS; ++c) st_async(map_cta(sm + p.off_tq + at, c), bits, map_cta(t_ready, c));
           } else if (LQER_IN_BOUNDS(p.status, at, 4, 8 * rplane, 734)) {
-            *reinterpret_cast<uint32_t*>(ly.tq + at) = bits | (next << 16);
+            *reinterpret_cast<uint32_t*>(ly.tq + at) = bits;
           }
         }
       }
@@ -705,7 +803,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
             }
           }
           if (!have_t) {
-            ok = LOCAL ? wait_cluster(t_ready, 0, &s_ws) : wait_count(ly.tcount, ly.t_expect, &s_ws);
+            ok = LOCAL ? wait_cluster(t_ready, 0, &s_ws) : wait_count(ly.tcount, ly.t_expect, &s_t_state, &s_ws);
             have_t = true;
             if (!ok) break;
           }
@@ -891,13 +989,12 @@ static bool plan_with(const PackedMeta* metas, int n, int M, int CS, Plan& q) {
     ++q.total;
   }
   // In the time of a stage: the stages, what a tile costs beyond them (many CTAs hand over more sums in less time), the rounds in which
-  // X is quantised, and what T costs the clusters that form it, which get fewer tiles for that (see launch_decode_cluster for how many
-  // they are).  Fitted to calls of 3, 8, 9 and 16 rows with clusters of 2, 4 and 8; us for the four groups of a 4096 / 11008 and of a
+  // X is quantised, and what T costs the clusters that form it, which get fewer tiles for that.  Fitted to calls of 3, 8, 9 and 16 rows with clusters of 2, 4 and 8; us for the four groups of a 4096 / 11008 and of a
   // 5120 / 13824 layer (qkv, o, gate and up, down), 3 rows: 17.9 10.8 25.3 28.8 with 2, 15.1 10.2 25.9 14.4 with 4, 18.4 11.1 31.3 18.4 with 8;
   // 21.6 13.1 31.6 37.6, 21.7 12.2 35.4 28.5, 25.7 12.0 41.3 22.6; 16 rows: 26.3 19.5 34.1 -, 23.7 13.6 31.8 25.6, 28.8 15.5 47.4 24.8;
   // 33.3 25.6 45.3 -, 28.7 18.6 43.1 46.1, 36.1 17.2 57.6 31.1.
   const double tile_cost = CS == 8 ? (MT == 1 ? 2.0 : 3.5) : CS == 4 ? (MT == 1 ? 0.7 : 1.2) : (MT == 1 ? 0.3 : 0.6);
-  const int most = std::max(q.resident / 4 / n, 1);
+  const int most = std::max(q.resident / 4 / n, 1);  // clusters that form a layer's T: a quarter of the places, whatever the rank
   auto share = [&](int i) { return (metas[i].n_tiles + q.clusters[i] - 1) / q.clusters[i]; };
   // few stages: T's way through global memory would take longer than they do
   q.local = r_blocks_max > 0 && r_blocks_max <= 8;
@@ -998,11 +1095,6 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
   p.slots = q.slots;
   p.off_red = q.off_red; p.red_bytes = q.red_bytes;
   p.off_xq = q.off_xq; p.off_xe = q.off_xe; p.off_tpart = q.off_tpart; p.off_trecv = q.off_trecv; p.off_tq = q.off_tq; p.off_ring = q.off_ring;
-  // The clusters that form a layer's T wait for one another, and all others of the layer, placed after them, wait for these.  A launch
-  // that runs beside others may get its places one by one, and until all of its T clusters have theirs the ones that do
-  // cannot leave.  At most a quarter of the places go to such clusters (one to each layer at least), so that four launches on as many
-  // streams cannot hold each other up for good.
-  // (plan_with sees to it.)
   int begin = 0;
   size_t t_off = 0;
   for (int i = 0; i < kMaxLayers; ++i) {
@@ -1023,7 +1115,7 @@ cudaError_t launch_decode_cluster(const lqer_call_t* calls, const PackedMeta* me
     ly.tq = static_cast<uint8_t*>(scratch) + t_off;
     ly.tcount = counts + 2 * g;
     // the warps of an owner count their 16-blocks of T in
-    ly.t_expect = M * m.r_blocks + p.stall;
+    ly.t_expect = M * m.r_blocks + (p.stall != 0 || (kDebugBounds && p.lag > 0) ? 1 : 0);
     ly.t_blocks = q.t_blocks[g]; ly.t_clusters = q.t_clusters[g]; ly.t_tiles = q.t_tiles[g];
     if (i < n) t_off += decode_cluster_scratch_bytes(m);
     if (i < n) begin += q.clusters[g];

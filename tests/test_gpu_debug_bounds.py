@@ -139,6 +139,43 @@ def test_weight_stages_that_land_late_lose_nothing():
     assert r.returncode == 0 and "late-stages-ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
 
 
+def test_whoever_waits_for_the_clusters_that_form_t_in_vain_forms_it():
+    # the cluster kernel under the same hook: T never counts as complete (as if its clusters waited for places that other launches hold), so every
+    # warp that needs it forms it.  The sums are the same in the same order: Y is that of the ordinary call, and no wait runs out.
+    code = textwrap.dedent("""
+        import torch
+        import paper_2402_02446_b200 as L
+        dev = "cuda:0"
+        g = torch.Generator(device=dev); g.manual_seed(9)
+        draw = lambda *s: torch.randn(s, generator=g, device=dev)
+        # one rank block to a cluster, two, six and more than warps are; one, two, four and eight CTAs that share K; a ragged last block of ranks
+        for K, N, k, M, w_bits in ((1040, 20008, 40, 5, 4), (2112, 264, 256, 3, 4), (2048, 2048, 256, 16, 4), (4096, 1032, 130, 9, 4),
+                                   (1040, 648, 136, 8, 2), (256, 4104, 200, 16, 4), (64, 4104, 36, 4, 4), (12288, 520, 200, 12, 4)):
+            cfg = L.default_config(); cfg.w_bits = w_bits
+            Pg = L.prepare_weights(draw(K, N) * 0.02, draw(K, k) / K ** 0.5, draw(k, N) * 0.01, cfg)
+            # X of many binades: the fp64 sums round, so their order shows
+            X = draw(M, K) * torch.exp2(torch.randint(-30, 31, (M, K // 16), generator=g, device=dev).float()).repeat_interleave(16, 1)
+            for x in (X, X.bfloat16()):
+                ws = L.new_workspace(M, Pg)
+                Y = L.linear_ex(x, Pg, ws).clone()
+                assert L.poll_status(ws) == 0
+                L.debug_converter_lag(1)
+                try:
+                    before = L.launch_count()
+                    alone = L.linear_ex(x, Pg, ws)
+                    assert L.launch_count() - before == 1
+                    assert L.poll_status(ws) == 0, (K, M)
+                finally:
+                    L.debug_converter_lag(0)
+                assert torch.equal(alone, Y), (K, M, k)
+                assert torch.equal(L.linear_ex(x, Pg, ws), Y) and L.poll_status(ws) == 0
+            Pg.release()
+        print("t-alone-ok")
+    """)
+    r = _run(["-c", code])
+    assert r.returncode == 0 and "t-alone-ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
+
+
 def test_the_ordinary_build_has_no_such_hook():
     import paper_2402_02446_b200 as L
     from paper_2402_02446_b200 import binding

@@ -179,3 +179,22 @@ def test_replays_of_a_launch_placed_as_a_whole():
         assert L.poll_status(ws) == 0
         assert worst_ratio(y.cpu().numpy(), olqer.forward(X, P)) <= 1.0, rep
     Pg.release()
+
+
+def test_many_streams_of_launches_whose_t_comes_from_several_clusters():
+    # ten streams of two priorities, ranks of 256: their clusters that form T are more than the device has places.  Nobody waits for good.
+    spec, P, Pg = _layer(12288, 520, 256, 910)
+    X = _t(gen.make_activations(spec, M=8))
+    want = L.linear(X, Pg, L.new_workspace(8, Pg))
+    assert worst_ratio(want.cpu().numpy(), olqer.forward(X.cpu().numpy(), P)) <= 1.0
+    streams = [torch.cuda.Stream(priority=-(i % 2)) for i in range(10)]
+    spaces = [L.new_workspace(8, Pg) for _ in streams]
+    Ys = [[torch.full_like(want, float("nan")) for _ in range(20)] for _ in streams]
+    torch.cuda.synchronize()
+    for rep in range(20):
+        for s, w, ys in zip(streams, spaces, Ys):
+            L.linear(X, Pg, w, ys[rep], stream=s)
+    torch.cuda.synchronize()
+    assert all(L.poll_status(w) == 0 for w in spaces)
+    assert all(torch.equal(y, want) for ys in Ys for y in ys)
+    Pg.release()
