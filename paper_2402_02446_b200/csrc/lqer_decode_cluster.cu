@@ -221,11 +221,15 @@ __device__ __forceinline__ void load_x_block(float (&v)[16], const void* X, int 
 // order in which the lanes get the weights: word t of every block pair (4-bit mantissas: K 32 (i >> 1) + 8 t + 4 (i & 1) of the step),
 // or word t of every slab (2-bit ones: K 64 (i >> 2) + 16 t + 4 (i & 3)).  Four planes, of the MMAs 2 m and 2 m + 1 of every step: [step][MMA where MT
 // == 2][token, lane t][16 bytes], the 16 bytes being both MMAs' words of one tile, or one MMA's of two.
+// The planes lie 16, 64 and 80 bytes beyond multiples of 128 from the first, so that the lanes that store neighbouring blocks meet four to a bank
+// (with none of that sixteen: 16 rows, K = 2048 in clusters of four, 2 us of 8).
+__host__ __device__ constexpr uint32_t plane_bytes(int steps, int mt) { return (uint32_t)steps * (512u * mt) + 16u; }
+__host__ __device__ constexpr uint32_t plane_offset(uint32_t m, uint32_t plane) { return m * plane + (m >> 1) * 32u; }
 // The sixteen K of a block (f0, f1: eight pairs of bf16 values) to their places.
 template <int WB, int MT>
 __device__ __forceinline__ void store_block(uint8_t* planes, uint32_t plane, int row, int block, const uint4& f0, const uint4& f1) {
   const int b = block & 3, slab = block >> 2;
-  uint8_t* at = planes + (uint32_t)((slab & 1) * 2 + (WB == 4 ? b >> 1 : 0)) * plane + (uint32_t)((slab >> 1) * (512 * MT) + (row >> 3) * 4) +
+  uint8_t* at = planes + plane_offset((slab & 1) * 2 + (WB == 4 ? b >> 1 : 0), plane) + (uint32_t)((slab >> 1) * (512 * MT) + (row >> 3) * 4) +
                 ((row & 7) * 4 + (WB == 4 ? (b & 1) * 2 : b)) * 16;
   const uint32_t next = WB == 4 ? 16u : plane;               // the block's second half: the next lane's, or the next pair of MMAs
   if (MT == 1) {
@@ -396,7 +400,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
   const int chunks = nth < 0 ? ly.t_tiles : f_all + (int)((uint32_t)(nth + 1) * (uint32_t)rest / (uint32_t)others) - tile_lo;
   const int s_lo = rank * ly.k_slabs / CS, s_hi = (rank + 1) * ly.k_slabs / CS, n_slabs = s_hi - s_lo;
   const int steps = (n_slabs + 1) / 2;                               // of two slabs (128 K)
-  const uint32_t plane = (uint32_t)p.steps_max * (512u * MT);
+  const uint32_t plane = plane_bytes(p.steps_max, MT);
   const uint32_t sm = smem_u32(smem);
   const uint32_t bar0 = smem_u32(s_bars);
   const uint32_t t_full = bar0, t_seen = bar0 + 8;
@@ -550,7 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
       asm volatile("prefetch.global.L2 [%0];" ::"l"(bt + (size_t)ly.r_blocks * kTileN * 16 + rb * kTileN + col));
     }
   // ---- zeros where no activation is written: rows beyond M, the second half of an odd last step, ranks beyond k_pad
-  for (int o = tid * 16; o < (int)(4 * plane); o += kWorkers * 16) *reinterpret_cast<uint4*>(smem + o) = make_uint4(0u, 0u, 0u, 0u);
+  for (int o = tid * 16; o < (int)plane_offset(4, plane); o += kWorkers * 16) *reinterpret_cast<uint4*>(smem + o) = make_uint4(0u, 0u, 0u, 0u);
   uint8_t* xq = smem + p.off_xq;
   int8_t* xe = reinterpret_cast<int8_t*>(smem + p.off_xe);
   const int xq_stride = p.steps_max * 128 + 16, xe_stride = p.steps_max * 8;
@@ -695,12 +699,12 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
             return convert_crumbs(w[o][m >> 1], m & 1, s2, c2, kc);
           }
         }, [&](int m, uint32_t (&b0)[2 * MT], uint32_t (&b1)[2 * MT]) {
-          uint4 v = *reinterpret_cast<const uint4*>(xs + m * plane);
+          uint4 v = *reinterpret_cast<const uint4*>(xs + plane_offset(m, plane));
           if (MT == 1) {
             b0[0] = v.x; b0[1] = v.y; b1[0] = v.z; b1[1] = v.w;
           } else {
             b0[0] = v.x; b0[2 * MT - 2] = v.y; b0[1] = v.z; b0[2 * MT - 1] = v.w;
-            v = *reinterpret_cast<const uint4*>(xs + m * plane + 512);
+            v = *reinterpret_cast<const uint4*>(xs + plane_offset(m, plane) + 512);
             b1[0] = v.x; b1[2 * MT - 2] = v.y; b1[1] = v.z; b1[2 * MT - 1] = v.w;
           }
         });
@@ -955,7 +959,7 @@ static bool plan_with(const PackedMeta* metas, int n, int M, int CS, Plan& q) {
   const int red = al(kUnits * kPhases * kUnit * token_stride(MT) * 4), stage = wb == 4 ? Stage<4>::kBytes : Stage<2>::kBytes;
   q.steps_max = ((k_slabs_max + CS - 1) / CS + 1) / 2;
   if ((long long)q.steps_max * 2048 * MT > kSmemMax) return false;
-  const int off = q.steps_max * 2048 * MT;
+  const int off = al((int)plane_offset(4, plane_bytes(q.steps_max, MT)));
   // X_q for the projection and the partial sums of T share their room with the sums of the tiles
   q.off_red = off;
   q.red_bytes = red;
