@@ -28,30 +28,17 @@
 // and on others not at all; a run of (tile, step) to each CTA of 148 without clusters, the sums exchanged through global memory, took
 // 94 us where this takes 64 (decoder layer of 4096 / 11008, 4 rows); copies of 0.5 to 2 KB, padded against bank conflicts, 118.
 #include <algorithm>
-#include <cstring>
 #include <mutex>
 
+#include "lqer_cluster_plan.h"
 #include "lqer_gemm_small.cuh"
 #include "lqer_mma_frag.cuh"
-#include "lqer_ring.h"
 
 namespace lqer {
 namespace dcl {
 using namespace mf;
 using sg::bf16_rn;
 using tc::smem_u32;
-
-constexpr int kColumnWarps = 4, kPhases = 3;                       // consumer warps: 32 columns of a tile each, and every third stage
-constexpr int kConsumers = kColumnWarps * kPhases, kEpilogue = 4;  // warps; one more is the producer, and one looks after T
-constexpr int kWorkerWarps = kConsumers + kEpilogue, kWorkers = kWorkerWarps * 32, kThreads = kWorkers + 64;
-constexpr int kMaxLayers = 4;                // layers of a launch, at most
-constexpr int kUnit = 16;                    // columns of a unit, one side of an MMA
-constexpr int kUnits = kTileN / kUnit;       // units of a tile
-constexpr int kRows = 16;
-constexpr int kMaxSlots = 20;                // ring slots, at most (RingCursor: each phase has its own of them, a third if the ring is filled again)
-constexpr int kRed = 3;                      // tiles whose sums may be under way
-constexpr int kSmemMax = 222 * 1024;
-constexpr int kLocalStages = 10, kLocalBlocks = 8;   // stages of a cluster that forms all of T itself, and blocks of T (of eight rows) to a warp, at most
 
 struct Layer {
   const void* X;
@@ -156,13 +143,10 @@ __device__ __forceinline__ void ldmatrix2(uint32_t (&r)[4], uint32_t addr) {
 // A stage in shared memory: two slabs of a packed weight tile, as they lie in the packed buffer.
 template <int WB>
 struct Stage {
-  static constexpr int kMant = WB == 4 ? kWTileNibbleBytes : 2048;   // bytes of a tile's mantissas
-  static constexpr int kTile = kMant + kTileN * 4;                   // and of the whole tile
+  static constexpr int kMant = slab_mantissa_bytes(WB);
+  static constexpr int kTile = slab_bytes(WB);
   static constexpr int kBytes = 2 * kTile;
 };
-// Words from column to column of a unit on its way to Y: tokens, two more against bank conflicts.
-__host__ __device__ constexpr int token_stride(int mt) { return 8 * mt + 2; }
-
 // Four consecutive columns of a row of Y (a lane of a quad of lanes that hold a 16-block of the row), all lanes calling.
 __device__ __forceinline__ void write_y4(const Params& p, const Layer& ly, int row, int col, float4 v, bool live) {
   if (p.y_type == kYMXINT8) {
@@ -221,10 +205,6 @@ __device__ __forceinline__ void load_x_block(float (&v)[16], const void* X, int 
 // order in which the lanes get the weights: word t of every block pair (4-bit mantissas: K 32 (i >> 1) + 8 t + 4 (i & 1) of the step),
 // or word t of every slab (2-bit ones: K 64 (i >> 2) + 16 t + 4 (i & 3)).  Four planes, of the MMAs 2 m and 2 m + 1 of every step: [step][MMA where MT
 // == 2][token, lane t][16 bytes], the 16 bytes being both MMAs' words of one tile, or one MMA's of two.
-// The planes lie 16, 64 and 80 bytes beyond multiples of 128 from the first, so that the lanes that store neighbouring blocks meet four to a bank
-// (with none of that sixteen: 16 rows, K = 2048 in clusters of four, 2 us of 8).
-__host__ __device__ constexpr uint32_t plane_bytes(int steps, int mt) { return (uint32_t)steps * (512u * mt) + 16u; }
-__host__ __device__ constexpr uint32_t plane_offset(uint32_t m, uint32_t plane) { return m * plane + (m >> 1) * 32u; }
 // The sixteen K of a block (f0, f1: eight pairs of bf16 values) to their places.
 template <int WB, int MT>
 __device__ __forceinline__ void store_block(uint8_t* planes, uint32_t plane, int row, int block, const uint4& f0, const uint4& f1) {
@@ -884,7 +864,6 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
   if (tid == 0 && s_ws.abort != 0) report_error(p.status, LQER_ERR_TIMEOUT, 730, blockIdx.x);
 }
 
-// Clusters of CS CTAs that the device holds at a time (0 if the query fails).
 static cudaLaunchConfig_t launch_config(int CS, int clusters, size_t smem, cudaLaunchAttribute* attr, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(clusters * CS);
@@ -899,20 +878,23 @@ static cudaLaunchConfig_t launch_config(int CS, int clusters, size_t smem, cudaL
   cfg.numAttrs = 2;
   return cfg;
 }
+// Clusters of CS CTAs that the device holds at a time (-1 if the query fails).
 template <int WB, int MT, bool LOCAL>
 static int resident_clusters(int CS) {
   static std::mutex mu;
   static int known[64][4] = {};
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
   std::lock_guard<std::mutex> lock(mu);
   int& n = known[dev][CS == 8 ? 3 : CS == 4 ? 2 : CS == 2 ? 1 : 0];
   if (n == 0) {
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = launch_config(CS, 1, kSmemMax, attr, nullptr);
     if (cudaFuncSetAttribute(decode_cluster_kernel<WB, MT, LOCAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, decode_cluster_kernel<WB, MT, LOCAL>, &cfg) != cudaSuccess)
+        cudaOccupancyMaxActiveClusters(&n, decode_cluster_kernel<WB, MT, LOCAL>, &cfg) != cudaSuccess) {
       n = 0;
+      return -1;
+    }
   }
   return n;
 }
@@ -936,130 +918,14 @@ static Entry entry_of(int wb, int mt, bool local) {
   return mt == 1 ? entry<2, 1>(local) : entry<2, 2>(local);
 }
 
-// The cluster size, the clusters of each layer and the shared memory of a launch over these layers: functions of the shapes (and of
-// what the device holds) alone.
-struct Plan {
-  int CS, steps_max, slots;
-  int off_red, red_bytes, off_xq, off_xe, off_tpart, off_trecv, off_tq, off_ring;
-  size_t smem;
-  int resident, clusters[kMaxLayers], total;
-  int t_blocks[kMaxLayers], t_clusters[kMaxLayers], t_tiles[kMaxLayers];
-  bool local;                               // every cluster forms all of T for itself
-  double cost;
-};
-static bool plan_with(const PackedMeta* metas, int n, int M, int CS, Plan& q) {
-  const int MT = M > 8 ? 2 : 1, wb = metas[0].w_bits;
-  int k_slabs_max = 0, r_blocks_max = 0;
-  for (int i = 0; i < n; ++i) {
-    k_slabs_max = std::max(k_slabs_max, (int)metas[i].k_slabs);
-    r_blocks_max = std::max(r_blocks_max, (int)metas[i].r_blocks);
-  }
-  q.CS = CS;
-  auto al = [](int v) { return (v + 127) / 128 * 128; };
-  const int red = al(kUnits * kPhases * kUnit * token_stride(MT) * 4), stage = wb == 4 ? Stage<4>::kBytes : Stage<2>::kBytes;
-  q.steps_max = ((k_slabs_max + CS - 1) / CS + 1) / 2;
-  if ((long long)q.steps_max * 2048 * MT > kSmemMax) return false;
-  const int off = al((int)plane_offset(4, plane_bytes(q.steps_max, MT)));
-  // X_q for the projection and the partial sums of T share their room with the sums of the tiles
-  q.off_red = off;
-  q.red_bytes = red;
-  q.off_xq = off;
-  q.off_xe = q.off_xq + al(8 * MT * (q.steps_max * 128 + 16));
-  q.off_tpart = q.off_xe + al(8 * MT * q.steps_max * 8);
-  const int t_width = std::max(8 * kWorkerWarps, 16 * r_blocks_max);
-  q.off_trecv = q.off_tpart + 64 * MT * t_width;
-  q.off_tq = r_blocks_max > 0 ? std::max(off + kRed * red, q.off_trecv + 64 * MT * 16 * r_blocks_max) : off + kRed * red;
-  q.off_ring = q.off_tq + 2048 * MT;
-  if (kSmemMax - q.off_ring < kPhases * stage) return false;
-  int stages_max = 0;
-  for (int i = 0; i < n; ++i) stages_max = std::max(stages_max, (int)metas[i].n_tiles * q.steps_max);
-  q.slots = std::min(std::min((kSmemMax - q.off_ring) / stage, kMaxSlots), stages_max);
-  q.smem = (size_t)q.off_ring + (size_t)q.slots * stage;
-  q.resident = std::min(entry_of(wb, MT, false).resident(CS), entry_of(wb, MT, true).resident(CS));
-  if (q.resident < n) return false;
-  // each layer has a cluster, the others go one by one where the time is longest, as long as every cluster keeps a tile
-  auto steps = [&](int i) { return ((metas[i].k_slabs + CS - 1) / CS + 1) / 2; };
-  q.total = n;
-  for (int i = 0; i < n; ++i) q.clusters[i] = 1;
-  while (q.total < q.resident) {
-    int best = -1;
-    double longest = 0.0;
-    for (int i = 0; i < n; ++i) {
-      const double len = (double)metas[i].n_tiles / q.clusters[i] * steps(i);
-      if (q.clusters[i] < metas[i].n_tiles && len > longest) { longest = len; best = i; }
-    }
-    if (best < 0) break;
-    ++q.clusters[best];
-    ++q.total;
-  }
-  // In the time of a stage: the stages, what a tile costs beyond them (many CTAs hand over more sums in less time), the rounds in which
-  // X is quantised, and what T costs the clusters that form it, which get fewer tiles for that.  Fitted to calls of 3, 8, 9 and 16 rows with clusters of 2, 4 and 8; us for the four groups of a 4096 / 11008 and of a
-  // 5120 / 13824 layer (qkv, o, gate and up, down), 3 rows: 17.9 10.8 25.3 28.8 with 2, 15.1 10.2 25.9 14.4 with 4, 18.4 11.1 31.3 18.4 with 8;
-  // 21.6 13.1 31.6 37.6, 21.7 12.2 35.4 28.5, 25.7 12.0 41.3 22.6; 16 rows: 26.3 19.5 34.1 -, 23.7 13.6 31.8 25.6, 28.8 15.5 47.4 24.8;
-  // 33.3 25.6 45.3 -, 28.7 18.6 43.1 46.1, 36.1 17.2 57.6 31.1.
-  const double tile_cost = CS == 8 ? (MT == 1 ? 2.0 : 3.5) : CS == 4 ? (MT == 1 ? 0.7 : 1.2) : (MT == 1 ? 0.3 : 0.6);
-  const int most = std::max(q.resident / 4 / n, 1);  // clusters that form a layer's T: a quarter of the places, whatever the rank
-  auto share = [&](int i) { return (metas[i].n_tiles + q.clusters[i] - 1) / q.clusters[i]; };
-  // few stages: T's way through global memory would take longer than they do
-  q.local = r_blocks_max > 0 && r_blocks_max <= 8;
-  for (int i = 0; i < n; ++i)
-    q.local = q.local && steps(i) * 8 * 2 * metas[i].r_blocks * MT <= kLocalBlocks * kWorkerWarps && share(i) * steps(i) <= kLocalStages;
-  q.cost = 0.0;
-  for (int i = 0; i < n; ++i) {
-    const int tiles = metas[i].n_tiles, formers = q.local ? 1 : std::min(q.clusters[i], most);
-    q.t_blocks[i] = (metas[i].r_blocks + formers - 1) / formers;
-    int f = !q.local && q.t_blocks[i] > 0 ? (metas[i].r_blocks + q.t_blocks[i] - 1) / q.t_blocks[i] : 0, tf = 0;
-    const double per_tile = steps(i) + tile_cost;
-    const double t_cost = metas[i].r_blocks > 0 ? 2.0 + 0.15 * MT * steps(i) * 16 * q.t_blocks[i] / kWorkerWarps : 0.0;
-    if (f > 0 && f < q.clusters[i]) {
-      // equal times: f * tf + (clusters - f) * (tf + t_cost / per_tile) = tiles
-      const double level = (tiles - (q.clusters[i] - f) * t_cost / per_tile) / q.clusters[i];
-      tf = std::max(1, (int)(level + 0.5));
-      if (tiles - f * tf < q.clusters[i] - f) tf = 0;
-    }
-    if (tf == 0) f = 0;                              // equal shares for all
-    q.t_clusters[i] = f;
-    q.t_tiles[i] = tf;
-    const int longest = (tiles - f * tf + q.clusters[i] - f - 1) / (q.clusters[i] - f);
-    q.cost = std::max(q.cost, std::max(longest * per_tile + (f > 0 ? 0.0 : t_cost), f > 0 ? tf * per_tile + t_cost : 0.0) +
-                                  (MT == 1 ? 3.0 : 3.5) * ((M * steps(i) * 8 + kWorkers - 1) / kWorkers));
-  }
-  return true;
-}
-static bool make_plan(const PackedMeta* metas, int n, int M, Plan& best) {
-  int k_slabs_min = metas[0].k_slabs;
-  for (int i = 1; i < n; ++i) k_slabs_min = std::min(k_slabs_min, (int)metas[i].k_slabs);
-  bool found = false;
-  for (int CS = 8; CS >= 1; CS >>= 1) {
-    if (CS > 1 && k_slabs_min < 2 * CS) continue;                    // at least one step of two slabs to a CTA
-    Plan q;
-    if (!plan_with(metas, n, M, CS, q)) continue;
-    if (!found || q.cost < best.cost) { best = q; found = true; }
-  }
-  return found;
-}
-// The plans of the last few shapes a thread has asked for (a call asks twice, and working one out takes about a microsecond).
 static bool plan(const PackedMeta* metas, int n, int M, Plan& q) {
-  struct Shape {
-    int dev, n, M, w_bits, k_slabs[kMaxLayers], N[kMaxLayers], k_pad[kMaxLayers];
-  };
-  struct Known {
-    Shape shape;
-    Plan plan;
-    bool found;
-  };
-  static thread_local Known known[8] = {};
-  static thread_local unsigned next = 0;
+  static thread_local PlanCache cache;
   Shape sh = {};
   if (cudaGetDevice(&sh.dev) != cudaSuccess) return false;
   sh.n = n; sh.M = M; sh.w_bits = metas[0].w_bits;
-  for (int i = 0; i < n; ++i) { sh.k_slabs[i] = metas[i].k_slabs; sh.N[i] = metas[i].N; sh.k_pad[i] = metas[i].k_pad; }
-  for (const Known& k : known)
-    if (std::memcmp(&k.shape, &sh, sizeof(sh)) == 0) { q = k.plan; return k.found; }
-  const bool found = make_plan(metas, n, M, q);
-  Known& k = known[next++ % 8];
-  k.shape = sh; k.plan = q; k.found = found;
-  return found;
+  for (int i = 0; i < n; ++i) { sh.k_slabs[i] = metas[i].k_slabs; sh.tiles[i] = metas[i].n_tiles; sh.r_blocks[i] = metas[i].r_blocks; }
+  const int mt = M > 8 ? 2 : 1;
+  return cache.find(sh, [&](int CS) { return std::min(entry_of(sh.w_bits, mt, false).resident(CS), entry_of(sh.w_bits, mt, true).resident(CS)); }, q);
 }
 }  // namespace dcl
 
