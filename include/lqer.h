@@ -328,7 +328,8 @@ lqer_status_t lqer_debug_bounds_shrink(long long bytes);
 
 /* Test hook of the checked build (host, process wide): in the launches of the tensor-memory small-batch GEMM that follow, a
  * group of warps that has nothing to convert in a batch of weights looks at that batch `cycles` SM clock cycles late (0 ..
- * 1e7; 0 restores), so that a wait that relied on its being in time would run out; and in launches of the cluster kernel (3 to 16
+ * 1e7; 0 restores), so that a wait that relied on its being in time would run out, and a tile's first K chunk is counted in four times as
+ * late, so that the CTAs that share in its sums give their shares up; and in launches of the cluster kernel (3 to 16
  * rows) every fifth stage of weights from the ring's second round on is copied that long after as many of its successors as the ring has
  * room for, so that a consumer that took a former stage for its own would show, and T is never reported complete, so that whoever
  * waits for it has to form it.  The ordinary build returns LQER_ERR_CONFIG. */

@@ -66,7 +66,7 @@ struct Params {
   int off_red, red_bytes, off_xq, off_xe, off_tpart, off_trecv, off_tq, off_ring;   // offsets in shared memory (the planes of X_q come first)
   long long wait_limit;
   long long lag;                            // checked build, test hook: see lqer_debug_converter_lag
-  int stall;                                // test hook: the sums of the first tile wait for bytes that never come (see also t_expect)
+  int stall;                                // test hook: the sums of the first tile and a cluster's own T_q wait for bytes that never come (see also t_expect)
 };
 
 __device__ __forceinline__ uint32_t cta_rank() {
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_cluster_kernel(const __gri
       tc::fence_barrier_init();
       tc::fence_proxy_async_smem();
       if (NT > 0 && own_rows > 0) tc::mbar_expect_tx(t_full, (uint32_t)(own_rows * t_cols * 8 * CS));
-      if (LOCAL) tc::mbar_expect_tx(t_ready, (uint32_t)(M * k_pad * 2));
+      if (LOCAL) tc::mbar_expect_tx(t_ready, (uint32_t)(M * k_pad * 2) + (p.stall ? 16u : 0u));
       for (int i = 0; i < min(chunks, kRed); ++i) tc::mbar_expect_tx(red_full(i), chunk_bytes + (p.stall && i == 0 ? 16u : 0u));
     }
     __syncwarp();

@@ -98,6 +98,11 @@ constexpr int kTaken = 1 << 8, kLeft = 1 << 20, kGaveUp = (int)0x80000000u;
 __device__ __forceinline__ int arrived(int v) { return v & 0xFF; }
 __device__ __forceinline__ int taken(int v) { return (v >> 8) & 0xFFF; }
 __device__ __forceinline__ int left(int v) { return (v >> 20) & 0x7FF; }
+__device__ __forceinline__ int ld_acquire(const int* p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
 // Rows [lo, hi) of a tile from its chunks' partial sums, by `nthreads` threads (a multiple of 64): four columns to a thread.
 __device__ __forceinline__ void finish_rows(const Params& p, const Layer& ly, const Item& c, int lo, int hi, int tid, int nthreads) {
   const int col0 = c.tile * BN, c4 = (tid & 63) * 4, step = nthreads >> 6;
@@ -131,7 +136,7 @@ __device__ __forceinline__ void finish_rows(const Params& p, const Layer& ly, co
 // same time is the same).  So none depends on another's progress.  The last one to leave puts the counter back to zero.
 // With the CTA of the last chunk alone, the sums of 64 rows and 7 chunks took 9 us, 4 now; 4096 x 4096, 20 / 64 / 128 tokens, the call
 // 22.3 / 29.2 / 40.8 us alone and 20.1 / 25 / 29.5 shared, 11008 x 4096 30.5 / 39.1 / 57.9 and 27.9 / 34 / 44.4.
-constexpr int kFinishWait = 40000;             // cycles
+constexpr int kFinishWait = 40000;             // cycles (not the launch's wait limit: giving up is no error)
 // old: the counter before this CTA's chunk arrived.
 template <bool WHOLE_CTA, bool RUN>
 __device__ __forceinline__ void finish_tile(const Params& p, const Item& c, int old, int tid, int* flag) {
@@ -145,9 +150,13 @@ __device__ __forceinline__ void finish_tile(const Params& p, const Item& c, int 
     bool ok = true;
     if (WHOLE_CTA && !last && share < shares) {  // (an epilogue comes here with the last chunk only)
       if (tid == 0) {
-        int v = *reinterpret_cast<volatile int*>(count);
-        for (const long long t0 = clock64(); arrived(v) != ly.chunks && clock64() - t0 < kFinishWait;) v = *reinterpret_cast<volatile int*>(count);
-        *flag = arrived(v) == ly.chunks || arrived(atomicOr(count, kGaveUp)) == ly.chunks ? 1 : 0;
+        int v = ld_acquire(count);
+        for (const long long t0 = clock64(); arrived(v) != ly.chunks && clock64() - t0 < kFinishWait;) v = ld_acquire(count);
+        if (arrived(v) != ly.chunks) {
+          v = atomicOr(count, kGaveUp);
+          __threadfence();
+        }
+        *flag = arrived(v) == ly.chunks ? 1 : 0;
       }
       __syncthreads();
       ok = *flag != 0;
@@ -468,6 +477,8 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
         if (RUN && it.chunk + 1 < ly.chunks) continue;       // (the tile's other chunks are this CTA's too)
         __threadfence();
         epilogue_barrier();
+        if (kDebugBounds && p.lag > 0 && it.chunk == 0)  // test hook: a tile's first chunk is counted in long after the others
+          for (const long long t0 = clock64(); clock64() - t0 < 4 * p.lag;) { }
         if (next_item<RUN>(p, i, num_ctas) >= num_items) {
           if (et == 0) {
             at_end[0] = i;

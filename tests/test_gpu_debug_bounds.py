@@ -30,6 +30,7 @@ def test_small_parity_cases_pass_under_the_checked_build():
               "tests/test_gpu_parity.py", "tests/test_gpu_bf16_io.py", "tests/test_gpu_mxint8_io.py", "tests/test_gpu_w2.py",
               "tests/test_gpu_small_mma.py", "tests/test_gpu_small_batches.py", "tests/test_gpu_digit_prologue.py",
               "tests/test_gpu_decode_cluster.py", "tests/test_gpu_pair_tiles.py", "tests/test_gpu_batched_mixed_rows.py",
+              "tests/test_gpu_cluster_stages.py", "tests/test_gpu_small_sums.py",
               "-k", "not full and not stack and not sweep and not round"])
     assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
     assert " passed" in r.stdout
@@ -104,6 +105,42 @@ def test_converter_warps_that_come_late_to_a_batch_lose_nothing():
     """)
     r = _run(["-c", code])
     assert r.returncode == 0 and "late-converters-ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
+
+
+def test_shares_of_a_tile_that_are_given_up_are_summed_by_the_last_chunk():
+    # a tile's first chunk is counted in 400000 cycles after the others, ten times what these wait for it before they give their shares of the rows up:
+    # its CTA sums all rows.  Four shares and more, also where CTAs have several chunks; the counters are zero afterwards.
+    code = textwrap.dedent("""
+        import torch
+        import paper_2402_02446_b200 as L
+        dev = "cuda:0"
+        g = torch.Generator(device=dev); g.manual_seed(10)
+        draw = lambda *s: torch.randn(s, generator=g, device=dev)
+        for K, N, n in ((11008, 264, 1), (4096, 4096, 1), (8192, 2424, 15)):
+            Pg = L.prepare_weights(draw(K, N) * 0.02, draw(K, 40) / K ** 0.5, draw(40, N) * 0.01)
+            for M, dtype in ((17, torch.float32), (49, torch.bfloat16), (128, torch.float32)):
+                X = draw(M, K)
+                Ys = [torch.full((M, N), float("nan"), dtype=dtype, device=dev) for _ in range(n)]
+                calls = L.make_calls([(X, Pg, y) for y in Ys], torch.float32, dtype)
+                ws = torch.zeros(L.batched_workspace_bytes(calls), dtype=torch.uint8, device=dev)
+                L.linear_batched_ex(calls, ws, torch.float32, dtype)
+                assert L.poll_status(ws) == 0
+                want = [y.clone() for y in Ys]
+                ws[168192:] = 0xFF
+                L.debug_converter_lag(100_000)
+                try:
+                    L.linear_batched_ex(calls, ws, torch.float32, dtype)
+                    assert L.poll_status(ws) == 0, (K, M)
+                finally:
+                    L.debug_converter_lag(0)
+                assert all(torch.equal(y, w) for y, w in zip(Ys, want)), (K, M)
+                L.linear_batched_ex(calls, ws, torch.float32, dtype)
+                assert L.poll_status(ws) == 0 and all(torch.equal(y, w) for y, w in zip(Ys, want)), (K, M)
+            Pg.release()
+        print("given-up-ok")
+    """)
+    r = _run(["-c", code])
+    assert r.returncode == 0 and "given-up-ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
 
 
 def test_weight_stages_that_land_late_lose_nothing():

@@ -42,6 +42,7 @@ CASES = [
     ("small_gemm_ring", FAM_DECODE, binding.PATH_SMALL_TMEM, 9, 1024, 640, 40),
     ("decode_cluster_T_exchange", FAM_DECODE, binding.PATH_AUTO, 5, 1040, 20008, 40),   # T_q of other clusters, counters left behind
     ("decode_cluster_sums", FAM_DECODE, binding.PATH_AUTO, 5, 1040, 20008, 0),          # no rank: the first of several rounds
+    ("decode_cluster_own_T", FAM_DECODE, binding.PATH_AUTO, 5, 256, 256, 8),            # a cluster that forms all of T itself
     ("small_mma_flags", FAM_DECODE, binding.PATH_SMALL, 9, 1024, 640, 40),      # the polls of the prologue's flags
     ("prologue_tc_row_tile", FAM_PROLOGUE, binding.PATH_TENSOR_PROLOGUE, 300, 1024, 640, 32),
     ("digit_prologue_ring", FAM_PROLOGUE, binding.PATH_TENSOR_PROLOGUE, 300, 1040, 640, 136),   # several K ranges: one of them stalls
