@@ -706,12 +706,12 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
       const long rounds = (items + ctas - 1) / ctas, cost = rounds * (len + extra);
       if (best < 0 || cost < best) { best = cost; group_chunks = c; best_rounds = rounds; best_len = len; }
     }
-    // Several rounds of chunks though each tile could have an SM to itself: above 32 rows the rounds cost 2 M / 3 slabs' time (0.4 us) each beside
+    // Several rounds of chunks though each tile could have an SM to itself: the rounds cost 2 M / 3 slabs' time (0.4 us) each, 16 at least, beside
     // their slabs (partial sums of every chunk, and of all CTAs at a time), a CTA that takes a tile's chunks one after the other 4 + M / 8
-    // and 3 + M / 17 for each chunk's partial sums.  Two layers of 4096 x 11008, us, apart / one after the other: 32 rows 46.8 / 46.0,
-    // 64 rows 64.3 / 51.9, 128 rows 103 / 70.5.  (The sums are the same, bit for bit.)
-    if (!use_mma && M > 32 && alike && group_chunks > 1 && best_rounds > 1 && tiles <= ctas &&
-        slabs + 4 + M / 8 + group_chunks * (3 + M / 17) < best_rounds * (best_len + 2 * M / 3))
+    // and 3 + M / 17 for each chunk's partial sums.  us, apart / one after the other: two layers of 4096 x 11008, 20 rows 41.1 / 45.3, 32 rows
+    // 46.8 / 45.2, 64 rows 64.3 / 50.6, 128 rows 103 / 70.0; of 2048 x 11008, 32 rows 40.2 / 32.8.  (The sums are the same, bit for bit.)
+    if (!use_mma && alike && group_chunks > 1 && best_rounds > 1 && tiles <= ctas &&
+        slabs + 4 + M / 8 + group_chunks * (3 + M / 17) < best_rounds * (best_len + std::max(16, 2 * M / 3)))
       p.run = 0;                                             // all of a tile's chunks: see below
   }
   for (int i = 0; i < MAX_LAYERS; ++i) {
@@ -768,7 +768,7 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
   p.stall = take_stall(kFamDecode) ? 1 : 0;
   if (use_mma) return launch_gemm_mma(p, s);
   const int ctas = std::min(p.num_items / p.run, sms);
-  if (p.run > 1) return M <= 64 ? launch_nt<64, true>(tmaps, p, ctas, s) : launch_nt<128, true>(tmaps, p, ctas, s);
+  if (p.run > 1) return M <= 32 ? launch_nt<32, true>(tmaps, p, ctas, s) : M <= 64 ? launch_nt<64, true>(tmaps, p, ctas, s) : launch_nt<128, true>(tmaps, p, ctas, s);
   return M <= 32 ? launch_nt<32, false>(tmaps, p, ctas, s) : M <= 64 ? launch_nt<64, false>(tmaps, p, ctas, s) : launch_nt<128, false>(tmaps, p, ctas, s);
 }
 

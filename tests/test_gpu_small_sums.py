@@ -80,10 +80,10 @@ def _oracle(W, A, B, cols):
     return olqer.prepare_weights(h(W[:, cols]), h(A), h(B[:, cols]))         # (columns are independent)
 
 
-# two layers of 76 tiles (the last with one half) and three chunks: 228 items where 76 CTAs can take a tile each; 33 rows up
-@pytest.mark.parametrize("M", [33, 64, 65, 128])
-def test_ctas_with_all_chunks_of_a_tile(M):
-    K, N, k = 4096, 9592, 40
+# two layers of 76 tiles (the last with one half) and three chunks: 228 items where 76 CTAs can take a tile each
+@pytest.mark.parametrize("M,K", [(17, 2048), (32, 4096), (33, 4096), (64, 4096), (65, 4096), (128, 4096)])
+def test_ctas_with_all_chunks_of_a_tile(M, K):
+    N, k = 9592, 40
     g = torch.Generator(device=DEV)
     g.manual_seed(1700 + M)
     W, A, B, P = _groups(K, N, k, 2, g)
