@@ -17,7 +17,7 @@
 // the shapes of all of them (launch_gemm_small), so a result does not depend on the number of SMs, but its last bits may on the layers
 // beside it.  Each chunk is summed from zero in tensor memory and, if a tile has more than one, leaves its fp32 partial in scratch;
 // the CTAs whose last chunk is of one tile add its chunks up together, in chunk order, a share of the rows each (finish_tile), and
-// none depends on another's help; or one CTA takes all chunks of a tile, one after the other, and adds them up (RUN).
+// none depends on another's help; or a CTA takes several or all chunks of a tile, one after the other (RUN).
 // Roles per CTA:
 //   warp 0      producer: bulk copies of packed weight tiles (issued before the dependency wait: weights
 //               depend on no earlier kernel) and TMA loads of activation tiles (after it)
@@ -31,6 +31,7 @@
 // MMA warp some 450 cycles beside the MMAs themselves (waits, the commit, the loop): with a slab to a step that was more
 // than the eight MMAs of 32 cycles.
 #include <algorithm>
+#include <type_traits>
 
 #include "lqer_gemm_small.cuh"
 #include "lqer_tc_ptx.cuh"
@@ -138,14 +139,14 @@ __device__ __forceinline__ void finish_rows(const Params& p, const Layer& ly, co
 // 22.3 / 29.2 / 40.8 us alone and 20.1 / 25 / 29.5 shared, 11008 x 4096 30.5 / 39.1 / 57.9 and 27.9 / 34 / 44.4.
 constexpr int kFinishWait = 40000;             // cycles (not the launch's wait limit: giving up is no error)
 // old: the counter before this CTA's chunk arrived.
-template <bool WHOLE_CTA, bool RUN>
+template <bool WHOLE_CTA, int RUN>
 __device__ __forceinline__ void finish_tile(const Params& p, const Item& c, int old, int tid, int* flag) {
   const Layer& ly = p.L[c.layer];
   int lo = 0, hi = p.M;
-  if (!RUN) {                                  // (otherwise all of the chunks were this CTA's)
+  if (RUN != kAllChunks) {                     // (otherwise all of the chunks were this CTA's)
     int* count = ly.counters + c.tile;
     // shares of some 96 rows of partial sums; where that makes one of them, the CTA of the last chunk is through sooner than the first's
-    const int shares = min((p.M * ly.chunks + 95) / 96, ly.chunks), rows = (p.M + shares - 1) / shares, share = shares > 1 ? taken(old) : ly.chunks;
+    const int shares = min((p.M * ly.chunks + 95) / 96, RUN == kSomeChunks ? p.takers : ly.chunks), rows = (p.M + shares - 1) / shares, share = shares > 1 ? taken(old) : ly.chunks;
     const bool last = arrived(old) == ly.chunks - 1;
     bool ok = true;
     if (WHOLE_CTA && !last && share < shares) {  // (an epilogue comes here with the last chunk only)
@@ -168,7 +169,7 @@ __device__ __forceinline__ void finish_tile(const Params& p, const Item& c, int 
   __threadfence();
   finish_rows(p, ly, c, lo, hi, tid, WHOLE_CTA ? NUM_THREADS : 128);
 }
-template <bool RUN>
+template <int RUN>
 __device__ __noinline__ void finish_by_epilogue(const Params& p, const Item c, int old, int tid) { finish_tile<false, RUN>(p, c, old, tid, nullptr); }
 
 // bf16_rn by the conversion instruction, which has one NaN for all.
@@ -262,7 +263,7 @@ __device__ __forceinline__ int batch_end(int s, int s_hi, int k_slabs) {
 }
 constexpr int RANK_EXP_OFFSET = 8 * kTileN * 16;
 static_assert(RANK_EXP_OFFSET + 8 * kTileN <= W_HALF_BYTES, "two rank slabs");
-template <int NT, bool RUN>
+template <int NT, int RUN>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constant__ Params p) {
   using C = Cfg<NT>;
@@ -323,7 +324,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
         pdl_wait();
         waited = true;
         for (int i = first_item<RUN>(p, cta), q = 0; q < npend; i = next_item<RUN>(p, i, num_ctas)) {
-          const Item it = item_of(p, i);
+          const Item it = item_of<RUN>(p, i);
           const int k_slabs = p.L[it.layer].k_slabs;
           for (int s = it.s_lo; s < it.s_hi && q < npend; ++q) {
             const int e = batch_end(s, it.s_hi, k_slabs);
@@ -338,7 +339,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
       bool ok = true;
       const uint32_t w_tile = (uint32_t)w_tile_bytes(p.w_bits);
       for (int i = first_item<RUN>(p, cta); i < num_items && ok; i = next_item<RUN>(p, i, num_ctas)) {
-        const Item it = item_of(p, i);
+        const Item it = item_of<RUN>(p, i);
         const Layer& ly = p.L[it.layer];
         const int k_slabs = ly.k_slabs, r_blocks = ly.r_blocks, b_tile_stride = r_blocks * kTileN * 17;
         const int nt0 = 2 * it.tile;
@@ -391,7 +392,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     uint32_t cv = 0, cv_ph = 0, pk = 0, acc = 0, acc_ph = 1;
     bool first_pass = true, ok = true;
     for (int i = first_item<RUN>(p, cta); i < num_items && ok; i = next_item<RUN>(p, i, num_ctas)) {
-      const Item it = item_of(p, i);
+      const Item it = item_of<RUN>(p, i);
       const int k_slabs = p.L[it.layer].k_slabs, r_blocks = p.L[it.layer].r_blocks;
       ok = __all_sync(0xFFFFFFFFu, mbar_wait(acc_empty(acc), acc_ph, abort_flag)) != 0;
       if (!ok) break;
@@ -462,7 +463,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     bool ok = true;
     pdl_wait();                                    // Y, the scratch and the counters may be in use by the kernel before
     for (int i = first_item<RUN>(p, cta); i < num_items && ok; i = next_item<RUN>(p, i, num_ctas), ++tile_it) {
-      const Item it = item_of(p, i);
+      const Item it = item_of<RUN>(p, i);
       const Layer& ly = p.L[it.layer];
       const int acc = tile_it % C::ACCS;
       if (!mbar_wait<true>(acc_full(acc), (tile_it / C::ACCS) & 1, abort_flag)) { ok = false; break; }
@@ -474,7 +475,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
       if (ly.chunks > 1) {
         // count this chunk in; the CTA's last one is seen to by all of its threads at the end (every other role is about to fall
         // idle), another one by the epilogue where it is the tile's last to arrive
-        if (RUN && it.chunk + 1 < ly.chunks) continue;       // (the tile's other chunks are this CTA's too)
+        if (RUN == kAllChunks && it.chunk + 1 < ly.chunks) continue;       // (the tile's other chunks are this CTA's too)
         __threadfence();
         epilogue_barrier();
         if (kDebugBounds && p.lag > 0 && it.chunk == 0)  // test hook: a tile's first chunk is counted in long after the others
@@ -482,11 +483,11 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
         if (next_item<RUN>(p, i, num_ctas) >= num_items) {
           if (et == 0) {
             at_end[0] = i;
-            at_end[1] = RUN ? 0 : atomicAdd(ly.counters + it.tile, 1 + kTaken);
+            at_end[1] = RUN == kAllChunks ? 0 : atomicAdd(ly.counters + it.tile, 1 + kTaken);
           }
           break;
         }
-        if (RUN) { finish_by_epilogue<RUN>(p, it, 0, et); continue; }
+        if (RUN == kAllChunks) { finish_by_epilogue<RUN>(p, it, 0, et); continue; }
         if (et == 0) {
           const int old = atomicAdd(ly.counters + it.tile, 1);
           *last_flag = old;
@@ -510,7 +511,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
     bool ok = true;
     const int w_tile = w_tile_bytes(p.w_bits);
     for (int item = first_item<RUN>(p, cta); item < num_items && ok; item = next_item<RUN>(p, item, num_ctas)) {
-      const Item it = item_of(p, item);
+      const Item it = item_of<RUN>(p, item);
       const int k_slabs = p.L[it.layer].k_slabs, r_blocks = p.L[it.layer].r_blocks;
       const bool has_w = 2 * it.tile + half < p.L[it.layer].n_tiles;
       for (int s0 = it.s_lo; s0 < it.s_hi && ok; ++batch_no) {
@@ -602,7 +603,7 @@ gemm_small_kernel(const __grid_constant__ TensorMaps tmaps, const __grid_constan
 
   // ------------------------------------------------------------------ teardown
   __syncthreads();                      // every role is done (or has given up): the flags below are final for this CTA
-  if (at_end[0] >= 0 && abort_flag->abort == 0) finish_tile<true, RUN>(p, item_of(p, at_end[0]), at_end[1], threadIdx.x, last_flag);
+  if (at_end[0] >= 0 && abort_flag->abort == 0) finish_tile<true, RUN>(p, item_of<RUN>(p, at_end[0]), at_end[1], threadIdx.x, last_flag);
   if (abort_flag->abort != 0) {
     const long long t0 = clock64();
     while (clock64() - t0 < 400000) { }
@@ -632,7 +633,7 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-template <int NT, bool RUN>
+template <int NT, int RUN>
 static cudaError_t launch_nt(const TensorMaps& tmaps, const Params& p, int ctas, cudaStream_t s) {
   using C = Cfg<NT>;
   static OncePerDevice once;
@@ -677,23 +678,23 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
   const int sms = sm_count();
   if (sms < 1) return cudaErrorInvalidDevice;
   int group_chunks = 1;
-  p.run = 1;
+  p.run = p.takers = 1;
   if (n > 1) {
     // The cut that makes (rounds of items over the SMs) x (slabs per item + what an item costs beside its slabs) smallest,
     // a function of the shapes alone.  The register-operand kernel runs two CTAs per SM, an item each at a time, and an item costs
     // it about ten slabs' worth of time (activation copy, rank term, partial sums); this file's kernel one, and four.
     // The cut is also how long a chain of sums in tensor memory gets, and these cut off what does not fit: two layers of
     // 4096 x 11008 in one piece instead of three chunks a tile are 7 times as far from 64 bits (one sign, block exponents over a dozen
-    // binades: 1.9e-6 and 2.7e-7), although that was the faster way.  So the time model below, which knows more of what an item
-    // costs, does not choose the cut, only who takes a tile's chunks.
+    // binades: 1.9e-6 and 2.7e-7), although that was the faster way.  So what is known better of an item's costs, below, may
+    // make the chunks smaller, not larger.
     const int ctas = use_mma ? 2 * 148 : 148, extra = use_mma ? 10 : 4;
-    long best = -1, best_rounds = 0, best_len = 0, tiles = 0, slabs = 0;
-    bool alike = true;                                       // one number of chunks for all layers
+    long best = -1, best_rounds = 0, best_len = 0, tiles = 0;
+    const int slabs = layers[0].meta->k_slabs, most = small_gemm_chunks(*layers[0].meta);
+    bool alike = !use_mma;                                   // one K and one number of chunks for all layers
     for (int i = 0; i < n; ++i) {
       const PackedMeta& m = *layers[i].meta;
       tiles += small_gemm_col_tiles(m);
-      slabs = std::max(slabs, (long)m.k_slabs);
-      alike = alike && m.k_slabs == layers[0].meta->k_slabs && small_gemm_chunks(m) == small_gemm_chunks(*layers[0].meta);
+      alike = alike && m.k_slabs == slabs && small_gemm_chunks(m) == most;
     }
     for (int c = 1; c <= 16; ++c) {
       long items = 0, len = 0;
@@ -706,13 +707,24 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
       const long rounds = (items + ctas - 1) / ctas, cost = rounds * (len + extra);
       if (best < 0 || cost < best) { best = cost; group_chunks = c; best_rounds = rounds; best_len = len; }
     }
-    // Several rounds of chunks though each tile could have an SM to itself: the rounds cost 2 M / 3 slabs' time (0.4 us) each, 16 at least, beside
-    // their slabs (partial sums of every chunk, and of all CTAs at a time), a CTA that takes a tile's chunks one after the other 4 + M / 8
-    // and 3 + M / 17 for each chunk's partial sums.  us, apart / one after the other: two layers of 4096 x 11008, 20 rows 41.1 / 45.3, 32 rows
-    // 46.8 / 45.2, 64 rows 64.3 / 50.6, 128 rows 103 / 70.0; of 2048 x 11008, 32 rows 40.2 / 32.8.  (The sums are the same, bit for bit.)
-    if (!use_mma && alike && group_chunks > 1 && best_rounds > 1 && tiles <= ctas &&
-        slabs + 4 + M / 8 + group_chunks * (3 + M / 17) < best_rounds * (best_len + std::max(16, 2 * M / 3)))
-      p.run = 0;                                             // all of a tile's chunks: see below
+    // Several rounds of chunks though the tiles fit the SMs at once: then one or more CTAs may have a tile for themselves and take runs of its chunks.
+    // In slabs' time (0.4 us), a round costs 6 c - 16 + 4 M / 7 (c chunks a tile), 16 at least, beside its slabs: partial sums of every chunk, of
+    // all CTAs at a time; a run costs 3 + M / 17 for each chunk beside its slabs, and 4 + M / 8 at the end if all chunks are its own, 19 + M / 20
+    // if their sums meet in scratch.  us, in rounds / in runs of all, or of half of the chunks: two layers of 4096 x 11008, 3 chunks, 20 rows 41.1 /
+    // 45.3, 32 rows 46.8 / 45.2, 64 rows 64.3 / 50.6, 128 rows 103 / 70.0; of 2048 x 11008, 32 rows 40.2 / 32.8; three of 4352 x 4352, 5 chunks,
+    // 20 rows 40.2 / 36.9, 64 rows 77.8 / 44.5, 128 rows 137 / 65.7, and in 6 chunks 34.6, 41.9, 63.6.
+    if (alike && group_chunks > 1 && best_rounds > 1 && tiles <= ctas) {
+      long least = best_rounds * (best_len + std::max(16, 6 * group_chunks - 16 + 4 * M / 7));
+      for (int c = group_chunks; c <= most; ++c) {
+        const int stages = (slabs + c - 1) / c;
+        if ((slabs + stages - 1) / stages != c) continue;
+        for (int takers = 1; takers < c && takers * tiles <= ctas; ++takers) {
+          const int run = (c + takers - 1) / takers;
+          const long cost = run * (stages + 3 + M / 17) + (takers == 1 ? 4 + M / 8 : 19 + M / 20);
+          if ((takers - 1) * run < c && cost < least) { least = cost; group_chunks = c; p.run = run; p.takers = takers; }
+        }
+      }
+    }
   }
   for (int i = 0; i < MAX_LAYERS; ++i) {
     const SmallGemmLayer& src = layers[i < n ? i : 0];
@@ -749,10 +761,10 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
     ly.chunks = (m.k_slabs + ly.chunk_stages - 1) / ly.chunk_stages;
     ly.partial_extent = ly.chunks > 1 ? (size_t)small_gemm_col_tiles(m) * ly.chunks * M * 256 * 4 : 0;
     ly.item_begin = item_begin;
-    if (i < n) item_begin += small_gemm_col_tiles(m) * ly.chunks;
+    if (i < n) item_begin += small_gemm_col_tiles(m) * (p.run > 1 ? p.takers * p.run : ly.chunks);
   }
   p.n = n;
-  if (p.run == 0) p.run = p.L[0].chunks;
+  p.chunks = p.L[0].chunks;
   p.num_items = item_begin;
   p.status = st;
   p.M = M;
@@ -768,8 +780,12 @@ cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_
   p.stall = take_stall(kFamDecode) ? 1 : 0;
   if (use_mma) return launch_gemm_mma(p, s);
   const int ctas = std::min(p.num_items / p.run, sms);
-  if (p.run > 1) return M <= 32 ? launch_nt<32, true>(tmaps, p, ctas, s) : M <= 64 ? launch_nt<64, true>(tmaps, p, ctas, s) : launch_nt<128, true>(tmaps, p, ctas, s);
-  return M <= 32 ? launch_nt<32, false>(tmaps, p, ctas, s) : M <= 64 ? launch_nt<64, false>(tmaps, p, ctas, s) : launch_nt<128, false>(tmaps, p, ctas, s);
+  const auto go = [&](auto run) {
+    constexpr int RUN = decltype(run)::value;
+    return M <= 32 ? launch_nt<32, RUN>(tmaps, p, ctas, s) : M <= 64 ? launch_nt<64, RUN>(tmaps, p, ctas, s) : launch_nt<128, RUN>(tmaps, p, ctas, s);
+  };
+  if (p.run == 1) return go(std::integral_constant<int, kNoRuns>());
+  return p.takers == 1 ? go(std::integral_constant<int, kAllChunks>()) : go(std::integral_constant<int, kSomeChunks>());
 }
 
 }  // namespace lqer

@@ -31,7 +31,9 @@ struct Params {
   Layer L[MAX_LAYERS];
   int n;                       // layers in this launch
   int num_items;
-  int run;                     // neighbouring items that one CTA takes, one after the other: 1, or all chunks of a tile (RUN kernels)
+  // Runs of chunks (RUN below): a CTA takes `run` chunks of a tile, one after the other, or what is left of them; `takers` CTAs to a tile, `chunks` in
+  // every layer.  (A tile has takers * run places in the list of items, the last of them possibly empty.)
+  int run, takers, chunks;
   DeviceStatus* status;
   int M;
   int lr_shift;
@@ -49,29 +51,32 @@ struct Params {
 struct Item {
   int layer, tile, chunk, s_lo, s_hi;      // tile: index of the 256-column tile
 };
+enum { kNoRuns = 0, kAllChunks, kSomeChunks };   // RUN: a CTA's item is a chunk, all chunks of a tile, or `run` of them
+template <int RUN = kNoRuns>
 __device__ __forceinline__ Item item_of(const Params& p, int i) {
   int l = 0;
 #pragma unroll
   for (int q = 1; q < MAX_LAYERS; ++q)
     if (q < p.n && i >= p.L[q].item_begin) l = q;
   const Layer& ly = p.L[l];
-  const int local = i - ly.item_begin;
+  const int local = i - ly.item_begin, places = RUN == kSomeChunks ? p.takers * p.run : ly.chunks;
   Item it;
   it.layer = l;
-  it.tile = local / ly.chunks;
-  it.chunk = local - it.tile * ly.chunks;
+  it.tile = local / places;
+  it.chunk = local - it.tile * places;
   it.s_lo = it.chunk * ly.chunk_stages;
   it.s_hi = it.chunk == ly.chunks - 1 ? ly.spt : it.s_lo + ly.chunk_stages;
   return it;
 }
 
 // The items that a CTA takes: its first, and the one after item i.
-template <bool RUN>
+template <int RUN>
 __device__ __forceinline__ int first_item(const Params& p, int cta) { return RUN ? cta * p.run : cta; }
-template <bool RUN>
+template <int RUN>
 __device__ __forceinline__ int next_item(const Params& p, int i, int num_ctas) {
-  if (!RUN) return i + num_ctas;
-  return (i + 1) % p.run != 0 ? i + 1 : i + 1 + (num_ctas - 1) * p.run;
+  if (RUN == kNoRuns) return i + num_ctas;
+  const int n = i + 1;
+  return n % p.run != 0 && (RUN == kAllChunks || n % (p.takers * p.run) < p.chunks) ? n : (i / p.run + num_ctas) * p.run;
 }
 
 __device__ __forceinline__ uint32_t bf16_rn(float v) {

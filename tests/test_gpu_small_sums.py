@@ -80,18 +80,19 @@ def _oracle(W, A, B, cols):
     return olqer.prepare_weights(h(W[:, cols]), h(A), h(B[:, cols]))         # (columns are independent)
 
 
-# two layers of 76 tiles (the last with one half) and three chunks: 228 items where 76 CTAs can take a tile each
-@pytest.mark.parametrize("M,K", [(17, 2048), (32, 4096), (33, 4096), (64, 4096), (65, 4096), (128, 4096)])
-def test_ctas_with_all_chunks_of_a_tile(M, K):
-    N, k = 9592, 40
+# Two layers of 76 tiles (the last with one half) and three chunks: 228 items where 76 CTAs can take a tile each.  Two of 52 tiles and five chunks: two
+# CTAs take three and two chunks of each.  Three of 51 tiles: five chunks would do, two CTAs take three of six each.
+@pytest.mark.parametrize("M,K,N,n", [(17, 2048, 9592, 2), (32, 4096, 9592, 2), (33, 4096, 9592, 2), (64, 4096, 9592, 2), (65, 4096, 9592, 2), (128, 4096, 9592, 2),
+                                     (17, 4096, 6408, 2), (64, 4096, 6408, 2), (128, 4096, 6408, 2), (20, 4352, 4232, 3), (128, 4352, 4232, 3)])
+def test_ctas_with_runs_of_a_tiles_chunks(M, K, N, n):
+    k = 40
     g = torch.Generator(device=DEV)
     g.manual_seed(1700 + M)
-    W, A, B, P = _groups(K, N, k, 2, g)
+    W, A, B, P = _groups(K, N, k, n, g)
     X = torch.randn((M, K), generator=g, device=DEV)
     cols = torch.cat([torch.arange(0, 64), torch.arange(N - 136, N)]).to(DEV)
     lone = [L.linear(X, p, L.new_workspace(M, p)) for p in P]
-    for y, w, a, b in zip(lone, W, A, B):
-        assert worst_ratio(y[:, cols].cpu().numpy(), olqer.forward(X.cpu().numpy(), _oracle(w, a, b, cols))) <= 1.0
+    oracle = [_oracle(w, a, b, cols) for w, a, b in zip(W, A, B)]
     for dtype in (torch.float32, torch.bfloat16):
         Ys = [torch.full((M, N), float("nan"), device=DEV, dtype=dtype) for _ in P]
         calls = L.make_calls([(X, p, y) for p, y in zip(P, Ys)], torch.float32, dtype)
@@ -101,8 +102,13 @@ def test_ctas_with_all_chunks_of_a_tile(M, K):
             before = L.launch_count()
             L.linear_batched_ex(calls, ws, torch.float32, dtype)
             assert L.poll_status(ws) == 0 and L.launch_count() - before == 2
-            # the layer alone has the same cut, one CTA to a chunk
-            assert all(torch.equal(y, z.to(dtype)) for y, z in zip(Ys, lone))
+            if dtype == torch.float32:
+                for y, o in zip(Ys, oracle):
+                    assert worst_ratio(y[:, cols].cpu().numpy(), olqer.forward(X.cpu().numpy(), o)) <= 1.0
+                whole = [y.clone() for y in Ys]
+                if n == 2:                              # the layer alone has the same cut, one CTA to a chunk
+                    assert all(torch.equal(y, z) for y, z in zip(Ys, lone))
+            assert all(torch.equal(y, z.to(dtype)) for y, z in zip(Ys, whole))
     for p in P:
         p.release()
 
