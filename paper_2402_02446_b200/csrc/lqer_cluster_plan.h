@@ -86,7 +86,8 @@ inline bool plan_with(const Shape& sh, int CS, int resident, Plan& q) {
     q.clusters[i] = clusters;
     length[i] = clusters < sh.tiles[i] ? (double)sh.tiles[i] / clusters * steps[i] : 0.0;
   };
-  // (to begin with, nearly what each one's part of the work comes to: one by one no layer gets more than that and one, so none gets less than n - 1 below it)
+  // (to begin with, nearly what each one's part of the work comes to: one by one no layer gets more than that and one, so none gets
+  // less than n - 1 below it)
   double work = 0.0;
   for (int i = 0; i < n; ++i) work += (double)sh.tiles[i] * steps[i];
   q.total = 0;
@@ -103,10 +104,11 @@ inline bool plan_with(const Shape& sh, int CS, int resident, Plan& q) {
     ++q.total;
   }
   // In the time of a stage: the stages, what a tile costs beyond them (many CTAs hand over more sums in less time), the rounds in which
-  // X is quantised, and what T costs the clusters that form it, which get fewer tiles for that.  Fitted to calls of 3, 8, 9 and
-  // 16 rows with clusters of 2, 4 and 8; us for the four groups of a 4096 / 11008 and of a 5120 / 13824 layer (qkv, o, gate and up, down), 3 rows: 17.9 10.8 25.3 28.8 with 2, 15.1 10.2 25.9 14.4 with 4, 18.4 11.1 31.3 18.4 with 8;
-  // 21.6 13.1 31.6 37.6, 21.7 12.2 35.4 28.5, 25.7 12.0 41.3 22.6; 16 rows: 26.3 19.5 34.1 -, 23.7 13.6 31.8 25.6, 28.8 15.5 47.4 24.8;
-  // 33.3 25.6 45.3 -, 28.7 18.6 43.1 46.1, 36.1 17.2 57.6 31.1.
+  // X is quantised, and what T costs the clusters that form it, which get fewer tiles for that.  Fitted to calls of 3, 8, 9 and 16 rows with
+  // clusters of 2, 4 and 8.  us for the groups (qkv, o, gate and up, down) of a 4096 / 11008 and of a 5120 / 13824 layer, 2 | 4 | 8:
+  //    3 rows: 18.0 10.9 25.5 28.2 | 15.0 10.6 26.0 13.9 | 17.8 10.7 30.5 18.6;  21.9 12.9 31.6 36.0 | 21.9 12.5 35.8 28.2 | 24.7 11.9 41.4 22.6
+  //   16 rows: 23.5 17.4 31.6 -    | 20.5 13.3 30.7 22.2 | 27.5 14.6 45.9 23.2;  29.4 21.7 41.7 -    | 27.5 16.9 42.4 39.3 | 34.7 16.3 56.9 29.2
+  // (At hidden sizes of 1024 to 2048 the model is at times off: 1536 / 4096, rank 32, 16 rows, gate and up 13.9 with 4, 11.6 with 2.)
   const double tile_cost = CS == 8 ? (MT == 1 ? 2.0 : 3.5) : CS == 4 ? (MT == 1 ? 0.7 : 1.2) : (MT == 1 ? 0.3 : 0.6);
   const int most = std::max(q.resident / 4 / n, 1);  // clusters that form a layer's T: a quarter of the places, whatever the rank
   auto share = [&](int i) { return (sh.tiles[i] + q.clusters[i] - 1) / q.clusters[i]; };

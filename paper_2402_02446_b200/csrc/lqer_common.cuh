@@ -582,7 +582,7 @@ int gemm_small_max_layers();
 // would take the launch.
 cudaError_t launch_gemm_small(const SmallGemmLayer* layers, int n, int M, int y_type, bool tensor_memory_form, int epoch,
                               DeviceStatus* st, cudaStream_t s);
-// The kernels for few rows hold a lane's place in the packed W section in 32 bits; the GEMMs take larger sections.
+// The column-owner kernel holds a lane's place in the packed W section in 32 bits; the others take larger sections.
 inline bool w_offsets_fit(const PackedMeta& m) { return m.off_b - m.off_w <= 0xFFFFFFFFull; }
 // The layer for 3 to 16 rows in one launch (lqer_decode_cluster.cu), up to decode_cluster_max_layers() independent layers with one M
 // and one set of formats.  scratch: decode_cluster_scratch_bytes per layer; counts: two zeroed counters per layer, zero again

@@ -1,4 +1,4 @@
-// The layer for M <= 16 tokens in one launch (paper Section 3.1 / 3.2: Y = X_q W_q + q(X_q A_q) B_q; Section 2.1: few
+// The layer for 3 to 16 tokens in one launch (paper Section 3.1 / 3.2: Y = X_q W_q + q(X_q A_q) B_q; Section 2.1: few
 // tokens per step make it memory bound on its weights).
 //
 // A cluster of CS CTAs owns a range of weight tiles (128 columns); its CTAs share the contraction: CTA q takes the slabs
@@ -932,13 +932,15 @@ static bool plan(const PackedMeta* metas, int n, int M, Plan& q) {
 // Whether n layers with one M go out as one launch of this kernel: at 3 to 16 rows, up to four layers, wherever X_q fits.  Measured on one
 // B200, us a call in a chain of such calls over weights beyond L2, the same sums through two CTAs to an SM with a ring of each lane's own
 // pieces (before) / this kernel; for 16 rows the kernels that share a prologue, which took the larger of these calls / this kernel:
-//   4096 x 4096, rank 32 alone   4 rows 11.2 / 10.3   8 rows 11.4 / 10.5   16 rows 14.7 / 13.6
-//   three of them                4 rows 20.8 / 15.1   8 rows 21.3 / 15.6   16 rows 28.1 / 21.6
-//   two of 4096 x 11008          4 rows 30.3 / 25.3   8 rows 30.8 / 25.6   16 rows 33.1 / 31.6
-//   11008 x 4096 alone           4 rows 17.2 / 14.4   8 rows 18.4 / 15.4   16 rows 28.9 / 25.5
-//   two of 5120 x 13824, rank 64 4 rows 43.8 / 32.0   8 rows 44.5 / 33.0   16 rows 45.8 / 45.2
-//   the same, rank 256           3 rows 48.9 / 34.6   8 rows 53.2 / 36.3   16 rows 52.7 / 48.0
-//   2048 x 2048, rank 32 alone   4 rows 8.9 / 7.0;  rank 64, 16 rows 10.7 / 11.7 (the one size found where the smaller CTAs were faster)
+//   4096 x 4096, rank 32 alone   4 rows 11.2 / 10.5   8 rows 11.4 / 10.7   16 rows 14.7 / 13.1
+//   three of them                4 rows 20.8 / 15.3   8 rows 21.3 / 15.6   16 rows 28.1 / 20.7
+//   two of 4096 x 11008          4 rows 30.3 / 25.6   8 rows 30.8 / 26.1   16 rows 33.1 / 30.6
+//   11008 x 4096 alone           4 rows 17.2 / 13.9   8 rows 18.4 / 14.9   16 rows 28.9 / 22.4
+//   two of 5120 x 13824, rank 64 4 rows 43.8 / 31.7   8 rows 44.5 / 32.9   16 rows 45.8 / 41.7
+//   the same, rank 256           3 rows 48.9 / 34.4   8 rows 53.2 / 36.1   16 rows 52.7 / 46.9
+//   2048 x 2048, rank 32 alone   4 rows 8.9 / 7.2;  rank 64, 16 rows 10.7 / 10.6
+// and a whole layer of hidden 1024 to 2048 at 16 rows: 1024, rank 0 26.2 / 29.0, rank 32 42.3 / 42.8; 1984, rank 0 41.5 / 42.1; 2048, rank 64
+// 62.5 / 51.6.  (Short contractions of 9 and more rows without a rank are where the smaller CTAs were as fast or faster.)
 // One and two rows keep the column-owner kernel, whose launches several layers share bit for bit.
 int decode_cluster_max_layers() { return dcl::kMaxLayers; }
 bool decode_cluster_takes(const PackedMeta* metas, int n, int M) {

@@ -181,7 +181,8 @@ __device__ __forceinline__ uint16_t bf16_rn_cvt(uint32_t v) {
 // A finished chunk from its accumulator to Y or to the partial sums, by the epilogue's warps: warp q of them has a quarter of the
 // lanes; a lane holds a weight column, its columns are the tokens.  Each warp is alone on its scheduler by then and bound by its own
 // instructions, so bf16 is the conversion's (7 us for 64 tokens with bf16_rn, 4 now), and a partial sum's address is a constant away
-// from the one before.  (All 28 warps at the end took no less time.)
+// from the one before.  (All 28 warps at the end took no less time.  The kernel spills 64 - 76 bytes a thread, mostly around the call of
+// finish_by_epilogue; every further live value costs 1 - 2 us.)
 template <int NT>
 __device__ __forceinline__ void store_chunk(const Params& p, const Item& c, uint32_t tmem_base, int acc, int q) {
   const Layer& ly = p.L[c.layer];

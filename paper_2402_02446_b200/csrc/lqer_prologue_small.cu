@@ -76,7 +76,7 @@ __device__ __forceinline__ double ld_dsmem(const double* local, uint32_t cta) {
 // first blocks before it waits for the kernel before, on which they do not depend) and eight quads of X per thread.  With eight
 // warps of 128 registers and 16 blocks a round it took 14 - 21 us at 64 rows, K = 5120 - 13824 and rank 32 (5 - 9 of them to
 // quantise, 2 - 5 for the products); the layer's four calls with their GEMMs 172 us, 158 with sixteen (4096 / 11008: 140 and 128;
-// rank 256 210, with four quads of X a round 236).
+// rank 256 210, with four quads of X a round 236).  They spill for it: 196 bytes stored and 80 loaded by a thread, 340 and 184 with TPW == 2.
 template <int TPW>
 __global__ void __launch_bounds__(kThreads, 2) prologue_small_kernel(const __grid_constant__ Params p) {
   __shared__ __align__(16) uint8_t s_xq[kRows * kXqStride];

@@ -1,8 +1,8 @@
 """Batches of 3 to 16 rows in one launch: a cluster of CTAs per range of columns, the contraction shared by its CTAs.
 
-Sizes sit at the edges of what the kernel cuts: contractions that give a CTA one slab, half a step or a ragged last block,
-column ranges of less than a warp's octets, of several rounds with a nearly empty last one (owners to whom nothing comes), ranks
-of no, one, several and sixteen blocks, and both sides of the eight-token tile.
+Sizes sit at the edges of what the kernel cuts: contractions that give a CTA one slab, half a step or a ragged last block, fewer columns than
+a tile of 128, one and several tiles to a cluster with a nearly empty last one, ranks of no, one, several and sixteen blocks, and both
+sides of the eight-token tile.
 """
 import numpy as np
 import pytest
@@ -132,8 +132,8 @@ def test_groups_share_one_launch(M):
 
 
 def test_streams_with_a_workspace_each():
-    # four streams of calls whose T comes from several clusters (one block of ranks each, two, and a launch placed as a whole),
-    # beside a stream that keeps the SMs busy: nobody waits for good, and every result is the lone call's
+    # four streams of calls whose T comes from several clusters (one block of ranks each, two, four), beside a stream that keeps the SMs
+    # busy: nobody waits for good, and every result is the lone call's
     shapes = [(4096, 1032, 256), (4096, 1032, 64), (12288, 520, 256), (1040, 4104, 256)]
     layers = [_layer(*s, 905 + i) for i, s in enumerate(shapes)]
     rows = (3, 16, 8, 5)
@@ -162,8 +162,8 @@ def test_streams_with_a_workspace_each():
         l[2].release()
 
 
-def test_replays_of_a_launch_placed_as_a_whole():
-    # long K and a high rank: one CTA to an SM and more T clusters than a quarter of the places (a cooperative launch), captured
+def test_replays_of_a_launch_whose_t_comes_from_several_clusters():
+    # long K and a high rank: four clusters form T, which reaches the others through global memory and counters; captured
     spec, P, Pg = _layer(12288, 520, 256, 909)
     x, y, ws = torch.zeros((8, spec.K), device=DEV), torch.zeros((8, spec.N), device=DEV), L.new_workspace(8, Pg)
     L.linear(x, Pg, ws, y)
