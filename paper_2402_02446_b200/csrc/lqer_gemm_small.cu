@@ -146,7 +146,8 @@ __device__ __forceinline__ void finish_tile(const Params& p, const Item& c, int 
   if (RUN != kAllChunks) {                     // (otherwise all of the chunks were this CTA's)
     int* count = ly.counters + c.tile;
     // shares of some 96 rows of partial sums; where that makes one of them, the CTA of the last chunk is through sooner than the first's
-    const int shares = min((p.M * ly.chunks + 95) / 96, RUN == kSomeChunks ? p.takers : ly.chunks), rows = (p.M + shares - 1) / shares, share = shares > 1 ? taken(old) : ly.chunks;
+    const int shares = min((p.M * ly.chunks + 95) / 96, RUN == kSomeChunks ? p.takers : ly.chunks);
+    const int rows = (p.M + shares - 1) / shares, share = shares > 1 ? taken(old) : ly.chunks;
     const bool last = arrived(old) == ly.chunks - 1;
     bool ok = true;
     if (WHOLE_CTA && !last && share < shares) {  // (an epilogue comes here with the last chunk only)
